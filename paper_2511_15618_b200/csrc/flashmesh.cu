@@ -10,6 +10,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <new>
 #include <utility>
@@ -19,11 +20,12 @@
 #include "fm_common.cuh"
 #include "fm_gemm_tc.cuh"
 #include "fm_kernels.cuh"
+#include "fm_prefill.cuh"
 
 namespace {
 
 constexpr int STACK_LEVEL[5] = {0, 1, 2, 1, 0};
-constexpr int PREFILL_CHUNK = 256;      // conditioning rows projected per launch group
+constexpr int PREFILL_ROWS = 8192;      // coordinate rows of a prefill chunk, at most
 constexpr int FM_ROPE_SLACK = 64;       // the HF-Blocks of the face level query positions up to 4 faces ahead
 
 struct LayerDev {
@@ -91,10 +93,21 @@ struct fm_ctx {
   int ssq_n, ssq_ld;    // slots the last producer filled, floats between slots
   bool use_pdl;
   bool debug_sync;      // FM_DEBUG_SYNC: wait for and check every launch
-  // prefill temporaries
-  bf16* pre_a;
-  float* pre_o;
-  int* prompt_off_dev;
+  // prefill: activations of one chunk (see fm_prefill.cuh)
+  struct Prefill {
+    int rows[3];                         // row capacity per level
+    float *x[3], *ssq;
+    bf16 *a, *q, *kbuf, *vbuf, *attn, *wide;      // wide: FFN hidden, shorten operands, upsampled triples, prefix operands
+    size_t wide_bytes;
+    int prefix_rows;                     // conditioning rows projected per launch
+    pf::Row* map[3];
+    char* plan;                          // device copy of the host's plan
+    size_t plan_bytes;
+    pf::LayerPtr* layers;
+    int n_layers;
+  } pre;
+  std::vector<char> plan_host;
+  int* limits_dev;
   // generate
   GenOut* gen_dev;
   long long* stats_dev;
@@ -328,10 +341,37 @@ void carve(fm_ctx* c, Carver& cv) {
   for (int s = 0; s < 5; ++s) n_layers += c->cfg.layers[s];
   c->tmaps_cap = (size_t)6 * n_layers + 128;
   c->tmaps = cv.take<CUtensorMap>(c->tmaps_cap);
-  // prefill temporaries
-  c->pre_a = cv.take<bf16>((size_t)PREFILL_CHUNK * d);
-  c->pre_o = cv.take<float>((size_t)PREFILL_CHUNK * 2 * dm.Hkv * dm.dh);
-  c->prompt_off_dev = cv.take<int>(B + 1);
+  // prefill: one chunk of coordinate rows and its vertices and faces
+  {
+    auto& pr = c->pre;
+    const size_t all = B * (size_t)dm.max_tokens, R = align_up(all < (size_t)PREFILL_ROWS ? all + 16 : (size_t)PREFILL_ROWS, 128);
+    pr.rows[0] = (int)R;
+    pr.rows[1] = (int)align_up(R / 3 + B + 16, 128);
+    pr.rows[2] = (int)align_up(R / 9 + B + 16, 128);
+    for (int l = 0; l < 3; ++l) { pr.x[l] = cv.take<float>(pr.rows[l] * d); pr.map[l] = cv.take<pf::Row>(pr.rows[l]); }
+    pr.ssq = cv.take<float>((d + 127) / 128 * tc::MAX_SPLIT * R);
+    pr.a = cv.take<bf16>(R * 2 * d);
+    pr.q = cv.take<bf16>(R * hd);
+    pr.kbuf = cv.take<bf16>(R * dm.Hkv * dm.dh);
+    pr.vbuf = cv.take<bf16>(R * dm.Hkv * dm.dh);
+    pr.attn = cv.take<bf16>(R * 2 * hd);
+    pr.n_layers = n_layers;
+    const size_t per_prefix_row = (size_t)n_layers * d * sizeof(bf16);
+    size_t wide = R * 2 * dm.dff * sizeof(bf16);
+    const size_t cat = pr.rows[1] * 6 * d * sizeof(bf16), least = 256 * per_prefix_row;
+    wide = wide > cat ? wide : cat;                          // (the triples, 3d floats a row, take as much as the operands)
+    wide = dm.P > 0 && wide < least ? least : wide;
+    pr.wide = cv.take<bf16>(wide / sizeof(bf16));
+    pr.wide_bytes = wide;
+    const size_t fit = wide / per_prefix_row / 256 * 256, want = align_up(B * (size_t)dm.P, 256);
+    pr.prefix_rows = (int)(fit < want ? fit : want);
+    // prompt offsets, segments, query tiles of all chunks
+    const size_t chunks = all / (R - 16) + 2, segs = B + chunks;
+    pr.plan_bytes = (B + 2) * sizeof(int) + segs * sizeof(pf::Seg) + (all / 8 + 8 * segs + 64) * sizeof(int2) + 256;
+    pr.plan = cv.take<char>(pr.plan_bytes);
+    pr.layers = cv.take<pf::LayerPtr>(n_layers);
+    c->limits_dev = cv.take<int>(B);
+  }
   c->gen_dev = cv.take<GenOut>(1);
   c->stats_dev = cv.take<long long>(FM_MAX_DRAFT + 4);
   cv.off = align_up(cv.off, 256);
@@ -357,12 +397,20 @@ int upload_bf16(bf16* dst, const float* src, size_t n, std::vector<uint16_t>& tm
 // 128 rows (zeros), K cut into slabs of 64; slab (t, k) is stored as the 16 KB image the MMA reads
 // from shared memory (row r at r*128 bytes, its 16-byte chunk c at position c ^ (r & 7): the
 // 128-byte swizzle), slabs of one tile one after the other.
-int upload_packed(bf16* dst, const float* src, size_t M, size_t K, std::vector<uint16_t>& tmp) {
+// The first rot_rows rows are heads of rot_dh rows whose rotary pairs (i, i + dh/2) are stored side by
+// side, at (2i, 2i + 1): a thread that owns neighbouring outputs can rotate them.  Queries and keys
+// share the order, so their products do not change.
+int upload_packed(bf16* dst, const float* src, size_t M, size_t K, std::vector<uint16_t>& tmp, size_t rot_rows = 0, size_t rot_dh = 1) {
   if (src == nullptr) return FM_ERR_INVALID_ARG;
   const size_t tiles = (M + 127) / 128, slabs = K / 64;
   tmp.assign(tiles * 128 * K, 0);
   for (size_t m = 0; m < M; ++m) {
-    const size_t t = m / 128, r = m % 128;
+    size_t to = m;
+    if (m < rot_rows) {
+      const size_t i = m % rot_dh, half = rot_dh / 2;
+      to = m - i + (i < half ? 2 * i : 2 * (i - half) + 1);
+    }
+    const size_t t = to / 128, r = to % 128;
     for (size_t k = 0; k < K; ++k) {
       uint32_t u;
       memcpy(&u, src + m * K + k, 4);
@@ -394,7 +442,7 @@ int upload_f32(float* dst, const float* src, size_t n) {
     if ((ctx)->debug_sync) debug_sync_check(ctx, #kern);                 \
   } while (0)
 
-enum ProfClass { PROF_GEMM = 0, PROF_ATTN = 1, PROF_OTHER = 2 };
+enum ProfClass { PROF_GEMM = 0, PROF_ATTN = 1, PROF_OTHER = 2, PROF_NONE = 3 };
 
 // Diagnostic mode (environment FM_DEBUG_SYNC): wait for every launch and name the first one that
 // ends with an error; nothing is launched after it.  Not used while a graph is being captured.
@@ -495,7 +543,7 @@ int tmap_for(fm_ctx* c, const void* base, uint64_t rows, uint64_t cols, uint32_t
     if (k.base == base && k.rows == rows && k.cols == cols && k.box_rows == box_rows && k.parts == parts) return (int)i;
   }
   if (c->tmaps_host.size() >= c->tmaps_cap || c->capturing) return -1;   // descriptors are made before capture
-  const int idx = add_tmap_operand(c, base, rows, cols, parts, box_rows);
+  const int idx = parts == 0 ? add_tmap_bf16(c, base, rows, cols, box_rows) : add_tmap_operand(c, base, rows, cols, parts, box_rows);
   if (idx < 0) return -1;
   c->tmap_keys.push_back({base, rows, cols, box_rows, parts});
   cudaMemcpyAsync(c->tmaps + idx, &c->tmaps_host[idx], sizeof(CUtensorMap), cudaMemcpyHostToDevice, c->stream);
@@ -931,6 +979,267 @@ __global__ void set_limits_kernel(Dims dm, SeqState st, int batch, const int* __
   st.t_end[b] = want < cap ? (int)want : cap;
 }
 
+// ------------------------------------------------------------------------------------------
+// prefill
+// ------------------------------------------------------------------------------------------
+// One GEMM of the prefill.  Rows per tile: the choice that minimises waves x (slabs x the longer of a
+// slab's copy at 64 B per clock and its MMAs, + about 2000 clocks of start-up and epilogue).
+void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, pf::Epi e, int layers = 1, int w_tile0 = 0) {
+  if (R <= 0) return;
+  const int parts = mode == pf::PF_PREFIX ? 1 : 2, tiles_m = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
+  int NT = 32;
+  double best = 0.0;
+  for (int nt = 32; nt <= 256 / parts; nt *= 2) {
+    const double tiles = (double)tiles_m * ((R + nt - 1) / nt) * layers, waves = ceil(tiles / c->n_sm);
+    const double copy = (tc::BM * 128 + parts * nt * 128) / 64.0, mma = 2.0 * (parts * nt > 64 ? parts * nt : 64);
+    const double cost = waves * (slabs * (copy > mma ? copy : mma) + 12.0 * parts * nt) + 2000.0;
+    if (nt == 32 || cost < best) { best = cost; NT = nt; }
+  }
+  const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, NT, (uint32_t)parts);
+  if (tA < 0) { c->launch_error = FM_ERR_CUDA; return; }
+  int stages = (200 * 1024) / pf::stage_bytes(NT, parts);
+  stages = stages > 4 ? 4 : stages;
+  const int tiles_n = (R + NT - 1) / NT, tiles = tiles_m * tiles_n * layers;
+  if (mode == pf::PF_RESID && e.ssq_out != nullptr) c->ssq_n = tiles_m * 4;        // slots the next consumer adds
+  pf::Gemm g{W, c->tmaps + tA, M, K, R, NT, stages, tiles_m, tiles_n, tiles, w_tile0, c->st.status};
+  const dim3 grid(tiles < c->n_sm ? tiles : c->n_sm), one(1, 1, 1);
+  const int smem = pf::smem_bytes(NT, parts, stages);
+  switch (mode) {
+    case pf::PF_F32: launch_pdl(c, one, pf::gemm_kernel<pf::PF_F32, 2>, grid, pf::THREADS, smem, g, e); break;
+    case pf::PF_GELU: launch_pdl(c, one, pf::gemm_kernel<pf::PF_GELU, 2>, grid, pf::THREADS, smem, g, e); break;
+    case pf::PF_RESID: launch_pdl(c, one, pf::gemm_kernel<pf::PF_RESID, 2>, grid, pf::THREADS, smem, g, e); break;
+    case pf::PF_QKV: launch_pdl(c, one, pf::gemm_kernel<pf::PF_QKV, 2>, grid, pf::THREADS, smem, g, e); break;
+    default: launch_pdl(c, one, pf::gemm_kernel<pf::PF_PREFIX, 1>, grid, pf::THREADS, smem, g, e); break;
+  }
+}
+
+struct PfChunk {
+  const pf::Seg* segs;                   // device
+  const int2* tiles[3];
+  int n_segs, rows[3], n_tiles[3], tile_rows[3];
+  bool direct[3], ends;                  // the cache can be written by the projection itself; some prompt ends here
+};
+
+// Fewer rows than this go through the decode pass's GEMM, which splits K over a cluster.
+constexpr int PF_SMALL = 256;
+
+template <int DH, int C, int QW>
+void pf_attention(fm_ctx* c, dim3 grid, const pf::Attn& at) {
+  launch_pdl(c, dim3(1, 1, 1), pf::attn_kernel<DH, C, QW>, grid, pf::AttnCfg<DH, C, QW>::THREADS, pf::AttnCfg<DH, C, QW>::BYTES, at);
+}
+
+// one stack on the chunk's rows of its level
+void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const float* next_gain, bool want_a) {
+  const Dims& dm = c->dm;
+  auto& pr = c->pre;
+  const int level = STACK_LEVEL[s], R = ch.rows[level], d = dm.d, hd = dm.H * dm.dh, kvw = dm.Hkv * dm.dh, qkvw = hd + 2 * kvw;
+  const int nl = (int)c->layers[s].size(), ld = pr.rows[0];
+  const bool small = R <= PF_SMALL && ch.direct[level];
+  float* x = pr.x[level];
+  int tK = -1, tV = -1;
+  if (!ch.direct[level]) {
+    tK = tmap_for(c, pr.kbuf, pr.rows[0], kvw, c->attn_chunk, 0);
+    tV = tmap_for(c, pr.vbuf, pr.rows[0], kvw, c->attn_chunk, 0);
+    if (tK < 0 || tV < 0) { c->launch_error = FM_ERR_CUDA; return; }
+  }
+  for (int l = 0; l < nl; ++l) {
+    const LayerDev& L = c->layers[s][l];
+    const bool last = l == nl - 1;
+    if (last && stash_ring != nullptr && ch.ends)
+      launch_pdl(c, dim3(1, 1, 1), pf::stash_kernel, ch.n_segs, row_threads(d / 4), 0, dm, ch.segs, level, (const float*)x, stash_ring);
+    const float qscale = (float)(1.4426950408889634 / sqrt((double)dm.dh));
+    pf::Epi eq{};
+    eq.ssq_in = pr.ssq; eq.ssq_n = c->ssq_n; eq.ld_ssq = ld; eq.inv_d = 1.f / d; eq.eps = dm.eps;
+    tc::Epi sq{};
+    sq.ssq_in = pr.ssq; sq.ssq_n = c->ssq_n; sq.ld_ssq = ld; sq.inv_d_in = 1.f / d; sq.eps = dm.eps;
+    if (small) {
+      sq.dm = dm; sq.st = c->st; sq.batch = c->batch; sq.level = level; sq.rows = pr.map[level]; sq.rope_tab = c->rope_tab;
+      sq.q_out = pr.q; sq.Kc = L.K; sq.Vc = L.V; sq.qscale = qscale;
+      gemm(c, L.Wqkv, pad128(qkvw), 0, pr.a, ld, 0, qkvw, d, R, nullptr, tc::EPI_QKV, sq, 2);
+    } else {
+      eq.dm = dm; eq.rows = pr.map[level]; eq.level = level; eq.rope = c->rope_tab; eq.qscale = qscale;
+      eq.q = pr.q; eq.kbuf = pr.kbuf; eq.vbuf = pr.vbuf;
+      if (ch.direct[level]) { eq.Kc = L.K; eq.Vc = L.V; }
+      pf_gemm(c, pf::PF_QKV, L.Wqkv, pr.a, ld, qkvw, d, R, eq);
+    }
+    pf::Attn at{dm, ch.segs, ch.tiles[level], level, pr.q, c->tmaps + L.tmK, c->tmaps + L.tmV, tK < 0 ? nullptr : c->tmaps + tK,
+                tV < 0 ? nullptr : c->tmaps + tV, pr.attn, c->st.status};
+    const dim3 grid(dm.H, ch.n_tiles[level]);
+    const int qw = ch.tile_rows[level] / 16;
+    if (dm.dh == 64) {
+      if (qw == 8) pf_attention<64, 128, 8>(c, grid, at);
+      else if (qw == 2) pf_attention<64, 128, 2>(c, grid, at);
+      else pf_attention<64, 128, 1>(c, grid, at);
+    } else {
+      if (qw == 8) pf_attention<128, 64, 8>(c, grid, at);
+      else pf_attention<128, 64, 2>(c, grid, at);
+    }
+    if (!ch.direct[level])
+      launch_pdl(c, dim3(1, 1, 1), pf::cache_kernel, R, 128, 0, dm, ch.segs, (const pf::Row*)pr.map[level], level, (const bf16*)pr.kbuf,
+                 (const bf16*)pr.vbuf, L.K, L.V);
+    const float* gain2 = last ? next_gain : c->layers[s][l + 1].g1;
+    const bool out2 = !last || want_a;
+    if (small) {
+      tc::Epi eo{};
+      eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq_out = ld;
+      gemm(c, L.Wo, pad128(d), 0, pr.attn, ld, 0, d, hd, R, nullptr, tc::EPI_RESID, eo, 2);
+      tc::Epi e1 = epi_plain(pr.wide, 2 * dm.dff);
+      e1.lo_off = dm.dff;
+      e1.ssq_in = pr.ssq; e1.ssq_n = c->ssq_n; e1.ld_ssq = ld; e1.inv_d_in = 1.f / d; e1.eps = dm.eps;
+      gemm(c, L.W1, pad128(dm.dff), 0, pr.a, ld, 0, dm.dff, d, R, nullptr, tc::EPI_GELU, e1, 2);
+      eo.gain = gain2;
+      if (!out2) { eo.a_out = nullptr; eo.ssq_out = nullptr; }
+      gemm(c, L.W2, pad128(d), 0, pr.wide, ld, 0, d, dm.dff, R, nullptr, tc::EPI_RESID, eo, 2);
+      continue;
+    }
+    pf::Epi eo{};
+    eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq = ld;
+    pf_gemm(c, pf::PF_RESID, L.Wo, pr.attn, ld, d, hd, R, eo);
+    eq.out = pr.wide; eq.ldo = 2 * dm.dff; eq.lo_off = dm.dff; eq.ssq_n = c->ssq_n;
+    pf_gemm(c, pf::PF_GELU, L.W1, pr.a, ld, dm.dff, d, R, eq);
+    eo.gain = gain2;
+    if (!out2) { eo.a_out = nullptr; eo.ssq_out = nullptr; }
+    pf_gemm(c, pf::PF_RESID, L.W2, pr.wide, ld, d, dm.dff, R, eo);
+  }
+}
+
+// one chunk through the hourglass
+void pf_chunk(fm_ctx* c, const PfChunk& ch, const int* prompt, const int* prompt_off) {
+  const Dims& dm = c->dm;
+  auto& pr = c->pre;
+  const int d = dm.d, th = row_threads(d / 4);
+  const dim3 one(1, 1, 1);
+  LAUNCH(c, pf::map_kernel, dim3(ch.n_segs, 3), 256, 0, dm, ch.segs, pr.map[0], pr.map[1], pr.map[2]);
+  // (a full barrier: later prologues may read the maps before their dependency wait)
+  LAUNCH(c, pf::embed_kernel, ch.rows[0], th, 0, dm, c->st, (const pf::Row*)pr.map[0], prompt, prompt_off, (const bf16*)c->E, pr.x[0],
+         (const float*)c->layers[0][0].g1, pr.a, pr.ssq);
+  c->ssq_n = 1;
+  for (int up = 1; up <= 2; ++up) {                          // down: coordinate and vertex stacks, each followed by a shortening
+    pf_stack(c, ch, up - 1, nullptr, nullptr, false);
+    launch_pdl(c, one, pf::gather_kernel, dim3(ch.rows[up], 3), th, 0, dm, ch.segs, (const pf::Row*)pr.map[up], up, (const float*)pr.x[up - 1],
+               (const float*)(up == 1 ? c->hc_ring : c->hv_ring), pr.wide);
+    const bf16* S = up == 1 ? c->S_cv : c->S_vf;
+    if (ch.rows[up] <= PF_SMALL) {
+      tc::Epi es{};
+      es.x = pr.x[up]; es.ldx = d; es.add = 0; es.gain = c->layers[up][0].g1; es.a_out = pr.a; es.lda = 2 * d; es.lo_off = d;
+      es.ssq_out = pr.ssq; es.ld_ssq_out = pr.rows[0];
+      gemm(c, S, pad128(d), 0, pr.wide, pr.rows[1], 0, d, 3 * d, ch.rows[up], nullptr, tc::EPI_RESID, es, 2);
+    } else {
+      pf::Epi es{};
+      es.x = pr.x[up]; es.ldx = d; es.add = 0; es.gain = c->layers[up][0].g1; es.a_out = pr.a; es.lda = 2 * d; es.lo_off = d;
+      es.ssq_out = pr.ssq; es.ld_ssq = pr.rows[0];
+      pf_gemm(c, pf::PF_RESID, S, pr.wide, pr.rows[1], d, 3 * d, ch.rows[up], es);
+    }
+  }
+  pf_stack(c, ch, 2, c->zf, nullptr, true);
+  for (int low = 1; low >= 0; --low) {                       // up
+    const bf16* U = low == 1 ? c->U_fv : c->U_vc;
+    if (ch.rows[low + 1] <= PF_SMALL) {
+      gemm(c, U, pad128(3 * d), 0, pr.a, pr.rows[0], 0, 3 * d, d, ch.rows[low + 1], nullptr, tc::EPI_F32, epi_plain(pr.wide, 3 * d), 2);
+    } else {
+      pf::Epi eu{};
+      eu.out = pr.wide; eu.ldo = 3 * d;
+      pf_gemm(c, pf::PF_F32, U, pr.a, pr.rows[0], 3 * d, d, ch.rows[low + 1], eu);
+    }
+    launch_pdl(c, one, pf::upsample_kernel, ch.rows[low], th, 0, dm, ch.segs, (const pf::Row*)pr.map[low], low,
+               (const float*)reinterpret_cast<float*>(pr.wide), low == 1 ? c->hv_ring : c->hc_ring, low == 1 ? c->trif_ring : c->triv_ring, pr.x[low],
+               (const float*)c->layers[low == 1 ? 3 : 4][0].g1, pr.a, pr.ssq);
+    c->ssq_n = 1;
+    pf_stack(c, ch, low == 1 ? 3 : 4, low == 1 ? c->zv : c->zc, low == 1 ? nullptr : c->g_out, true);
+  }
+  if (ch.ends)
+    launch_pdl(c, one, pf::last_rows_kernel, ch.n_segs, 128, 0, dm, ch.segs, (const bf16*)pr.a, (const float*)pr.ssq, c->ssq_n, pr.rows[0], c->a_norm, c->ssq);
+}
+
+int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off) {
+  const Dims& dm = c->dm;
+  auto& pr = c->pre;
+  const int B = c->batch;
+  // ---- plan: sequences packed into chunks, cut at multiples of 9 (faces)
+  std::vector<pf::Seg> segs;
+  std::vector<int2> tiles;
+  std::vector<PfChunk> chunks;
+  std::vector<size_t> seg_at, tile_at;
+  int b = 0, done = 0;
+  while (b < B) {
+    PfChunk ch{};
+    ch.direct[0] = ch.direct[1] = ch.direct[2] = true;
+    seg_at.push_back(segs.size());
+    while (b < B && ch.rows[0] < pr.rows[0]) {
+      const int total = 1 + off[b + 1] - off[b], room = pr.rows[0] - ch.rows[0];
+      int n = total - done;
+      if (n > room) n = room - room % 9;
+      if (n == 0) break;
+      pf::Seg s{};
+      s.b = b;
+      s.last = done + n == total;
+      for (int l = 0; l < 3; ++l) {
+        const int ratio = fm_ratio(l);
+        s.p0[l] = done / ratio;
+        s.n[l] = (done + n - 1) / ratio - s.p0[l] + 1;
+        s.r0[l] = ch.rows[l];
+        ch.rows[l] += s.n[l];
+        if (s.p0[l] + s.n[l] > dm.cap[l]) ch.direct[l] = false;
+      }
+      ch.ends = ch.ends || s.last;
+      ch.n_segs++;
+      segs.push_back(s);
+      done += n;
+      if (s.last) { ++b; done = 0; }
+    }
+    for (int l = 0; l < 3; ++l) {
+      const size_t t0 = tiles.size();
+      tile_at.push_back(t0);
+      // query rows per CTA: the most that still give every SM one (see pf::AttnCfg)
+      ch.tile_rows[l] = dm.dh == 64 ? 16 : 32;
+      for (int rows = 128; rows >= 32; rows /= 4) {
+        int n = 0;
+        for (int k = 0; k < ch.n_segs; ++k) n += (segs[seg_at.back() + k].n[l] + rows - 1) / rows;
+        if (n * dm.H >= c->n_sm) { ch.tile_rows[l] = rows; break; }
+      }
+      for (int k = 0; k < ch.n_segs; ++k)
+        for (int q = 0; q < segs[seg_at.back() + k].n[l]; q += ch.tile_rows[l]) tiles.push_back(make_int2(k, q));
+      // longest first: rows late in a long segment see the most keys
+      const pf::Seg* sg = segs.data() + seg_at.back();
+      std::sort(tiles.begin() + t0, tiles.end(), [&](const int2& x, const int2& y) { return sg[x.x].p0[l] + x.y > sg[y.x].p0[l] + y.y; });
+      ch.n_tiles[l] = (int)(tiles.size() - t0);
+    }
+    chunks.push_back(ch);
+  }
+  const size_t o_seg = align_up((B + 1) * sizeof(int), 16), o_tile = align_up(o_seg + segs.size() * sizeof(pf::Seg), 16);
+  const size_t bytes = o_tile + tiles.size() * sizeof(int2);
+  if (bytes > pr.plan_bytes) return FM_ERR_CAPACITY;
+  c->plan_host.resize(bytes);
+  memcpy(c->plan_host.data(), off, (B + 1) * sizeof(int));
+  memcpy(c->plan_host.data() + o_seg, segs.data(), segs.size() * sizeof(pf::Seg));
+  memcpy(c->plan_host.data() + o_tile, tiles.data(), tiles.size() * sizeof(int2));
+  CUDA_OK(cudaMemcpyAsync(pr.plan, c->plan_host.data(), bytes, cudaMemcpyHostToDevice, c->stream));   // pageable: read before it returns
+  const int* off_dev = reinterpret_cast<const int*>(pr.plan);
+  LAUNCH(c, init_state_kernel, (dm.max_batch + 127) / 128, 128, 0, dm, c->st, B, off_dev);
+  // ---- per-layer prefix keys/values: K_pre = Wk rms(c, g1), V_pre = Wv rms(c, g1), no rotation; all layers in one launch
+  const int prefix_total = B * dm.P, kvw = 2 * dm.Hkv * dm.dh;
+  for (int r0 = 0; r0 < prefix_total; r0 += pr.prefix_rows) {
+    const int rows = prefix_total - r0 < pr.prefix_rows ? prefix_total - r0 : pr.prefix_rows;
+    LAUNCH(c, pf::prefix_norm_kernel, dim3(rows, rows < 2048 ? 4 : 1), row_threads(dm.d / 4), 0, cond + (size_t)r0 * dm.d, pr.layers, pr.n_layers,
+           pr.prefix_rows, pr.wide, dm.d, dm.eps);
+    pf::Epi e{};
+    e.dm = dm; e.layers = pr.layers; e.row_first = r0; e.rows_layer = pr.prefix_rows;
+    pf_gemm(c, pf::PF_PREFIX, nullptr, pr.wide, (size_t)pr.n_layers * pr.prefix_rows, kvw, dm.d, rows, e, pr.n_layers, dm.H * dm.dh / tc::BM);
+  }
+  // ---- BOS + prompt
+  for (size_t i = 0; i < chunks.size(); ++i) {
+    PfChunk& ch = chunks[i];
+    ch.segs = reinterpret_cast<const pf::Seg*>(pr.plan + o_seg) + seg_at[i];
+    for (int l = 0; l < 3; ++l) ch.tiles[l] = reinterpret_cast<const int2*>(pr.plan + o_tile) + tile_at[3 * i + l];
+    pf_chunk(c, ch, prompt, off_dev);
+  }
+  tc::Epi el = epi_plain(c->logits, dm.Vpad);
+  el.ssq_in = c->ssq; el.ssq_n = 1; el.ld_ssq = c->ssq_ld; el.inv_d_in = 1.f / dm.d; el.eps = dm.eps;
+  gemm(c, c->W_out, dm.Vpad, 0, c->a_norm, align_up((size_t)dm.max_batch * dm.R1, 16), 0, dm.V, dm.d, B, nullptr, tc::EPI_F32, el, 2);
+  launch_pdl(c, dim3(1, 1, 1), pf::finish_kernel, B, 256, 0, dm, c->st, (const float*)c->logits, prompt, off_dev);
+  return FM_OK;
+}
+
 // one decode pass of fm_generate
 void step_body(fm_ctx* c) {
   const Dims& dm = c->dm;
@@ -938,6 +1247,15 @@ void step_body(fm_ctx* c) {
   forward(c, nullptr);
   LAUNCH(c, accept_kernel, 1, accept_threads(c->batch), 0, dm, c->st, c->batch, (const int*)nullptr, (const int*)nullptr,
          (int*)nullptr, (int*)nullptr, (int*)nullptr, (const GenOut*)c->gen_dev, 1);
+}
+
+// Walk through `body` without launching anything: afterwards the descriptors of its launches exist (they
+// are made on first use, with a copy that a stream capture cannot hold).
+template <typename F>
+void make_descriptors(fm_ctx* c, F&& body) {
+  c->only_class = PROF_NONE;
+  body();
+  c->only_class = -1;
 }
 
 void drop_graph(fm_ctx* c) {
@@ -1013,8 +1331,7 @@ void run_cached(fm_ctx* c, fm_ctx::CallGraph& g, const void* k0, const void* k1,
 void ensure_graph(fm_ctx* c) {
   if (c->graph_unavailable || (c->graph_exec != nullptr && c->graph_batch == c->batch)) return;
   drop_graph(c);
-  draft(c, nullptr, nullptr, nullptr);             // makes the draft path's TMA descriptors exist
-  cudaStreamSynchronize(c->stream);
+  make_descriptors(c, [&] { step_body(c); });
   if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();
     c->graph_unavailable = true;
@@ -1108,7 +1425,7 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
     for (size_t l = 0; l < c->layers[s].size(); ++l) {
       const fm_layer_weights& hw = w->stack[s][l];
       LayerDev& L = c->layers[s][l];
-      TRY(upload_packed(L.Wqkv, hw.Wqkv, qkvw, d, tmp));
+      TRY(upload_packed(L.Wqkv, hw.Wqkv, qkvw, d, tmp, (size_t)(dm.H + dm.Hkv) * dm.dh, dm.dh));
       TRY(upload_packed(L.Wo, hw.Wo, d, hd, tmp));
       TRY(upload_packed(L.W1, hw.W1, (size_t)dm.dff, d, tmp));
       TRY(upload_packed(L.W2, hw.W2, d, (size_t)dm.dff, tmp));
@@ -1175,6 +1492,23 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
   TRYCUDA(cudaFuncSetAttribute(tc::gemm_tc_kernel<tc::EPI_RESID_CAT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::max_smem_bytes()));
   TRYCUDA(cudaFuncSetAttribute(tc::gemm_tc_kernel<tc::EPI_UP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::max_smem_bytes()));
   TRYCUDA(cudaFuncSetAttribute(tc::gemm_tc_kernel<tc::EPI_QKV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::max_smem_bytes()));
+  {
+    const int most = 216 * 1024;                             // a ring of at most 200 KB and what lies behind it
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_F32, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_GELU, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_RESID, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_QKV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_PREFIX, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<64, 128, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<64, 128, 8>::BYTES));
+    TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<64, 128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<64, 128, 2>::BYTES));
+    TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<64, 128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<64, 128, 1>::BYTES));
+    TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<128, 64, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<128, 64, 8>::BYTES));
+    TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<128, 64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<128, 64, 2>::BYTES));
+    std::vector<pf::LayerPtr> lp;
+    for (int s = 0; s < 5; ++s)
+      for (auto& L : c->layers[s]) lp.push_back({L.Wqkv, L.g1, L.K, L.V, STACK_LEVEL[s], 0});
+    TRYCUDA(cudaMemcpy(c->pre.layers, lp.data(), lp.size() * sizeof(pf::LayerPtr), cudaMemcpyHostToDevice));
+  }
   TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<64, 128, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64, 128, 8>::BYTES));
   TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<128, 64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128, 64, 4>::BYTES));
   std::vector<double> freq(dm.dh / 2);
@@ -1249,6 +1583,7 @@ int fm_profile_class(fm_ctx* c, int32_t cls, int32_t reps, fm_profile* out) {
   if (c == nullptr || out == nullptr || reps < 1 || (cls != PROF_GEMM && cls != PROF_ATTN)) return FM_ERR_INVALID_ARG;
   if (c->phase < 1) return FM_ERR_BAD_STATE;
   memset(out, 0, sizeof(*out));
+  make_descriptors(c, [&] { forward(c, nullptr); });
   CUDA_OK(cudaStreamSynchronize(c->stream));
   if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); return FM_ERR_CUDA; }
   const int64_t l0 = c->launches;
@@ -1324,29 +1659,8 @@ int fm_prefill(fm_ctx* c, int32_t batch, const float* cond, const int32_t* promp
   CUDA_OK(cudaMemsetAsync(c->attn_ticket, 0, c->attn_ticket_n * sizeof(int), c->stream));
   c->plen_host.assign(batch, 0);
   for (int b = 0; b < batch; ++b) c->plen_host[b] = prompt_off[b + 1] - prompt_off[b];
-  CUDA_OK(cudaMemcpyAsync(c->prompt_off_dev, prompt_off, (batch + 1) * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  CUDA_OK(cudaStreamSynchronize(c->stream));       // prompt_off is caller memory: finish reading it now
-  LAUNCH(c, init_state_kernel, (dm.max_batch + 127) / 128, 128, 0, dm, c->st, batch, c->prompt_off_dev);
-  // per-layer prefix keys/values: K_pre = Wk rms(c, g1), V_pre = Wv rms(c, g1), no rotation
-  const int rows_total = batch * dm.P, kvw = 2 * dm.Hkv * dm.dh;
-  for (int r0 = 0; r0 < rows_total; r0 += PREFILL_CHUNK) {
-    const int rows = rows_total - r0 < PREFILL_CHUNK ? rows_total - r0 : PREFILL_CHUNK;
-    for (int s = 0; s < 5; ++s)
-      for (auto& L : c->layers[s]) {
-        LAUNCH(c, rmsnorm_kernel, rows, 256, 0, cond + (size_t)r0 * dm.d, L.g1, c->pre_a, dm.d, dm.eps);
-        gemm(c, L.Wqkv, pad128((size_t)(dm.H + 2 * dm.Hkv) * dm.dh), dm.H * dm.dh, c->pre_a, PREFILL_CHUNK, 0, kvw, dm.d, rows,
-             nullptr, tc::EPI_F32, epi_plain(c->pre_o, kvw));
-        LAUNCH(c, prefix_store_kernel, rows, 128, 0, dm, STACK_LEVEL[s], r0, c->pre_o, L.K, L.V);
-      }
-  }
-  // BOS + prompt through the multi-row forward, D+1 rows per sequence and pass, all rows kept
-  const int passes = (1 + longest + dm.R1 - 1) / dm.R1;
-  for (int i = 0; i < passes; ++i) {
-    LAUNCH(c, prefill_feed_kernel, batch, 32, 0, dm, c->st, batch, prompt, c->prompt_off_dev);
-    LAUNCH(c, row_count_kernel, 1, 32, 0, dm, c->st, batch);
-    forward(c, nullptr);
-    LAUNCH(c, prefill_advance_kernel, (batch + 127) / 128, 128, 0, dm, c->st, batch);
-  }
+  const int rc = prefill_run(c, cond, prompt, prompt_off);
+  if (rc != FM_OK) return rc;
   LAUNCH(c, arm_kernel, (batch + 127) / 128, 128, 0, dm, c->st, batch);
   LAUNCH(c, row_count_kernel, 1, 32, 0, dm, c->st, batch);
   CUDA_OK(cudaGetLastError());
@@ -1360,7 +1674,7 @@ int fm_set_max_faces(fm_ctx* c, const int32_t* max_faces) {
   if (c == nullptr || max_faces == nullptr) return FM_ERR_INVALID_ARG;
   if (c->phase < 1) return FM_ERR_BAD_STATE;
   for (int b = 0; b < c->batch; ++b) if (max_faces[b] < 0) return FM_ERR_INVALID_ARG;
-  int* tmp = reinterpret_cast<int*>(c->pre_o);       // scratch that no pass is using now
+  int* tmp = c->limits_dev;
   CUDA_OK(cudaMemcpyAsync(tmp, max_faces, c->batch * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   LAUNCH(c, set_limits_kernel, (c->batch + 127) / 128, 128, 0, c->dm, c->st, c->batch, tmp);
   LAUNCH(c, arm_kernel, (c->batch + 127) / 128, 128, 0, c->dm, c->st, c->batch);

@@ -69,6 +69,9 @@ __device__ inline bool fm_row_map(const Dims& dm, const SeqState& st, int batch,
   return ratio * p <= Lb + n - 1;
 }
 
+// One row of a packed prefill chunk: sequence, level-local position, segment, cache slot behind the prefix.
+struct alignas(16) PackedRow { int b, p, seg, slot; };
+
 __device__ inline float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

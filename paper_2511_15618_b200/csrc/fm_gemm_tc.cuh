@@ -81,6 +81,7 @@ struct Epi {
   float* ssq_out; int ld_ssq_out;//            [M tiles * split][ld] partial sums of squares of the new x rows (may be null)
   Dims dm; SeqState st;          // EPI_QKV
   int batch, level;
+  const PackedRow* rows;         //            (b, p) of every row when the rows are packed (prefill); null: rows of a pass
   const float2* rope_tab;
   bf16* q_out;                   //            [rows, H*dh], rotated and scaled by qscale
   bf16* Kc; bf16* Vc;            //            caches [B, Hkv, slots, dh]
@@ -96,6 +97,14 @@ struct Epi {
   float* tri_ring;               //            where the triples of this pass go [B, fm_ring(level), 3d]
   int d_model;
 };
+
+__device__ inline bool row_of(const Epi& e, int row, int& b, int& p) {
+  if (e.rows == nullptr) return fm_row_map(e.dm, e.st, e.batch, e.level, row, b, p);
+  const PackedRow r = e.rows[row];
+  b = r.b;
+  p = r.p;
+  return true;
+}
 
 __device__ inline uint64_t smem_desc_sw128(uint32_t addr) {
   // K-major operand, 128-byte swizzle: start address, leading offset 1 (unused), stride between
@@ -216,18 +225,9 @@ __device__ inline void store_hi_lo2(bf16* p, float a, float b, int lo_off) {
 
 __device__ inline float gelu_erf_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 
-// Pair slot q (0..63) of a 128-column tile -> its two columns.  Rotary pairs are (i, i + dh/2)
-// inside a head, so with heads of 64 a tile holds two heads with 32 pairs each, with heads of
-// 128 one head with 64 pairs.  The other epilogues use the same map (any bijection would do).
-// Epilogues without rotation pair neighbouring columns (2q, 2q + 1), so that a thread's two values
-// leave in one store.
-template <bool ROT>
-__device__ inline void pair_cols(int q, bool head128, int& ca, int& cb) {
-  if (!ROT) { ca = 2 * q; cb = ca + 1; }
-  else if (head128) { ca = q; cb = q + 64; }
-  else { ca = (q >> 5) * 64 + (q & 31); cb = ca + 32; }
-}
-
+// Pair slot q (0..63) of a 128-column tile holds columns (2q, 2q + 1): a thread's two values leave in one
+// store, and in the QKV projection, whose weight rows are stored with the rotary pairs (i, i + dh/2) of
+// a head side by side, they are one rotary pair.
 // grid (M/128 tiles, split, N tiles of the token rows), cluster (1, split, 1); block 128.  Warp 0 lane 0 feeds TMA, warp 1
 // lane 0 issues MMAs, all four warps read the accumulator back (warp w owns TMEM lanes 32w..32w+31).
 // SIDE: the launch has side rows (side_bytes(N, split) > 0); a separate instantiation, because the
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
       for (int n0 = 0; n0 < ns; n0 += 32) {
         const int n = n0 + lane;
         int b = 0, p = 0;
-        const bool valid = n < ns && fm_row_map(e.dm, e.st, e.batch, e.level, row0 + n, b, p);
+        const bool valid = n < ns && row_of(e, row0 + n, b, p);
         if (n < ns) { s_rb[n] = valid ? b : -1; s_rp[n] = p; }
         if ((MODE == EPI_RESID_CAT || MODE == EPI_UP) && n < ns && valid) {
           // first position of the sequence at the other level of the pair, last position at the lower one
@@ -440,13 +440,11 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   // (indices, gains, rotary angles) is prepared here, before the wait.
   const int lgS = 31 - __clz(S);                           // S is 1, 2, 4 or 8
   const int lgPW = 6 - lgS, PW = 1 << lgPW;
-  const bool head128 = MODE == EPI_QKV && e.dm.dh == 128;
   const int items = ns * PW;
   uint32_t dst0 = 0, dbar = 0;
   float* recv_own;                                         // S == 1: this thread's row run in the local buffer
   {
-    const int q = MODE != EPI_QKV ? (tid >> 1) : (head128 ? (tid & 63) : ((tid >> 6) * 32 + (tid & 31)));
-    const int h = MODE != EPI_QKV ? (tid & 1) : (head128 ? (tid >> 6) : ((tid >> 5) & 1));
+    const int q = tid >> 1, h = tid & 1;
     const int owner = q >> lgPW, cc = q & (PW - 1);
     recv_own = recv + (((size_t)z * PW + cc) * 2 + h) * NP;
     if (S > 1) {
@@ -459,9 +457,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   float pre_ga = 1.f, pre_gb = 1.f;
   float2 pre_cs = make_float2(1.f, 0.f);                   // first item's rotary angle when the side rows are not used
   if (tid < items) {
-    int ca, cb;
-    pair_cols<MODE == EPI_QKV>(z * PW + (tid & (PW - 1)), head128, ca, cb);
-    const int ma = tile_m * BM + ca, mb = tile_m * BM + cb;
+    const int ma = tile_m * BM + 2 * (z * PW + (tid & (PW - 1))), mb = ma + 1;
     if (IS_RESID && e.gain != nullptr) {
       if (ma < g.M) pre_ga = e.gain[ma];
       if (mb < g.M) pre_gb = e.gain[mb];
@@ -472,8 +468,8 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     }
     if (MODE == EPI_QKV && want_side && !use_side) {
       int b, p;
-      const bool valid = fm_row_map(e.dm, e.st, e.batch, e.level, row0 + (tid >> lgPW), b, p);
-      const int head = ma / e.dm.dh, i = ma - head * e.dm.dh;
+      const bool valid = row_of(e, row0 + (tid >> lgPW), b, p);
+      const int head = ma / e.dm.dh, i = (ma - head * e.dm.dh) >> 1;
       if (valid && ma < g.M && head < e.dm.H + e.dm.Hkv) pre_cs = e.rope_tab[(size_t)p * (e.dm.dh >> 1) + i];
     }
   }
@@ -496,9 +492,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   ptx::grid_dep_wait();                                    // everything below touches activations
   float pre_xa = 0.f, pre_xb = 0.f;                        // first item's residual values, same case
   if (IS_RESID && want_side && !use_side && tid < items) {
-    int ca, cb;
-    pair_cols<MODE == EPI_QKV>(z * PW + (tid & (PW - 1)), head128, ca, cb);
-    const int ma = tile_m * BM + ca, mb = tile_m * BM + cb;
+    const int ma = tile_m * BM + 2 * (z * PW + (tid & (PW - 1))), mb = ma + 1;
     const float* xr = k_x + (size_t)(k_row0 + (tid >> lgPW)) * k_ldx;
     if (ma < k_M) pre_xa = xr[ma];
     if (mb < k_M) pre_xb = xr[mb];
@@ -555,8 +549,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     const int it = it0 + tid;
     const bool active = it < items, first = it0 == 0;
     const int n = active ? it >> lgPW : 0, cc = active ? it & (PW - 1) : 0;
-    int ca, cb;
-    pair_cols<MODE == EPI_QKV>(z * PW + cc, head128, ca, cb);
+    const int ca = 2 * (z * PW + cc);
     float va[MAX_SPLIT], vb[MAX_SPLIT];
 #pragma unroll
     for (int r = 0; r < MAX_SPLIT; ++r) {                  // all loads first, then the sums in rank order
@@ -571,7 +564,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     const float inv = s_inv[n];
     ya *= inv;
     yb *= inv;
-    const int ma = tile_m * BM + ca, mb = tile_m * BM + cb;
+    const int ma = tile_m * BM + ca, mb = ma + 1;
     const bool a_ok = active && ma < k_M, b_ok = active && mb < k_M;
     const size_t row = (size_t)(k_row0 + n);
     if (MODE == EPI_F32) {
@@ -657,32 +650,26 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
         if (active && child && (cc & (L - 1)) == 0)
           k_ssqo[(size_t)(((((tile_m % (dd / BM)) << lgS) + z) << (lgPW - lgL)) + (cc >> lgL)) * k_ldssq + crow] = sqv;
       }
-    } else {  // EPI_QKV: (ya, yb) is the rotary pair (i, i + dh/2) of one head
-      const int dh = k_dh, half = dh >> 1, H = k_H, Hkv = k_Hkv;
-      const int head = ma / dh, i = ma - head * dh;
+    } else {  // EPI_QKV: (ya, yb) is the rotary pair (i, i + dh/2) of one head, stored at (c, c + 1), c = 2i
+      const int dh = k_dh, H = k_H, Hkv = k_Hkv;
+      const int head = ma / dh, c = ma - head * dh;
       if (a_ok && head < H + 2 * Hkv) {
         const int b = s_rb[n], p = s_rp[n];
         const bool valid = b >= 0;
         const int slots = k_P + k_cap;
         if (head < H + Hkv) {
           float2 cs = make_float2(1.f, 0.f);
-          if (use_side) { if (valid) cs = reinterpret_cast<const float2*>(side)[n * 64 + i]; }
+          if (use_side) { if (valid) cs = reinterpret_cast<const float2*>(side)[n * 64 + (c >> 1)]; }
           else if (first) cs = pre_cs;
-          else if (want_side && valid) cs = e.rope_tab[(size_t)p * half + i];
+          else if (want_side && valid) cs = e.rope_tab[(size_t)p * (dh >> 1) + (c >> 1)];
           const float y1 = ya * cs.x - yb * cs.y, y2 = yb * cs.x + ya * cs.y;
-          if (head < H) {
-            bf16* q = k_q + (row * H + head) * dh;
-            q[i] = __float2bfloat16(valid ? y1 * k_qs : 0.f);
-            q[half + i] = __float2bfloat16(valid ? y2 * k_qs : 0.f);
-          } else if (valid) {
-            bf16* dst = k_K + (((size_t)b * Hkv + (head - H)) * slots + k_P + (p % k_cap)) * dh;
-            dst[i] = __float2bfloat16(y1);
-            dst[half + i] = __float2bfloat16(y2);
-          }
+          if (head < H)
+            *reinterpret_cast<__nv_bfloat162*>(k_q + (row * H + head) * dh + c) =
+                valid ? __floats2bfloat162_rn(y1 * k_qs, y2 * k_qs) : __floats2bfloat162_rn(0.f, 0.f);
+          else if (valid)
+            *reinterpret_cast<__nv_bfloat162*>(k_K + (((size_t)b * Hkv + (head - H)) * slots + k_P + (p % k_cap)) * dh + c) = __floats2bfloat162_rn(y1, y2);
         } else if (valid) {
-          bf16* dst = k_V + (((size_t)b * Hkv + (head - H - Hkv)) * slots + k_P + (p % k_cap)) * dh;
-          dst[i] = __float2bfloat16(ya);
-          dst[half + i] = __float2bfloat16(yb);
+          *reinterpret_cast<__nv_bfloat162*>(k_V + (((size_t)b * Hkv + (head - H - Hkv)) * slots + k_P + (p % k_cap)) * dh + c) = __floats2bfloat162_rn(ya, yb);
         }
       }
     }
@@ -697,9 +684,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
       const bool active = it < nci;
       const int cc = it & (PW - 1);
       const size_t crow = active ? (size_t)s_carry[it >> lgPW] : 0;
-      int ca, cb;
-      pair_cols<false>(z * PW + cc, false, ca, cb);
-      const int col = (tile_m * BM + ca) % dd;
+      const int col = (tile_m * BM + 2 * (z * PW + cc)) % dd;
       float2 x0 = make_float2(0.f, 0.f);
       if (active) x0 = __ldcg(reinterpret_cast<const float2*>(k_x + crow * k_ldx + col));
       if (active && k_aout != nullptr) {

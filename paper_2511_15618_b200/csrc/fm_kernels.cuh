@@ -133,22 +133,6 @@ __global__ void rope_table_kernel(float2* __restrict__ tab, const double* __rest
   tab[i] = make_float2((float)c, (float)s);
 }
 
-// prefix keys/values of one layer: kv fp32 [rows, 2*Hkv*dh] (rows = chunk of b*P+j) -> slots [0,P)
-__global__ void prefix_store_kernel(Dims dm, int level, int row0, const float* __restrict__ kv,
-                                    bf16* __restrict__ Kc, bf16* __restrict__ Vc) {
-  const int r = row0 + blockIdx.x;
-  const int b = r / dm.P, j = r - b * dm.P;
-  const int slots = dm.P + dm.cap[level];
-  const int n = dm.Hkv * dm.dh;
-  const float* src = kv + (size_t)blockIdx.x * 2 * n;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    const int hk = t / dm.dh, i = t - hk * dm.dh;
-    const size_t o = (((size_t)b * dm.Hkv + hk) * slots + j) * dm.dh + i;
-    Kc[o] = __float2bfloat16(src[t]);
-    Vc[o] = __float2bfloat16(src[n + t]);
-  }
-}
-
 // ------------------------------------------------------------------------------------------
 // hourglass carry rings
 // ------------------------------------------------------------------------------------------
@@ -378,36 +362,8 @@ __global__ void accept_kernel(Dims dm, SeqState st, int batch, const int* __rest
   }
 }
 // ------------------------------------------------------------------------------------------
-// prefill helpers
+// start of decoding
 // ------------------------------------------------------------------------------------------
-// next chunk of BOS + prompt: cand[b][j] = u_{L+j}, nrow = min(R1, inputs left)
-__global__ void prefill_feed_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ prompt,
-                                    const int* __restrict__ prompt_off) {
-  const int b = blockIdx.x;
-  if (b >= batch) return;
-  const int L = st.L[b], total = 1 + st.plen[b];
-  const int n = max(0, min(dm.R1, total - L));
-  for (int j = threadIdx.x; j < dm.R1; j += blockDim.x) {
-    const int pos = L + j;
-    int tok = dm.n_bins + 2;
-    if (j < n) tok = pos == 0 ? dm.n_bins : prompt[prompt_off[b] + pos - 1];
-    st.cand[b * dm.R1 + j] = tok;
-    if (j < n && pos >= 1) st.hist[b * FM_HIST + ((pos - 1) & (FM_HIST - 1))] = tok;            // input u_pos is mesh token t_{pos-1}
-  }
-  if (threadIdx.x == 0) st.nrow[b] = n;
-}
-
-// all fed rows are accepted; when the prompt is used up the argmax of the last row is the main token
-__global__ void prefill_advance_kernel(Dims dm, SeqState st, int batch) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= batch) return;
-  const int n = st.nrow[b];
-  if (n <= 0) return;
-  const int L = st.L[b] + n;
-  st.L[b] = L;
-  if (L == 1 + st.plen[b]) st.main_tok[b] = st.o[b * dm.R1 + n - 1];
-}
-
 // set the rows of the first verify pass (and after fm_set_max_faces)
 __global__ void arm_kernel(Dims dm, SeqState st, int batch) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -529,8 +485,9 @@ __global__ void draft_q_kernel(Dims dm, SeqState st, int batch, int stage, int l
     float2 cs = make_float2(1.f, 0.f);
     if (dm.theta != 0.f) cs = rope_tab[(size_t)pos * half + k];
     const float x1 = src[head * dm.dh + k], x2 = src[head * dm.dh + half + k];
-    dst[head * dm.dh + k] = __float2bfloat16((x1 * cs.x - x2 * cs.y) * qscale);
-    dst[head * dm.dh + half + k] = __float2bfloat16((x2 * cs.x + x1 * cs.y) * qscale);
+    // the caches hold rotary pairs side by side
+    *reinterpret_cast<__nv_bfloat162*>(dst + head * dm.dh + 2 * k) =
+        __floats2bfloat162_rn((x1 * cs.x - x2 * cs.y) * qscale, (x2 * cs.x + x1 * cs.y) * qscale);
   }
 }
 

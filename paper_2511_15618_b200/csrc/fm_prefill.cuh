@@ -1,0 +1,795 @@
+// Prefill: BOS + prompt of all sequences as one packed multi-row forward.
+//
+// The rows of a chunk are the coordinate positions of up to a few thousand prompt tokens, sequence
+// segments one after the other; segments start at multiples of 9, so every vertex and face of a
+// segment has its children in the same chunk, and only the two hiddens before the segment come from
+// the carry rings.  Each projection is then a real GEMM (weights read once per chunk instead of once
+// per D + 1 tokens), and the attention of a segment streams a key once per 128 query rows.
+#pragma once
+#include "fm_common.cuh"
+#include "fm_gemm_tc.cuh"
+#include "fm_kernels.cuh"
+#include "fm_ptx.cuh"
+
+namespace pf {
+
+// One sequence's share of a chunk: level-local positions [p0, p0 + n) at rows [r0, r0 + n).
+struct Seg {
+  int b, last;                   // sequence; last != 0: the segment ends with the prompt
+  int p0[3], n[3], r0[3];
+};
+typedef PackedRow Row;
+
+// Pointers of one layer, for launches that span layers.
+struct LayerPtr { const bf16* Wqkv; const float* g1; bf16* K; bf16* V; int level, pad; };
+
+// ------------------------------------------------------------------------------------------
+// GEMM
+// ------------------------------------------------------------------------------------------
+// y[n][m] = sum_k W[m, k] A[n, k].  Tile: 128 output features (the MMA's M axis) x NT rows (N axis).
+// Operand rows with two bfloat16 terms lie as [hi | lo] tiles behind one another and form one operand of
+// 2 NT rows, so a weight slab is loaded once for both.  One persistent CTA per SM walks over the tiles
+// (feature tiles innermost: neighbouring CTAs share their operand rows in L2); a ring of shared-memory
+// stages decouples the copies from the MMA thread, and two accumulators in tensor memory let the
+// epilogue of a tile run under the MMAs of the next.  A thread of the epilogue owns one feature (its
+// tensor-memory lane), so a warp stores 32 neighbouring features of a row at a time.
+// Bound: tensor cores and, below 128 rows per tile, the stream from L2 (48 KB per 512 MMA clocks).
+enum Mode { PF_F32 = 0, PF_GELU = 1, PF_RESID = 2, PF_QKV = 3, PF_PREFIX = 4 };
+
+constexpr int THREADS = 192;     // producer warp, MMA warp, four epilogue warps
+constexpr int MAX_STAGES = 6;
+
+struct Gemm {
+  const bf16* W; const CUtensorMap* tmA;
+  int M, K, R, NT, stages;
+  int tiles_m, tiles_n, tiles;   // tiles = tiles_m * tiles_n * layers (PF_PREFIX), else tiles_m * tiles_n
+  int w_tile0;
+  int* status;
+};
+struct Epi {
+  const float* ssq_in; int ssq_n, ld_ssq; float inv_d, eps;     // RMSNorm scale of the operand rows (null: none)
+  void* out; int ldo, lo_off;                                   // PF_F32: fp32, PF_GELU: [hi | lo] bf16
+  float* x; int ldx, add; const float* gain; bf16* a_out; int lda; float* ssq_out;      // PF_RESID
+  Dims dm; const Row* rows; int level; const float2* rope; float qscale;                // PF_QKV
+  bf16 *q, *kbuf, *vbuf, *Kc, *Vc;                              // keys and values: into the cache, or (Kc null) into kbuf / vbuf
+  const LayerPtr* layers; int row_first, rows_layer;            // PF_PREFIX: operand rows of layer z at z * rows_layer
+};
+
+inline int stage_bytes(int NT, int parts) { return tc::BM * 128 + parts * NT * 128; }
+inline int smem_bytes(int NT, int parts, int stages) { return stages * stage_bytes(NT, parts) + 2 * 256 * 4 + 256 + 1024; }
+
+__device__ inline void ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,"
+      "%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+        "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
+__device__ inline void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ inline bool epi_sync_or(bool v) {                 // barrier of the epilogue warps; true if it was true for any thread
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"((uint32_t)v) : "memory");
+  return r != 0;
+}
+
+// One step of a transposing butterfly: afterwards a lane holds half as many rows, summed over pairs of lanes.
+template <int H>
+__device__ inline void fold(float* v, int lane) {
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const float send = (lane & H) ? v[i] : v[i + H], keep = (lane & H) ? v[i + H] : v[i];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, H);
+  }
+}
+
+template <int MODE, int PARTS>
+__global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Epi e) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const int NT = g.NT, ST = g.stages;
+  const int stage = tc::BM * 128 + PARTS * NT * 128;
+  float* s_inv = reinterpret_cast<float*>(sm + ST * stage);                  // [2][256]
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_inv + 512);
+  uint64_t* empty = full + MAX_STAGES;
+  uint64_t* acc_full = empty + MAX_STAGES;
+  uint64_t* acc_empty = acc_full + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  __shared__ int s_fail;
+  __shared__ Row s_row[2][MODE == PF_QKV ? 128 : 1];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int slabs = g.K / tc::BK;
+  uint32_t ncols = 32;
+  while ((int)ncols < 2 * PARTS * NT) ncols <<= 1;
+  const int acc_cols = (int)ncols / 2;
+  if (tid == 0) {
+    s_fail = 0;
+    for (int i = 0; i < ST; ++i) { ptx::mbar_init(full + i, 1); ptx::mbar_init(empty + i, 1); }
+    for (int i = 0; i < 2; ++i) { ptx::mbar_init(acc_full + i, 1); ptx::mbar_init(acc_empty + i, 128); }
+    ptx::fence_mbar_init();
+    ptx::prefetch_tmap(g.tmA);
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(tmem_slot)), "r"(ncols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = *tmem_slot;
+  ptx::grid_dep_launch();
+  const int per_z = g.tiles_m * g.tiles_n;
+  auto tile_of = [&](int t, int& z, int& tm, int& tn) {
+    z = MODE == PF_PREFIX ? t / per_z : 0;
+    const int u = t - z * per_z;
+    tn = u / g.tiles_m;
+    tm = u - tn * g.tiles_m;
+  };
+  if (warp == 0 && lane == 0) {
+    // ---- producer.  Weights do not depend on the previous kernel: the first stages' slabs are requested
+    // before the dependency wait.
+    auto wsrc = [&](int z, int tm) {
+      const bf16* W = MODE == PF_PREFIX ? e.layers[z].Wqkv : g.W;
+      return W + (size_t)(g.w_tile0 + tm) * slabs * (tc::BM * tc::BK);
+    };
+    int done = 0;                                            // slabs whose weights are already on their way
+    if ((int)blockIdx.x < g.tiles) {
+      int z, tm, tn;
+      tile_of(blockIdx.x, z, tm, tn);
+      const bf16* W = wsrc(z, tm);
+      done = slabs < ST ? slabs : ST;
+      for (int i = 0; i < done; ++i) {
+        ptx::mbar_expect_tx(full + i, stage);
+        ptx::bulk_load(sm + i * stage, W + (size_t)i * (tc::BM * tc::BK), tc::BM * 128, full + i);
+      }
+    }
+    ptx::grid_dep_wait();
+    int it = 0;
+    for (int t = blockIdx.x; t < g.tiles; t += gridDim.x) {
+      int z, tm, tn;
+      tile_of(t, z, tm, tn);
+      const bf16* W = wsrc(z, tm);
+      const int row = tn * NT + (MODE == PF_PREFIX ? z * e.rows_layer : 0);
+      for (int s = 0; s < slabs; ++s, ++it) {
+        const int st = it % ST;
+        unsigned char* dst = sm + st * stage;
+        if (it >= done) {
+          if (it >= ST && !ptx::mbar_wait(empty + st, ((it / ST) - 1) & 1)) { s_fail = 1; break; }
+          ptx::mbar_expect_tx(full + st, stage);
+          ptx::bulk_load(dst, W + (size_t)s * (tc::BM * tc::BK), tc::BM * 128, full + st);
+        }
+        ptx::tma_load_3d(dst + tc::BM * 128, g.tmA, s * tc::BK, row, 0, full + st);
+      }
+      if (s_fail) break;
+    }
+  } else if (warp == 1 && lane == 0) {
+    // ---- MMA issuer
+    const uint32_t idesc = tc::instr_desc_bf16(PARTS * NT);
+    int it = 0, k = 0;
+    for (int t = blockIdx.x; t < g.tiles; t += gridDim.x, ++k) {
+      const int buf = k & 1;
+      if (k >= 2 && !ptx::mbar_wait(acc_empty + buf, ((k >> 1) - 1) & 1)) { s_fail = 1; break; }
+      tc::fence_after();
+      bool bad = false;
+      for (int s = 0; s < slabs; ++s, ++it) {
+        const int st = it % ST;
+        if (!ptx::mbar_wait(full + st, (it / ST) & 1)) { s_fail = 1; bad = true; break; }
+        tc::fence_after();
+        const uint32_t a_addr = ptx::smem_u32(sm + st * stage);
+        const uint64_t da = tc::smem_desc_sw128(a_addr), db = tc::smem_desc_sw128(a_addr + tc::BM * 128);
+#pragma unroll
+        for (int kk = 0; kk < tc::BK / 16; ++kk)
+          tc::mma_ss(tmem + buf * acc_cols, da + 2 * kk, db + 2 * kk, idesc, (s > 0 || kk > 0) ? 1u : 0u);
+        tc::commit(empty + st);
+      }
+      if (bad) break;
+      tc::commit(acc_full + buf);
+    }
+  } else if (warp >= 2) {
+    // ---- epilogue: warp w reads tensor-memory lanes 32 (w mod 4) .. + 31
+    const int w4 = warp & 3, et = tid - 64;
+    ptx::grid_dep_wait();
+    int k = 0;
+    for (int t = blockIdx.x; t < g.tiles; t += gridDim.x, ++k) {
+      int z, tm, tn;
+      tile_of(t, z, tm, tn);
+      const int buf = k & 1, n0 = tn * NT, nrows = min(NT, g.R - n0);
+      const int m = tm * tc::BM + w4 * 32 + lane;
+      const bool m_ok = m < g.M;
+      float* inv = s_inv + buf * 256;
+      if (MODE != PF_PREFIX) {
+        for (int n = et; n < nrows; n += 128) {
+          float v = 1.f;
+          if (e.ssq_in != nullptr) {
+            float ss = 0.f;
+#pragma unroll 8
+            for (int s = 0; s < e.ssq_n; ++s) ss += __ldcg(e.ssq_in + (size_t)s * e.ld_ssq + n0 + n);
+            v = rsqrtf(ss * e.inv_d + e.eps);
+          }
+          inv[n] = v;
+          if (MODE == PF_QKV) s_row[buf][n] = e.rows[n0 + n];
+        }
+      }
+      float gain = 1.f;
+      if (MODE == PF_RESID && e.gain != nullptr && m_ok) gain = e.gain[m];
+      // (the barrier also publishes inv; all epilogue threads leave together when a wait ran out)
+      const bool late = !ptx::mbar_wait(acc_full + buf, (k >> 1) & 1);
+      if (epi_sync_or(late)) { if (late) s_fail = 1; break; }
+      tc::fence_after();
+      for (int c0 = 0; c0 < nrows; c0 += 32) {
+        uint32_t r[32];
+        float y[32];
+        ld32(tmem + buf * acc_cols + ((uint32_t)(w4 * 32) << 16) + c0, r);
+        if (PARTS == 2) {
+          uint32_t r2[32];
+          ld32(tmem + buf * acc_cols + ((uint32_t)(w4 * 32) << 16) + NT + c0, r2);
+          ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(r[j]) + __uint_as_float(r2[j]);
+        } else {
+          ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(r[j]);
+        }
+        if (c0 + 32 >= nrows) {                              // accumulator is in registers: the next tile may overwrite it
+          tc::fence_before();
+          ptx::mbar_arrive(acc_empty + buf);
+        }
+        const int nv = min(32, nrows - c0);
+        const size_t row = (size_t)(n0 + c0);
+        if (MODE != PF_PREFIX) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) y[j] *= inv[c0 + j];  // (rows behind nrows: stale scale, never stored)
+        }
+        if (MODE == PF_F32) {
+          float* o = reinterpret_cast<float*>(e.out) + row * e.ldo + m;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (j < nv && m_ok) o[(size_t)j * e.ldo] = y[j];
+        } else if (MODE == PF_GELU) {
+          bf16* o = reinterpret_cast<bf16*>(e.out) + row * e.ldo + m;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (j < nv && m_ok) tc::store_hi_lo(o + (size_t)j * e.ldo, tc::gelu_erf_f(y[j]), e.lo_off);
+        } else if (MODE == PF_RESID) {
+          float* xr = e.x + row * e.ldx + m;
+          if (e.add) {
+            float x0[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) x0[j] = (j < nv && m_ok) ? xr[(size_t)j * e.ldx] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) y[j] += x0[j];
+          }
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (j < nv && m_ok) xr[(size_t)j * e.ldx] = y[j];
+          if (e.a_out != nullptr) {
+            bf16* ao = e.a_out + row * e.lda + m;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (j < nv && m_ok) tc::store_hi_lo(ao + (size_t)j * e.lda, __fmul_rn(y[j], gain), e.lo_off);
+          }
+          if (e.ssq_out != nullptr) {
+            // sums of squares of 32 rows over the warp's 32 features: lane i ends up with row c0 + i
+#pragma unroll
+            for (int j = 0; j < 32; ++j) y[j] = m_ok ? y[j] * y[j] : 0.f;
+            fold<16>(y, lane); fold<8>(y, lane); fold<4>(y, lane); fold<2>(y, lane); fold<1>(y, lane);
+            if (lane < nv) e.ssq_out[(size_t)(tm * 4 + w4) * e.ld_ssq + row + lane] = y[0];
+          }
+        } else if (MODE == PF_QKV) {
+          // Q and K heads are stored with their rotary pairs side by side: the partner is the neighbouring lane
+          const int dh = e.dm.dh, H = e.dm.H, Hkv = e.dm.Hkv;
+          const int head = m / dh, i = m - head * dh;        // (the same head for the whole warp: dh is 64 or 128)
+          if (head < H + Hkv && e.dm.theta != 0.f) {
+            const float2* tab = e.rope + (i >> 1);
+            float2 cs[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) cs[j] = j < nv ? tab[(size_t)s_row[buf][c0 + j].p * (dh >> 1)] : make_float2(1.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              const float o = __shfl_xor_sync(0xffffffffu, y[j], 1);
+              y[j] = (lane & 1) ? y[j] * cs[j].x + o * cs[j].y : y[j] * cs[j].x - o * cs[j].y;
+            }
+          }
+          if (head < H) {
+            bf16* o = e.q + row * (size_t)(H * dh) + m;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (j < nv && m_ok) o[(size_t)j * (H * dh)] = __float2bfloat16(y[j] * e.qscale);
+          } else {
+            const bool is_k = head < H + Hkv;
+            const int hk = head - H - (is_k ? 0 : Hkv);
+            if (e.Kc != nullptr) {
+              const size_t slots = e.dm.P + e.dm.cap[e.level];
+              bf16* o = (is_k ? e.Kc : e.Vc) + (hk * slots + e.dm.P) * dh + i;
+#pragma unroll
+              for (int j = 0; j < 32; ++j) {
+                const Row rw = s_row[buf][c0 + j];
+                if (j < nv && m_ok) o[(rw.b * (Hkv * slots) + rw.slot) * dh] = __float2bfloat16(y[j]);
+              }
+            } else {
+              bf16* o = (is_k ? e.kbuf : e.vbuf) + row * (size_t)(Hkv * dh) + hk * dh + i;
+#pragma unroll
+              for (int j = 0; j < 32; ++j)
+                if (j < nv && m_ok) o[(size_t)j * (Hkv * dh)] = __float2bfloat16(y[j]);
+            }
+          }
+        } else {  // PF_PREFIX
+          const int dh = e.dm.dh, Hkv = e.dm.Hkv, P = e.dm.P;
+          const LayerPtr L = e.layers[z];
+          const int head = m / dh, i = m - head * dh;
+          const int hk = head < Hkv ? head : head - Hkv;
+          const int slots = P + e.dm.cap[L.level];
+          bf16* dst = (head < Hkv ? L.K : L.V) + i;
+          int b = (e.row_first + (int)row) / P, s = e.row_first + (int)row - b * P;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            if (j < nv && m_ok) dst[(((size_t)b * Hkv + hk) * slots + s) * dh] = __float2bfloat16(y[j]);
+            if (++s == P) { s = 0; ++b; }
+          }
+        }
+      }
+    }
+  }
+  __syncwarp();
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (s_fail) {
+    if (tid == 0) atomicExch(g.status, -5);
+    ptx::drain_delay();                                      // stages already requested may still be landing
+  }
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+}
+
+// ------------------------------------------------------------------------------------------
+// row-wise kernels
+// ------------------------------------------------------------------------------------------
+// (b, p, segment, cache slot) of every row of the three levels; grid (segments, 3)
+__global__ void map_kernel(Dims dm, const Seg* __restrict__ segs, Row* m0, Row* m1, Row* m2) {
+  const int l = blockIdx.y;
+  const Seg& s = segs[blockIdx.x];
+  Row* m = (l == 0 ? m0 : l == 1 ? m1 : m2) + s.r0[l];
+  for (int i = threadIdx.x; i < s.n[l]; i += blockDim.x) m[i] = Row{s.b, s.p0[l] + i, (int)blockIdx.x, (s.p0[l] + i) % dm.cap[l]};
+}
+
+// operand row [hi | lo] of x * g and the row's sum of squares, four columns per thread and step
+__device__ inline void entry_row(const float4* xr, int row, int d, const float* __restrict__ g, bf16* __restrict__ a,
+                                 float* __restrict__ ssq) {
+  __shared__ float sh[32];
+  float ss = 0.f;
+  for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
+    const float4 v = xr[i];
+    const float4 gg = g != nullptr ? reinterpret_cast<const float4*>(g)[i] : make_float4(1.f, 1.f, 1.f, 1.f);
+    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    bf16* p = a + (size_t)row * 2 * d + 4 * i;
+    tc::store_hi_lo2(p, __fmul_rn(v.x, gg.x), __fmul_rn(v.y, gg.y), d);
+    tc::store_hi_lo2(p + 2, __fmul_rn(v.z, gg.z), __fmul_rn(v.w, gg.w), d);
+  }
+  ss = block_sum(ss, sh);
+  if (threadIdx.x == 0) ssq[row] = ss;
+}
+
+__global__ void embed_kernel(Dims dm, SeqState st, const Row* __restrict__ rows, const int* __restrict__ prompt,
+                             const int* __restrict__ prompt_off, const bf16* __restrict__ E, float* __restrict__ x,
+                             const float* __restrict__ g, bf16* __restrict__ a, float* __restrict__ ssq) {
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
+  const int row = blockIdx.x, d = dm.d;
+  const Row r = rows[row];
+  int tok = r.p == 0 ? dm.n_bins : prompt[prompt_off[r.b] + r.p - 1];
+  if (tok < 0 || tok >= dm.V) {                      // never index outside the table
+    if (threadIdx.x == 0) atomicExch(st.status, -1);
+    tok = dm.n_bins + 2;
+  }
+  float4* xr = reinterpret_cast<float4*>(x + (size_t)row * d);
+  const __nv_bfloat162* er = reinterpret_cast<const __nv_bfloat162*>(E + (size_t)tok * d);
+  for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
+    const float2 lo = __bfloat1622float2(er[2 * i]), hi = __bfloat1622float2(er[2 * i + 1]);
+    xr[i] = make_float4(lo.x, lo.y, hi.x, hi.y);
+  }
+  entry_row(xr, row, d, g, a, ssq);                  // every thread reads the columns it wrote
+}
+
+// operand rows of a shorten GEMM: row u of level `lu` <- hiddens 3u-2, 3u-1, 3u of the level below,
+// from its residual rows or, before the segment, from the carry ring; grid (rows of the level, 3)
+__global__ void gather_kernel(Dims dm, const Seg* __restrict__ segs, const Row* __restrict__ rows, int lu,
+                              const float* __restrict__ x_low, const float* __restrict__ ring, bf16* __restrict__ out) {
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
+  const int row = blockIdx.x, part = blockIdx.y, d = dm.d, lb = lu - 1, rs = fm_ring(lb);
+  const Row r = rows[row];
+  const Seg& s = segs[r.seg];
+  const int pos = 3 * r.p - 2 + part;
+  const float4* src = reinterpret_cast<const float4*>(pos >= s.p0[lb] ? x_low + (size_t)(s.r0[lb] + pos - s.p0[lb]) * d
+                                                                      : ring + ((size_t)r.b * rs + ((pos + rs) % rs)) * d);
+  bf16* o = out + (size_t)row * 6 * d + part * d;
+  for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
+    const float4 v = pos >= 0 ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    tc::store_hi_lo2(o + 4 * i, v.x, v.y, 3 * d);
+    tc::store_hi_lo2(o + 4 * i + 2, v.z, v.w, 3 * d);
+  }
+}
+
+// x[row] (the pre-shorten hidden) += its parent's upsampled slot; the last hiddens and triples of a
+// segment go into the carry rings for what comes after it; operand row and sum of squares for the stack
+// above.  The parent of every row is a row of the same segment.
+__global__ void upsample_kernel(Dims dm, const Seg* __restrict__ segs, const Row* __restrict__ rows, int level,
+                                const float* __restrict__ tri, float* __restrict__ h_ring, float* __restrict__ tri_ring,
+                                float* __restrict__ x, const float* __restrict__ g, bf16* __restrict__ a, float* __restrict__ ssq) {
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
+  const int row = blockIdx.x, d = dm.d, rs = fm_ring(level), rsu = fm_ring(level + 1);
+  const Row r = rows[row];
+  const Seg& s = segs[r.seg];
+  const int up = r.p / 3, slot = r.p - 3 * up;
+  const float4* t = reinterpret_cast<const float4*>(tri + ((size_t)(s.r0[level + 1] + up - s.p0[level + 1]) * 3 + slot) * d);
+  float4* xr = reinterpret_cast<float4*>(x + (size_t)row * d);
+  float4* hr = r.p >= s.p0[level] + s.n[level] - rs ? reinterpret_cast<float4*>(h_ring + ((size_t)r.b * rs + r.p % rs) * d) : nullptr;
+  // a triple is stored whole, by the block of its first child (its other children may lie behind the segment)
+  float4* tr = slot == 0 && up >= s.p0[level + 1] + s.n[level + 1] - rsu ? reinterpret_cast<float4*>(tri_ring + ((size_t)r.b * rsu + up % rsu) * 3 * d) : nullptr;
+  for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
+    const float4 h = xr[i], u = t[i];
+    if (hr != nullptr) hr[i] = h;
+    if (tr != nullptr) { tr[i] = u; tr[d / 4 + i] = t[d / 4 + i]; tr[d / 2 + i] = t[d / 2 + i]; }
+    xr[i] = make_float4(h.x + u.x, h.y + u.y, h.z + u.z, h.w + u.w);
+  }
+  entry_row(xr, row, d, g, a, ssq);
+}
+
+// the residual row of a prompt's last position, as it enters the last layer of a stack (split node)
+__global__ void stash_kernel(Dims dm, const Seg* __restrict__ segs, int level, const float* __restrict__ x, float* __restrict__ ring) {
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
+  const Seg& s = segs[blockIdx.x];
+  if (!s.last) return;
+  const int k = s.n[level] - 1, p = s.p0[level] + k, rs = fm_ring(level);
+  const float4* src = reinterpret_cast<const float4*>(x + (size_t)(s.r0[level] + k) * dm.d);
+  float4* dst = reinterpret_cast<float4*>(ring + ((size_t)s.b * rs + p % rs) * dm.d);
+  for (int i = threadIdx.x; i < dm.d / 4; i += blockDim.x) dst[i] = src[i];
+}
+
+// keys and values of the chunk -> cache, where its attention still needed entries that they replace
+__global__ void cache_kernel(Dims dm, const Seg* __restrict__ segs, const Row* __restrict__ rows, int level, const bf16* __restrict__ kbuf,
+                             const bf16* __restrict__ vbuf, bf16* __restrict__ Kc, bf16* __restrict__ Vc) {
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
+  const int row = blockIdx.x, cap = dm.cap[level], kvw = dm.Hkv * dm.dh;
+  const Row r = rows[row];
+  const Seg& s = segs[r.seg];
+  if (r.p < s.p0[level] + s.n[level] - cap) return;          // a later row of the segment takes this slot
+  const int slots = dm.P + cap;
+  for (int i = threadIdx.x; i < kvw / 8; i += blockDim.x) {
+    const int hk = 8 * i / dm.dh, c = 8 * i - hk * dm.dh;
+    const size_t to = (((size_t)r.b * dm.Hkv + hk) * slots + dm.P + r.slot) * dm.dh + c;
+    *reinterpret_cast<uint4*>(Kc + to) = reinterpret_cast<const uint4*>(kbuf + (size_t)row * kvw)[i];
+    *reinterpret_cast<uint4*>(Vc + to) = reinterpret_cast<const uint4*>(vbuf + (size_t)row * kvw)[i];
+  }
+}
+
+// operand row and sum of squares of a prompt's last position -> row b of the logits GEMM
+__global__ void last_rows_kernel(Dims dm, const Seg* __restrict__ segs, const bf16* __restrict__ a, const float* __restrict__ ssq,
+                                 int ssq_n, int ld, bf16* __restrict__ a_out, float* __restrict__ ssq_out) {
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
+  const Seg& s = segs[blockIdx.x];
+  if (!s.last) return;
+  const int row = s.r0[0] + s.n[0] - 1;
+  const uint4* src = reinterpret_cast<const uint4*>(a + (size_t)row * 2 * dm.d);
+  uint4* dst = reinterpret_cast<uint4*>(a_out + (size_t)s.b * 2 * dm.d);
+  for (int i = threadIdx.x; i < dm.d / 4; i += blockDim.x) dst[i] = src[i];
+  if (threadIdx.x == 0) {
+    float t = 0.f;
+    for (int k = 0; k < ssq_n; ++k) t += ssq[(size_t)k * ld + row];
+    ssq_out[s.b] = t;
+  }
+}
+
+// state behind the prompt: the first main token is the argmax of the last position
+__global__ void finish_kernel(Dims dm, SeqState st, const float* __restrict__ logits, const int* __restrict__ prompt,
+                              const int* __restrict__ prompt_off) {
+  ptx::grid_dep_launch();
+  ptx::grid_dep_wait();
+  const int b = blockIdx.x, n = st.plen[b];
+  const Top2 t = block_top2(logits + (size_t)b * dm.Vpad, dm, n);
+  for (int i = max(0, n - FM_HIST) + threadIdx.x; i < n; i += blockDim.x) st.hist[b * FM_HIST + (i & (FM_HIST - 1))] = prompt[prompt_off[b] + i];
+  if (threadIdx.x == 0) { st.L[b] = n + 1; st.main_tok[b] = t.i1; }
+}
+
+// ------------------------------------------------------------------------------------------
+// conditioning
+// ------------------------------------------------------------------------------------------
+// operand rows of the prefix projections: a[z][row] = bf16(rms(c_row) * g1 of layer z); grid (rows, layer groups)
+__global__ void prefix_norm_kernel(const float* __restrict__ c, const LayerPtr* __restrict__ layers, int n_layers, int rows_layer,
+                                   bf16* __restrict__ a, int d, float eps) {
+  __shared__ float sh[32];
+  const float* xr = c + (size_t)blockIdx.x * d;              // caller memory: only known to be float-aligned
+  float ss = 0.f;
+  for (int i = threadIdx.x; i < d / 4; i += blockDim.x) { const float4 v = make_float4(xr[4 * i], xr[4 * i + 1], xr[4 * i + 2], xr[4 * i + 3]); ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w; }
+  ss = block_sum(ss, sh);
+  const float inv = rsqrtf(ss / (float)d + eps);
+  for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
+    const float4 v = make_float4(xr[4 * i], xr[4 * i + 1], xr[4 * i + 2], xr[4 * i + 3]);
+    for (int z = blockIdx.y; z < n_layers; z += gridDim.y) {
+      const float4 g = reinterpret_cast<const float4*>(layers[z].g1)[i];
+      uint2 o;
+      o.x = ptx::pack_bf16(v.x * inv * g.x, v.y * inv * g.y);
+      o.y = ptx::pack_bf16(v.z * inv * g.z, v.w * inv * g.w);
+      *reinterpret_cast<uint2*>(a + ((size_t)z * rows_layer + blockIdx.x) * d + 4 * i) = o;
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// attention
+// ------------------------------------------------------------------------------------------
+// Causal attention of a chunk's rows.  A CTA takes 128 query rows (eight warps of 16) of one segment and
+// head; a producer warp streams first the cache entries of earlier chunks (prefix slots included),
+// then the keys and values of the chunk itself through a ring of TMA stages.  The chunk's own entries
+// come from the cache too, except where a windowed level's ring would give a slot to a new position
+// while an earlier row of the chunk still needs the old one: then they come from the projection's
+// output, and the cache is written afterwards.
+struct Attn {
+  Dims dm;
+  const Seg* segs; const int2* tiles;        // (segment, first query row)
+  int level;
+  const bf16* q;                             // [rows, H*dh], rotated and scaled by log2(e)/sqrt(dh)
+  const CUtensorMap *tmK, *tmV;              // cache as 2-D [B*Hkv*slots, dh], box C x 64
+  const CUtensorMap *tmKn, *tmVn;            // the chunk's [rows, Hkv*dh], same box; null: they are in the cache already
+  bf16* out;                                 // [rows, 2*H*dh] as [hi | lo]
+  int* status;
+};
+
+// QW of the eight warps share a key, the others split the keys of a tile among them and are merged at
+// the end: few rows then still make enough CTAs, each with a short chain of key steps.
+template <int DH, int C, int QW>
+struct AttnCfg {
+  static constexpr int NW = 8, KW = NW / QW, STAGES = 3, SUB = C / KW < 64 ? C / KW : 64, HALVES = DH / 64;
+  static_assert(SUB >= 16, "a warp takes at least 16 keys of a tile");
+  static constexpr int ROWS = QW * 16;
+  static constexpr int TILE = C * DH * 2, STAGE = 2 * TILE;
+  static constexpr int BYTES = STAGES * STAGE + 64 + 1024;
+  static constexpr int THREADS = (NW + 1) * 32;
+};
+
+template <int DH, int C, int QW>
+__global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1) attn_kernel(const Attn a) {
+  using CF = AttnCfg<DH, C, QW>;
+  constexpr int NW = CF::NW, KS = DH / 16, SUB = CF::SUB, KW = CF::KW;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + CF::STAGES * CF::STAGE);
+  uint64_t* empty = full + CF::STAGES;
+  __shared__ int s_fail;
+  const Dims& dm = a.dm;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
+  const int h = blockIdx.x, hk = h / (dm.H / dm.Hkv), level = a.level;
+  ptx::grid_dep_launch();
+  // (segments and tiles were written before the pass)
+  const int2 tile = a.tiles[blockIdx.y];
+  const Seg& sg = a.segs[tile.x];
+  const int b = sg.b, p0 = sg.p0[level], n = sg.n[level], r0 = sg.r0[level], q0 = tile.y, nq = min(CF::ROWS, n - q0);
+  const int P = dm.P, cap = dm.cap[level], W = dm.window[level], slots = P + cap;
+  const int used = P + min(cap, p0);                         // cache slots that earlier chunks have filled
+  const bool linear = p0 <= cap;
+  const int q_last = q0 + nq - 1, vis_lo = W > 0 ? max(0, p0 + q0 - W + 1) : 0;      // lowest position any row sees
+  // key tiles: [0, tp) prefix (and what shares its last tile), [tc0, tc1) cache, [tn0, tn1) this chunk
+  const int tc1 = (used + C - 1) / C, tp = min(tc1, (P + C - 1) / C);
+  const int tc0 = linear ? max(tp, min(tc1, (P + vis_lo) / C)) : tp;
+  const int tn0 = max(0, vis_lo - p0) / C, tn1 = q_last / C + 1;
+  const int n_old = tp + tc1 - tc0, n_tiles = n_old + tn1 - tn0;
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    for (int i = 0; i < CF::STAGES; ++i) { ptx::mbar_init(full + i, 1); ptx::mbar_init(empty + i, NW); }
+    ptx::fence_mbar_init();
+  }
+  __syncthreads();
+  if (warp == NW) {
+    if (lane == 0) {
+      ptx::grid_dep_wait();
+      for (int i = 0; i < n_tiles; ++i) {
+        const int st = i % CF::STAGES;
+        if (i >= CF::STAGES && !ptx::mbar_wait(empty + st, ((i / CF::STAGES) - 1) & 1)) { s_fail = 1; break; }
+        unsigned char* Ks = sm + st * CF::STAGE;
+        unsigned char* Vs = Ks + CF::TILE;
+        ptx::mbar_expect_tx(full + st, CF::STAGE);
+        const bool old = i < n_old, cached = old || a.tmKn == nullptr;
+        const int row = !cached ? r0 + (tn0 + i - n_old) * C
+                                : (b * dm.Hkv + hk) * slots + (i < tp ? i * C : old ? (tc0 + i - tp) * C : P + p0 + (tn0 + i - n_old) * C);
+        const CUtensorMap* mk = cached ? a.tmK : a.tmKn;
+        const CUtensorMap* mv = cached ? a.tmV : a.tmVn;
+#pragma unroll
+        for (int hf = 0; hf < CF::HALVES; ++hf) {
+          const int x = cached ? hf * 64 : hk * DH + hf * 64;
+          ptx::tma_load_2d(Ks + hf * C * 128, mk, x, row, full + st);
+          ptx::tma_load_2d(Vs + hf * C * 128, mv, x, row, full + st);
+        }
+      }
+    }
+    __syncwarp();
+  } else {
+    ptx::grid_dep_wait();
+    uint32_t qa[KS][4];
+    const int qw = warp % QW, kw = warp / QW;
+    const int w0 = q0 + qw * 16;                             // this warp's first query row of the segment
+    const bool live = qw * 16 < nq;
+#pragma unroll
+    for (int hr = 0; hr < 2; ++hr) {
+      const int i = g + hr * 8;
+      const bool ok = qw * 16 + i < nq;
+      const bf16* qp = a.q + ((size_t)(r0 + w0 + (ok ? i : 0)) * dm.H + h) * DH;
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) {
+        qa[ks][hr] = ok ? *reinterpret_cast<const uint32_t*>(qp + ks * 16 + 2 * t4) : 0u;
+        qa[ks][2 + hr] = ok ? *reinterpret_cast<const uint32_t*>(qp + ks * 16 + 8 + 2 * t4) : 0u;
+      }
+    }
+    float o[DH / 8][4];
+    float mrun[2] = {-INFINITY, -INFINITY}, lrun[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < DH / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+    const int wrap_q = p0 > 0 ? (p0 - 1) / cap : 0, wrap_r = p0 - 1 - wrap_q * cap;
+    const int pr_lo = p0 + w0, pr_hi = pr_lo + 15;           // positions of the warp's rows
+    for (int i = 0; i < n_tiles; ++i) {
+      const int st = i % CF::STAGES;
+      const bool old = i < n_old;
+      const int k0 = old ? (i < tp ? i : tc0 + i - tp) * C : (tn0 + i - n_old) * C;    // first slot, or first chunk row
+      if (!__all_sync(0xffffffffu, ptx::mbar_wait(full + st, (i / CF::STAGES) & 1))) { s_fail = 1; break; }
+      const uint32_t Ks_u = ptx::smem_u32(sm + st * CF::STAGE), Vs_u = Ks_u + CF::TILE;
+#pragma unroll 1
+      for (int sub = kw; sub < C / SUB; sub += KW) {
+        const int s_lo = k0 + sub * SUB, s_hi = s_lo + SUB - 1;
+        bool skip, all_vis;
+        if (old) {
+          skip = s_lo >= used || (linear && s_lo >= P && W > 0 && s_hi - P < pr_lo - W + 1);
+          all_vis = s_hi < P || (linear && s_hi < used && (W == 0 || max(s_lo - P, 0) >= pr_hi - W + 1));
+        } else {
+          skip = p0 + s_lo > pr_hi || (W > 0 && p0 + s_hi < pr_lo - W + 1);
+          all_vis = p0 + s_hi <= pr_lo && (W == 0 || p0 + s_lo >= pr_hi - W + 1);
+        }
+        if (skip || !live) continue;                         // the same for the whole warp
+        float s[SUB / 8][4];
+#pragma unroll
+        for (int nt = 0; nt < SUB / 8; ++nt) s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+#pragma unroll
+        for (int kb = 0; kb < SUB / 16; ++kb)
+#pragma unroll
+          for (int ks = 0; ks < KS; ++ks) {
+            const int key = sub * SUB + kb * 16 + (lane & 7) + (lane >> 4) * 8;
+            const int ch = ks * 2 + ((lane >> 3) & 1);
+            uint32_t b0, b1, b2, b3;
+            ptx::ldmatrix_x4(b0, b1, b2, b3, Ks_u + (ch >> 3) * C * 128 + ptx::swz128(key, ch & 7));
+            ptx::mma_bf16_16816(s[2 * kb], qa[ks], b0, b1);
+            ptx::mma_bf16_16816(s[2 * kb + 1], qa[ks], b2, b3);
+          }
+        if (!all_vis) {
+#pragma unroll
+          for (int nt = 0; nt < SUB / 8; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const int k = s_lo + nt * 8 + 2 * t4 + e;      // slot or chunk row
+              int kp;                                        // its position; -1 prefix, -2 nothing there
+              if (old) {
+                const int r = k - P;
+                kp = k < P ? -1 : (k >= used ? -2 : (linear ? r : r + (r <= wrap_r ? wrap_q : wrap_q - 1) * cap));
+              } else {
+                kp = p0 + k;
+              }
+#pragma unroll
+              for (int hr = 0; hr < 2; ++hr) {
+                const int pr = pr_lo + g + hr * 8;
+                const bool vis = kp == -1 || (kp >= 0 && kp <= pr && (W == 0 || kp >= pr - W + 1));
+                if (!vis) s[nt][hr * 2 + e] = -INFINITY;
+              }
+            }
+        }
+        float scale[2], base[2];
+#pragma unroll
+        for (int hr = 0; hr < 2; ++hr) {
+          float mx = -INFINITY;
+#pragma unroll
+          for (int nt = 0; nt < SUB / 8; ++nt) mx = fmaxf(mx, fmaxf(s[nt][hr * 2], s[nt][hr * 2 + 1]));
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+          const float mnew = fmaxf(mrun[hr], mx);
+          base[hr] = mnew == -INFINITY ? 0.f : mnew;
+          scale[hr] = mnew == mrun[hr] ? 1.f : exp2f(mrun[hr] - base[hr]);
+          mrun[hr] = mnew;
+        }
+        float ls[2] = {0.f, 0.f};
+#pragma unroll
+        for (int nt = 0; nt < SUB / 8; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            s[nt][e] = exp2f(s[nt][e] - base[e >> 1]);
+            ls[e >> 1] += s[nt][e];
+          }
+#pragma unroll
+        for (int hr = 0; hr < 2; ++hr) lrun[hr] = lrun[hr] * scale[hr] + ls[hr];     // per lane; the quad is added at the end
+        if (__any_sync(0xffffffffu, scale[0] != 1.f || scale[1] != 1.f)) {
+#pragma unroll
+          for (int i2 = 0; i2 < DH / 8; ++i2) {
+            o[i2][0] *= scale[0]; o[i2][1] *= scale[0];
+            o[i2][2] *= scale[1]; o[i2][3] *= scale[1];
+          }
+        }
+#pragma unroll
+        for (int kb = 0; kb < SUB / 16; ++kb) {
+          uint32_t pa[4];
+          pa[0] = ptx::pack_bf16(s[2 * kb][0], s[2 * kb][1]);
+          pa[1] = ptx::pack_bf16(s[2 * kb][2], s[2 * kb][3]);
+          pa[2] = ptx::pack_bf16(s[2 * kb + 1][0], s[2 * kb + 1][1]);
+          pa[3] = ptx::pack_bf16(s[2 * kb + 1][2], s[2 * kb + 1][3]);
+#pragma unroll
+          for (int dp = 0; dp < DH / 16; ++dp) {
+            const int key = sub * SUB + kb * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
+            const int ch = dp * 2 + (lane >> 4);
+            uint32_t b0, b1, b2, b3;
+            ptx::ldmatrix_x4_trans(b0, b1, b2, b3, Vs_u + (ch >> 3) * C * 128 + ptx::swz128(key, ch & 7));
+            ptx::mma_bf16_16816(o[2 * dp], pa, b0, b1);
+            ptx::mma_bf16_16816(o[2 * dp + 1], pa, b2, b3);
+          }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(empty + st);
+    }
+#pragma unroll
+    for (int hr = 0; hr < 2; ++hr) {
+      lrun[hr] += __shfl_xor_sync(0xffffffffu, lrun[hr], 1);
+      lrun[hr] += __shfl_xor_sync(0xffffffffu, lrun[hr], 2);
+    }
+    if (KW == 1) {
+#pragma unroll
+      for (int hr = 0; hr < 2; ++hr) {
+        const float inv = 1.f / lrun[hr];
+        const int i = g + hr * 8;
+        if (qw * 16 + i < nq) {
+          bf16* op = a.out + ((size_t)(r0 + w0 + i) * 2 * dm.H + h) * DH;
+#pragma unroll
+          for (int c = 0; c < DH / 8; ++c) tc::store_hi_lo2(op + c * 8 + 2 * t4, o[c][hr * 2] * inv, o[c][hr * 2 + 1] * inv, dm.H * DH);
+        }
+      }
+    } else {
+      asm volatile("bar.sync 1, 256;" ::: "memory");         // the compute warps are done with the ring
+      float* mine = reinterpret_cast<float*>(sm) + warp * 16 * (DH + 2);      // [16][DH + 2]: output, maximum, sum
+#pragma unroll
+      for (int hr = 0; hr < 2; ++hr) {
+        float* row = mine + (g + hr * 8) * (DH + 2);
+#pragma unroll
+        for (int c = 0; c < DH / 8; ++c) *reinterpret_cast<float2*>(row + c * 8 + 2 * t4) = make_float2(o[c][hr * 2], o[c][hr * 2 + 1]);
+        if (t4 == 0) { row[DH] = mrun[hr]; row[DH + 1] = lrun[hr]; }
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      const float* base = reinterpret_cast<const float*>(sm);
+      for (int e = threadIdx.x; e < nq * (DH / 2); e += NW * 32) {
+        const int i = e / (DH / 2), c = 2 * (e - i * (DH / 2));
+        const float* row = base + ((i >> 4) * 16 + (i & 15)) * (DH + 2);
+        float m = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) m = fmaxf(m, row[k * QW * 16 * (DH + 2) + DH]);
+        float l = 0.f, o0 = 0.f, o1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < KW; ++k) {
+          const float* r = row + k * QW * 16 * (DH + 2);
+          const float w = r[DH] == -INFINITY ? 0.f : exp2f(r[DH] - m);
+          l += w * r[DH + 1];
+          o0 += w * r[c];
+          o1 += w * r[c + 1];
+        }
+        const float inv = 1.f / l;
+        tc::store_hi_lo2(a.out + ((size_t)(r0 + q0 + i) * 2 * dm.H + h) * DH + c, o0 * inv, o1 * inv, dm.H * DH);
+      }
+    }
+  }
+  __syncthreads();
+  if (s_fail) {                                              // a bounded wait gave up: report
+    if (threadIdx.x == 0) atomicExch(a.status, -5);
+    ptx::drain_delay();
+  }
+}
+
+}  // namespace pf

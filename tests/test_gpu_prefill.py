@@ -1,0 +1,39 @@
+"""The packed prefill against the oracle at the sizes where it changes form: one query tile and a row more, the
+last size of the split-K GEMMs and the first of the tiled ones, ragged batches, windows whose ring is shorter
+than a chunk (keys of the chunk outside the cache), more positions than one chunk holds."""
+import numpy as np
+import pytest
+
+import fm_synth as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("faces,window,kw", [
+    ((0, 1, 3), (0, 0, 0), {}),
+    ((14, 15), (0, 0, 0), {}),                                        # 127 and 136 rows
+    ((28, 1), (0, 0, 0), {"n_kv_heads": 1}),                          # 263 rows together
+    ((29, 120, 2), (0, 0, 0), {}),
+    ((40, 7), (30, 11, 5), {}),                                       # rings shorter than the prompt
+    ((100,), (50, 0, 3), {"n_kv_heads": 1}),
+    ((90, 20), (0, 0, 0), {"n_heads": 1, "n_kv_heads": 1, "head_dim": 128}),
+    ((60,), (20, 9, 0), {"n_heads": 1, "n_kv_heads": 1, "head_dim": 128}),
+    ((35, 2), (0, 0, 0), {"d_model": 192, "d_ff": 320}),              # partly empty last tiles
+    ((950, 30), (0, 0, 0), {}),                                       # cut into two chunks
+    ((950,), (700, 0, 0), {}),                                        # two chunks and a ring that wraps
+])
+def test_prefill_lockstep(faces, window, kw):
+    from oracle.lockstep import run_lockstep
+    from paper_2511_15618_b200 import FlashMesh
+    B, D = len(faces), 9
+    base = dict(d_model=128, n_heads=2, n_kv_heads=2, head_dim=64, d_ff=256, weight_std=0.1, out_std=0.02)
+    base.update(kw)
+    cfg = S.toy_config(**base, draft_len=D, layers=(1, 2, 2, 1, 2), window=window, max_batch=B, batch=B, gen_faces=2,
+                       max_tokens=1 + 9 * (max(faces) + 4) + D + 2)
+    w = S.make_weights(cfg)
+    conds = [S.make_condition(cfg, b) for b in range(B)]
+    prompts = [S.fill_prompt(cfg, b, f) if f else [] for b, f in enumerate(faces)]
+    dev = FlashMesh(cfg, w)
+    rep = run_lockstep(cfg, w, conds, prompts, dev, 2, 60, prefill_chunk=512)
+    assert rep["done"] and rep["emitted"] == 18 * B and dev.device_status() == 0
+    print(faces, {k: rep[k] for k in ("steps", "max_logit_err", "max_draft_err", "overrides")})
