@@ -19,6 +19,7 @@
 #include "fm_attention.cuh"
 #include "fm_common.cuh"
 #include "fm_gemm_tc.cuh"
+#include "fm_gemm_rows.cuh"
 #include "fm_kernels.cuh"
 #include "fm_prefill.cuh"
 
@@ -90,7 +91,7 @@ struct fm_ctx {
   size_t tmaps_cap, tmaps_uploaded;
   // per-tile sums of squares of the residual rows (RMSNorm statistics handed between GEMMs)
   float* ssq;
-  int ssq_n, ssq_ld;    // slots the last producer filled, floats between slots
+  int ssq_n, ssq_ld;    // slots the last producer filled, floats between rows
   bool use_pdl;
   bool debug_sync;      // FM_DEBUG_SYNC: wait for and check every launch
   // prefill: activations of one chunk (see fm_prefill.cuh)
@@ -123,6 +124,7 @@ struct fm_ctx {
   int only_class;       // -1, or the kernel class (ProfClass) that alone is launched (fm_profile_class)
   int cur_class;        // class of the launch being enqueued
   double class_bytes;   // weight bytes of the GEMM launches enqueued by fm_profile_class
+  int rows_max;         // rows up to which the few-row GEMM is used
   int split_target;     // CTAs a GEMM launch aims for (M tiles x K splits)
   int stage_cap;        // tuning knob: upper bound on the GEMM ring depth (0 = none)
   int n_sm;                                  // SMs of the device
@@ -256,8 +258,8 @@ void carve(fm_ctx* c, Carver& cv) {
   const size_t Rc = align_up(B * dm.R1, 16), Rv = align_up(B * dm.mv, 16), Rf = align_up(B * dm.mf, 16);
   c->xc = cv.take<float>(Rc * d); c->xv = cv.take<float>(Rv * d); c->xf = cv.take<float>(Rf * d);
   c->qbuf = cv.take<bf16>(Rc * hd);
-  c->ssq_ld = (int)Rc;
-  c->ssq = cv.take<float>((size_t)((d + 127) / 128) * tc::MAX_SPLIT * Rc);
+  c->ssq_ld = (int)((d + 127) / 128 * 16);                   // a slot per 8 features, at most
+  c->ssq = cv.take<float>((size_t)c->ssq_ld * Rc);
   c->logits = cv.take<float>(Rc * dm.Vpad); c->tmp3d = cv.take<float>(Rv * 3 * d);
   // GEMM operand rows of the backbone hold two bfloat16 terms per value: [hi | lo]
   c->a_norm = cv.take<bf16>(Rc * 2 * d); c->a_up = cv.take<bf16>(Rc * 2 * d); c->a_cat = cv.take<bf16>(Rv * 6 * d); c->a_cat2 = cv.take<bf16>(Rf * 6 * d);
@@ -349,7 +351,7 @@ void carve(fm_ctx* c, Carver& cv) {
     pr.rows[1] = (int)align_up(R / 3 + B + 16, 128);
     pr.rows[2] = (int)align_up(R / 9 + B + 16, 128);
     for (int l = 0; l < 3; ++l) { pr.x[l] = cv.take<float>(pr.rows[l] * d); pr.map[l] = cv.take<pf::Row>(pr.rows[l]); }
-    pr.ssq = cv.take<float>((d + 127) / 128 * tc::MAX_SPLIT * R);
+    pr.ssq = cv.take<float>((size_t)c->ssq_ld * R);
     pr.a = cv.take<bf16>(R * 2 * d);
     pr.q = cv.take<bf16>(R * hd);
     pr.kbuf = cv.take<bf16>(R * dm.Hkv * dm.dh);
@@ -602,16 +604,60 @@ tc::Epi epi_plain(void* out, int ldo) {
   return e;
 }
 
-// y[n][m] = W[w_row0 + m, :] . A[a_row0 + n, :], n < R, m < M, finished by the epilogue `mode`
-// (see fm_gemm_tc.cuh).  W: packed weight slabs of a matrix with K columns (w_row0 a multiple of
-// 128), A: [a_rows_alloc, a_parts * K] bf16 (rows padded to 16; a_parts = 2: [hi | lo] terms).  The
-// K split (= cluster size) depends on the shapes only.
-void gemm(fm_ctx* c, const bf16* W, size_t w_rows_alloc, int w_row0, const bf16* A, size_t a_rows_alloc, int a_row0,
-          int M, int K, int R, const int* n_active, int mode, tc::Epi e, int a_parts = 1, int stacked = 1, int z_rows = 0,
-          int z_w_rows = 0) {
-  if (R <= 0) return;
-  (void)w_rows_alloc;
-  if (w_row0 % tc::BM != 0) { c->launch_error = FM_ERR_UNSUPPORTED; return; }
+template <int MODE>
+void launch_rows(fm_ctx* c, int mtn, int fj, dim3 grid, int smem, const rg::Args& g, const tc::Epi& e) {
+  const dim3 one(1, 1, 1);
+  if (mtn == 1) {
+    if (fj == 1) launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 1, 1>, grid, rg::THREADS, smem, g, e);
+    else if (fj == 2) launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 1, 2>, grid, rg::THREADS, smem, g, e);
+    else launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 1, 4>, grid, rg::THREADS, smem, g, e);
+  } else {
+    if (fj == 1) launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 2, 1>, grid, rg::THREADS, smem, g, e);
+    else if (fj == 2) launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 2, 2>, grid, rg::THREADS, smem, g, e);
+    else launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 2, 4>, grid, rg::THREADS, smem, g, e);
+  }
+}
+// The few-row form (fm_gemm_rows.cuh), with as few features per CTA as give every SM at most one CTA.  For
+// up to 16 rows (above that the operand rows that every CTA reads cost more than the cluster exchange of the
+// other form: 24 rows 4.0 / 9.8 us for the output projection and the second FFN matrix) whose weights per
+// CTA fit beside a neighbour's; returns false where it does not apply.
+bool gemm_rows(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, int a_row0, int M, int K, int R, const int* n_active, int mode,
+               const tc::Epi& e, int parts, int stacked, int z_rows, int z_w_rows) {
+  if (R > c->rows_max || M < 8) return false;
+  int FT = 8;
+  while (FT < 32 && (M + FT - 1) / FT * stacked > c->n_sm) FT *= 2;
+  const int mtn = (parts * R + 15) / 16, smem = rg::smem_bytes(FT, K, mtn);
+  if (smem > 100 * 1024) return false;
+  if (e.ssq_out != nullptr && c->dm.d % FT != 0) return false;
+  const rg::Args g{W, A, parts * K, M, K, R, parts, w_row0 / tc::BM, a_row0, stacked > 1 ? z_rows : 0, stacked > 1 ? z_w_rows / tc::BM : 0,
+                   n_active, c->st.status};
+  const dim3 grid((M + FT - 1) / FT, stacked);
+  switch (mode) {
+    case tc::EPI_F32: launch_rows<tc::EPI_F32>(c, mtn, FT / 8, grid, smem, g, e); break;
+    case tc::EPI_BF16: launch_rows<tc::EPI_BF16>(c, mtn, FT / 8, grid, smem, g, e); break;
+    case tc::EPI_GELU: launch_rows<tc::EPI_GELU>(c, mtn, FT / 8, grid, smem, g, e); break;
+    case tc::EPI_RESID: launch_rows<tc::EPI_RESID>(c, mtn, FT / 8, grid, smem, g, e); break;
+    case tc::EPI_RESID_CAT: launch_rows<tc::EPI_RESID_CAT>(c, mtn, FT / 8, grid, smem, g, e); break;
+    case tc::EPI_UP: launch_rows<tc::EPI_UP>(c, mtn, FT / 8, grid, smem, g, e); break;
+    default: launch_rows<tc::EPI_QKV>(c, mtn, FT / 8, grid, smem, g, e); break;
+  }
+  if (e.ssq_out != nullptr) c->ssq_n = c->dm.d / FT;         // slots the next consumer adds
+  return true;
+}
+
+template <int MODE>
+cudaError_t allow_rows_smem() {
+  const int most = 101 * 1024;
+  cudaError_t r = cudaSuccess;
+  auto set = [&](const void* k) { if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most); };
+  set((const void*)rg::gemm_rows_kernel<MODE, 1, 1>); set((const void*)rg::gemm_rows_kernel<MODE, 1, 2>); set((const void*)rg::gemm_rows_kernel<MODE, 1, 4>);
+  set((const void*)rg::gemm_rows_kernel<MODE, 2, 1>); set((const void*)rg::gemm_rows_kernel<MODE, 2, 2>); set((const void*)rg::gemm_rows_kernel<MODE, 2, 4>);
+  return r;
+}
+
+// The tensor-memory form (fm_gemm_tc.cuh).  The K split (= cluster size) depends on the shapes only.
+void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_rows_alloc, int a_row0, int M, int K, int R,
+                const int* n_active, int mode, tc::Epi e, int a_parts, int stacked, int z_rows, int z_w_rows) {
   const int tiles = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
   // Few rows: one N tile, K split over a cluster so that enough SMs stream weights.  Many rows:
   // N tiles of 32 rows as well (each weight slab then comes from HBM once and from L2 for the other
@@ -639,14 +685,11 @@ void gemm(fm_ctx* c, const bf16* W, size_t w_rows_alloc, int w_row0, const bf16*
     const int fit = (112 * 1024 - tc::smem_bytes(N, 0, a_parts, side_b)) / tc::stage_bytes(N, a_parts);
     stages = stages > fit ? (fit < 2 ? 2 : fit) : stages;
   }
-  const long pi = prof_open(c, PROF_GEMM, 2.0 * M * K);            // algorithmic bytes: the weight matrix once
   tc::Args g{W, c->tmaps + tA, M, K, N, R, split, stages, a_parts, w_row0 / tc::BM, a_row0, stacked > 1 ? z_rows : 0,
              stacked > 1 ? z_w_rows / tc::BM : 0, n_active, c->st.status};
   e.row0 = 0;
   const int smem = tc::smem_bytes(N, stages, a_parts, side_b);
   const dim3 grid(tiles, split, n_tiles), cl(1, split, 1);
-  c->cur_class = PROF_GEMM;
-  if (c->only_class == PROF_GEMM) c->class_bytes += 2.0 * M * K * (stacked > 1 ? stacked : 1);
   switch (mode) {
     case tc::EPI_F32: launch_pdl(c, cl, tc::gemm_tc_kernel<tc::EPI_F32, false>, grid, 128, smem, g, e); break;
     case tc::EPI_BF16: launch_pdl(c, cl, tc::gemm_tc_kernel<tc::EPI_BF16, false>, grid, 128, smem, g, e); break;
@@ -662,10 +705,26 @@ void gemm(fm_ctx* c, const bf16* W, size_t w_rows_alloc, int w_row0, const bf16*
       else launch_pdl(c, cl, tc::gemm_tc_kernel<tc::EPI_QKV, false>, grid, 128, smem, g, e);
       break;
   }
-  c->cur_class = PROF_OTHER;
-  prof_close(c, pi);
   if ((mode == tc::EPI_RESID || mode == tc::EPI_RESID_CAT) && e.ssq_out != nullptr) c->ssq_n = tiles * split * (split == 1 ? 2 : 1);     // slots the next consumer adds
   if (mode == tc::EPI_UP && e.ssq_out != nullptr) c->ssq_n = (c->dm.d / tc::BM) * split * (split == 1 ? 2 : 1);   // tiles within d
+}
+
+// y[n][m] = W[w_row0 + m, :] . A[a_row0 + n, :], n < R, m < M, finished by the epilogue `mode`
+// (see fm_gemm_tc.cuh).  W: packed weight slabs of a matrix with K columns (w_row0 a multiple of
+// 128), A: [a_rows_alloc, a_parts * K] bf16 (rows padded to 16; a_parts = 2: [hi | lo] terms).
+void gemm(fm_ctx* c, const bf16* W, size_t w_rows_alloc, int w_row0, const bf16* A, size_t a_rows_alloc, int a_row0,
+          int M, int K, int R, const int* n_active, int mode, tc::Epi e, int a_parts = 1, int stacked = 1, int z_rows = 0,
+          int z_w_rows = 0) {
+  if (R <= 0) return;
+  (void)w_rows_alloc;
+  if (w_row0 % tc::BM != 0) { c->launch_error = FM_ERR_UNSUPPORTED; return; }
+  const long pi = prof_open(c, PROF_GEMM, 2.0 * M * K);            // algorithmic bytes: the weight matrix once
+  c->cur_class = PROF_GEMM;
+  if (c->only_class == PROF_GEMM) c->class_bytes += 2.0 * M * K * (stacked > 1 ? stacked : 1);
+  if (!gemm_rows(c, W, w_row0, A, a_row0, M, K, R, n_active, mode, e, a_parts, stacked, z_rows, z_w_rows))
+    gemm_split(c, W, w_row0, A, a_rows_alloc, a_row0, M, K, R, n_active, mode, e, a_parts, stacked, z_rows, z_w_rows);
+  c->cur_class = PROF_OTHER;
+  prof_close(c, pi);
 }
 
 // rows fed at each level in this pass (n_active[level]); n_active[3] = unfinished sequences
@@ -761,7 +820,7 @@ void forward(fm_ctx* c, float* logits_out) {
     // parent belongs to an earlier pass that parent's stored slot.  Up: the upsampling GEMM's
     // epilogue adds slot r of parent u to child row 3u + r, whose residual row still holds the
     // pre-shorten hidden, and hands the child rows to the stack above.
-    LAUNCH(c, embed_kernel, Rc + 3 * (Rv + Rf), row_threads(d), 0, dm, c->st, B, c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, Rc,
+    LAUNCH(c, embed_kernel, Rc + 3 * (Rv + Rf), row_threads(d), 0, dm, c->st, B, c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc,
            (const float*)c->hc_ring, (const float*)c->hv_ring, c->a_cat, c->a_cat2, Rv, Rf);
     c->ssq_n = 1;
     tc::Epi cat{};
@@ -787,7 +846,7 @@ void forward(fm_ctx* c, float* logits_out) {
     eu.level = 1; eu.x = c->xc; eu.gain = c->layers[4][0].g1; eu.tri_ring = c->triv_ring;
     gemm(c, c->U_vc, pad128(3 * d), 0, c->a_norm, Rc_alloc, 0, 3 * d, d, Rv, na, tc::EPI_UP, eu, 2);
   } else {
-    LAUNCH(c, embed_kernel, Rc, row_threads(d), 0, dm, c->st, B, c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, Rc,
+    LAUNCH(c, embed_kernel, Rc, row_threads(d), 0, dm, c->st, B, c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc,
            (const float*)nullptr, (const float*)nullptr, (bf16*)nullptr, (bf16*)nullptr, 0, 0);
     c->ssq_n = 1;
     run_stack(c, 0, c->xc, nullptr, nullptr, false);
@@ -801,12 +860,12 @@ void forward(fm_ctx* c, float* logits_out) {
     run_stack(c, 2, c->xf, c->zf, nullptr, true);                  // leaves bf16(xf) in a_norm
     gemm(c, c->U_fv, pad128(3 * d), 0, c->a_norm, Rc_alloc, 0, 3 * d, d, Rf, na + 2, tc::EPI_F32, epi_plain(c->tmp3d, 3 * d), 2);
     launch_pdl(c, dim3(1, 1, 1), upsample_add_kernel, Rv + Rf, row_threads(d), 0, dm, c->st, B, 1, (const float*)c->hv_ring, (const float*)c->tmp3d,
-               c->trif_ring, c->xv, (const float*)c->layers[3][0].g1, c->a_norm, c->ssq, Rv);
+               c->trif_ring, c->xv, (const float*)c->layers[3][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rv);
     c->ssq_n = 1;
     run_stack(c, 3, c->xv, c->zv, nullptr, true);                  // leaves bf16(xv) in a_norm
     gemm(c, c->U_vc, pad128(3 * d), 0, c->a_norm, Rc_alloc, 0, 3 * d, d, Rv, na + 1, tc::EPI_F32, epi_plain(c->tmp3d, 3 * d), 2);
     launch_pdl(c, dim3(1, 1, 1), upsample_add_kernel, Rc + Rv, row_threads(d), 0, dm, c->st, B, 0, (const float*)c->hc_ring, (const float*)c->tmp3d,
-               c->triv_ring, c->xc, (const float*)c->layers[4][0].g1, c->a_norm, c->ssq, Rc);
+               c->triv_ring, c->xc, (const float*)c->layers[4][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc);
     c->ssq_n = 1;
   }
   run_stack(c, 4, c->xc, c->zc, c->g_out, true, nullptr, c->fuse_hourglass ? c->a_up : nullptr);   // leaves bf16(xc * g_out) and its sums of squares
@@ -1033,7 +1092,7 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
   const Dims& dm = c->dm;
   auto& pr = c->pre;
   const int level = STACK_LEVEL[s], R = ch.rows[level], d = dm.d, hd = dm.H * dm.dh, kvw = dm.Hkv * dm.dh, qkvw = hd + 2 * kvw;
-  const int nl = (int)c->layers[s].size(), ld = pr.rows[0];
+  const int nl = (int)c->layers[s].size(), ld = pr.rows[0], ldq = c->ssq_ld;
   const bool small = R <= PF_SMALL && ch.direct[level];
   float* x = pr.x[level];
   int tK = -1, tV = -1;
@@ -1049,9 +1108,9 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
       launch_pdl(c, dim3(1, 1, 1), pf::stash_kernel, ch.n_segs, row_threads(d / 4), 0, dm, ch.segs, level, (const float*)x, stash_ring);
     const float qscale = (float)(1.4426950408889634 / sqrt((double)dm.dh));
     pf::Epi eq{};
-    eq.ssq_in = pr.ssq; eq.ssq_n = c->ssq_n; eq.ld_ssq = ld; eq.inv_d = 1.f / d; eq.eps = dm.eps;
+    eq.ssq_in = pr.ssq; eq.ssq_n = c->ssq_n; eq.ld_ssq = ldq; eq.inv_d = 1.f / d; eq.eps = dm.eps;
     tc::Epi sq{};
-    sq.ssq_in = pr.ssq; sq.ssq_n = c->ssq_n; sq.ld_ssq = ld; sq.inv_d_in = 1.f / d; sq.eps = dm.eps;
+    sq.ssq_in = pr.ssq; sq.ssq_n = c->ssq_n; sq.ld_ssq = ldq; sq.inv_d_in = 1.f / d; sq.eps = dm.eps;
     if (small) {
       sq.dm = dm; sq.st = c->st; sq.batch = c->batch; sq.level = level; sq.rows = pr.map[level]; sq.rope_tab = c->rope_tab;
       sq.q_out = pr.q; sq.Kc = L.K; sq.Vc = L.V; sq.qscale = qscale;
@@ -1081,11 +1140,11 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
     const bool out2 = !last || want_a;
     if (small) {
       tc::Epi eo{};
-      eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq_out = ld;
+      eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq_out = ldq;
       gemm(c, L.Wo, pad128(d), 0, pr.attn, ld, 0, d, hd, R, nullptr, tc::EPI_RESID, eo, 2);
       tc::Epi e1 = epi_plain(pr.wide, 2 * dm.dff);
       e1.lo_off = dm.dff;
-      e1.ssq_in = pr.ssq; e1.ssq_n = c->ssq_n; e1.ld_ssq = ld; e1.inv_d_in = 1.f / d; e1.eps = dm.eps;
+      e1.ssq_in = pr.ssq; e1.ssq_n = c->ssq_n; e1.ld_ssq = ldq; e1.inv_d_in = 1.f / d; e1.eps = dm.eps;
       gemm(c, L.W1, pad128(dm.dff), 0, pr.a, ld, 0, dm.dff, d, R, nullptr, tc::EPI_GELU, e1, 2);
       eo.gain = gain2;
       if (!out2) { eo.a_out = nullptr; eo.ssq_out = nullptr; }
@@ -1093,7 +1152,7 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
       continue;
     }
     pf::Epi eo{};
-    eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq = ld;
+    eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq = ldq;
     pf_gemm(c, pf::PF_RESID, L.Wo, pr.attn, ld, d, hd, R, eo);
     eq.out = pr.wide; eq.ldo = 2 * dm.dff; eq.lo_off = dm.dff; eq.ssq_n = c->ssq_n;
     pf_gemm(c, pf::PF_GELU, L.W1, pr.a, ld, dm.dff, d, R, eq);
@@ -1112,7 +1171,7 @@ void pf_chunk(fm_ctx* c, const PfChunk& ch, const int* prompt, const int* prompt
   LAUNCH(c, pf::map_kernel, dim3(ch.n_segs, 3), 256, 0, dm, ch.segs, pr.map[0], pr.map[1], pr.map[2]);
   // (a full barrier: later prologues may read the maps before their dependency wait)
   LAUNCH(c, pf::embed_kernel, ch.rows[0], th, 0, dm, c->st, (const pf::Row*)pr.map[0], prompt, prompt_off, (const bf16*)c->E, pr.x[0],
-         (const float*)c->layers[0][0].g1, pr.a, pr.ssq);
+         (const float*)c->layers[0][0].g1, pr.a, pr.ssq, c->ssq_ld);
   c->ssq_n = 1;
   for (int up = 1; up <= 2; ++up) {                          // down: coordinate and vertex stacks, each followed by a shortening
     pf_stack(c, ch, up - 1, nullptr, nullptr, false);
@@ -1122,12 +1181,12 @@ void pf_chunk(fm_ctx* c, const PfChunk& ch, const int* prompt, const int* prompt
     if (ch.rows[up] <= PF_SMALL) {
       tc::Epi es{};
       es.x = pr.x[up]; es.ldx = d; es.add = 0; es.gain = c->layers[up][0].g1; es.a_out = pr.a; es.lda = 2 * d; es.lo_off = d;
-      es.ssq_out = pr.ssq; es.ld_ssq_out = pr.rows[0];
+      es.ssq_out = pr.ssq; es.ld_ssq_out = c->ssq_ld;
       gemm(c, S, pad128(d), 0, pr.wide, pr.rows[1], 0, d, 3 * d, ch.rows[up], nullptr, tc::EPI_RESID, es, 2);
     } else {
       pf::Epi es{};
       es.x = pr.x[up]; es.ldx = d; es.add = 0; es.gain = c->layers[up][0].g1; es.a_out = pr.a; es.lda = 2 * d; es.lo_off = d;
-      es.ssq_out = pr.ssq; es.ld_ssq = pr.rows[0];
+      es.ssq_out = pr.ssq; es.ld_ssq = c->ssq_ld;
       pf_gemm(c, pf::PF_RESID, S, pr.wide, pr.rows[1], d, 3 * d, ch.rows[up], es);
     }
   }
@@ -1143,12 +1202,12 @@ void pf_chunk(fm_ctx* c, const PfChunk& ch, const int* prompt, const int* prompt
     }
     launch_pdl(c, one, pf::upsample_kernel, ch.rows[low], th, 0, dm, ch.segs, (const pf::Row*)pr.map[low], low,
                (const float*)reinterpret_cast<float*>(pr.wide), low == 1 ? c->hv_ring : c->hc_ring, low == 1 ? c->trif_ring : c->triv_ring, pr.x[low],
-               (const float*)c->layers[low == 1 ? 3 : 4][0].g1, pr.a, pr.ssq);
+               (const float*)c->layers[low == 1 ? 3 : 4][0].g1, pr.a, pr.ssq, c->ssq_ld);
     c->ssq_n = 1;
     pf_stack(c, ch, low == 1 ? 3 : 4, low == 1 ? c->zv : c->zc, low == 1 ? nullptr : c->g_out, true);
   }
   if (ch.ends)
-    launch_pdl(c, one, pf::last_rows_kernel, ch.n_segs, 128, 0, dm, ch.segs, (const bf16*)pr.a, (const float*)pr.ssq, c->ssq_n, pr.rows[0], c->a_norm, c->ssq);
+    launch_pdl(c, one, pf::last_rows_kernel, ch.n_segs, 128, 0, dm, ch.segs, (const bf16*)pr.a, (const float*)pr.ssq, c->ssq_n, c->ssq_ld, c->a_norm, c->ssq);
 }
 
 int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off) {
@@ -1492,6 +1551,13 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
   TRYCUDA(cudaFuncSetAttribute(tc::gemm_tc_kernel<tc::EPI_RESID_CAT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::max_smem_bytes()));
   TRYCUDA(cudaFuncSetAttribute(tc::gemm_tc_kernel<tc::EPI_UP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::max_smem_bytes()));
   TRYCUDA(cudaFuncSetAttribute(tc::gemm_tc_kernel<tc::EPI_QKV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::max_smem_bytes()));
+  TRYCUDA(allow_rows_smem<tc::EPI_F32>());
+  TRYCUDA(allow_rows_smem<tc::EPI_BF16>());
+  TRYCUDA(allow_rows_smem<tc::EPI_GELU>());
+  TRYCUDA(allow_rows_smem<tc::EPI_RESID>());
+  TRYCUDA(allow_rows_smem<tc::EPI_RESID_CAT>());
+  TRYCUDA(allow_rows_smem<tc::EPI_UP>());
+  TRYCUDA(allow_rows_smem<tc::EPI_QKV>());
   {
     const int most = 216 * 1024;                             // a ring of at most 200 KB and what lies behind it
     TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_F32, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
@@ -1538,6 +1604,8 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
     c->debug_sync = ds != nullptr && ds[0] == '1';
     const char* ncg = getenv("FM_NO_CALL_GRAPH");
     c->call_graphs_off = ncg != nullptr && ncg[0] == '1';
+    const char* rm = getenv("FM_ROWS_MAX");
+    c->rows_max = rm != nullptr && atoi(rm) < rg::MAX_ROWS ? atoi(rm) : rg::MAX_ROWS;
     const char* t = getenv("FM_SPLIT_TARGET");
     c->split_target = t != nullptr && atoi(t) > 0 ? atoi(t) : 160;
     int dev = 0, sms = 148;

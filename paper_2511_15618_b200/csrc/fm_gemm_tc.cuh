@@ -69,7 +69,7 @@ struct Args {
 
 struct Epi {
   int row0;                      // first output row of this launch (N tiles beyond the first)
-  const float* ssq_in;           // [ssq_n][ld_ssq] partial sums of squares of the operand rows; null = no scale
+  const float* ssq_in;           // [rows][ld_ssq] partial sums of squares of the operand rows, ssq_n of them each; null = no scale
   int ssq_n, ld_ssq;
   float inv_d_in, eps;
   void* out; int ldo;            // EPI_F32 / EPI_BF16 / EPI_GELU
@@ -78,7 +78,7 @@ struct Epi {
   float* x; int ldx; int add;    // EPI_RESID: residual stream, add = 0 replaces it
   const float* gain;             //            gain of the next norm (null = 1)
   bf16* a_out; int lda;          //            next GEMM's operand rows (may be null)
-  float* ssq_out; int ld_ssq_out;//            [M tiles * split][ld] partial sums of squares of the new x rows (may be null)
+  float* ssq_out; int ld_ssq_out;//            [rows][ld] partial sums of squares of the new x rows, a slot per tile and rank (may be null)
   Dims dm; SeqState st;          // EPI_QKV
   int batch, level;
   const PackedRow* rows;         //            (b, p) of every row when the rows are packed (prefill); null: rows of a pass
@@ -416,13 +416,13 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const int slot = sub + 8 * k;
-          v[k] = (n < ns && slot < e.ssq_n) ? __ldcg(e.ssq_in + (size_t)slot * e.ld_ssq + row0 + n) : 0.f;
+          v[k] = (n < ns && slot < e.ssq_n) ? __ldcg(e.ssq_in + (size_t)(row0 + n) * e.ld_ssq + slot) : 0.f;
         }
         float ss = 0.f;
 #pragma unroll
         for (int k = 0; k < 8; ++k) ss += v[k];
         for (int slot = sub + 64; slot < e.ssq_n; slot += 8)             // more than 64 slots: not expected
-          ss += (n < ns) ? __ldcg(e.ssq_in + (size_t)slot * e.ld_ssq + row0 + n) : 0.f;
+          ss += (n < ns) ? __ldcg(e.ssq_in + (size_t)(row0 + n) * e.ld_ssq + slot) : 0.f;
         ss += __shfl_xor_sync(0xffffffffu, ss, 1);
         ss += __shfl_xor_sync(0xffffffffu, ss, 2);
         ss += __shfl_xor_sync(0xffffffffu, ss, 4);
@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
         float sqv = __fmaf_rn(xa, xa, __fmul_rn(xb, xb));
         for (int o = L >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
         if (active && (cc & (L - 1)) == 0)
-          k_ssqo[(size_t)((((tile_m << lgS) + z) << (lgPW - lgL)) + (cc >> lgL)) * k_ldssq + k_row0 + n] = sqv;
+          k_ssqo[row * k_ldssq + ((((tile_m << lgS) + z) << (lgPW - lgL)) + (cc >> lgL))] = sqv;
       }
     } else if (MODE == EPI_UP) {
       // (ya, yb): columns (ma, ma + 1) of the triple of parent row n = slot ma / d, column ma % d
@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
         float sqv = __fmaf_rn(xa, xa, __fmul_rn(xb, xb));
         for (int o = L >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
         if (active && child && (cc & (L - 1)) == 0)
-          k_ssqo[(size_t)(((((tile_m % (dd / BM)) << lgS) + z) << (lgPW - lgL)) + (cc >> lgL)) * k_ldssq + crow] = sqv;
+          k_ssqo[crow * k_ldssq + (((((tile_m % (dd / BM)) << lgS) + z) << (lgPW - lgL)) + (cc >> lgL))] = sqv;
       }
     } else {  // EPI_QKV: (ya, yb) is the rotary pair (i, i + dh/2) of one head, stored at (c, c + 1), c = 2i
       const int dh = k_dh, H = k_H, Hkv = k_Hkv;
@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
         float sqv = __fmaf_rn(x0.x, x0.x, __fmul_rn(x0.y, x0.y));
         for (int o = L >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
         if (active && (cc & (L - 1)) == 0)
-          k_ssqo[(size_t)(((((tile_m % (dd / BM)) << lgS) + z) << (lgPW - lgL)) + (cc >> lgL)) * k_ldssq + crow] = sqv;
+          k_ssqo[crow * k_ldssq + (((((tile_m % (dd / BM)) << lgS) + z) << (lgPW - lgL)) + (cc >> lgL))] = sqv;
       }
     }
   }

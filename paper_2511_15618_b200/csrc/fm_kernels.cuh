@@ -42,7 +42,7 @@ __device__ inline void store_hi_lo(bf16* p, float v, int lo_off) {
 // filled).
 // ------------------------------------------------------------------------------------------
 __device__ inline void stack_entry_row(const float* xr, int row, int d, const float* __restrict__ g,
-                                       bf16* __restrict__ a_out, float* __restrict__ ssq) {
+                                       bf16* __restrict__ a_out, float* __restrict__ ssq, int ld_ssq) {
   __shared__ float sh[32];
   float ss = 0.f;
   for (int i = threadIdx.x; i < d; i += blockDim.x) {
@@ -51,7 +51,7 @@ __device__ inline void stack_entry_row(const float* xr, int row, int d, const fl
     store_hi_lo(a_out + (size_t)row * 2 * d + i, __fmul_rn(v, g[i]), d);
   }
   ss = block_sum(ss, sh);
-  if (threadIdx.x == 0) ssq[row] = ss;
+  if (threadIdx.x == 0) ssq[(size_t)row * ld_ssq] = ss;
 }
 
 // first level-local position of sequence b in this pass
@@ -64,7 +64,7 @@ __device__ inline int fm_first_pos(const SeqState& st, int b, int level) {
 // a1. candidate embedding: x[row] = E[cand[b][j]]  (zeros for rows that are not fed)
 // ------------------------------------------------------------------------------------------
 __global__ void embed_kernel(Dims dm, SeqState st, int batch, const bf16* __restrict__ E, float* __restrict__ x,
-                             const float* __restrict__ g, bf16* __restrict__ a_out, float* __restrict__ ssq,
+                             const float* __restrict__ g, bf16* __restrict__ a_out, float* __restrict__ ssq, int ld_ssq,
                              int rows, const float* __restrict__ hc_ring, const float* __restrict__ hv_ring,
                              bf16* __restrict__ cat_v, bf16* __restrict__ cat_f, int rows_v, int rows_f) {
   if ((int)blockIdx.x >= rows) {
@@ -102,7 +102,7 @@ __global__ void embed_kernel(Dims dm, SeqState st, int batch, const bf16* __rest
   for (int i = threadIdx.x; i < dm.d; i += blockDim.x)
     x[(size_t)row * dm.d + i] = valid ? __bfloat162float(E[(size_t)tok * dm.d + i]) : 0.f;
   __syncthreads();
-  stack_entry_row(x + (size_t)row * dm.d, row, dm.d, g, a_out, ssq);
+  stack_entry_row(x + (size_t)row * dm.d, row, dm.d, g, a_out, ssq, ld_ssq);
 }
 
 // RMSNorm of read-only fp32 rows (conditioning vectors, draft features) -> bf16 operand rows
@@ -180,7 +180,7 @@ __global__ void shorten_gather_kernel(Dims dm, SeqState st, int batch, int level
 // rows_up): this pass's triples go into the ring.
 __global__ void upsample_add_kernel(Dims dm, SeqState st, int batch, int level, const float* __restrict__ h_ring,
                                     const float* __restrict__ tri_new, float* __restrict__ tri_ring, float* __restrict__ x,
-                                    const float* __restrict__ g, bf16* __restrict__ a_out, float* __restrict__ ssq, int rows) {
+                                    const float* __restrict__ g, bf16* __restrict__ a_out, float* __restrict__ ssq, int ld_ssq, int rows) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int rs = fm_ring(level), rsu = fm_ring(level + 1), d = dm.d;
@@ -202,7 +202,7 @@ __global__ void upsample_add_kernel(Dims dm, SeqState st, int batch, int level, 
                                         : tri_ring + ((size_t)b * rsu + (up % rsu)) * 3 * d + (p % 3) * d;
   for (int i = threadIdx.x; i < d; i += blockDim.x) x[(size_t)row * d + i] = valid ? h[i] + t[i] : 0.f;
   __syncthreads();
-  stack_entry_row(x + (size_t)row * d, row, d, g, a_out, ssq);
+  stack_entry_row(x + (size_t)row * d, row, d, g, a_out, ssq, ld_ssq);
 }
 
 // ------------------------------------------------------------------------------------------

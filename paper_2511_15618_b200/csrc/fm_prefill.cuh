@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
           if (e.ssq_in != nullptr) {
             float ss = 0.f;
 #pragma unroll 8
-            for (int s = 0; s < e.ssq_n; ++s) ss += __ldcg(e.ssq_in + (size_t)s * e.ld_ssq + n0 + n);
+            for (int s = 0; s < e.ssq_n; ++s) ss += __ldcg(e.ssq_in + (size_t)(n0 + n) * e.ld_ssq + s);
             v = rsqrtf(ss * e.inv_d + e.eps);
           }
           inv[n] = v;
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
 #pragma unroll
             for (int j = 0; j < 32; ++j) y[j] = m_ok ? y[j] * y[j] : 0.f;
             fold<16>(y, lane); fold<8>(y, lane); fold<4>(y, lane); fold<2>(y, lane); fold<1>(y, lane);
-            if (lane < nv) e.ssq_out[(size_t)(tm * 4 + w4) * e.ld_ssq + row + lane] = y[0];
+            if (lane < nv) e.ssq_out[(row + lane) * e.ld_ssq + tm * 4 + w4] = y[0];
           }
         } else if (MODE == PF_QKV) {
           // Q and K heads are stored with their rotary pairs side by side: the partner is the neighbouring lane
@@ -358,7 +358,7 @@ __global__ void map_kernel(Dims dm, const Seg* __restrict__ segs, Row* m0, Row* 
 
 // operand row [hi | lo] of x * g and the row's sum of squares, four columns per thread and step
 __device__ inline void entry_row(const float4* xr, int row, int d, const float* __restrict__ g, bf16* __restrict__ a,
-                                 float* __restrict__ ssq) {
+                                 float* __restrict__ ssq, int ld_ssq) {
   __shared__ float sh[32];
   float ss = 0.f;
   for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
@@ -370,12 +370,12 @@ __device__ inline void entry_row(const float4* xr, int row, int d, const float* 
     tc::store_hi_lo2(p + 2, __fmul_rn(v.z, gg.z), __fmul_rn(v.w, gg.w), d);
   }
   ss = block_sum(ss, sh);
-  if (threadIdx.x == 0) ssq[row] = ss;
+  if (threadIdx.x == 0) ssq[(size_t)row * ld_ssq] = ss;
 }
 
 __global__ void embed_kernel(Dims dm, SeqState st, const Row* __restrict__ rows, const int* __restrict__ prompt,
                              const int* __restrict__ prompt_off, const bf16* __restrict__ E, float* __restrict__ x,
-                             const float* __restrict__ g, bf16* __restrict__ a, float* __restrict__ ssq) {
+                             const float* __restrict__ g, bf16* __restrict__ a, float* __restrict__ ssq, int ld_ssq) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int row = blockIdx.x, d = dm.d;
@@ -391,7 +391,7 @@ __global__ void embed_kernel(Dims dm, SeqState st, const Row* __restrict__ rows,
     const float2 lo = __bfloat1622float2(er[2 * i]), hi = __bfloat1622float2(er[2 * i + 1]);
     xr[i] = make_float4(lo.x, lo.y, hi.x, hi.y);
   }
-  entry_row(xr, row, d, g, a, ssq);                  // every thread reads the columns it wrote
+  entry_row(xr, row, d, g, a, ssq, ld_ssq);                  // every thread reads the columns it wrote
 }
 
 // operand rows of a shorten GEMM: row u of level `lu` <- hiddens 3u-2, 3u-1, 3u of the level below,
@@ -419,7 +419,7 @@ __global__ void gather_kernel(Dims dm, const Seg* __restrict__ segs, const Row* 
 // above.  The parent of every row is a row of the same segment.
 __global__ void upsample_kernel(Dims dm, const Seg* __restrict__ segs, const Row* __restrict__ rows, int level,
                                 const float* __restrict__ tri, float* __restrict__ h_ring, float* __restrict__ tri_ring,
-                                float* __restrict__ x, const float* __restrict__ g, bf16* __restrict__ a, float* __restrict__ ssq) {
+                                float* __restrict__ x, const float* __restrict__ g, bf16* __restrict__ a, float* __restrict__ ssq, int ld_ssq) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int row = blockIdx.x, d = dm.d, rs = fm_ring(level), rsu = fm_ring(level + 1);
@@ -437,7 +437,7 @@ __global__ void upsample_kernel(Dims dm, const Seg* __restrict__ segs, const Row
     if (tr != nullptr) { tr[i] = u; tr[d / 4 + i] = t[d / 4 + i]; tr[d / 2 + i] = t[d / 2 + i]; }
     xr[i] = make_float4(h.x + u.x, h.y + u.y, h.z + u.z, h.w + u.w);
   }
-  entry_row(xr, row, d, g, a, ssq);
+  entry_row(xr, row, d, g, a, ssq, ld_ssq);
 }
 
 // the residual row of a prompt's last position, as it enters the last layer of a stack (split node)
@@ -483,8 +483,8 @@ __global__ void last_rows_kernel(Dims dm, const Seg* __restrict__ segs, const bf
   for (int i = threadIdx.x; i < dm.d / 4; i += blockDim.x) dst[i] = src[i];
   if (threadIdx.x == 0) {
     float t = 0.f;
-    for (int k = 0; k < ssq_n; ++k) t += ssq[(size_t)k * ld + row];
-    ssq_out[s.b] = t;
+    for (int k = 0; k < ssq_n; ++k) t += ssq[(size_t)row * ld + k];
+    ssq_out[(size_t)s.b * ld] = t;
   }
 }
 
