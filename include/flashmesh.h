@@ -261,8 +261,8 @@ int fm_verify(fm_ctx* ctx, const int32_t* cand /*DEV*/, int32_t* argmax /*DEV*/,
  * paper).  Some hosts of this library carve the workspace of fm_create out of an arena that is
  * sized and committed once at start-up -- a serving process with a fixed memory plan, a plug-in that
  * is forbidden to call cudaMalloc because an allocation would synchronise the device under its
- * real-time loop -- and want the attention kernel's split-KV scratch (per-group partial results and
- * the ticket counters of the final merge) kept out of that arena.  This call does what fm_verify
+ * real-time loop -- and want the attention kernel's split-KV scratch (per-group partial results) kept
+ * out of that arena.  This call does what fm_verify
  * does, same arguments, same results, but points the attention kernel at a fixed array of
  * FM_STATIC_SCRATCH_BYTES bytes that is part of the library image: every GPU that loads the library
  * holds that many bytes until the process exits.  It allocates nothing (no cudaMalloc, no
@@ -273,8 +273,7 @@ int fm_verify(fm_ctx* ctx, const int32_t* cand /*DEV*/, int32_t* argmax /*DEV*/,
  *   - Every GPU has its own copy of the array: the device the context was created on must be the
  *     current device at every call (FM_ERR_BAD_STATE otherwise).  The first call on a device looks
  *     up the array's device address; make that first call before any stream capture is begun.
- *   - All contexts and all calls share the one array.  It keeps the previous call's contents (the
- *     call clears the counters that must start at zero), and two calls whose kernels overlap on
+ *   - All contexts and all calls share the one array.  Two calls whose kernels overlap on
  *     the GPU -- different streams, different contexts -- race on it: serialise them. */
 #define FM_STATIC_SCRATCH_BYTES (4 * 1024 * 1024)
 int fm_verify_static_scratch(fm_ctx* ctx, const int32_t* cand /*DEV*/, int32_t* argmax /*DEV*/, float* logits /*DEV*/,
@@ -340,10 +339,10 @@ int fm_profile_end(fm_ctx* ctx, fm_profile* out /*HOST*/);
 
 /* How the attention kernel cuts a level's cache (no counterpart in the paper; for reports and
  * tests): slots per chunk, chunks per group (one CTA streams one group; fixed when the context is
- * created) and the number of groups the full cache has.  A (sequence, kv-head) whose cache holds n
- * slots, prefix included, is read by ceil(ceil(n / chunk) / chunks_per_group) CTAs, whose partial
- * results go through the scratch buffers when there is more than one.  level: 0 coordinate,
- * 1 vertex, 2 face.  HOST out pointers, any may be NULL. */
+ * created) and the number of groups the full cache has.  Chunk c belongs to group c mod groups, so a
+ * (sequence, kv-head) whose cache holds n slots, prefix included, is read by
+ * min(ceil(n / chunk), groups) CTAs, whose partial results go through the scratch buffer when there
+ * is more than one.  level: 0 coordinate, 1 vertex, 2 face.  HOST out pointers, any may be NULL. */
 int fm_attention_layout(const fm_ctx* ctx, int32_t level, int32_t* chunk_slots, int32_t* chunks_per_group,
                         int32_t* max_groups);
 
@@ -361,9 +360,7 @@ int fm_selftest_wait_timeout(fm_ctx* ctx, int64_t limit_cycles);
 
 const char* fm_strerror(int code);
 /* Device status word: 0, or FM_ERR_TIMEOUT if a bounded wait inside a kernel gave up, or
- * FM_ERR_INVALID_ARG if a kernel met an out-of-range token id (it then used PAD), or
- * FM_ERR_CAPACITY if the attention kernel was asked to merge more cache groups than it can stage
- * (it then wrote nothing; fm_create sizes the groups so that this does not happen).  The word is
+ * FM_ERR_INVALID_ARG if a kernel met an out-of-range token id (it then used PAD).  The word is
  * cleared by fm_prefill.  Synchronises the stream. */
 int fm_device_status(fm_ctx* ctx);
 

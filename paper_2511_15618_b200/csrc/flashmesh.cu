@@ -41,7 +41,7 @@ inline int round_up(int v, int a) { return (v + a - 1) / a * a; }
 
 }  // namespace
 
-// Attention scratch (group partials, then tickets) for fm_verify_static_scratch: lives in the
+// Attention scratch (group partials) for fm_verify_static_scratch: lives in the
 // library image, so every GPU that loads the library holds these bytes until the process exits.
 static __device__ __align__(256) unsigned char g_static_attn_scratch[FM_STATIC_SCRATCH_BYTES];
 
@@ -82,7 +82,6 @@ struct fm_ctx {
   int attn_mt_draft[3];                      // query tiles of the draft modules' attention launches per level
   // attention scratch and TMA descriptors
   float* attn_part;
-  int* attn_ticket;
   int attn_chunk, attn_G[3], attn_max_groups[3], attn_mt[3];
   CUtensorMap* tmaps;                    // device array
   std::vector<CUtensorMap> tmaps_host;
@@ -129,7 +128,6 @@ struct fm_ctx {
   int stage_cap;        // tuning knob: upper bound on the GEMM ring depth (0 = none)
   int n_sm;                                  // SMs of the device
   int device;                                // ordinal of the device the context was created on
-  size_t attn_ticket_n;                      // entries of attn_ticket
   int split_target_deep;                     // the same for launches whose CTAs stream long K ranges
   int launch_error;     // first error met while enqueueing (capacity, descriptor creation)
   // one decode pass (draft, teacher edit, verify, accept) captured as a CUDA graph
@@ -298,10 +296,10 @@ void carve(fm_ctx* c, Carver& cv) {
     c->d_q = cv.take<bf16>(rows * hd); c->d_attn = cv.take<bf16>(rows * 2 * hd); c->d_a = cv.take<bf16>(rows * d);
     c->d_h1 = cv.take<bf16>(rows * 2 * dm.hf);
   }
-  // attention: chunk size, chunks per group (fixed per level so that the reduction order of a row
-  // never depends on the cache length), group partials (max over levels), tickets
+  // attention: chunk size, number of groups (fixed per level so that the reduction order of a row
+  // never depends on the cache length), group partials (max over levels)
   c->attn_chunk = dm.dh == 64 ? 128 : 64;
-  size_t part_max = 0, ticket_max = 0;
+  size_t part_max = 0;
   for (int l = 0; l < 3; ++l) {
     const int max_chunks = (dm.P + dm.cap[l] + c->attn_chunk - 1) / c->attn_chunk;
     c->attn_mt[l] = (fm_rows_per_seq(dm, l) * (dm.H / dm.Hkv) + 15) / 16;
@@ -309,12 +307,10 @@ void carve(fm_ctx* c, Carver& cv) {
     const int dq = !dm.full ? 0 : (l == 0 ? (dm.nc > 3 * dm.nv + 9 * dm.Ef ? dm.nc : 3 * dm.nv + 9 * dm.Ef) : (l == 1 ? (dm.nv > 3 * dm.Ef ? dm.nv : 3 * dm.Ef) : dm.Ef));
     c->attn_mt_draft[l] = (dq * (dm.H / dm.Hkv) + 15) / 16;
     const int mt_max = c->attn_mt[l] > c->attn_mt_draft[l] ? c->attn_mt[l] : c->attn_mt_draft[l];
-    // Chunks per group: the number of groups (1 .. what the merge can stage: 24, fewer for wide
-    // heads) that minimises waves x (chunks per CTA + a CTA's fixed cost), with the cache full.
-    // The fixed cost (pipeline start, merge of the warps, and with several groups the partials,
-    // the ticket and the last CTA's merge) was measured at batch 16 as about 5 chunk times:
-    // 87 / 70 / 63 / 61 us per launch with at most 8 / 16 / 32 / 64 chunks per group.
-    const int g_cap = dm.dh == 64 ? AttnCfg<64, 128, 8>::MAX_GROUPS : AttnCfg<128, 64, 4>::MAX_GROUPS;
+    // Number of groups (1 .. what the merge holds: 24): the one that minimises waves x (chunks per CTA + a
+    // CTA's fixed cost), with the cache full.  The fixed cost (pipeline start, merge of the warps, and with
+    // several groups the partials and the merge launch) was measured at batch 16 as about 5 chunk times.
+    const int g_cap = dm.dh == 64 ? AttnCfg<64, 128, 4>::MAX_GROUPS : AttnCfg<128, 64, 4>::MAX_GROUPS;
     const size_t tiles_l = (size_t)dm.Hkv * B * c->attn_mt[l];      // the verify pass decides the grouping
     int G = max_chunks;
     double best = 0.0;
@@ -333,12 +329,8 @@ void carve(fm_ctx* c, Carver& cv) {
     c->attn_max_groups[l] = (max_chunks + G - 1) / G;
     const size_t need = B * dm.Hkv * (size_t)mt_max * c->attn_max_groups[l] * 16 * (dm.dh + 2);
     part_max = need > part_max ? need : part_max;
-    const size_t tk = B * dm.Hkv * (size_t)mt_max;
-    ticket_max = tk > ticket_max ? tk : ticket_max;
   }
   c->attn_part = cv.take<float>(part_max);
-  c->attn_ticket = cv.take<int>(ticket_max);
-  c->attn_ticket_n = ticket_max;
   int n_layers = 0;
   for (int s = 0; s < 5; ++s) n_layers += c->cfg.layers[s];
   c->tmaps_cap = (size_t)6 * n_layers + 128;
@@ -624,10 +616,10 @@ void launch_rows(fm_ctx* c, int mtn, int fj, dim3 grid, int smem, const rg::Args
 bool gemm_rows(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, int a_row0, int M, int K, int R, const int* n_active, int mode,
                const tc::Epi& e, int parts, int stacked, int z_rows, int z_w_rows) {
   if (R > c->rows_max || M < 8) return false;
-  int FT = 8;
+  int FT = K > 1536 ? 16 : 8;                              // long K: fewer CTAs, each of which reads all operand rows
   while (FT < 32 && (M + FT - 1) / FT * stacked > c->n_sm) FT *= 2;
   const int mtn = (parts * R + 15) / 16, smem = rg::smem_bytes(FT, K, mtn);
-  if (smem > 100 * 1024) return false;
+  if (smem > 140 * 1024) return false;
   if (e.ssq_out != nullptr && c->dm.d % FT != 0) return false;
   const rg::Args g{W, A, parts * K, M, K, R, parts, w_row0 / tc::BM, a_row0, stacked > 1 ? z_rows : 0, stacked > 1 ? z_w_rows / tc::BM : 0,
                    n_active, c->st.status};
@@ -647,7 +639,7 @@ bool gemm_rows(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, int a_row0, 
 
 template <int MODE>
 cudaError_t allow_rows_smem() {
-  const int most = 101 * 1024;
+  const int most = 141 * 1024;
   cudaError_t r = cudaSuccess;
   auto set = [&](const void* k) { if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most); };
   set((const void*)rg::gemm_rows_kernel<MODE, 1, 1>); set((const void*)rg::gemm_rows_kernel<MODE, 1, 2>); set((const void*)rg::gemm_rows_kernel<MODE, 1, 4>);
@@ -736,17 +728,26 @@ __global__ void row_count_kernel(Dims dm, SeqState st, int batch) {
 inline int row_threads(int d) { return d >= 512 ? 512 : (d >= 256 ? 256 : 128); }
 inline int accept_threads(int batch) { return batch >= 32 ? 1024 : 32 * (batch < 1 ? 1 : batch); }
 
-void attention(fm_ctx* c, int level, const LayerDev& L) {
+// the streaming launch and, where a level's cache is cut into several groups, the merge
+void launch_attention(fm_ctx* c, const AttnArgs& a) {
   const Dims& dm = c->dm;
-  const int groups = c->attn_max_groups[level];
-  AttnArgs a{dm, c->st, c->batch, level, c->qbuf, c->tmaps + L.tmK, c->tmaps + L.tmV, c->attn_part, c->attn_ticket,
-             c->a_attn, c->attn_G[level], groups, c->attn_mt[level]};
-  const dim3 grid(groups, dm.Hkv * c->attn_mt[level], c->batch);
-  const long pi = prof_open(c, PROF_ATTN, 0.0);
+  const dim3 grid(a.max_groups, dm.Hkv * a.MT, c->batch), merge(dm.Hkv * a.MT * c->batch, 4), one(1, 1, 1);
   c->cur_class = PROF_ATTN;
-  if (dm.dh == 64) launch_pdl(c, dim3(1, 1, 1), attn_stream_kernel<64, 128, 8>, grid, AttnCfg<64, 128, 8>::THREADS, AttnCfg<64, 128, 8>::BYTES, a);
-  else launch_pdl(c, dim3(1, 1, 1), attn_stream_kernel<128, 64, 4>, grid, AttnCfg<128, 64, 4>::THREADS, AttnCfg<128, 64, 4>::BYTES, a);
+  if (dm.dh == 64) {
+    launch_pdl(c, one, attn_stream_kernel<64, 128, 4>, grid, AttnCfg<64, 128, 4>::THREADS, AttnCfg<64, 128, 4>::BYTES, a);
+    if (a.max_groups > 1) launch_pdl(c, one, attn_merge_kernel<64, 128>, merge, 128, 0, a);
+  } else {
+    launch_pdl(c, one, attn_stream_kernel<128, 64, 4>, grid, AttnCfg<128, 64, 4>::THREADS, AttnCfg<128, 64, 4>::BYTES, a);
+    if (a.max_groups > 1) launch_pdl(c, one, attn_merge_kernel<128, 64>, merge, 128, 0, a);
+  }
   c->cur_class = PROF_OTHER;
+}
+
+void attention(fm_ctx* c, int level, const LayerDev& L) {
+  AttnArgs a{c->dm, c->st, c->batch, level, c->qbuf, c->tmaps + L.tmK, c->tmaps + L.tmV, c->attn_part, c->a_attn,
+             c->attn_max_groups[level], c->attn_mt[level]};
+  const long pi = prof_open(c, PROF_ATTN, 0.0);
+  launch_attention(c, a);
   prof_close(c, pi);
 }
 
@@ -902,16 +903,10 @@ void attention_draft(fm_ctx* c, int s, int nq, const bf16* q, bf16* out) {
   const Dims& dm = c->dm;
   const int level = STACK_LEVEL[s];
   const LayerDev& L = c->layers[s].back();
-  const int groups = c->attn_max_groups[level];
   const int MT = (nq * (dm.H / dm.Hkv) + 15) / 16;
   if (MT > c->attn_mt_draft[level] && MT > c->attn_mt[level]) { c->launch_error = FM_ERR_CAPACITY; return; }
-  AttnArgs a{dm, c->st, c->batch, level, q, c->tmaps + L.tmK, c->tmaps + L.tmV, c->attn_part, c->attn_ticket,
-             out, c->attn_G[level], groups, MT, nq, dm.max_batch};
-  const dim3 grid(groups, dm.Hkv * MT, c->batch);
-  c->cur_class = PROF_ATTN;
-  if (dm.dh == 64) launch_pdl(c, dim3(1, 1, 1), attn_stream_kernel<64, 128, 8>, grid, AttnCfg<64, 128, 8>::THREADS, AttnCfg<64, 128, 8>::BYTES, a);
-  else launch_pdl(c, dim3(1, 1, 1), attn_stream_kernel<128, 64, 4>, grid, AttnCfg<128, 64, 4>::THREADS, AttnCfg<128, 64, 4>::BYTES, a);
-  c->cur_class = PROF_OTHER;
+  AttnArgs a{dm, c->st, c->batch, level, q, c->tmaps + L.tmK, c->tmaps + L.tmV, c->attn_part, out, c->attn_max_groups[level], MT, nq, dm.max_batch};
+  launch_attention(c, a);
 }
 
 // One stage of HF-Blocks (Eq. 3-5) on the fp32 features hf_feature() names: T offsets, each with its
@@ -1575,7 +1570,7 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
       for (auto& L : c->layers[s]) lp.push_back({L.Wqkv, L.g1, L.K, L.V, STACK_LEVEL[s], 0});
     TRYCUDA(cudaMemcpy(c->pre.layers, lp.data(), lp.size() * sizeof(pf::LayerPtr), cudaMemcpyHostToDevice));
   }
-  TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<64, 128, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64, 128, 8>::BYTES));
+  TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<64, 128, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64, 128, 4>::BYTES));
   TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<128, 64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128, 64, 4>::BYTES));
   std::vector<double> freq(dm.dh / 2);
   for (int i = 0; i < dm.dh / 2; ++i)
@@ -1721,10 +1716,8 @@ int fm_prefill(fm_ctx* c, int32_t batch, const float* cond, const int32_t* promp
   if (prompt_off[batch] > 0 && prompt == nullptr) return FM_ERR_INVALID_ARG;
   c->batch = batch;
   c->launch_error = FM_OK;                         // a new start clears an earlier enqueue error
-  // ... and whatever a kernel that gave up on a bounded wait left behind: the status word, and
-  // the tickets of attention tiles whose last CTA never came to reset them
+  // ... and the status word of a kernel that gave up on a bounded wait
   CUDA_OK(cudaMemsetAsync(c->st.status, 0, sizeof(int), c->stream));
-  CUDA_OK(cudaMemsetAsync(c->attn_ticket, 0, c->attn_ticket_n * sizeof(int), c->stream));
   c->plen_host.assign(batch, 0);
   for (int b = 0; b < batch; ++b) c->plen_host[b] = prompt_off[b + 1] - prompt_off[b];
   const int rc = prefill_run(c, cond, prompt, prompt_off);
@@ -1813,18 +1806,14 @@ int fm_verify(fm_ctx* c, const int32_t* cand, int32_t* argmax, float* logits, fl
 int fm_verify_static_scratch(fm_ctx* c, const int32_t* cand, int32_t* argmax, float* logits, float* margin) {
   if (c == nullptr || cand == nullptr) return FM_ERR_INVALID_ARG;
   if (c->phase < 1) return FM_ERR_BAD_STATE;
-  // what the attention kernel needs: the largest level's group partials, then one ticket per
-  // (sequence, kv-head, query tile)
+  // what the attention kernel needs: the largest level's group partials
   const Dims& dm = c->dm;
-  size_t part_floats = 0, tickets = 0;
+  size_t part_floats = 0;
   for (int l = 0; l < 3; ++l) {
-    const size_t per = (size_t)dm.max_batch * dm.Hkv * c->attn_mt[l];
-    const size_t need = per * c->attn_max_groups[l] * 16 * (dm.dh + 2);
+    const size_t need = (size_t)dm.max_batch * dm.Hkv * c->attn_mt[l] * c->attn_max_groups[l] * 16 * (dm.dh + 2);
     part_floats = need > part_floats ? need : part_floats;
-    tickets = per > tickets ? per : tickets;
   }
-  const size_t ticket_off = align_up(part_floats * sizeof(float), 256);
-  if (ticket_off + tickets * sizeof(int) > (size_t)FM_STATIC_SCRATCH_BYTES) return FM_ERR_CAPACITY;
+  if (part_floats * sizeof(float) > (size_t)FM_STATIC_SCRATCH_BYTES) return FM_ERR_CAPACITY;
   // Device address of the static array, looked up once per device with that device current (the
   // array's name is only a host-side handle; a kernel must be given this address).  Every GPU
   // holds its own copy of the array, so the address must be the one of the context's device:
@@ -1844,18 +1833,13 @@ int fm_verify_static_scratch(fm_ctx* c, const int32_t* cand, int32_t* argmax, fl
     }
   }
   unsigned char* base = static_cast<unsigned char*>(dev_addr[dev]);
-  // tickets must start at zero; the array keeps whatever the last call (of any context) left
-  CUDA_OK(cudaMemsetAsync(base + ticket_off, 0, tickets * sizeof(int), c->stream));
   float* saved_part = c->attn_part;
-  int* saved_ticket = c->attn_ticket;
   c->attn_part = reinterpret_cast<float*>(base);
-  c->attn_ticket = reinterpret_cast<int*>(base + ticket_off);
   const bool was_off = c->call_graphs_off;
   c->call_graphs_off = true;                       // the scratch pointers differ from the cached graph's
   const int rc = fm_verify(c, cand, argmax, logits, margin);
   c->call_graphs_off = was_off;
   c->attn_part = saved_part;
-  c->attn_ticket = saved_ticket;
   return rc;
 }
 
