@@ -529,15 +529,36 @@ int add_tmap_operand(fm_ctx* c, const void* base, uint64_t rows, uint64_t K, uin
   return (int)c->tmaps_host.size() - 1;
 }
 
+// The same rows for stages of one or two K slabs: a 4-D tensor (64 columns, rows, parts, K / 64) whose box brings, slab
+// after slab, the hi and the lo tile; what lies behind the last slab reads as zero.
+int add_tmap_stage(fm_ctx* c, const void* base, uint64_t rows, uint64_t K, uint32_t parts, uint32_t box_rows) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (fn == nullptr) return -1;
+  CUtensorMap m;
+  const cuuint64_t gdim[4] = {64, rows, parts, K / 64};
+  const cuuint64_t gstride[3] = {parts * K * 2, K * 2, 128};
+  const cuuint32_t box[4] = {64, box_rows, parts, (cuuint32_t)pf::stage_slabs((int)box_rows, (int)parts)};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  if (fn(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), gdim, gstride, box, estr,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return -1;
+  c->tmaps_host.push_back(m);
+  return (int)c->tmaps_host.size() - 1;
+}
+
 // index of the tensor map for a bf16 matrix / box, created on first use (all call sites are
 // visited by the first pass, before any timing or capture)
+constexpr uint32_t TMAP_STAGE = 16;      // added to `parts`: the 4-D form; parts = 0: a plain 2-D map
 int tmap_for(fm_ctx* c, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t parts) {
   for (size_t i = 0; i < c->tmap_keys.size(); ++i) {
     const auto& k = c->tmap_keys[i];
     if (k.base == base && k.rows == rows && k.cols == cols && k.box_rows == box_rows && k.parts == parts) return (int)i;
   }
   if (c->tmaps_host.size() >= c->tmaps_cap || c->capturing) return -1;   // descriptors are made before capture
-  const int idx = parts == 0 ? add_tmap_bf16(c, base, rows, cols, box_rows) : add_tmap_operand(c, base, rows, cols, parts, box_rows);
+  const int idx = parts == 0 ? add_tmap_bf16(c, base, rows, cols, box_rows)
+                  : parts >= TMAP_STAGE ? add_tmap_stage(c, base, rows, cols, parts - TMAP_STAGE, box_rows)
+                                        : add_tmap_operand(c, base, rows, cols, parts, box_rows);
   if (idx < 0) return -1;
   c->tmap_keys.push_back({base, rows, cols, box_rows, parts});
   cudaMemcpyAsync(c->tmaps + idx, &c->tmaps_host[idx], sizeof(CUtensorMap), cudaMemcpyHostToDevice, c->stream);
@@ -1049,13 +1070,13 @@ void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_al
     const double cost = waves * (slabs * (copy > mma ? copy : mma) + 12.0 * parts * nt) + 2000.0;
     if (nt == 32 || cost < best) { best = cost; NT = nt; }
   }
-  const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, NT, (uint32_t)parts);
+  const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, NT, TMAP_STAGE + (uint32_t)parts);
   if (tA < 0) { c->launch_error = FM_ERR_CUDA; return; }
   int stages = (200 * 1024) / pf::stage_bytes(NT, parts);
-  stages = stages > 4 ? 4 : stages;
+  stages = stages > pf::MAX_STAGES ? pf::MAX_STAGES : stages;
   const int tiles_n = (R + NT - 1) / NT, tiles = tiles_m * tiles_n * layers;
   if (mode == pf::PF_RESID && e.ssq_out != nullptr) c->ssq_n = tiles_m * 4;        // slots the next consumer adds
-  pf::Gemm g{W, c->tmaps + tA, M, K, R, NT, stages, tiles_m, tiles_n, tiles, w_tile0, c->st.status};
+  pf::Gemm g{W, c->tmaps + tA, M, K, R, NT, stages, pf::stage_slabs(NT, parts), tiles_m, tiles_n, tiles, w_tile0, c->st.status};
   const dim3 grid(tiles < c->n_sm ? tiles : c->n_sm), one(1, 1, 1);
   const int smem = pf::smem_bytes(NT, parts, stages);
   switch (mode) {

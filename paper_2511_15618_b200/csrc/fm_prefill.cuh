@@ -33,15 +33,18 @@ struct LayerPtr { const bf16* Wqkv; const float* g1; bf16* K; bf16* V; int level
 // stages decouples the copies from the MMA thread, and two accumulators in tensor memory let the
 // epilogue of a tile run under the MMAs of the next.  A thread of the epilogue owns one feature (its
 // tensor-memory lane), so a warp stores 32 neighbouring features of a row at a time.
-// Bound: tensor cores and, below 128 rows per tile, the stream from L2 (48 KB per 512 MMA clocks).
+// One thread needs about 420 clocks to request a weight slab and an operand slab of 64 k, and 128 threads
+// need 35 000 clocks for the GELU of a tile (its MMAs take 8 200): hence a producer warp for each of the two
+// streams, (for narrow tiles) stages of two slabs and eight epilogue warps.
 enum Mode { PF_F32 = 0, PF_GELU = 1, PF_RESID = 2, PF_QKV = 3, PF_PREFIX = 4 };
 
-constexpr int THREADS = 192;     // producer warp, MMA warp, four epilogue warps
-constexpr int MAX_STAGES = 6;
+constexpr int THREADS = 384;     // weight producer, operand producer, MMA warp, one idle warp, eight epilogue warps
+constexpr int EPI_WARPS = 8;
+constexpr int MAX_STAGES = 4;     // (deeper rings were no faster)
 
 struct Gemm {
   const bf16* W; const CUtensorMap* tmA;
-  int M, K, R, NT, stages;
+  int M, K, R, NT, stages, slabs;  // slabs of 64 k per stage: 1 or 2
   int tiles_m, tiles_n, tiles;   // tiles = tiles_m * tiles_n * layers (PF_PREFIX), else tiles_m * tiles_n
   int w_tile0;
   int* status;
@@ -55,7 +58,8 @@ struct Epi {
   const LayerPtr* layers; int row_first, rows_layer;            // PF_PREFIX: operand rows of layer z at z * rows_layer
 };
 
-inline int stage_bytes(int NT, int parts) { return tc::BM * 128 + parts * NT * 128; }
+inline int stage_slabs(int NT, int parts) { return parts * NT > 128 ? 1 : 2; }      // slabs of 64 k per stage
+inline int stage_bytes(int NT, int parts) { return stage_slabs(NT, parts) * (tc::BM * 128 + parts * NT * 128); }
 inline int smem_bytes(int NT, int parts, int stages) { return stages * stage_bytes(NT, parts) + 2 * 256 * 4 + 256 + 1024; }
 
 __device__ inline void ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -71,7 +75,7 @@ __device__ inline void ld32(uint32_t taddr, uint32_t (&r)[32]) {
 __device__ inline void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ inline bool epi_sync_or(bool v) {                 // barrier of the epilogue warps; true if it was true for any thread
   uint32_t r;
-  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
                : "=r"(r) : "r"((uint32_t)v) : "memory");
   return r != 0;
 }
@@ -86,12 +90,26 @@ __device__ inline void fold(float* v, int lane) {
   }
 }
 
+// [hi | lo] operand values of 32 rows: neighbouring lanes hold neighbouring features; of two rows the even
+// lane stores the first and the odd lane the second, both features in one 4-byte store per term.  `p`: the
+// lane pair's first feature of the first row.
+__device__ inline void store_rows_hi_lo(bf16* p, int ld, int lo_off, const float (&y)[32], int nv, bool ok, int lane) {
+  const bool odd = lane & 1;
+#pragma unroll
+  for (int j = 0; j < 32; j += 2) {
+    const float other = __shfl_xor_sync(0xffffffffu, odd ? y[j] : y[j + 1], 1);
+    const float a = odd ? other : y[j], b = odd ? y[j + 1] : other;
+    const int n = j + (odd ? 1 : 0);
+    if (n < nv && ok) tc::store_hi_lo2(p + (size_t)n * ld, a, b, lo_off);
+  }
+}
+
 template <int MODE, int PARTS>
 __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Epi e) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int NT = g.NT, ST = g.stages;
-  const int stage = tc::BM * 128 + PARTS * NT * 128;
+  const int NT = g.NT, ST = g.stages, SLABS = g.slabs;
+  const int w_slab = tc::BM * 128, a_slab = PARTS * NT * 128, stage = SLABS * (w_slab + a_slab);
   float* s_inv = reinterpret_cast<float*>(sm + ST * stage);                  // [2][256]
   uint64_t* full = reinterpret_cast<uint64_t*>(s_inv + 512);
   uint64_t* empty = full + MAX_STAGES;
@@ -101,18 +119,18 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
   __shared__ int s_fail;
   __shared__ Row s_row[2][MODE == PF_QKV ? 128 : 1];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int slabs = g.K / tc::BK;
+  const int slabs = g.K / tc::BK, steps = (slabs + SLABS - 1) / SLABS;
   uint32_t ncols = 32;
   while ((int)ncols < 2 * PARTS * NT) ncols <<= 1;
   const int acc_cols = (int)ncols / 2;
   if (tid == 0) {
     s_fail = 0;
-    for (int i = 0; i < ST; ++i) { ptx::mbar_init(full + i, 1); ptx::mbar_init(empty + i, 1); }
-    for (int i = 0; i < 2; ++i) { ptx::mbar_init(acc_full + i, 1); ptx::mbar_init(acc_empty + i, 128); }
+    for (int i = 0; i < ST; ++i) { ptx::mbar_init(full + i, 2); ptx::mbar_init(empty + i, 1); }
+    for (int i = 0; i < 2; ++i) { ptx::mbar_init(acc_full + i, 1); ptx::mbar_init(acc_empty + i, EPI_WARPS); }
     ptx::fence_mbar_init();
     ptx::prefetch_tmap(g.tmA);
   }
-  if (warp == 1) {
+  if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(tmem_slot)), "r"(ncols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -129,43 +147,35 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
     tm = u - tn * g.tiles_m;
   };
   if (warp == 0 && lane == 0) {
-    // ---- producer.  Weights do not depend on the previous kernel: the first stages' slabs are requested
-    // before the dependency wait.
-    auto wsrc = [&](int z, int tm) {
-      const bf16* W = MODE == PF_PREFIX ? e.layers[z].Wqkv : g.W;
-      return W + (size_t)(g.w_tile0 + tm) * slabs * (tc::BM * tc::BK);
-    };
-    int done = 0;                                            // slabs whose weights are already on their way
-    if ((int)blockIdx.x < g.tiles) {
-      int z, tm, tn;
-      tile_of(blockIdx.x, z, tm, tn);
-      const bf16* W = wsrc(z, tm);
-      done = slabs < ST ? slabs : ST;
-      for (int i = 0; i < done; ++i) {
-        ptx::mbar_expect_tx(full + i, stage);
-        ptx::bulk_load(sm + i * stage, W + (size_t)i * (tc::BM * tc::BK), tc::BM * 128, full + i);
-      }
-    }
-    ptx::grid_dep_wait();
+    // ---- weights: they do not depend on the previous kernel and start before the dependency wait
     int it = 0;
-    for (int t = blockIdx.x; t < g.tiles; t += gridDim.x) {
+    for (int t = blockIdx.x; t < g.tiles && !s_fail; t += gridDim.x) {
       int z, tm, tn;
       tile_of(t, z, tm, tn);
-      const bf16* W = wsrc(z, tm);
-      const int row = tn * NT + (MODE == PF_PREFIX ? z * e.rows_layer : 0);
-      for (int s = 0; s < slabs; ++s, ++it) {
-        const int st = it % ST;
-        unsigned char* dst = sm + st * stage;
-        if (it >= done) {
-          if (it >= ST && !ptx::mbar_wait(empty + st, ((it / ST) - 1) & 1)) { s_fail = 1; break; }
-          ptx::mbar_expect_tx(full + st, stage);
-          ptx::bulk_load(dst, W + (size_t)s * (tc::BM * tc::BK), tc::BM * 128, full + st);
-        }
-        ptx::tma_load_3d(dst + tc::BM * 128, g.tmA, s * tc::BK, row, 0, full + st);
+      const bf16* W = (MODE == PF_PREFIX ? e.layers[z].Wqkv : g.W) + (size_t)(g.w_tile0 + tm) * slabs * (tc::BM * tc::BK);
+      for (int s = 0; s < steps; ++s, ++it) {
+        const int st = it % ST, bytes = min(SLABS, slabs - s * SLABS) * w_slab;
+        if (it >= ST && !ptx::mbar_wait(empty + st, ((it / ST) - 1) & 1)) { s_fail = 1; break; }
+        ptx::mbar_expect_tx(full + st, bytes);
+        ptx::bulk_load(sm + st * stage, W + (size_t)s * SLABS * (tc::BM * tc::BK), bytes, full + st);
       }
-      if (s_fail) break;
     }
   } else if (warp == 1 && lane == 0) {
+    // ---- operand rows: one copy brings the hi and lo tiles of a stage (zeros behind the last slab)
+    ptx::grid_dep_wait();
+    int it = 0;
+    for (int t = blockIdx.x; t < g.tiles && !s_fail; t += gridDim.x) {
+      int z, tm, tn;
+      tile_of(t, z, tm, tn);
+      const int row = tn * NT + (MODE == PF_PREFIX ? z * e.rows_layer : 0);
+      for (int s = 0; s < steps; ++s, ++it) {
+        const int st = it % ST;
+        if (it >= ST && !ptx::mbar_wait(empty + st, ((it / ST) - 1) & 1)) { s_fail = 1; break; }
+        ptx::mbar_expect_tx(full + st, SLABS * a_slab);
+        ptx::tma_load_4d(sm + st * stage + SLABS * w_slab, g.tmA, 0, row, 0, s * SLABS, full + st);
+      }
+    }
+  } else if (warp == 2 && lane == 0) {
     // ---- MMA issuer
     const uint32_t idesc = tc::instr_desc_bf16(PARTS * NT);
     int it = 0, k = 0;
@@ -174,23 +184,25 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
       if (k >= 2 && !ptx::mbar_wait(acc_empty + buf, ((k >> 1) - 1) & 1)) { s_fail = 1; break; }
       tc::fence_after();
       bool bad = false;
-      for (int s = 0; s < slabs; ++s, ++it) {
-        const int st = it % ST;
+      for (int s = 0; s < steps; ++s, ++it) {
+        const int st = it % ST, n = min(SLABS, slabs - s * SLABS);
         if (!ptx::mbar_wait(full + st, (it / ST) & 1)) { s_fail = 1; bad = true; break; }
         tc::fence_after();
-        const uint32_t a_addr = ptx::smem_u32(sm + st * stage);
-        const uint64_t da = tc::smem_desc_sw128(a_addr), db = tc::smem_desc_sw128(a_addr + tc::BM * 128);
+        const uint32_t base = ptx::smem_u32(sm + st * stage);
+        for (int j = 0; j < n; ++j) {
+          const uint64_t da = tc::smem_desc_sw128(base + j * w_slab), db = tc::smem_desc_sw128(base + SLABS * w_slab + j * a_slab);
 #pragma unroll
-        for (int kk = 0; kk < tc::BK / 16; ++kk)
-          tc::mma_ss(tmem + buf * acc_cols, da + 2 * kk, db + 2 * kk, idesc, (s > 0 || kk > 0) ? 1u : 0u);
+          for (int kk = 0; kk < tc::BK / 16; ++kk)
+            tc::mma_ss(tmem + buf * acc_cols, da + 2 * kk, db + 2 * kk, idesc, (s > 0 || j > 0 || kk > 0) ? 1u : 0u);
+        }
         tc::commit(empty + st);
       }
       if (bad) break;
       tc::commit(acc_full + buf);
     }
-  } else if (warp >= 2) {
-    // ---- epilogue: warp w reads tensor-memory lanes 32 (w mod 4) .. + 31
-    const int w4 = warp & 3, et = tid - 64;
+  } else if (warp >= 4) {
+    // ---- epilogue: warp w reads tensor-memory lanes 32 (w mod 4) .. + 31; warps w and w + 4 share the rows
+    const int w4 = warp & 3, et = tid - 128;
     ptx::grid_dep_wait();
     int k = 0;
     for (int t = blockIdx.x; t < g.tiles; t += gridDim.x, ++k) {
@@ -201,7 +213,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
       const bool m_ok = m < g.M;
       float* inv = s_inv + buf * 256;
       if (MODE != PF_PREFIX) {
-        for (int n = et; n < nrows; n += 128) {
+        for (int n = et; n < nrows; n += EPI_WARPS * 32) {
           float v = 1.f;
           if (e.ssq_in != nullptr) {
             float ss = 0.f;
@@ -219,7 +231,9 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
       const bool late = !ptx::mbar_wait(acc_full + buf, (k >> 1) & 1);
       if (epi_sync_or(late)) { if (late) s_fail = 1; break; }
       tc::fence_after();
-      for (int c0 = 0; c0 < nrows; c0 += 32) {
+      const int c_first = (warp >= 8 ? 32 : 0);
+      if (c_first >= nrows && lane == 0) ptx::mbar_arrive(acc_empty + buf);          // nothing to read for this warp
+      for (int c0 = c_first; c0 < nrows; c0 += 64) {
         uint32_t r[32];
         float y[32];
         ld32(tmem + buf * acc_cols + ((uint32_t)(w4 * 32) << 16) + c0, r);
@@ -234,11 +248,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
 #pragma unroll
           for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(r[j]);
         }
-        if (c0 + 32 >= nrows) {                              // accumulator is in registers: the next tile may overwrite it
+        if (c0 + 64 >= nrows) {                              // this warp's share is in registers
           tc::fence_before();
-          ptx::mbar_arrive(acc_empty + buf);
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(acc_empty + buf);
         }
-        const int nv = min(32, nrows - c0);
+      const int nv = min(32, nrows - c0);
         const size_t row = (size_t)(n0 + c0);
         if (MODE != PF_PREFIX) {
 #pragma unroll
@@ -250,10 +265,9 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
           for (int j = 0; j < 32; ++j)
             if (j < nv && m_ok) o[(size_t)j * e.ldo] = y[j];
         } else if (MODE == PF_GELU) {
-          bf16* o = reinterpret_cast<bf16*>(e.out) + row * e.ldo + m;
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (j < nv && m_ok) tc::store_hi_lo(o + (size_t)j * e.ldo, tc::gelu_erf_f(y[j]), e.lo_off);
+          for (int j = 0; j < 32; ++j) y[j] = tc::gelu_erf_f(y[j]);
+          store_rows_hi_lo(reinterpret_cast<bf16*>(e.out) + row * e.ldo + (m & ~1), e.ldo, e.lo_off, y, nv, m_ok, lane);
         } else if (MODE == PF_RESID) {
           float* xr = e.x + row * e.ldx + m;
           if (e.add) {
@@ -267,10 +281,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
           for (int j = 0; j < 32; ++j)
             if (j < nv && m_ok) xr[(size_t)j * e.ldx] = y[j];
           if (e.a_out != nullptr) {
-            bf16* ao = e.a_out + row * e.lda + m;
+            float v[32];
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (j < nv && m_ok) tc::store_hi_lo(ao + (size_t)j * e.lda, __fmul_rn(y[j], gain), e.lo_off);
+            for (int j = 0; j < 32; ++j) v[j] = __fmul_rn(y[j], gain);
+            store_rows_hi_lo(e.a_out + row * e.lda + (m & ~1), e.lda, e.lo_off, v, nv, m_ok, lane);
           }
           if (e.ssq_out != nullptr) {
             // sums of squares of 32 rows over the warp's 32 features: lane i ends up with row c0 + i
