@@ -63,6 +63,7 @@ struct fm_ctx {
   // activations
   float *xc, *xv, *xf, *logits, *tmp3d;
   bf16 *qbuf, *a_norm, *a_up, *a_cat, *a_cat2, *a_attn, *a_ff;
+  PackedRow* row_map[3];                   // (sequence, position, -, cache slot) of the rows of a pass per level, b = -1: not fed
   bool fuse_hourglass;                     // shorten gather and upsample add inside the adjacent GEMM epilogues
   float *hc_ring, *hv_ring, *trif_ring, *triv_ring, *zc, *zv, *zf;
   // draft
@@ -254,6 +255,7 @@ void carve(fm_ctx* c, Carver& cv) {
   c->st.status = cv.take<int>(1); c->st.n_active = cv.take<int>(4); c->st.step = cv.take<int>(1);
   // activations (row counts padded to 16 so that later tiles never run off the end)
   const size_t Rc = align_up(B * dm.R1, 16), Rv = align_up(B * dm.mv, 16), Rf = align_up(B * dm.mf, 16);
+  c->row_map[0] = cv.take<PackedRow>(Rc); c->row_map[1] = cv.take<PackedRow>(Rv); c->row_map[2] = cv.take<PackedRow>(Rf);
   c->xc = cv.take<float>(Rc * d); c->xv = cv.take<float>(Rv * d); c->xf = cv.take<float>(Rf * d);
   c->qbuf = cv.take<bf16>(Rc * hd);
   c->ssq_ld = (int)((d + 127) / 128 * 16);                   // a slot per 8 features, at most
@@ -722,6 +724,55 @@ void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_ro
   if (mode == tc::EPI_UP && e.ssq_out != nullptr) c->ssq_n = (c->dm.d / tc::BM) * split * (split == 1 ? 2 : 1);   // tiles within d
 }
 
+// The tiled form (fm_prefill.cuh).  Rows per tile: the choice that minimises waves x (slabs x the longer of a
+// slab's copy at 64 B per clock and its MMAs, + about 2000 clocks of start-up and epilogue).
+void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, pf::Epi e, int layers = 1, int w_tile0 = 0,
+             const int* n_active = nullptr) {
+  if (R <= 0) return;
+  const int parts = mode == pf::PF_PREFIX ? 1 : 2, tiles_m = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
+  int NT = 32;
+  double best = 0.0;
+  for (int nt = 32; nt <= 256 / parts; nt *= 2) {
+    const double tiles = (double)tiles_m * ((R + nt - 1) / nt) * layers, waves = ceil(tiles / c->n_sm);
+    const double copy = (tc::BM * 128 + parts * nt * 128) / 64.0, mma = 2.0 * (parts * nt > 64 ? parts * nt : 64);
+    const double cost = waves * (slabs * (copy > mma ? copy : mma) + 12.0 * parts * nt) + 2000.0;
+    if (nt == 32 || cost < best) { best = cost; NT = nt; }
+  }
+  const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, NT, TMAP_STAGE + (uint32_t)parts);
+  if (tA < 0) { c->launch_error = FM_ERR_CUDA; return; }
+  int stages = (200 * 1024) / pf::stage_bytes(NT, parts);
+  stages = stages > pf::MAX_STAGES ? pf::MAX_STAGES : stages;
+  const int tiles_n = (R + NT - 1) / NT, tiles = tiles_m * tiles_n * layers;
+  if (mode == pf::PF_RESID && e.ssq_out != nullptr) c->ssq_n = tiles_m * 4;        // slots the next consumer adds
+  pf::Gemm g{W, c->tmaps + tA, M, K, R, NT, stages, pf::stage_slabs(NT, parts), tiles_m, tiles_n, tiles, w_tile0, n_active, c->st.status};
+  const dim3 grid(tiles < c->n_sm ? tiles : c->n_sm), one(1, 1, 1);
+  const int smem = pf::smem_bytes(NT, parts, stages);
+  switch (mode) {
+    case pf::PF_F32: launch_pdl(c, one, pf::gemm_kernel<pf::PF_F32, 2>, grid, pf::THREADS, smem, g, e); break;
+    case pf::PF_GELU: launch_pdl(c, one, pf::gemm_kernel<pf::PF_GELU, 2>, grid, pf::THREADS, smem, g, e); break;
+    case pf::PF_RESID: launch_pdl(c, one, pf::gemm_kernel<pf::PF_RESID, 2>, grid, pf::THREADS, smem, g, e); break;
+    case pf::PF_QKV: launch_pdl(c, one, pf::gemm_kernel<pf::PF_QKV, 2>, grid, pf::THREADS, smem, g, e); break;
+    default: launch_pdl(c, one, pf::gemm_kernel<pf::PF_PREFIX, 1>, grid, pf::THREADS, smem, g, e); break;
+  }
+}
+
+// Whether a projection of more than 16 rows goes to the tiled form, whose CTAs hold all of K and need no exchange, or
+// to the split-K form.  Measured at d = 1024 (us, tiled / split): 73 rows QKV 6.9 / 10.2, first FFN matrix 9.0 / 10.1,
+// output projection 9.0 / 6.2; 253 rows 7.5 / 12.9, 9.6 / 15.2, 9.1 / 9.0, second FFN matrix 23 / 14; 20 rows 6.8 / 5.8.
+bool tiled_gemm(fm_ctx* c, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, const int* n_active, int mode, const tc::Epi& e) {
+  const bool resid = mode == tc::EPI_RESID;
+  if (!resid && mode != tc::EPI_F32 && mode != tc::EPI_GELU && !(mode == tc::EPI_QKV && e.rows != nullptr && e.stash_ring == nullptr)) return false;
+  if (R < (resid ? (K <= 1536 ? 257 : 401) : 64)) return false;
+  pf::Epi t{};
+  t.ssq_in = e.ssq_in; t.ssq_n = e.ssq_n; t.ld_ssq = resid ? e.ld_ssq_out : e.ld_ssq; t.inv_d = e.inv_d_in; t.eps = e.eps;
+  t.out = e.out; t.ldo = e.ldo; t.lo_off = e.lo_off;
+  t.x = e.x; t.ldx = e.ldx; t.add = e.add; t.gain = e.gain; t.a_out = e.a_out; t.lda = e.lda; t.ssq_out = e.ssq_out;
+  if (mode == tc::EPI_QKV) { t.dm = e.dm; t.rows = e.rows; t.level = e.level; t.rope = e.rope_tab; t.qscale = e.qscale; t.q = e.q_out; t.Kc = e.Kc; t.Vc = e.Vc; }
+  const int m = resid ? pf::PF_RESID : mode == tc::EPI_F32 ? pf::PF_F32 : mode == tc::EPI_GELU ? pf::PF_GELU : pf::PF_QKV;
+  pf_gemm(c, m, W, A, a_rows_alloc, M, K, R, t, 1, 0, n_active);
+  return true;
+}
+
 // y[n][m] = W[w_row0 + m, :] . A[a_row0 + n, :], n < R, m < M, finished by the epilogue `mode`
 // (see fm_gemm_tc.cuh).  W: packed weight slabs of a matrix with K columns (w_row0 a multiple of
 // 128), A: [a_rows_alloc, a_parts * K] bf16 (rows padded to 16; a_parts = 2: [hi | lo] terms).
@@ -734,7 +785,8 @@ void gemm(fm_ctx* c, const bf16* W, size_t w_rows_alloc, int w_row0, const bf16*
   const long pi = prof_open(c, PROF_GEMM, 2.0 * M * K);            // algorithmic bytes: the weight matrix once
   c->cur_class = PROF_GEMM;
   if (c->only_class == PROF_GEMM) c->class_bytes += 2.0 * M * K * (stacked > 1 ? stacked : 1);
-  if (!gemm_rows(c, W, w_row0, A, a_row0, M, K, R, n_active, mode, e, a_parts, stacked, z_rows, z_w_rows))
+  if (!gemm_rows(c, W, w_row0, A, a_row0, M, K, R, n_active, mode, e, a_parts, stacked, z_rows, z_w_rows) &&
+      !(stacked == 1 && a_parts == 2 && w_row0 == 0 && a_row0 == 0 && tiled_gemm(c, W, A, a_rows_alloc, M, K, R, n_active, mode, e)))
     gemm_split(c, W, w_row0, A, a_rows_alloc, a_row0, M, K, R, n_active, mode, e, a_parts, stacked, z_rows, z_w_rows);
   c->cur_class = PROF_OTHER;
   prof_close(c, pi);
@@ -795,7 +847,7 @@ void run_stack(fm_ctx* c, int s, float* x, float* stash_ring, const float* next_
     }
     eq.ssq_in = c->ssq; eq.ssq_n = c->ssq_n; eq.ld_ssq = c->ssq_ld; eq.inv_d_in = 1.f / d; eq.eps = dm.eps;
     eq.dm = dm; eq.st = c->st; eq.batch = c->batch; eq.level = level; eq.rope_tab = c->rope_tab;
-    eq.q_out = c->qbuf; eq.Kc = L.K; eq.Vc = L.V;
+    eq.q_out = c->qbuf; eq.Kc = L.K; eq.Vc = L.V; eq.rows = c->row_map[level];
     eq.qscale = (float)(1.4426950408889634 / sqrt((double)dm.dh));   // 1/sqrt(dh) * log2(e)
     gemm(c, L.Wqkv, pad128(qkvw), 0, l == 0 && a_entry != nullptr ? a_entry : c->a_norm, Rc_alloc, 0, qkvw, d, rows, na, tc::EPI_QKV, eq, 2);
     attention(c, level, L);
@@ -842,7 +894,7 @@ void forward(fm_ctx* c, float* logits_out) {
     // parent belongs to an earlier pass that parent's stored slot.  Up: the upsampling GEMM's
     // epilogue adds slot r of parent u to child row 3u + r, whose residual row still holds the
     // pre-shorten hidden, and hands the child rows to the stack above.
-    LAUNCH(c, embed_kernel, Rc + 3 * (Rv + Rf), row_threads(d), 0, dm, c->st, B, c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc,
+    LAUNCH(c, embed_kernel, Rc + 3 * (Rv + Rf) + 1, row_threads(d), 0, dm, c->st, B, c->row_map[0], c->row_map[1], c->row_map[2], c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc,
            (const float*)c->hc_ring, (const float*)c->hv_ring, c->a_cat, c->a_cat2, Rv, Rf);
     c->ssq_n = 1;
     tc::Epi cat{};
@@ -868,7 +920,7 @@ void forward(fm_ctx* c, float* logits_out) {
     eu.level = 1; eu.x = c->xc; eu.gain = c->layers[4][0].g1; eu.tri_ring = c->triv_ring;
     gemm(c, c->U_vc, pad128(3 * d), 0, c->a_norm, Rc_alloc, 0, 3 * d, d, Rv, na, tc::EPI_UP, eu, 2);
   } else {
-    LAUNCH(c, embed_kernel, Rc, row_threads(d), 0, dm, c->st, B, c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc,
+    LAUNCH(c, embed_kernel, Rc + 1, row_threads(d), 0, dm, c->st, B, c->row_map[0], c->row_map[1], c->row_map[2], c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc,
            (const float*)nullptr, (const float*)nullptr, (bf16*)nullptr, (bf16*)nullptr, 0, 0);
     c->ssq_n = 1;
     run_stack(c, 0, c->xc, nullptr, nullptr, false);
@@ -1057,46 +1109,12 @@ __global__ void set_limits_kernel(Dims dm, SeqState st, int batch, const int* __
 // ------------------------------------------------------------------------------------------
 // prefill
 // ------------------------------------------------------------------------------------------
-// One GEMM of the prefill.  Rows per tile: the choice that minimises waves x (slabs x the longer of a
-// slab's copy at 64 B per clock and its MMAs, + about 2000 clocks of start-up and epilogue).
-void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, pf::Epi e, int layers = 1, int w_tile0 = 0) {
-  if (R <= 0) return;
-  const int parts = mode == pf::PF_PREFIX ? 1 : 2, tiles_m = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
-  int NT = 32;
-  double best = 0.0;
-  for (int nt = 32; nt <= 256 / parts; nt *= 2) {
-    const double tiles = (double)tiles_m * ((R + nt - 1) / nt) * layers, waves = ceil(tiles / c->n_sm);
-    const double copy = (tc::BM * 128 + parts * nt * 128) / 64.0, mma = 2.0 * (parts * nt > 64 ? parts * nt : 64);
-    const double cost = waves * (slabs * (copy > mma ? copy : mma) + 12.0 * parts * nt) + 2000.0;
-    if (nt == 32 || cost < best) { best = cost; NT = nt; }
-  }
-  const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, NT, TMAP_STAGE + (uint32_t)parts);
-  if (tA < 0) { c->launch_error = FM_ERR_CUDA; return; }
-  int stages = (200 * 1024) / pf::stage_bytes(NT, parts);
-  stages = stages > pf::MAX_STAGES ? pf::MAX_STAGES : stages;
-  const int tiles_n = (R + NT - 1) / NT, tiles = tiles_m * tiles_n * layers;
-  if (mode == pf::PF_RESID && e.ssq_out != nullptr) c->ssq_n = tiles_m * 4;        // slots the next consumer adds
-  pf::Gemm g{W, c->tmaps + tA, M, K, R, NT, stages, pf::stage_slabs(NT, parts), tiles_m, tiles_n, tiles, w_tile0, c->st.status};
-  const dim3 grid(tiles < c->n_sm ? tiles : c->n_sm), one(1, 1, 1);
-  const int smem = pf::smem_bytes(NT, parts, stages);
-  switch (mode) {
-    case pf::PF_F32: launch_pdl(c, one, pf::gemm_kernel<pf::PF_F32, 2>, grid, pf::THREADS, smem, g, e); break;
-    case pf::PF_GELU: launch_pdl(c, one, pf::gemm_kernel<pf::PF_GELU, 2>, grid, pf::THREADS, smem, g, e); break;
-    case pf::PF_RESID: launch_pdl(c, one, pf::gemm_kernel<pf::PF_RESID, 2>, grid, pf::THREADS, smem, g, e); break;
-    case pf::PF_QKV: launch_pdl(c, one, pf::gemm_kernel<pf::PF_QKV, 2>, grid, pf::THREADS, smem, g, e); break;
-    default: launch_pdl(c, one, pf::gemm_kernel<pf::PF_PREFIX, 1>, grid, pf::THREADS, smem, g, e); break;
-  }
-}
-
 struct PfChunk {
   const pf::Seg* segs;                   // device
   const int2* tiles[3];
   int n_segs, rows[3], n_tiles[3], tile_rows[3];
   bool direct[3], ends;                  // the cache can be written by the projection itself; some prompt ends here
 };
-
-// Fewer rows than this go through the decode pass's GEMM, which splits K over a cluster.
-constexpr int PF_SMALL = 256;
 
 template <int DH, int C, int QW>
 void pf_attention(fm_ctx* c, dim3 grid, const pf::Attn& at) {
@@ -1109,7 +1127,6 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
   auto& pr = c->pre;
   const int level = STACK_LEVEL[s], R = ch.rows[level], d = dm.d, hd = dm.H * dm.dh, kvw = dm.Hkv * dm.dh, qkvw = hd + 2 * kvw;
   const int nl = (int)c->layers[s].size(), ld = pr.rows[0], ldq = c->ssq_ld;
-  const bool small = R <= PF_SMALL && ch.direct[level];
   float* x = pr.x[level];
   int tK = -1, tV = -1;
   if (!ch.direct[level]) {
@@ -1123,18 +1140,17 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
     if (last && stash_ring != nullptr && ch.ends)
       launch_pdl(c, dim3(1, 1, 1), pf::stash_kernel, ch.n_segs, row_threads(d / 4), 0, dm, ch.segs, level, (const float*)x, stash_ring);
     const float qscale = (float)(1.4426950408889634 / sqrt((double)dm.dh));
-    pf::Epi eq{};
-    eq.ssq_in = pr.ssq; eq.ssq_n = c->ssq_n; eq.ld_ssq = ldq; eq.inv_d = 1.f / d; eq.eps = dm.eps;
-    tc::Epi sq{};
-    sq.ssq_in = pr.ssq; sq.ssq_n = c->ssq_n; sq.ld_ssq = ldq; sq.inv_d_in = 1.f / d; sq.eps = dm.eps;
-    if (small) {
-      sq.dm = dm; sq.st = c->st; sq.batch = c->batch; sq.level = level; sq.rows = pr.map[level]; sq.rope_tab = c->rope_tab;
-      sq.q_out = pr.q; sq.Kc = L.K; sq.Vc = L.V; sq.qscale = qscale;
-      gemm(c, L.Wqkv, pad128(qkvw), 0, pr.a, ld, 0, qkvw, d, R, nullptr, tc::EPI_QKV, sq, 2);
+    if (ch.direct[level]) {
+      tc::Epi eq{};
+      eq.ssq_in = pr.ssq; eq.ssq_n = c->ssq_n; eq.ld_ssq = ldq; eq.inv_d_in = 1.f / d; eq.eps = dm.eps;
+      eq.dm = dm; eq.st = c->st; eq.batch = c->batch; eq.level = level; eq.rows = pr.map[level]; eq.rope_tab = c->rope_tab;
+      eq.q_out = pr.q; eq.Kc = L.K; eq.Vc = L.V; eq.qscale = qscale;
+      gemm(c, L.Wqkv, pad128(qkvw), 0, pr.a, ld, 0, qkvw, d, R, nullptr, tc::EPI_QKV, eq, 2);
     } else {
+      pf::Epi eq{};
+      eq.ssq_in = pr.ssq; eq.ssq_n = c->ssq_n; eq.ld_ssq = ldq; eq.inv_d = 1.f / d; eq.eps = dm.eps;
       eq.dm = dm; eq.rows = pr.map[level]; eq.level = level; eq.rope = c->rope_tab; eq.qscale = qscale;
       eq.q = pr.q; eq.kbuf = pr.kbuf; eq.vbuf = pr.vbuf;
-      if (ch.direct[level]) { eq.Kc = L.K; eq.Vc = L.V; }
       pf_gemm(c, pf::PF_QKV, L.Wqkv, pr.a, ld, qkvw, d, R, eq);
     }
     pf::Attn at{dm, ch.segs, ch.tiles[level], level, pr.q, c->tmaps + L.tmK, c->tmaps + L.tmV, tK < 0 ? nullptr : c->tmaps + tK,
@@ -1152,29 +1168,16 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
     if (!ch.direct[level])
       launch_pdl(c, dim3(1, 1, 1), pf::cache_kernel, R, 128, 0, dm, ch.segs, (const pf::Row*)pr.map[level], level, (const bf16*)pr.kbuf,
                  (const bf16*)pr.vbuf, L.K, L.V);
-    const float* gain2 = last ? next_gain : c->layers[s][l + 1].g1;
-    const bool out2 = !last || want_a;
-    if (small) {
-      tc::Epi eo{};
-      eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq_out = ldq;
-      gemm(c, L.Wo, pad128(d), 0, pr.attn, ld, 0, d, hd, R, nullptr, tc::EPI_RESID, eo, 2);
-      tc::Epi e1 = epi_plain(pr.wide, 2 * dm.dff);
-      e1.lo_off = dm.dff;
-      e1.ssq_in = pr.ssq; e1.ssq_n = c->ssq_n; e1.ld_ssq = ldq; e1.inv_d_in = 1.f / d; e1.eps = dm.eps;
-      gemm(c, L.W1, pad128(dm.dff), 0, pr.a, ld, 0, dm.dff, d, R, nullptr, tc::EPI_GELU, e1, 2);
-      eo.gain = gain2;
-      if (!out2) { eo.a_out = nullptr; eo.ssq_out = nullptr; }
-      gemm(c, L.W2, pad128(d), 0, pr.wide, ld, 0, d, dm.dff, R, nullptr, tc::EPI_RESID, eo, 2);
-      continue;
-    }
-    pf::Epi eo{};
-    eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq = ldq;
-    pf_gemm(c, pf::PF_RESID, L.Wo, pr.attn, ld, d, hd, R, eo);
-    eq.out = pr.wide; eq.ldo = 2 * dm.dff; eq.lo_off = dm.dff; eq.ssq_n = c->ssq_n;
-    pf_gemm(c, pf::PF_GELU, L.W1, pr.a, ld, dm.dff, d, R, eq);
-    eo.gain = gain2;
-    if (!out2) { eo.a_out = nullptr; eo.ssq_out = nullptr; }
-    pf_gemm(c, pf::PF_RESID, L.W2, pr.wide, ld, d, dm.dff, R, eo);
+    tc::Epi eo{};
+    eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq_out = ldq;
+    gemm(c, L.Wo, pad128(d), 0, pr.attn, ld, 0, d, hd, R, nullptr, tc::EPI_RESID, eo, 2);
+    tc::Epi e1 = epi_plain(pr.wide, 2 * dm.dff);
+    e1.lo_off = dm.dff;
+    e1.ssq_in = pr.ssq; e1.ssq_n = c->ssq_n; e1.ld_ssq = ldq; e1.inv_d_in = 1.f / d; e1.eps = dm.eps;
+    gemm(c, L.W1, pad128(dm.dff), 0, pr.a, ld, 0, dm.dff, d, R, nullptr, tc::EPI_GELU, e1, 2);
+    eo.gain = last ? next_gain : c->layers[s][l + 1].g1;
+    if (last && !want_a) { eo.a_out = nullptr; eo.ssq_out = nullptr; }
+    gemm(c, L.W2, pad128(d), 0, pr.wide, ld, 0, d, dm.dff, R, nullptr, tc::EPI_RESID, eo, 2);
   }
 }
 
@@ -1193,29 +1196,14 @@ void pf_chunk(fm_ctx* c, const PfChunk& ch, const int* prompt, const int* prompt
     pf_stack(c, ch, up - 1, nullptr, nullptr, false);
     launch_pdl(c, one, pf::gather_kernel, dim3(ch.rows[up], 3), th, 0, dm, ch.segs, (const pf::Row*)pr.map[up], up, (const float*)pr.x[up - 1],
                (const float*)(up == 1 ? c->hc_ring : c->hv_ring), pr.wide);
-    const bf16* S = up == 1 ? c->S_cv : c->S_vf;
-    if (ch.rows[up] <= PF_SMALL) {
-      tc::Epi es{};
-      es.x = pr.x[up]; es.ldx = d; es.add = 0; es.gain = c->layers[up][0].g1; es.a_out = pr.a; es.lda = 2 * d; es.lo_off = d;
-      es.ssq_out = pr.ssq; es.ld_ssq_out = c->ssq_ld;
-      gemm(c, S, pad128(d), 0, pr.wide, pr.rows[1], 0, d, 3 * d, ch.rows[up], nullptr, tc::EPI_RESID, es, 2);
-    } else {
-      pf::Epi es{};
-      es.x = pr.x[up]; es.ldx = d; es.add = 0; es.gain = c->layers[up][0].g1; es.a_out = pr.a; es.lda = 2 * d; es.lo_off = d;
-      es.ssq_out = pr.ssq; es.ld_ssq = c->ssq_ld;
-      pf_gemm(c, pf::PF_RESID, S, pr.wide, pr.rows[1], d, 3 * d, ch.rows[up], es);
-    }
+    tc::Epi es{};
+    es.x = pr.x[up]; es.ldx = d; es.add = 0; es.gain = c->layers[up][0].g1; es.a_out = pr.a; es.lda = 2 * d; es.lo_off = d;
+    es.ssq_out = pr.ssq; es.ld_ssq_out = c->ssq_ld;
+    gemm(c, up == 1 ? c->S_cv : c->S_vf, pad128(d), 0, pr.wide, pr.rows[1], 0, d, 3 * d, ch.rows[up], nullptr, tc::EPI_RESID, es, 2);
   }
   pf_stack(c, ch, 2, c->zf, nullptr, true);
   for (int low = 1; low >= 0; --low) {                       // up
-    const bf16* U = low == 1 ? c->U_fv : c->U_vc;
-    if (ch.rows[low + 1] <= PF_SMALL) {
-      gemm(c, U, pad128(3 * d), 0, pr.a, pr.rows[0], 0, 3 * d, d, ch.rows[low + 1], nullptr, tc::EPI_F32, epi_plain(pr.wide, 3 * d), 2);
-    } else {
-      pf::Epi eu{};
-      eu.out = pr.wide; eu.ldo = 3 * d;
-      pf_gemm(c, pf::PF_F32, U, pr.a, pr.rows[0], 3 * d, d, ch.rows[low + 1], eu);
-    }
+    gemm(c, low == 1 ? c->U_fv : c->U_vc, pad128(3 * d), 0, pr.a, pr.rows[0], 0, 3 * d, d, ch.rows[low + 1], nullptr, tc::EPI_F32, epi_plain(pr.wide, 3 * d), 2);
     launch_pdl(c, one, pf::upsample_kernel, ch.rows[low], th, 0, dm, ch.segs, (const pf::Row*)pr.map[low], low,
                (const float*)reinterpret_cast<float*>(pr.wide), low == 1 ? c->hv_ring : c->hc_ring, low == 1 ? c->trif_ring : c->triv_ring, pr.x[low],
                (const float*)c->layers[low == 1 ? 3 : 4][0].g1, pr.a, pr.ssq, c->ssq_ld);

@@ -81,7 +81,7 @@ struct Epi {
   float* ssq_out; int ld_ssq_out;//            [rows][ld] partial sums of squares of the new x rows, a slot per tile and rank (may be null)
   Dims dm; SeqState st;          // EPI_QKV
   int batch, level;
-  const PackedRow* rows;         //            (b, p) of every row when the rows are packed (prefill); null: rows of a pass
+  const PackedRow* rows;         //            (b, p) of every row, b = -1: not fed; null: worked out from the state
   const float2* rope_tab;
   bf16* q_out;                   //            [rows, H*dh], rotated and scaled by qscale
   bf16* Kc; bf16* Vc;            //            caches [B, Hkv, slots, dh]
@@ -103,7 +103,7 @@ __device__ inline bool row_of(const Epi& e, int row, int& b, int& p) {
   const PackedRow r = e.rows[row];
   b = r.b;
   p = r.p;
-  return true;
+  return r.b >= 0;
 }
 
 __device__ inline uint64_t smem_desc_sw128(uint32_t addr) {

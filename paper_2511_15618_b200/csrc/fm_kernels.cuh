@@ -63,10 +63,23 @@ __device__ inline int fm_first_pos(const SeqState& st, int b, int level) {
 // ------------------------------------------------------------------------------------------
 // a1. candidate embedding: x[row] = E[cand[b][j]]  (zeros for rows that are not fed)
 // ------------------------------------------------------------------------------------------
-__global__ void embed_kernel(Dims dm, SeqState st, int batch, const bf16* __restrict__ E, float* __restrict__ x,
+__global__ void embed_kernel(Dims dm, SeqState st, int batch, PackedRow* map_c, PackedRow* map_v, PackedRow* map_f, const bf16* __restrict__ E, float* __restrict__ x,
                              const float* __restrict__ g, bf16* __restrict__ a_out, float* __restrict__ ssq, int ld_ssq,
                              int rows, const float* __restrict__ hc_ring, const float* __restrict__ hv_ring,
                              bf16* __restrict__ cat_v, bf16* __restrict__ cat_f, int rows_v, int rows_f) {
+  if (blockIdx.x == gridDim.x - 1) {
+    // the last block writes down which sequence and position every row of the pass is, per level
+    for (int l = 0; l < 3; ++l) {
+      PackedRow* m = l == 0 ? map_c : l == 1 ? map_v : map_f;
+      const int n = batch * fm_rows_per_seq(dm, l);
+      for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        int b, p;
+        const bool valid = fm_row_map(dm, st, batch, l, i, b, p);
+        m[i] = PackedRow{valid ? b : -1, valid ? p : 0, 0, valid ? p % dm.cap[l] : 0};
+      }
+    }
+    return;
+  }
   if ((int)blockIdx.x >= rows) {
     // Blocks behind the coordinate rows prepare the operand rows of the two shorten GEMMs (used when
     // the gather is fused into the producing GEMM's epilogue): part k of parent row u pools position

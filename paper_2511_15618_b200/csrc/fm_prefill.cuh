@@ -47,6 +47,7 @@ struct Gemm {
   int M, K, R, NT, stages, slabs;  // slabs of 64 k per stage: 1 or 2
   int tiles_m, tiles_n, tiles;   // tiles = tiles_m * tiles_n * layers (PF_PREFIX), else tiles_m * tiles_n
   int w_tile0;
+  const int* n_active;           // skip when *n_active == 0 (may be null)
   int* status;
 };
 struct Epi {
@@ -106,6 +107,11 @@ __device__ inline void store_rows_hi_lo(bf16* p, int ld, int lo_off, const float
 
 template <int MODE, int PARTS>
 __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Epi e) {
+  if (g.n_active != nullptr && *g.n_active == 0) {           // the whole grid leaves; keep the launch chain ordered
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
+    return;
+  }
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int NT = g.NT, ST = g.stages, SLABS = g.slabs;
@@ -322,7 +328,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
 #pragma unroll
               for (int j = 0; j < 32; ++j) {
                 const Row rw = s_row[buf][c0 + j];
-                if (j < nv && m_ok) o[(rw.b * (Hkv * slots) + rw.slot) * dh] = __float2bfloat16(y[j]);
+                if (j < nv && m_ok && rw.b >= 0) o[(rw.b * (Hkv * slots) + rw.slot) * dh] = __float2bfloat16(y[j]);
               }
             } else {
               bf16* o = (is_k ? e.kbuf : e.vbuf) + row * (size_t)(Hkv * dh) + hk * dh + i;
