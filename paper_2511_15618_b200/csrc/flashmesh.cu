@@ -642,7 +642,9 @@ bool gemm_rows(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, int a_row0, 
   int FT = K > 1536 ? 16 : 8;                              // long K: fewer CTAs, each of which reads all operand rows
   while (FT < 32 && (M + FT - 1) / FT * stacked > c->n_sm) FT *= 2;
   const int mtn = (parts * R + 15) / 16, smem = rg::smem_bytes(FT, K, mtn);
-  if (smem > 140 * 1024) return false;
+  // (weights of more than 64 KB only where an SM gets one CTA: a ring of slabs for larger ones was slower than the
+  // other form, 11.4 against 10.7 us per launch on the Large model)
+  if (smem > 140 * 1024 || (smem > 100 * 1024 && (M + FT - 1) / FT * stacked > c->n_sm)) return false;
   if (e.ssq_out != nullptr && c->dm.d % FT != 0) return false;
   const rg::Args g{W, A, parts * K, M, K, R, parts, w_row0 / tc::BM, a_row0, stacked > 1 ? z_rows : 0, stacked > 1 ? z_w_rows / tc::BM : 0,
                    n_active, c->st.status};
