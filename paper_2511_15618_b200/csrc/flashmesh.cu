@@ -83,6 +83,7 @@ struct fm_ctx {
   int attn_mt_draft[3];                      // query tiles of the draft modules' attention launches per level
   // attention scratch and TMA descriptors
   float* attn_part;
+  bool attn_two[3];                          // two CTAs per SM
   int attn_chunk, attn_G[3], attn_max_groups[3], attn_mt[3];
   CUtensorMap* tmaps;                    // device array
   std::vector<CUtensorMap> tmaps_host;
@@ -309,23 +310,29 @@ void carve(fm_ctx* c, Carver& cv) {
     const int dq = !dm.full ? 0 : (l == 0 ? (dm.nc > 3 * dm.nv + 9 * dm.Ef ? dm.nc : 3 * dm.nv + 9 * dm.Ef) : (l == 1 ? (dm.nv > 3 * dm.Ef ? dm.nv : 3 * dm.Ef) : dm.Ef));
     c->attn_mt_draft[l] = (dq * (dm.H / dm.Hkv) + 15) / 16;
     const int mt_max = c->attn_mt[l] > c->attn_mt_draft[l] ? c->attn_mt[l] : c->attn_mt_draft[l];
-    // Number of groups (1 .. what the merge holds: 24): the one that minimises waves x (chunks per CTA + a
-    // CTA's fixed cost), with the cache full.  The fixed cost (pipeline start, merge of the warps, and with
-    // several groups the partials and the merge launch) was measured at batch 16 as about 5 chunk times.
-    const int g_cap = dm.dh == 64 ? AttnCfg<64, 128, 4>::MAX_GROUPS : AttnCfg<128, 64, 4>::MAX_GROUPS;
-    const size_t tiles_l = (size_t)dm.Hkv * B * c->attn_mt[l];      // the verify pass decides the grouping
+    // Number of groups (1 .. what the merge holds: 24): the one that takes the fewest chunk times with the cache
+    // full.  Up to one CTA per SM: chunks per CTA + a CTA's fixed cost (pipeline start, merge of the warps, and
+    // with several groups the partials and the merge launch: about 3 and 6 chunk times).  More CTAs run two to an
+    // SM (three stages each) and share the memory bandwidth; that pays where there are more tiles than SMs (256
+    // tiles of a batch of 16: 54 us in 1.7 waves of one CTA per SM, 48 us in one wave of two), else by a wide margin only.
+    const int g_cap = AttnCfg<64, 128, 4, 5>::MAX_GROUPS;
+    const int tiles_l = dm.Hkv * (int)B * c->attn_mt[l];            // the verify pass decides the grouping
     int G = max_chunks;
     double best = 0.0;
+    c->attn_two[l] = false;
     for (int ng = 1; ng <= g_cap && ng <= max_chunks; ++ng) {
       const int Gc = (max_chunks + ng - 1) / ng, groups = (max_chunks + Gc - 1) / Gc;
-      const size_t waves = (tiles_l * groups + 147) / 148;
-      const double cost = (double)waves * (Gc + (groups == 1 ? 3 : 6));
-      if (ng == 1 || cost < best) { best = cost; G = Gc; }
+      const long n = (long)tiles_l * groups, r = n % 296;
+      const double fix = groups == 1 ? 3.0 : 6.0;
+      const bool two = n > 148;
+      const double cost = !two ? Gc + fix : (n / 296) * 2.0 * Gc + (r > 148 ? Gc * (r / 148.0) : r > 0 ? Gc : 0.0) + fix * ((n + 295) / 296);
+      if (ng == 1 || cost < best * (two && !c->attn_two[l] ? 0.8 : 1.0)) { best = cost; G = Gc; c->attn_two[l] = two; }
     }
     const char* gm = getenv("FM_ATTN_G");                 // tuning knob: chunks per group, all levels
     if (gm != nullptr && atoi(gm) > 0) {
       const int G_min = (max_chunks + g_cap - 1) / g_cap;
       G = atoi(gm) < G_min ? G_min : atoi(gm);
+      c->attn_two[l] = (long)tiles_l * ((max_chunks + G - 1) / G) > 148;
     }
     c->attn_G[l] = G;
     c->attn_max_groups[l] = (max_chunks + G - 1) / G;
@@ -808,11 +815,14 @@ void launch_attention(fm_ctx* c, const AttnArgs& a) {
   const Dims& dm = c->dm;
   const dim3 grid(a.max_groups, dm.Hkv * a.MT, c->batch), merge(dm.Hkv * a.MT * c->batch, 4), one(1, 1, 1);
   c->cur_class = PROF_ATTN;
+  const bool two = a.draft_nq == 0 && c->attn_two[a.level];
   if (dm.dh == 64) {
-    launch_pdl(c, one, attn_stream_kernel<64, 128, 4>, grid, AttnCfg<64, 128, 4>::THREADS, AttnCfg<64, 128, 4>::BYTES, a);
+    if (two) launch_pdl(c, one, attn_stream_kernel<64, 128, 4, 3>, grid, AttnCfg<64, 128, 4, 3>::THREADS, AttnCfg<64, 128, 4, 3>::BYTES, a);
+    else launch_pdl(c, one, attn_stream_kernel<64, 128, 4, 5>, grid, AttnCfg<64, 128, 4, 5>::THREADS, AttnCfg<64, 128, 4, 5>::BYTES, a);
     if (a.max_groups > 1) launch_pdl(c, one, attn_merge_kernel<64, 128>, merge, 128, 0, a);
   } else {
-    launch_pdl(c, one, attn_stream_kernel<128, 64, 4>, grid, AttnCfg<128, 64, 4>::THREADS, AttnCfg<128, 64, 4>::BYTES, a);
+    if (two) launch_pdl(c, one, attn_stream_kernel<128, 64, 4, 3>, grid, AttnCfg<128, 64, 4, 3>::THREADS, AttnCfg<128, 64, 4, 3>::BYTES, a);
+    else launch_pdl(c, one, attn_stream_kernel<128, 64, 4, 5>, grid, AttnCfg<128, 64, 4, 5>::THREADS, AttnCfg<128, 64, 4, 5>::BYTES, a);
     if (a.max_groups > 1) launch_pdl(c, one, attn_merge_kernel<128, 64>, merge, 128, 0, a);
   }
   c->cur_class = PROF_OTHER;
@@ -1581,8 +1591,10 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
       for (auto& L : c->layers[s]) lp.push_back({L.Wqkv, L.g1, L.K, L.V, STACK_LEVEL[s], 0});
     TRYCUDA(cudaMemcpy(c->pre.layers, lp.data(), lp.size() * sizeof(pf::LayerPtr), cudaMemcpyHostToDevice));
   }
-  TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<64, 128, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64, 128, 4>::BYTES));
-  TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<128, 64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128, 64, 4>::BYTES));
+  TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<64, 128, 4, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64, 128, 4, 5>::BYTES));
+  TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<64, 128, 4, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64, 128, 4, 3>::BYTES));
+  TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<128, 64, 4, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128, 64, 4, 5>::BYTES));
+  TRYCUDA(cudaFuncSetAttribute(attn_stream_kernel<128, 64, 4, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128, 64, 4, 3>::BYTES));
   std::vector<double> freq(dm.dh / 2);
   for (int i = 0; i < dm.dh / 2; ++i)
     freq[i] = dm.theta != 0.f ? pow((double)dm.theta, -2.0 * (double)i / (double)dm.dh) : 0.0;

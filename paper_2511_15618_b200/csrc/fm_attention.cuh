@@ -43,12 +43,12 @@ struct AttnArgs {
   int out_row_stride;
 };
 
-template <int DH, int C, int NW>
+template <int DH, int C, int NW, int ST>
 struct AttnCfg {
   static_assert(C % (16 * NW) == 0, "a compute warp owns a multiple of 16 slots of a chunk");
-  // Five stages of 32 KB: with the 64 KB of the projection in front (few rows, d = 1024) exactly what an SM
-  // holds, so that most of a group is on chip before the queries are.
-  static constexpr int STAGES = 5;
+  // Stages of 32 KB.  Five: with the 64 KB of the projection in front (few rows, d = 1024) exactly what an SM
+  // holds, so that most of a group is on chip before the queries are.  Three: two CTAs per SM.
+  static constexpr int STAGES = ST;
   static constexpr int KPW = C / NW;                        // slots of a chunk per warp
   static constexpr int HALVES = DH / 64;
   static constexpr int TILE = C * DH * 2;                   // bytes of one K (or V) tile
@@ -104,9 +104,9 @@ __device__ inline size_t attn_out_at(const AttnArgs& a, const AttnWork& w, int b
 }
 
 // grid (max_groups, Hkv * MT, batch); block (NW + 1) warps: NW compute warps and one producer warp.
-template <int DH, int C, int NW>
+template <int DH, int C, int NW, int ST>
 __global__ void __launch_bounds__((NW + 1) * 32, 1) attn_stream_kernel(const AttnArgs a) {
-  using CF = AttnCfg<DH, C, NW>;
+  using CF = AttnCfg<DH, C, NW, ST>;
   constexpr int KS = DH / 16, KB = CF::KPW / 16, NT = CF::KPW / 8;     // k-steps of Q K^T; 16-slot blocks and 8-slot tiles per warp
   const Dims& dm = a.dm;
   const int u = blockIdx.x, NG = a.max_groups;
