@@ -1636,7 +1636,7 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
     // (the upsampling epilogue lists at most 128 carried rows per slot: one per sequence)
     c->fuse_hourglass = c->dm.d % tc::BM == 0 && c->dm.max_batch <= 128 && !(nf != nullptr && nf[0] == '1');
     const char* sc = getenv("FM_STAGE_CAP");
-    c->stage_cap = sc != nullptr ? atoi(sc) : 4;        // measured: deeper rings cost more than they prefetch
+    c->stage_cap = sc != nullptr ? atoi(sc) : 3;        // (2 / 3 / 4 stages: 9.4 / 8.8 / 9.2 us per launch at batch 16, 11.5 / 10.1 / 10.7 us on Large)
   }
   *out = c;
   return FM_OK;
