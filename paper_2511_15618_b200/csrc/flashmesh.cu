@@ -1125,6 +1125,8 @@ struct PfChunk {
   const pf::Seg* segs;                   // device
   const int2* tiles[3];
   int n_segs, rows[3], n_tiles[3], tile_rows[3];
+  const int2* end_tiles;                 // the last row of every prompt that ends in the chunk
+  int n_ends;
   bool direct[3], ends;                  // the cache can be written by the projection itself; some prompt ends here
 };
 
@@ -1134,7 +1136,9 @@ void pf_attention(fm_ctx* c, dim3 grid, const pf::Attn& at) {
 }
 
 // one stack on the chunk's rows of its level
-void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const float* next_gain, bool want_a) {
+// `ends_only`: behind the last layer only the prompts' last positions matter (keys and values of all rows, everything
+// else for those rows alone); their attention output and residual rows are left in row b of the decode buffers.
+void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, bool want_a, bool ends_only = false) {
   const Dims& dm = c->dm;
   auto& pr = c->pre;
   const int level = STACK_LEVEL[s], R = ch.rows[level], d = dm.d, hd = dm.H * dm.dh, kvw = dm.Hkv * dm.dh, qkvw = hd + 2 * kvw;
@@ -1167,9 +1171,13 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
     }
     pf::Attn at{dm, ch.segs, ch.tiles[level], level, pr.q, c->tmaps + L.tmK, c->tmaps + L.tmV, tK < 0 ? nullptr : c->tmaps + tK,
                 tV < 0 ? nullptr : c->tmaps + tV, pr.attn, c->st.status};
-    const dim3 grid(dm.H, ch.n_tiles[level]);
-    const int qw = ch.tile_rows[level] / 16;
-    if (dm.dh == 64) {
+    const bool ends = last && ends_only;
+    if (ends) at.tiles = ch.end_tiles;
+    const dim3 grid(dm.H, ends ? ch.n_ends : ch.n_tiles[level]);
+    const int qw = ends ? (dm.dh == 64 ? 1 : 2) : ch.tile_rows[level] / 16;
+    if (ends && ch.n_ends == 0) {
+      // (no prompt ends here: only the keys and values are needed)
+    } else if (dm.dh == 64) {
       if (qw == 8) pf_attention<64, 128, 8>(c, grid, at);
       else if (qw == 2) pf_attention<64, 128, 2>(c, grid, at);
       else pf_attention<64, 128, 1>(c, grid, at);
@@ -1180,6 +1188,11 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
     if (!ch.direct[level])
       launch_pdl(c, dim3(1, 1, 1), pf::cache_kernel, R, 128, 0, dm, ch.segs, (const pf::Row*)pr.map[level], level, (const bf16*)pr.kbuf,
                  (const bf16*)pr.vbuf, L.K, L.V);
+    if (ends) {
+      if (ch.n_ends > 0)
+        launch_pdl(c, dim3(1, 1, 1), pf::last_rows_kernel, ch.n_segs, 256, 0, dm, ch.segs, (const bf16*)pr.attn, (const float*)x, c->a_attn, c->xc);
+      continue;
+    }
     tc::Epi eo{};
     eo.x = x; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = pr.a; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = pr.ssq; eo.ld_ssq_out = ldq;
     gemm(c, L.Wo, pad128(d), 0, pr.attn, ld, 0, d, hd, R, nullptr, tc::EPI_RESID, eo, 2);
@@ -1187,7 +1200,7 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, const floa
     e1.lo_off = dm.dff;
     e1.ssq_in = pr.ssq; e1.ssq_n = c->ssq_n; e1.ld_ssq = ldq; e1.inv_d_in = 1.f / d; e1.eps = dm.eps;
     gemm(c, L.W1, pad128(dm.dff), 0, pr.a, ld, 0, dm.dff, d, R, nullptr, tc::EPI_GELU, e1, 2);
-    eo.gain = last ? next_gain : c->layers[s][l + 1].g1;
+    eo.gain = last ? nullptr : c->layers[s][l + 1].g1;
     if (last && !want_a) { eo.a_out = nullptr; eo.ssq_out = nullptr; }
     gemm(c, L.W2, pad128(d), 0, pr.wide, ld, 0, d, dm.dff, R, nullptr, tc::EPI_RESID, eo, 2);
   }
@@ -1205,7 +1218,7 @@ void pf_chunk(fm_ctx* c, const PfChunk& ch, const int* prompt, const int* prompt
          (const float*)c->layers[0][0].g1, pr.a, pr.ssq, c->ssq_ld);
   c->ssq_n = 1;
   for (int up = 1; up <= 2; ++up) {                          // down: coordinate and vertex stacks, each followed by a shortening
-    pf_stack(c, ch, up - 1, nullptr, nullptr, false);
+    pf_stack(c, ch, up - 1, nullptr, false);
     launch_pdl(c, one, pf::gather_kernel, dim3(ch.rows[up], 3), th, 0, dm, ch.segs, (const pf::Row*)pr.map[up], up, (const float*)pr.x[up - 1],
                (const float*)(up == 1 ? c->hc_ring : c->hv_ring), pr.wide);
     tc::Epi es{};
@@ -1213,17 +1226,15 @@ void pf_chunk(fm_ctx* c, const PfChunk& ch, const int* prompt, const int* prompt
     es.ssq_out = pr.ssq; es.ld_ssq_out = c->ssq_ld;
     gemm(c, up == 1 ? c->S_cv : c->S_vf, pad128(d), 0, pr.wide, pr.rows[1], 0, d, 3 * d, ch.rows[up], nullptr, tc::EPI_RESID, es, 2);
   }
-  pf_stack(c, ch, 2, c->zf, nullptr, true);
+  pf_stack(c, ch, 2, c->zf, true);
   for (int low = 1; low >= 0; --low) {                       // up
     gemm(c, low == 1 ? c->U_fv : c->U_vc, pad128(3 * d), 0, pr.a, pr.rows[0], 0, 3 * d, d, ch.rows[low + 1], nullptr, tc::EPI_F32, epi_plain(pr.wide, 3 * d), 2);
     launch_pdl(c, one, pf::upsample_kernel, ch.rows[low], th, 0, dm, ch.segs, (const pf::Row*)pr.map[low], low,
                (const float*)reinterpret_cast<float*>(pr.wide), low == 1 ? c->hv_ring : c->hc_ring, low == 1 ? c->trif_ring : c->triv_ring, pr.x[low],
                (const float*)c->layers[low == 1 ? 3 : 4][0].g1, pr.a, pr.ssq, c->ssq_ld);
     c->ssq_n = 1;
-    pf_stack(c, ch, low == 1 ? 3 : 4, low == 1 ? c->zv : c->zc, low == 1 ? nullptr : c->g_out, true);
+    pf_stack(c, ch, low == 1 ? 3 : 4, low == 1 ? c->zv : c->zc, true, low == 0);
   }
-  if (ch.ends)
-    launch_pdl(c, one, pf::last_rows_kernel, ch.n_segs, 128, 0, dm, ch.segs, (const bf16*)pr.a, (const float*)pr.ssq, c->ssq_n, c->ssq_ld, c->a_norm, c->ssq);
 }
 
 int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off) {
@@ -1257,6 +1268,7 @@ int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off)
         if (s.p0[l] + s.n[l] > dm.cap[l]) ch.direct[l] = false;
       }
       ch.ends = ch.ends || s.last;
+      ch.n_ends += s.last ? 1 : 0;
       ch.n_segs++;
       segs.push_back(s);
       done += n;
@@ -1279,6 +1291,9 @@ int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off)
       std::sort(tiles.begin() + t0, tiles.end(), [&](const int2& x, const int2& y) { return sg[x.x].p0[l] + x.y > sg[y.x].p0[l] + y.y; });
       ch.n_tiles[l] = (int)(tiles.size() - t0);
     }
+    tile_at.push_back(tiles.size());
+    for (int k = 0; k < ch.n_segs; ++k)
+      if (segs[seg_at.back() + k].last) tiles.push_back(make_int2(k, segs[seg_at.back() + k].n[0] - 1));
     chunks.push_back(ch);
   }
   const size_t o_seg = align_up((B + 1) * sizeof(int), 16), o_tile = align_up(o_seg + segs.size() * sizeof(pf::Seg), 16);
@@ -1305,12 +1320,28 @@ int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off)
   for (size_t i = 0; i < chunks.size(); ++i) {
     PfChunk& ch = chunks[i];
     ch.segs = reinterpret_cast<const pf::Seg*>(pr.plan + o_seg) + seg_at[i];
-    for (int l = 0; l < 3; ++l) ch.tiles[l] = reinterpret_cast<const int2*>(pr.plan + o_tile) + tile_at[3 * i + l];
+    for (int l = 0; l < 3; ++l) ch.tiles[l] = reinterpret_cast<const int2*>(pr.plan + o_tile) + tile_at[4 * i + l];
+    ch.end_tiles = reinterpret_cast<const int2*>(pr.plan + o_tile) + tile_at[4 * i + 3];
     pf_chunk(c, ch, prompt, off_dev);
   }
-  tc::Epi el = epi_plain(c->logits, dm.Vpad);
-  el.ssq_in = c->ssq; el.ssq_n = 1; el.ld_ssq = c->ssq_ld; el.inv_d_in = 1.f / dm.d; el.eps = dm.eps;
-  gemm(c, c->W_out, dm.Vpad, 0, c->a_norm, align_up((size_t)dm.max_batch * dm.R1, 16), 0, dm.V, dm.d, B, nullptr, tc::EPI_F32, el, 2);
+  // ---- the last layer behind its attention and the logits, for the last position of every prompt
+  {
+    const LayerDev& L = c->layers[4].back();
+    const int d = dm.d, hd = dm.H * dm.dh;
+    const size_t ra = align_up((size_t)dm.max_batch * dm.R1, 16);
+    tc::Epi eo{};
+    eo.x = c->xc; eo.ldx = d; eo.add = 1; eo.gain = L.g2; eo.a_out = c->a_norm; eo.lda = 2 * d; eo.lo_off = d; eo.ssq_out = c->ssq; eo.ld_ssq_out = c->ssq_ld;
+    gemm(c, L.Wo, pad128(d), 0, c->a_attn, ra, 0, d, hd, B, nullptr, tc::EPI_RESID, eo, 2);
+    tc::Epi e1 = epi_plain(c->a_ff, 2 * dm.dff);
+    e1.lo_off = dm.dff;
+    e1.ssq_in = c->ssq; e1.ssq_n = c->ssq_n; e1.ld_ssq = c->ssq_ld; e1.inv_d_in = 1.f / d; e1.eps = dm.eps;
+    gemm(c, L.W1, pad128(dm.dff), 0, c->a_norm, ra, 0, dm.dff, d, B, nullptr, tc::EPI_GELU, e1, 2);
+    eo.gain = c->g_out;
+    gemm(c, L.W2, pad128(d), 0, c->a_ff, ra, 0, d, dm.dff, B, nullptr, tc::EPI_RESID, eo, 2);
+    tc::Epi el = epi_plain(c->logits, dm.Vpad);
+    el.ssq_in = c->ssq; el.ssq_n = c->ssq_n; el.ld_ssq = c->ssq_ld; el.inv_d_in = 1.f / d; el.eps = dm.eps;
+    gemm(c, c->W_out, dm.Vpad, 0, c->a_norm, ra, 0, dm.V, d, B, nullptr, tc::EPI_F32, el, 2);
+  }
   launch_pdl(c, dim3(1, 1, 1), pf::finish_kernel, B, 256, 0, dm, c->st, (const float*)c->logits, prompt, off_dev);
   return FM_OK;
 }

@@ -490,22 +490,19 @@ __global__ void cache_kernel(Dims dm, const Seg* __restrict__ segs, const Row* _
   }
 }
 
-// operand row and sum of squares of a prompt's last position -> row b of the logits GEMM
-__global__ void last_rows_kernel(Dims dm, const Seg* __restrict__ segs, const bf16* __restrict__ a, const float* __restrict__ ssq,
-                                 int ssq_n, int ld, bf16* __restrict__ a_out, float* __restrict__ ssq_out) {
+// attention output and residual row of a prompt's last position -> row b of the decode buffers
+__global__ void last_rows_kernel(Dims dm, const Seg* __restrict__ segs, const bf16* __restrict__ attn, const float* __restrict__ x,
+                                 bf16* __restrict__ attn_out, float* __restrict__ x_out) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const Seg& s = segs[blockIdx.x];
   if (!s.last) return;
-  const int row = s.r0[0] + s.n[0] - 1;
-  const uint4* src = reinterpret_cast<const uint4*>(a + (size_t)row * 2 * dm.d);
-  uint4* dst = reinterpret_cast<uint4*>(a_out + (size_t)s.b * 2 * dm.d);
-  for (int i = threadIdx.x; i < dm.d / 4; i += blockDim.x) dst[i] = src[i];
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int k = 0; k < ssq_n; ++k) t += ssq[(size_t)row * ld + k];
-    ssq_out[(size_t)s.b * ld] = t;
-  }
+  const size_t row = s.r0[0] + s.n[0] - 1;
+  const int hd = dm.H * dm.dh;
+  for (int i = threadIdx.x; i < hd / 4; i += blockDim.x)
+    reinterpret_cast<uint4*>(attn_out + (size_t)s.b * 2 * hd)[i] = reinterpret_cast<const uint4*>(attn + row * 2 * hd)[i];
+  for (int i = threadIdx.x; i < dm.d / 4; i += blockDim.x)
+    reinterpret_cast<float4*>(x_out + (size_t)s.b * dm.d)[i] = reinterpret_cast<const float4*>(x + row * dm.d)[i];
 }
 
 // state behind the prompt: the first main token is the argmax of the last position
