@@ -222,9 +222,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
         for (int n = et; n < nrows; n += EPI_WARPS * 32) {
           float v = 1.f;
           if (e.ssq_in != nullptr) {
+            const float* sq = e.ssq_in + (size_t)(n0 + n) * e.ld_ssq;
             float ss = 0.f;
+            if ((e.ssq_n & 3) == 0) {                        // (one round of wide loads: a scalar loop cost the epilogue 2 000 clocks)
 #pragma unroll 8
-            for (int s = 0; s < e.ssq_n; ++s) ss += __ldcg(e.ssq_in + (size_t)(n0 + n) * e.ld_ssq + s);
+              for (int s = 0; s < e.ssq_n; s += 4) { const float4 q = __ldcg(reinterpret_cast<const float4*>(sq + s)); ss += (q.x + q.y) + (q.z + q.w); }
+            } else {
+              for (int s = 0; s < e.ssq_n; ++s) ss += __ldcg(sq + s);
+            }
             v = rsqrtf(ss * e.inv_d + e.eps);
           }
           inv[n] = v;
