@@ -63,7 +63,6 @@ struct fm_ctx {
   // activations
   float *xc, *xv, *xf, *logits, *tmp3d;
   bf16 *qbuf, *a_norm, *a_up, *a_cat, *a_cat2, *a_attn, *a_ff;
-  PackedRow* row_map[3];                   // (sequence, position, -, cache slot) of the rows of a pass per level, b = -1: not fed
   bool fuse_hourglass;                     // shorten gather and upsample add inside the adjacent GEMM epilogues
   float *hc_ring, *hv_ring, *trif_ring, *triv_ring, *zc, *zv, *zf;
   // draft
@@ -71,7 +70,8 @@ struct fm_ctx {
   float *dh_y, *feat, *dlogits;
   float *label_g, *label_W, *label_margin;   // label head of the correction stage and its last results
   int* labels;
-  int *step_in, *step_cand, *step_nacc, *step_em, *step_kv;     // device side of fm_step_host
+  int* step_in;                              // fm_step_host: the host's candidates,
+  int *step_out, *step_out_dev;              // and its results in mapped host memory
   float* avg_rows;                           // [B*R1, Vpad] rows of the averaged merge
   // full draft modules: SP-Block attention (per head) and HF-Blocks (per offset), stacked per stage
   bf16 *spWq, *spWo; float* sp_ga;
@@ -145,7 +145,7 @@ struct fm_ctx {
     bool valid = false, failed = false;
     int64_t launches = 0;
     cudaGraphExec_t exec = nullptr;
-  } cg_verify, cg_draft;
+  } cg_verify, cg_draft, cg_step;
   bool call_graphs_off;   // plain launches only (diagnostic modes, calls that swap scratch buffers)
   int batch;
   bool gen_fresh;       // no fm_generate call since the last fm_prefill
@@ -252,11 +252,10 @@ void carve(fm_ctx* c, Carver& cv) {
   c->st.L = cv.take<int>(B); c->st.nrow = cv.take<int>(B); c->st.main_tok = cv.take<int>(B);
   c->st.done = cv.take<int>(B); c->st.t_end = cv.take<int>(B); c->st.plen = cv.take<int>(B);
   c->st.cand = cv.take<int>(B * dm.R1); c->st.o = cv.take<int>(B * dm.R1);
-  c->st.margin = cv.take<float>(B * dm.R1);
   c->st.status = cv.take<int>(1); c->st.n_active = cv.take<int>(4); c->st.step = cv.take<int>(1);
   // activations (row counts padded to 16 so that later tiles never run off the end)
   const size_t Rc = align_up(B * dm.R1, 16), Rv = align_up(B * dm.mv, 16), Rf = align_up(B * dm.mf, 16);
-  c->row_map[0] = cv.take<PackedRow>(Rc); c->row_map[1] = cv.take<PackedRow>(Rv); c->row_map[2] = cv.take<PackedRow>(Rf);
+  c->st.rows[0] = cv.take<PackedRow>(Rc); c->st.rows[1] = cv.take<PackedRow>(Rv); c->st.rows[2] = cv.take<PackedRow>(Rf);
   c->xc = cv.take<float>(Rc * d); c->xv = cv.take<float>(Rv * d); c->xf = cv.take<float>(Rf * d);
   c->qbuf = cv.take<bf16>(Rc * hd);
   c->ssq_ld = (int)((d + 127) / 128 * 16);                   // a slot per 8 features, at most
@@ -279,8 +278,7 @@ void carve(fm_ctx* c, Carver& cv) {
   c->label_g = cv.take<float>(d); c->label_W = cv.take<float>(3 * d);
   c->labels = cv.take<int>(B * dm.R1); c->label_margin = cv.take<float>(B * dm.R1);
   c->st.hist = cv.take<int>(B * FM_HIST);
-  c->step_in = cv.take<int>(B * dm.R1); c->step_cand = cv.take<int>(B * dm.R1); c->step_nacc = cv.take<int>(B);
-  c->step_em = cv.take<int>(B * dm.R1); c->step_kv = cv.take<int>(B * 3);
+  c->step_in = cv.take<int>(B * dm.R1);
   c->avg_rows = dm.avg ? cv.take<float>(B * dm.R1 * (size_t)dm.Vpad) : nullptr;
   c->hf_T[0] = 3 * dm.Ef; c->hf_T[1] = 3 * dm.nv + 9 * dm.Ef;
   c->draft_sets = dm.NH > c->hf_T[1] ? dm.NH : c->hf_T[1];
@@ -803,7 +801,7 @@ void gemm(fm_ctx* c, const bf16* W, size_t w_rows_alloc, int w_row0, const bf16*
 
 // rows fed at each level in this pass (n_active[level]); n_active[3] = unfinished sequences
 __global__ void row_count_kernel(Dims dm, SeqState st, int batch) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) count_rows(dm, st, batch);
+  count_rows(dm, st, batch);
 }
 
 // threads of a kernel that walks over one row of d values: one element per thread up to 512
@@ -859,7 +857,7 @@ void run_stack(fm_ctx* c, int s, float* x, float* stash_ring, const float* next_
     }
     eq.ssq_in = c->ssq; eq.ssq_n = c->ssq_n; eq.ld_ssq = c->ssq_ld; eq.inv_d_in = 1.f / d; eq.eps = dm.eps;
     eq.dm = dm; eq.st = c->st; eq.batch = c->batch; eq.level = level; eq.rope_tab = c->rope_tab;
-    eq.q_out = c->qbuf; eq.Kc = L.K; eq.Vc = L.V; eq.rows = c->row_map[level];
+    eq.q_out = c->qbuf; eq.Kc = L.K; eq.Vc = L.V; eq.rows = c->st.rows[level];
     eq.qscale = (float)(1.4426950408889634 / sqrt((double)dm.dh));   // 1/sqrt(dh) * log2(e)
     gemm(c, L.Wqkv, pad128(qkvw), 0, l == 0 && a_entry != nullptr ? a_entry : c->a_norm, Rc_alloc, 0, qkvw, d, rows, na, tc::EPI_QKV, eq, 2);
     attention(c, level, L);
@@ -885,16 +883,16 @@ void run_stack(fm_ctx* c, int s, float* x, float* stash_ring, const float* next_
   }
 }
 
-// the verify forward pass over st.cand / st.nrow (a1..a11)
-void forward(fm_ctx* c, float* logits_out) {
+// the verify forward pass over st.nrow rows of st.cand, or of `cand` (see embed_kernel) (a1..a11)
+void forward(fm_ctx* c, const int* cand, int merge, float* logits_out, int* o_out, float* margin_out) {
   const Dims& dm = c->dm;
   const int B = c->batch, d = dm.d;
   const int Rc = B * dm.R1, Rv = B * dm.mv, Rf = B * dm.mf;
   const size_t Rc_alloc = align_up((size_t)dm.max_batch * dm.R1, 16), Rv_alloc = align_up((size_t)dm.max_batch * dm.mv, 16);
   const int* na = c->st.n_active;
-  // The launch that opens a pass is a full barrier: the per-pass state (rows, lengths, row counts
-  // -- every call that changes them ends with a row count -- and candidates) is final before any
-  // later kernel's prologue can run.
+  // The launch that opens a pass waits for everything before it and only then lets the next prologues start: the
+  // per-pass state (rows, lengths, row counts and maps -- every call that changes them ends with a row count) is
+  // final before any of them reads it.
   const size_t Rf_alloc = align_up((size_t)dm.max_batch * dm.mf, 16);
   tc::Epi es{};
   es.ldx = d; es.add = 0; es.a_out = c->a_norm; es.lda = 2 * d; es.lo_off = d;
@@ -906,8 +904,8 @@ void forward(fm_ctx* c, float* logits_out) {
     // parent belongs to an earlier pass that parent's stored slot.  Up: the upsampling GEMM's
     // epilogue adds slot r of parent u to child row 3u + r, whose residual row still holds the
     // pre-shorten hidden, and hands the child rows to the stack above.
-    LAUNCH(c, embed_kernel, Rc + 3 * (Rv + Rf) + 1, row_threads(d), 0, dm, c->st, B, c->row_map[0], c->row_map[1], c->row_map[2], c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc,
-           (const float*)c->hc_ring, (const float*)c->hv_ring, c->a_cat, c->a_cat2, Rv, Rf);
+    launch_pdl(c, dim3(1, 1, 1), embed_kernel, Rc + 3 * (Rv + Rf), row_threads(d), 0, dm, c->st, B, cand, merge, (const bf16*)c->E, c->xc,
+               (const float*)c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc, (const float*)c->hc_ring, (const float*)c->hv_ring, c->a_cat, c->a_cat2, Rv, Rf);
     c->ssq_n = 1;
     tc::Epi cat{};
     cat.cat_out = c->a_cat; cat.cat_ring = c->hc_ring; cat.cat_tri = c->triv_ring;
@@ -932,8 +930,8 @@ void forward(fm_ctx* c, float* logits_out) {
     eu.level = 1; eu.x = c->xc; eu.gain = c->layers[4][0].g1; eu.tri_ring = c->triv_ring;
     gemm(c, c->U_vc, pad128(3 * d), 0, c->a_norm, Rc_alloc, 0, 3 * d, d, Rv, na, tc::EPI_UP, eu, 2);
   } else {
-    LAUNCH(c, embed_kernel, Rc + 1, row_threads(d), 0, dm, c->st, B, c->row_map[0], c->row_map[1], c->row_map[2], c->E, c->xc, c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc,
-           (const float*)nullptr, (const float*)nullptr, (bf16*)nullptr, (bf16*)nullptr, 0, 0);
+    launch_pdl(c, dim3(1, 1, 1), embed_kernel, Rc, row_threads(d), 0, dm, c->st, B, cand, merge, (const bf16*)c->E, c->xc,
+               (const float*)c->layers[0][0].g1, c->a_norm, c->ssq, c->ssq_ld, Rc, (const float*)nullptr, (const float*)nullptr, (bf16*)nullptr, (bf16*)nullptr, 0, 0);
     c->ssq_n = 1;
     run_stack(c, 0, c->xc, nullptr, nullptr, false);
     launch_pdl(c, dim3(1, 1, 1), shorten_gather_kernel, dim3(Rv + Rc, 3), row_threads(d), 0, dm, c->st, B, 1, (const float*)c->xc, c->hc_ring, c->a_cat, Rv);
@@ -958,7 +956,7 @@ void forward(fm_ctx* c, float* logits_out) {
   tc::Epi el = epi_plain(c->logits, dm.Vpad);
   el.ssq_in = c->ssq; el.ssq_n = c->ssq_n; el.ld_ssq = c->ssq_ld; el.inv_d_in = 1.f / d; el.eps = dm.eps;
   gemm(c, c->W_out, dm.Vpad, 0, c->a_norm, Rc_alloc, 0, dm.V, d, Rc, na, tc::EPI_F32, el, 2);
-  launch_pdl(c, dim3(1, 1, 1), verify_top2_kernel, Rc, 256, 0, dm, c->st, B, (const float*)c->logits, logits_out);
+  launch_pdl(c, dim3(1, 1, 1), verify_top2_kernel, Rc, 256, 0, dm, c->st, B, (const float*)c->logits, logits_out, o_out, margin_out);
 }
 
 // T problems of the same shape in one launch (grid.z): set t multiplies weight matrix t of the stacked
@@ -1018,7 +1016,7 @@ void hf_stage(fm_ctx* c, int k) {
 // a13: draft modules on the stashed split-node hiddens.  Reduced heads: SP = h + A rms(h), the
 // upsample matrices alone.  Full: the SP-Blocks' attention before the linear layer and an HF-Block
 // after every upsample (Sec. 3.1, Eq. 1-5; supplement "Three-Level Speculative Decoding").
-void draft(fm_ctx* c, float* logits_out, float* margin_out, const GenOut* gen) {
+void draft(fm_ctx* c, int* cand_out, float* logits_out, float* margin_out, const GenOut* gen) {
   const Dims& dm = c->dm;
   const int B = c->batch, d = dm.d;
   if (dm.D > 0) {
@@ -1030,7 +1028,8 @@ void draft(fm_ctx* c, float* logits_out, float* margin_out, const GenOut* gen) {
       // SP-Block attention: a = rms(z, ga); q = Wq a at the split node's position; o over the cache of
       // the level's last layer; u = Wo o; then the head's input is rms(z + u, g) instead of rms(z, g)
       const float qscale = (float)(1.4426950408889634 / sqrt((double)dm.dh));
-      LAUNCH(c, draft_prep_kernel, dim3(B, dm.NH), 256, 0, dm, c->st, B, c->zc, c->zv, c->zf, c->sp_ga, c->d_a);
+      launch_pdl(c, dim3(1, 1, 1), draft_prep_kernel, dim3(B, dm.NH), 256, 0, dm, c->st, B, (const float*)c->zc, (const float*)c->zv, (const float*)c->zf,
+                 (const float*)c->sp_ga, c->d_a);
       gemm_sets(c, c->spWq, round_up(hd, 128), hd, d, c->d_a, 1, dm.NH, tc::EPI_F32, epi_plain(c->d_qf, hd));
       const int cnt[3] = {dm.nc, dm.nv, dm.Ef}, stack_of[3] = {4, 3, 2};
       int h0 = 0;
@@ -1047,7 +1046,8 @@ void draft(fm_ctx* c, float* logits_out, float* margin_out, const GenOut* gen) {
       launch_pdl(c, dim3(1, 1, 1), sp_mid_kernel, dim3(B, dm.NH), 256, 0, dm, c->st, B, (const float*)c->zc, (const float*)c->zv,
                  (const float*)c->zf, (const float*)c->d_out, (const float*)c->head_g, c->dh_a);
     } else {
-      LAUNCH(c, draft_prep_kernel, dim3(B, dm.NH), 256, 0, dm, c->st, B, c->zc, c->zv, c->zf, c->head_g, c->dh_a);
+      launch_pdl(c, dim3(1, 1, 1), draft_prep_kernel, dim3(B, dm.NH), 256, 0, dm, c->st, B, (const float*)c->zc, (const float*)c->zv, (const float*)c->zf,
+                 (const float*)c->head_g, c->dh_a);
     }
     if (B <= 32) {                                               // the NH head matrices as one launch
       gemm(c, c->headA, (size_t)dm.NH * dpad, 0, c->dh_a, (size_t)dm.NH * MB + 16, 0, d, d, B, na, tc::EPI_F32, epi_plain(c->dh_y, d), 1,
@@ -1081,24 +1081,7 @@ void draft(fm_ctx* c, float* logits_out, float* margin_out, const GenOut* gen) {
   const bool lab = dm.has_label != 0 && dm.D > 0;
   launch_pdl(c, dim3(1, 1, 1), draft_pick_kernel, dim3(B, dm.R1), 256, 0, dm, c->st, B, (const float*)c->dlogits, logits_out, margin_out, gen,
              (const bf16*)c->up_in_v, (const float*)c->label_g, (const float*)c->label_W, lab ? c->labels : (int*)nullptr, c->label_margin,
-             c->avg_rows);
-}
-
-__global__ void verify_load_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ cand) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= batch * dm.R1) return;
-  const int b = i / dm.R1, j = i - b * dm.R1;
-  const int t = cand[i];
-  if (j == 0 && st.nrow[b] > 0 && t != st.main_tok[b]) atomicExch(st.status, FM_ERR_INVALID_ARG);
-  st.cand[i] = t;
-}
-
-// candidates of a host-driven pass: the host's entry where it gave one (>= 0), else the draft modules'
-__global__ void step_merge_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ host_cand, int* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= batch * dm.R1) return;
-  const int h = host_cand != nullptr ? host_cand[i] : -1;
-  out[i] = (h >= 0 && i % dm.R1 != 0) ? h : st.cand[i];          // slot 0 is always the pending main token
+             c->avg_rows, cand_out);
 }
 
 __global__ void init_state_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ prompt_off) {
@@ -1349,10 +1332,10 @@ int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off)
 // one decode pass of fm_generate
 void step_body(fm_ctx* c) {
   const Dims& dm = c->dm;
-  draft(c, nullptr, nullptr, (const GenOut*)c->gen_dev);
-  forward(c, nullptr);
-  LAUNCH(c, accept_kernel, 1, accept_threads(c->batch), 0, dm, c->st, c->batch, (const int*)nullptr, (const int*)nullptr,
-         (int*)nullptr, (int*)nullptr, (int*)nullptr, (const GenOut*)c->gen_dev, 1);
+  draft(c, nullptr, nullptr, nullptr, (const GenOut*)c->gen_dev);
+  forward(c, nullptr, 0, nullptr, nullptr, nullptr);
+  launch_pdl(c, dim3(1, 1, 1), accept_kernel, 1, accept_threads(c->batch), 0, dm, c->st, c->batch, (const int*)nullptr, (const int*)nullptr,
+             (int*)nullptr, (int*)nullptr, (int*)nullptr, (const GenOut*)c->gen_dev, 1);
 }
 
 // Walk through `body` without launching anything: afterwards the descriptors of its launches exist (they
@@ -1638,6 +1621,8 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
   TRYCUDA(cudaHostAlloc(reinterpret_cast<void**>(&c->host_done), 64, cudaHostAllocMapped));
   *c->host_done = 0;
   TRYCUDA(cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->host_done_dev), c->host_done, 0));
+  TRYCUDA(cudaHostAlloc(reinterpret_cast<void**>(&c->step_out), (size_t)dm.max_batch * (dm.R1 + 4) * sizeof(int), cudaHostAllocMapped));
+  TRYCUDA(cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->step_out_dev), c->step_out, 0));
   TRYCUDA(cudaDeviceSynchronize());
 #undef TRY
 #undef TRYCUDA
@@ -1700,14 +1685,14 @@ int fm_profile_class(fm_ctx* c, int32_t cls, int32_t reps, fm_profile* out) {
   if (c == nullptr || out == nullptr || reps < 1 || (cls != PROF_GEMM && cls != PROF_ATTN)) return FM_ERR_INVALID_ARG;
   if (c->phase < 1) return FM_ERR_BAD_STATE;
   memset(out, 0, sizeof(*out));
-  make_descriptors(c, [&] { forward(c, nullptr); });
+  make_descriptors(c, [&] { forward(c, nullptr, 0, nullptr, nullptr, nullptr); });
   CUDA_OK(cudaStreamSynchronize(c->stream));
   if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); return FM_ERR_CUDA; }
   const int64_t l0 = c->launches;
   c->only_class = cls;
   c->class_bytes = 0.0;
   c->capturing = true;
-  forward(c, nullptr);
+  forward(c, nullptr, 0, nullptr, nullptr, nullptr);
   c->capturing = false;
   c->only_class = -1;
   const int64_t n_launch = c->launches - l0;
@@ -1749,7 +1734,9 @@ int fm_destroy(fm_ctx* c) {
   drop_graph(c);
   drop_call_graph(c->cg_verify);
   drop_call_graph(c->cg_draft);
+  drop_call_graph(c->cg_step);
   if (c->host_done != nullptr) cudaFreeHost(c->host_done);
+  if (c->step_out != nullptr) cudaFreeHost(c->step_out);
   delete c;
   return FM_OK;
 }
@@ -1777,7 +1764,7 @@ int fm_prefill(fm_ctx* c, int32_t batch, const float* cond, const int32_t* promp
   const int rc = prefill_run(c, cond, prompt, prompt_off);
   if (rc != FM_OK) return rc;
   LAUNCH(c, arm_kernel, (batch + 127) / 128, 128, 0, dm, c->st, batch);
-  LAUNCH(c, row_count_kernel, 1, 32, 0, dm, c->st, batch);
+  LAUNCH(c, row_count_kernel, 1, 128, 0, dm, c->st, batch);
   CUDA_OK(cudaGetLastError());
   if (c->launch_error != FM_OK) return c->launch_error;
   c->phase = 1;
@@ -1793,7 +1780,7 @@ int fm_set_max_faces(fm_ctx* c, const int32_t* max_faces) {
   CUDA_OK(cudaMemcpyAsync(tmp, max_faces, c->batch * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   LAUNCH(c, set_limits_kernel, (c->batch + 127) / 128, 128, 0, c->dm, c->st, c->batch, tmp);
   LAUNCH(c, arm_kernel, (c->batch + 127) / 128, 128, 0, c->dm, c->st, c->batch);
-  LAUNCH(c, row_count_kernel, 1, 32, 0, c->dm, c->st, c->batch);
+  LAUNCH(c, row_count_kernel, 1, 128, 0, c->dm, c->st, c->batch);
   CUDA_OK(cudaStreamSynchronize(c->stream));       // max_faces is caller memory
   return FM_OK;
 }
@@ -1802,9 +1789,7 @@ int fm_draft(fm_ctx* c, int32_t* cand, float* draft_logits, float* draft_margin)
   if (c == nullptr) return FM_ERR_INVALID_ARG;
   if (c->phase < 1) return FM_ERR_BAD_STATE;
   run_cached(c, c->cg_draft, cand, draft_logits, draft_margin, nullptr, [&] {
-    draft(c, draft_logits, draft_margin, nullptr);
-    const int n = c->batch * c->dm.R1;
-    if (cand != nullptr) LAUNCH(c, copy_i32_kernel, (n + 127) / 128, 128, 0, c->st.cand, cand, n);
+    draft(c, cand, draft_logits, draft_margin, nullptr);
   });
   CUDA_OK(cudaGetLastError());
   if (c->launch_error != FM_OK) return c->launch_error;
@@ -1844,13 +1829,7 @@ int fm_draft_labels(fm_ctx* c, int32_t* labels, float* margin) {
 int fm_verify(fm_ctx* c, const int32_t* cand, int32_t* argmax, float* logits, float* margin) {
   if (c == nullptr || cand == nullptr) return FM_ERR_INVALID_ARG;
   if (c->phase < 1) return FM_ERR_BAD_STATE;
-  run_cached(c, c->cg_verify, cand, argmax, logits, margin, [&] {
-    const int n = c->batch * c->dm.R1;
-    LAUNCH(c, verify_load_kernel, (n + 127) / 128, 128, 0, c->dm, c->st, c->batch, cand);
-    forward(c, logits);
-    if (argmax != nullptr) LAUNCH(c, copy_i32_kernel, (n + 127) / 128, 128, 0, c->st.o, argmax, n);
-    if (margin != nullptr) LAUNCH(c, copy_f32_kernel, (n + 127) / 128, 128, 0, c->st.margin, margin, n);
-  });
+  run_cached(c, c->cg_verify, cand, argmax, logits, margin, [&] { forward(c, cand, 0, logits, argmax, margin); });
   CUDA_OK(cudaGetLastError());
   if (c->launch_error != FM_OK) return c->launch_error;
   c->phase = 2;
@@ -1900,20 +1879,25 @@ int fm_verify_static_scratch(fm_ctx* c, const int32_t* cand, int32_t* argmax, fl
 int fm_step_host(fm_ctx* c, const int32_t* cand, int32_t* n_acc, int32_t* emitted, int32_t* kv_len) {
   if (c == nullptr || n_acc == nullptr) return FM_ERR_INVALID_ARG;
   if (c->phase < 1) return FM_ERR_BAD_STATE;
-  const Dims& dm = c->dm;
-  const int n = c->batch * dm.R1;
+  // The candidates go in before the draft step, which does not touch them; the results are written to mapped host
+  // memory by the accept kernel, so that no copy stands between the kernels of the pass or behind them.
+  const int B = c->batch, R1 = c->dm.R1, n = B * R1;
+  if (cand != nullptr) CUDA_OK(cudaMemcpyAsync(c->step_in, cand, n * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  else CUDA_OK(cudaMemsetAsync(c->step_in, 0xff, n * sizeof(int), c->stream));
   int rc = fm_draft(c, nullptr, nullptr, nullptr);
   if (rc != FM_OK) return rc;
-  if (cand != nullptr) CUDA_OK(cudaMemcpyAsync(c->step_in, cand, n * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  LAUNCH(c, step_merge_kernel, (n + 127) / 128, 128, 0, dm, c->st, c->batch, cand != nullptr ? (const int*)c->step_in : (const int*)nullptr, c->step_cand);
-  rc = fm_verify(c, c->step_cand, nullptr, nullptr, nullptr);
+  run_cached(c, c->cg_step, c->step_in, nullptr, nullptr, nullptr, [&] { forward(c, c->step_in, 1, nullptr, nullptr, nullptr); });
+  CUDA_OK(cudaGetLastError());
+  if (c->launch_error != FM_OK) return c->launch_error;
+  c->phase = 2;
+  int* dev = c->step_out_dev;                        // [B] lengths, [B, R1] tokens, [B, 3] cache lengths
+  rc = fm_accept(c, nullptr, nullptr, dev, dev + B, dev + B + n);
   if (rc != FM_OK) return rc;
-  rc = fm_accept(c, nullptr, nullptr, c->step_nacc, c->step_em, c->step_kv);
-  if (rc != FM_OK) return rc;
-  CUDA_OK(cudaMemcpyAsync(n_acc, c->step_nacc, c->batch * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  if (emitted != nullptr) CUDA_OK(cudaMemcpyAsync(emitted, c->step_em, n * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  if (kv_len != nullptr) CUDA_OK(cudaMemcpyAsync(kv_len, c->step_kv, c->batch * 3 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_OK(cudaStreamSynchronize(c->stream));
+  const int* out = c->step_out;
+  memcpy(n_acc, out, B * sizeof(int));
+  if (emitted != nullptr) memcpy(emitted, out + B, n * sizeof(int));
+  if (kv_len != nullptr) memcpy(kv_len, out + B + n, B * 3 * sizeof(int));
   return FM_OK;
 }
 
@@ -1921,8 +1905,8 @@ int fm_accept(fm_ctx* c, const int32_t* force_len, const int32_t* force_tok, int
               int32_t* kv_len) {
   if (c == nullptr) return FM_ERR_INVALID_ARG;
   if (c->phase != 2) return FM_ERR_BAD_STATE;
-  LAUNCH(c, accept_kernel, 1, accept_threads(c->batch), 0, c->dm, c->st, c->batch, force_len, force_tok, n_acc, emitted, kv_len,
-         (const GenOut*)nullptr, 0);
+  launch_pdl(c, dim3(1, 1, 1), accept_kernel, 1, accept_threads(c->batch), 0, c->dm, c->st, c->batch, force_len, force_tok, n_acc, emitted, kv_len,
+             (const GenOut*)nullptr, 0);
   CUDA_OK(cudaGetLastError());
   if (c->launch_error != FM_OK) return c->launch_error;
   c->phase = 1;

@@ -30,6 +30,10 @@ struct Dims {
   int has_label;              // a label head was given
 };
 
+// One row of a level's activation matrix: sequence (-1: not fed), level-local position, segment (prefill), cache slot
+// behind the prefix.
+struct alignas(16) PackedRow { int b, p, seg, slot; };
+
 // Per-sequence decoding state, all int32 arrays of max_batch entries in device memory.
 struct SeqState {
   int* L;          // inputs consumed (coordinate KV length behind the prefix)
@@ -40,10 +44,10 @@ struct SeqState {
   int* plen;       // prompt length in tokens
   int* cand;       // [max_batch, R1] inputs of the current pass
   int* o;          // [max_batch, R1] masked argmax per row
-  float* margin;   // [max_batch, R1]
   int* status;     // device status word
   int* n_active;   // sequences with nrow > 0 in the current pass
   int* step;       // passes executed by fm_generate (schedule index)
+  PackedRow* rows[3];  // per level, the rows of the next / current pass
   int* hist;       // [max_batch, FM_HIST] accepted mesh tokens, token t_i at entry i mod FM_HIST
 };
 
@@ -68,9 +72,6 @@ __device__ inline bool fm_row_map(const Dims& dm, const SeqState& st, int batch,
   p = (Lb + ratio - 1) / ratio + k;
   return ratio * p <= Lb + n - 1;
 }
-
-// One row of a packed prefill chunk: sequence, level-local position, segment, cache slot behind the prefix.
-struct alignas(16) PackedRow { int b, p, seg, slot; };
 
 __device__ inline float warp_sum(float v) {
 #pragma unroll

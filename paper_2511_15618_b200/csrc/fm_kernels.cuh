@@ -63,23 +63,14 @@ __device__ inline int fm_first_pos(const SeqState& st, int b, int level) {
 // ------------------------------------------------------------------------------------------
 // a1. candidate embedding: x[row] = E[cand[b][j]]  (zeros for rows that are not fed)
 // ------------------------------------------------------------------------------------------
-__global__ void embed_kernel(Dims dm, SeqState st, int batch, PackedRow* map_c, PackedRow* map_v, PackedRow* map_f, const bf16* __restrict__ E, float* __restrict__ x,
+__global__ void embed_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ cand_in, int merge, const bf16* __restrict__ E, float* __restrict__ x,
                              const float* __restrict__ g, bf16* __restrict__ a_out, float* __restrict__ ssq, int ld_ssq,
                              int rows, const float* __restrict__ hc_ring, const float* __restrict__ hv_ring,
                              bf16* __restrict__ cat_v, bf16* __restrict__ cat_f, int rows_v, int rows_f) {
-  if (blockIdx.x == gridDim.x - 1) {
-    // the last block writes down which sequence and position every row of the pass is, per level
-    for (int l = 0; l < 3; ++l) {
-      PackedRow* m = l == 0 ? map_c : l == 1 ? map_v : map_f;
-      const int n = batch * fm_rows_per_seq(dm, l);
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        int b, p;
-        const bool valid = fm_row_map(dm, st, batch, l, i, b, p);
-        m[i] = PackedRow{valid ? b : -1, valid ? p : 0, 0, valid ? p % dm.cap[l] : 0};
-      }
-    }
-    return;
-  }
+  // Launched with the programmatic attribute: whatever precedes the pass has completed behind the wait, and only then
+  // may the prologues of the pass's kernels start, which read the per-pass state.
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   if ((int)blockIdx.x >= rows) {
     // Blocks behind the coordinate rows prepare the operand rows of the two shorten GEMMs (used when
     // the gather is fused into the producing GEMM's epilogue): part k of parent row u pools position
@@ -105,8 +96,19 @@ __global__ void embed_kernel(Dims dm, SeqState st, int batch, PackedRow* map_c, 
   int b, p;
   const bool valid = fm_row_map(dm, st, batch, 0, row, b, p);
   int tok = 0;
+  {
+    // the candidates of the pass: those of the draft step, the caller's (slot 0 has to be the pending main token), or
+    // (merge) the caller's where they are >= 0, never in slot 0
+    const int bb = row / dm.R1, j = row - bb * dm.R1;
+    const int own = cand_in != nullptr ? cand_in[row] : -1;
+    const bool take = cand_in != nullptr && (!merge || (own >= 0 && j != 0));
+    tok = take ? own : st.cand[row];
+    if (take && threadIdx.x == 0) {
+      if (j == 0 && st.nrow[bb] > 0 && own != st.main_tok[bb]) atomicExch(st.status, -1);
+      st.cand[row] = own;
+    }
+  }
   if (valid) {
-    tok = st.cand[b * dm.R1 + (row - b * dm.R1)];
     if (tok < 0 || tok >= dm.V) {                    // never index outside the table
       if (threadIdx.x == 0) atomicExch(st.status, -1);
       tok = dm.n_bins + 2;
@@ -260,24 +262,30 @@ __device__ inline Top2 block_top2(const float* __restrict__ z, const Dims& dm, i
 }
 
 __global__ void verify_top2_kernel(Dims dm, SeqState st, int batch, const float* __restrict__ logits,
-                                   float* __restrict__ logits_out) {
+                                   float* __restrict__ logits_out, int* __restrict__ o_out, float* __restrict__ margin_out) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int row = blockIdx.x;
   int b, p;
   const bool valid = fm_row_map(dm, st, batch, 0, row, b, p);
-  const int j = row % dm.R1;
-  const int bb = row / dm.R1;
-  if (bb >= batch) return;
+  if (row / dm.R1 >= batch) return;
   if (logits_out != nullptr)
     for (int i = threadIdx.x; i < dm.V; i += blockDim.x)
       logits_out[(size_t)row * dm.V + i] = valid ? logits[(size_t)row * dm.Vpad + i] : 0.f;
   if (!valid) {
-    if (threadIdx.x == 0) { st.o[bb * dm.R1 + j] = -1; st.margin[bb * dm.R1 + j] = 0.f; }
+    if (threadIdx.x == 0) {
+      st.o[row] = -1;
+      if (o_out != nullptr) o_out[row] = -1;
+      if (margin_out != nullptr) margin_out[row] = 0.f;
+    }
     return;
   }
   const Top2 t = block_top2(logits + (size_t)row * dm.Vpad, dm, p);
-  if (threadIdx.x == 0) { st.o[b * dm.R1 + j] = t.i1; st.margin[b * dm.R1 + j] = t.v1 - t.v2; }
+  if (threadIdx.x == 0) {
+    st.o[row] = t.i1;
+    if (o_out != nullptr) o_out[row] = t.i1;
+    if (margin_out != nullptr) margin_out[row] = t.v1 - t.v2;
+  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -342,8 +350,18 @@ __device__ inline void accept_one(const Dims& dm, const SeqState& st, int b, int
   }
 }
 
-// rows fed at each level in the next pass (n_active[level]); n_active[3] = unfinished sequences
+// rows fed at each level in the next pass (n_active[level]), n_active[3] = unfinished sequences, and which sequence and
+// position every row of the pass is; by one block, behind a barrier that follows the change of the state
 __device__ inline void count_rows(const Dims& dm, const SeqState& st, int batch) {
+  for (int l = 0; l < 3; ++l) {
+    const int n = batch * fm_rows_per_seq(dm, l);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      int b, p;
+      const bool valid = fm_row_map(dm, st, batch, l, i, b, p);
+      st.rows[l][i] = PackedRow{valid ? b : -1, valid ? p : 0, 0, valid ? p % dm.cap[l] : 0};
+    }
+  }
+  if (threadIdx.x != 0) return;
   int cnt[3] = {0, 0, 0}, act = 0;
   for (int b = 0; b < batch; ++b) {
     const int n = st.nrow[b], L = st.L[b];
@@ -363,12 +381,12 @@ __device__ inline void count_rows(const Dims& dm, const SeqState& st, int batch)
 __global__ void accept_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ force_len,
                               const int* __restrict__ force_tok, int* __restrict__ n_acc, int* __restrict__ emitted,
                               int* __restrict__ kv_len, const GenOut* __restrict__ gen, int step_end) {
+  ptx::grid_dep_wait();
   const int lane = threadIdx.x & 31;
   for (int b = threadIdx.x >> 5; b < batch; b += blockDim.x >> 5) accept_one(dm, st, b, lane, force_len, force_tok, n_acc, emitted, kv_len, gen);
   __syncthreads();
-  if (threadIdx.x != 0) return;
   count_rows(dm, st, batch);
-  if (step_end) {
+  if (threadIdx.x == 0 && step_end) {
     *st.step += 1;
     if (gen->stats != nullptr) gen->stats[0] += 1;
     if (gen->host_done != nullptr) { *gen->host_done = st.n_active[3]; __threadfence_system(); }
@@ -404,6 +422,8 @@ __device__ inline const float* head_split_node(const Dims& dm, int h, int b, int
 __global__ void draft_prep_kernel(Dims dm, SeqState st, int batch, const float* __restrict__ zc, const float* __restrict__ zv,
                                   const float* __restrict__ zf, const float* __restrict__ gains /*[NH,d]*/,
                                   bf16* __restrict__ a /*[NH, max_batch, d]*/) {
+  ptx::grid_dep_wait();                              // first: the prologues behind this kernel read the per-pass state
+  ptx::grid_dep_launch();
   __shared__ float sh[32];
   const int h = blockIdx.y, b = blockIdx.x, d = dm.d;
   if (b >= batch) return;
@@ -577,7 +597,8 @@ __global__ void draft_pick_kernel(Dims dm, SeqState st, int batch, const float* 
                                   const GenOut* __restrict__ gen, const bf16* __restrict__ point_feat /*[(nv+3Ef)*B, d]*/,
                                   const float* __restrict__ label_g, const float* __restrict__ label_W,
                                   int* __restrict__ labels /*[B, R1]*/, float* __restrict__ label_margin,
-                                  float* __restrict__ avg_rows /*[B*R1, Vpad] scratch of the averaged merge*/) {
+                                  float* __restrict__ avg_rows /*[B*R1, Vpad] scratch of the averaged merge*/,
+                                  int* __restrict__ cand_out /*[B, R1] or null*/) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int b = blockIdx.x, j = blockIdx.y;        // j = 0..D
@@ -615,11 +636,19 @@ __global__ void draft_pick_kernel(Dims dm, SeqState st, int batch, const float* 
     }
   }
   if (j == 0) {
-    if (threadIdx.x == 0) st.cand[b * dm.R1] = fin ? dm.n_bins + 2 : st.main_tok[b];
+    if (threadIdx.x == 0) {
+      const int t = fin ? dm.n_bins + 2 : st.main_tok[b];
+      st.cand[b * dm.R1] = t;
+      if (cand_out != nullptr) cand_out[b * dm.R1] = t;
+    }
     return;
   }
   if (fin) {
-    if (threadIdx.x == 0) { st.cand[b * dm.R1 + j] = dm.n_bins + 2; if (margin_out) margin_out[b * dm.D + j - 1] = 0.f; }
+    if (threadIdx.x == 0) {
+      st.cand[b * dm.R1 + j] = dm.n_bins + 2;
+      if (cand_out != nullptr) cand_out[b * dm.R1 + j] = dm.n_bins + 2;
+      if (margin_out) margin_out[b * dm.D + j - 1] = 0.f;
+    }
     if (logits_out)
       for (int i = threadIdx.x; i < dm.V; i += blockDim.x) logits_out[((size_t)b * dm.D + j - 1) * dm.V + i] = 0.f;
     return;
@@ -674,6 +703,7 @@ __global__ void draft_pick_kernel(Dims dm, SeqState st, int batch, const float* 
       }
     }
     st.cand[b * dm.R1 + j] = tok;
+    if (cand_out != nullptr) cand_out[b * dm.R1 + j] = tok;
     if (margin_out) margin_out[b * dm.D + j - 1] = t.v1 - t.v2;
   }
 }
