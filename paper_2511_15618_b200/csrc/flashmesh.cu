@@ -806,7 +806,7 @@ __global__ void row_count_kernel(Dims dm, SeqState st, int batch) {
 
 // threads of a kernel that walks over one row of d values: one element per thread up to 512
 inline int row_threads(int d) { return d >= 512 ? 512 : (d >= 256 ? 256 : 128); }
-inline int accept_threads(int batch) { return batch >= 32 ? 1024 : 32 * (batch < 1 ? 1 : batch); }
+inline int accept_threads(int batch) { return batch >= 32 ? 1024 : 32 * (batch < 4 ? 4 : batch); }
 
 // the streaming launch and, where a level's cache is cut into several groups, the merge
 void launch_attention(fm_ctx* c, const AttnArgs& a) {

@@ -303,41 +303,43 @@ __device__ inline void accept_one(const Dims& dm, const SeqState& st, int b, int
                                   const int* __restrict__ force_tok, int* __restrict__ n_acc, int* __restrict__ emitted,
                                   int* __restrict__ kv_len, const GenOut* __restrict__ gen) {
   const int R1 = dm.R1, eos = dm.n_bins + 1;
-  const int rows = st.nrow[b];
-  int a = 0;
+  // everything the decision needs, in one round of loads
+  const int rows = st.nrow[b], done = st.done[b], t_end = st.t_end[b];
   int L = st.L[b];
-  const int* o = (force_tok != nullptr ? force_tok : st.o) + b * R1;
+  const int ov = lane < R1 ? (force_tok != nullptr ? force_tok : st.o)[b * R1 + lane] : -1;
   const int cand = lane < R1 ? st.cand[b * R1 + lane] : -1;
-  if (rows > 0 && !st.done[b]) {
+  const int forced = force_len != nullptr ? force_len[b] : 0;
+  const bool plain = gen != nullptr && gen->plain;
+  int* out_tok = gen != nullptr ? gen->out_tok : nullptr;
+  int* out_len = gen != nullptr ? gen->out_len : nullptr;
+  const int stride = gen != nullptr ? gen->out_stride : 0, at0 = out_len != nullptr ? out_len[b] : 0;
+  int a = 0;
+  if (rows > 0 && !done) {
     // lane j holds candidate j; it matches if it is the main token or equals the argmax at row j-1
-    const bool match = lane < rows && (lane == 0 || cand == o[lane - 1]);
+    const int prev = __shfl_up_sync(0xffffffffu, ov, 1);
+    const bool match = lane < rows && (lane == 0 || cand == prev);
     const unsigned mm = __ballot_sync(0xffffffffu, match);
     a = __ffs(~mm) - 1;                              // length of the leading run of matches
-    if (gen != nullptr && gen->plain) a = 1;
-    if (force_len != nullptr) a = force_len[b];
+    if (plain) a = 1;
+    if (force_len != nullptr) a = forced;
     a = max(1, min(a, rows));
     const unsigned em = __ballot_sync(0xffffffffu, lane < a && cand == eos);
     bool fin = false;
     if (em) { a = __ffs(em); fin = true; }           // an accepted EOS ends the sequence
+    const int main_tok = __shfl_sync(0xffffffffu, ov, a - 1);
     if (lane < a) st.hist[b * FM_HIST + ((L - 1 + lane) & (FM_HIST - 1))] = cand;   // accepted token t_{L-1+lane}
     L += a;
-    if (L - 1 >= st.t_end[b]) fin = true;
-    if (gen != nullptr && gen->out_tok != nullptr && lane < a) {
-      const int at = gen->out_len[b] + lane;
-      if (at < gen->out_stride) gen->out_tok[(size_t)b * gen->out_stride + at] = cand;
-    }
-    __syncwarp();
+    if (L - 1 >= t_end) fin = true;
+    if (out_tok != nullptr && lane < a && at0 + lane < stride) out_tok[(size_t)b * stride + at0 + lane] = cand;
     if (lane == 0) {
       st.L[b] = L;
-      st.main_tok[b] = o[a - 1];
+      st.main_tok[b] = main_tok;
       st.done[b] = fin ? 1 : 0;
-      st.nrow[b] = fin ? 0 : min(R1, st.t_end[b] - (L - 1));
-      if (gen != nullptr) {
-        if (gen->out_len != nullptr) gen->out_len[b] += a;
-        if (gen->stats != nullptr) {
-          atomicAdd((unsigned long long*)&gen->stats[1], (unsigned long long)a);
-          atomicAdd((unsigned long long*)&gen->stats[2 + a], 1ull);
-        }
+      st.nrow[b] = fin ? 0 : min(R1, t_end - (L - 1));
+      if (out_len != nullptr) out_len[b] = at0 + a;
+      if (gen != nullptr && gen->stats != nullptr) {
+        atomicAdd((unsigned long long*)&gen->stats[1], (unsigned long long)a);
+        atomicAdd((unsigned long long*)&gen->stats[2 + a], 1ull);
       }
     }
   } else if (lane == 0) {
@@ -361,9 +363,9 @@ __device__ inline void count_rows(const Dims& dm, const SeqState& st, int batch)
       st.rows[l][i] = PackedRow{valid ? b : -1, valid ? p : 0, 0, valid ? p % dm.cap[l] : 0};
     }
   }
-  if (threadIdx.x != 0) return;
-  int cnt[3] = {0, 0, 0}, act = 0;
-  for (int b = 0; b < batch; ++b) {
+  if (threadIdx.x >= 32) return;
+  int cnt[3] = {0, 0, 0}, act = 0;                   // first warp, a sequence per lane
+  for (int b = threadIdx.x; b < batch; b += 32) {
     const int n = st.nrow[b], L = st.L[b];
     if (n <= 0) continue;
     act++;
@@ -372,12 +374,14 @@ __device__ inline void count_rows(const Dims& dm, const SeqState& st, int batch)
       cnt[l] += (L + n - 1) / r - (L + r - 1) / r + 1;
     }
   }
-  st.n_active[0] = cnt[0]; st.n_active[1] = cnt[1]; st.n_active[2] = cnt[2]; st.n_active[3] = act;
+  for (int l = 0; l < 3; ++l) cnt[l] = __reduce_add_sync(0xffffffffu, cnt[l]);
+  act = __reduce_add_sync(0xffffffffu, act);
+  if (threadIdx.x == 0) { st.n_active[0] = cnt[0]; st.n_active[1] = cnt[1]; st.n_active[2] = cnt[2]; st.n_active[3] = act; }
 }
 
 // One block; its warps walk over the sequences.  Afterwards thread 0 counts the rows of the next
-// pass and, inside fm_generate (step_end != 0), bumps the pass counter and tells the host how many
-// sequences are still running.
+// pass and, inside fm_generate (step_end != 0), bumps the pass counter and tells the host when no
+// sequence is running any more.
 __global__ void accept_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ force_len,
                               const int* __restrict__ force_tok, int* __restrict__ n_acc, int* __restrict__ emitted,
                               int* __restrict__ kv_len, const GenOut* __restrict__ gen, int step_end) {
@@ -389,7 +393,8 @@ __global__ void accept_kernel(Dims dm, SeqState st, int batch, const int* __rest
   if (threadIdx.x == 0 && step_end) {
     *st.step += 1;
     if (gen->stats != nullptr) gen->stats[0] += 1;
-    if (gen->host_done != nullptr) { *gen->host_done = st.n_active[3]; __threadfence_system(); }
+    // (mapped host memory, read after the stream was waited for: only the end is worth a write across the bus)
+    if (gen->host_done != nullptr && st.n_active[3] == 0) *gen->host_done = 0;
   }
 }
 // ------------------------------------------------------------------------------------------
