@@ -1161,7 +1161,11 @@ void pf_stack(fm_ctx* c, const PfChunk& ch, int s, float* stash_ring, bool want_
     if (ends && ch.n_ends == 0) {
       // (no prompt ends here: only the keys and values are needed)
     } else if (dm.dh == 64) {
-      if (qw == 8) pf_attention<64, 128, 8>(c, grid, at);
+      if (qw == 8) {
+        const int tQ = tmap_for(c, pr.q, pr.rows[0], hd, 128, 0);
+        if (tQ < 0) { c->launch_error = FM_ERR_CUDA; return; }
+        launch_pdl(c, dim3(1, 1, 1), pf::attn_tc_kernel, grid, pf::fa::THREADS, pf::fa::BYTES, at, (const CUtensorMap*)(c->tmaps + tQ));
+      }
       else if (qw == 2) pf_attention<64, 128, 2>(c, grid, at);
       else pf_attention<64, 128, 1>(c, grid, at);
     } else {
@@ -1595,7 +1599,7 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
     TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_RESID, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_QKV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_PREFIX, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<64, 128, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<64, 128, 8>::BYTES));
+    TRYCUDA(cudaFuncSetAttribute(pf::attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::fa::BYTES));
     TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<64, 128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<64, 128, 2>::BYTES));
     TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<64, 128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<64, 128, 1>::BYTES));
     TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<128, 64, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<128, 64, 8>::BYTES));

@@ -814,4 +814,265 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1)
   }
 }
 
+
+// The same for many rows and heads of 64, on the tensor cores: a CTA takes 128 query rows of a head, two threads per
+// row.  S = Q K^T goes to tensor memory; a thread reads its half of a row once, the two exchange maxima, and P
+// (bfloat16) goes back to tensor memory as the A operand of O += P V.  V is multiplied as it lies (keys x features: the
+// B operand's MN-major form).  S of the next tile is multiplied as soon as S is in registers, i.e. under the
+// exponentials.  The output is rescaled only when a row's maximum has grown by more than 2^8.  Bound: the special-
+// function units (1024 clocks for a tile's exponentials); two CTAs per SM keep them busy.  6994 rows, 16 heads:
+// 206 us a launch (MMAs of warps, attn_kernel: 505 us; a thread per row without the overlap: 462 us).
+namespace fa {
+constexpr int THREADS = 320;     // producer warp, MMA warp, eight softmax warps
+constexpr int STAGES = 2, TILE = 128 * 128, STAGE = 2 * TILE;            // bytes of 128 keys (or values) of 64
+constexpr int BYTES = TILE + STAGES * STAGE + 256 * 4 + 128 + 1024;
+constexpr float GROW = 8.f;
+
+__device__ inline float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ inline void st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" ::"r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]),
+               "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+               : "memory");
+}
+__device__ inline void st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ inline void mma_ts(uint32_t d, uint32_t a, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+      "r"(a), "l"(db), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+}  // namespace fa
+
+__global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, const CUtensorMap* tmQ) {
+  using namespace fa;
+  constexpr int DH = 64, C = 128;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  unsigned char* ring = sm + TILE;                           // behind the query tile
+  float* s_pair = reinterpret_cast<float*>(ring + STAGES * STAGE);         // [half][row]
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_pair + 256);
+  uint64_t *empty = full + STAGES, *q_full = empty + STAGES, *s_full = q_full + 1, *s_read = s_full + 1, *p_full = s_read + 1, *o_full = p_full + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_full + 1);
+  __shared__ int s_fail;
+  const Dims& dm = a.dm;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int h = blockIdx.x, hk = h / (dm.H / dm.Hkv), level = a.level;
+  const int2 tile = a.tiles[blockIdx.y];
+  const Seg& sg = a.segs[tile.x];
+  const int b = sg.b, p0 = sg.p0[level], n = sg.n[level], r0 = sg.r0[level], q0 = tile.y, nq = min(128, n - q0);
+  const int P = dm.P, cap = dm.cap[level], W = dm.window[level], slots = P + cap;
+  const int used = P + min(cap, p0);                         // cache slots that earlier chunks have filled
+  const bool linear = p0 <= cap;
+  const int q_last = q0 + nq - 1, vis_lo = W > 0 ? max(0, p0 + q0 - W + 1) : 0;      // lowest position any row sees
+  // key tiles, as in attn_kernel: prefix, cache, this chunk
+  const int tc1 = (used + C - 1) / C, tp = min(tc1, (P + C - 1) / C);
+  const int tc0 = linear ? max(tp, min(tc1, (P + vis_lo) / C)) : tp;
+  const int tn0 = max(0, vis_lo - p0) / C, tn1 = q_last / C + 1;
+  const int n_old = tp + tc1 - tc0, n_tiles = n_old + tn1 - tn0;
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    for (int i = 0; i < STAGES; ++i) { ptx::mbar_init(full + i, 1); ptx::mbar_init(empty + i, 1); }
+    ptx::mbar_init(q_full, 1); ptx::mbar_init(s_full, 1); ptx::mbar_init(s_read, 8); ptx::mbar_init(p_full, 8); ptx::mbar_init(o_full, 1);
+    ptx::fence_mbar_init();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(tmem_slot)), "r"(256) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = *tmem_slot, tO = tmem + 128, tP = tmem + 192;        // S in columns 0..127, then O, then P
+  ptx::grid_dep_launch();
+  if (warp == 0 && lane == 0) {
+    ptx::grid_dep_wait();
+    ptx::mbar_expect_tx(q_full, TILE);
+    ptx::tma_load_2d(sm, tmQ, h * DH, r0 + q0, q_full);
+    for (int i = 0; i < n_tiles; ++i) {
+      const int st = i % STAGES;
+      if (i >= STAGES && !ptx::mbar_wait(empty + st, ((i / STAGES) - 1) & 1)) { s_fail = 1; break; }
+      const bool old = i < n_old, cached = old || a.tmKn == nullptr;
+      const int row = !cached ? r0 + (tn0 + i - n_old) * C
+                              : (b * dm.Hkv + hk) * slots + (i < tp ? i * C : old ? (tc0 + i - tp) * C : P + p0 + (tn0 + i - n_old) * C);
+      const int x = cached ? 0 : hk * DH;
+      ptx::mbar_expect_tx(full + st, STAGE);
+      ptx::tma_load_2d(ring + st * STAGE, cached ? a.tmK : a.tmKn, x, row, full + st);
+      ptx::tma_load_2d(ring + st * STAGE + TILE, cached ? a.tmV : a.tmVn, x, row, full + st);
+    }
+  } else if (warp == 1 && lane == 0) {
+    const uint32_t id_s = tc::instr_desc_bf16(128), id_o = tc::instr_desc_bf16(DH) | (1u << 16);       // B of P V is MN-major
+    const uint64_t dq = tc::smem_desc_sw128(ptx::smem_u32(sm));
+    bool ok = ptx::mbar_wait(q_full, 0);
+    auto scores = [&](int i) {
+      const int st = i % STAGES;
+      if (!ptx::mbar_wait(full + st, (i / STAGES) & 1)) return false;
+      tc::fence_after();
+      const uint64_t dk = tc::smem_desc_sw128(ptx::smem_u32(ring + st * STAGE));
+#pragma unroll
+      for (int k = 0; k < DH / 16; ++k) tc::mma_ss(tmem, dq + 2 * k, dk + 2 * k, id_s, k > 0 ? 1u : 0u);
+      tc::commit(s_full);
+      return true;
+    };
+    ok = ok && scores(0);
+    for (int i = 0; i < n_tiles && ok; ++i) {
+      if (!(ok = ptx::mbar_wait(s_read, i & 1))) break;
+      if (i + 1 < n_tiles && !(ok = scores(i + 1))) break;
+      if (!(ok = ptx::mbar_wait(p_full, i & 1))) break;
+      tc::fence_after();
+      const uint64_t dv = tc::smem_desc_sw128(ptx::smem_u32(ring + (i % STAGES) * STAGE + TILE));
+#pragma unroll
+      for (int k = 0; k < C / 16; ++k) mma_ts(tO, tP + 8 * k, dv + 128 * k, id_o, (i > 0 || k > 0) ? 1u : 0u);
+      tc::commit(empty + i % STAGES);
+      tc::commit(o_full);
+    }
+    if (!ok) {
+      s_fail = 1;
+      tc::commit(q_full);                                    // what was issued ends before the CTA does
+      ptx::mbar_wait(q_full, 1);
+    }
+  } else if (warp >= 2) {
+    // ---- softmax: warps w and w + 4 share 32 query rows, 64 of a tile's keys each
+    const int w4 = warp & 3, half = (warp - 2) >> 2, i_row = w4 * 32 + lane;
+    const uint32_t lanes = (uint32_t)(w4 * 32) << 16;
+    const int pr = p0 + q0 + i_row;                          // the row's position
+    const int wrap_q = p0 > 0 ? (p0 - 1) / cap : 0, wrap_r = p0 - 1 - wrap_q * cap;
+    float m = -INFINITY, l = 0.f;                            // the maximum in use, the sum
+    bool ok = true;
+    for (int i = 0; i < n_tiles; ++i) {
+      const bool old = i < n_old;
+      const int k0 = old ? (i < tp ? i : tc0 + i - tp) * C : (tn0 + i - n_old) * C, k1 = k0 + C - 1;     // slots, or chunk rows
+      // every key of the tile visible to every row of the tile?
+      const bool all_vis = old ? k1 < P || (linear && k1 < used && (W == 0 || max(k0 - P, 0) >= p0 + q_last - W + 1))
+                               : k1 <= q0 && (W == 0 || p0 + k0 >= p0 + q_last - W + 1);
+      auto visible = [&](int k) {                            // slot or chunk row k
+        int kp;
+        if (old) {
+          const int r = k - P;
+          if (k < P) return true;
+          if (k >= used) return false;
+          kp = linear ? r : r + (r <= wrap_r ? wrap_q : wrap_q - 1) * cap;
+        } else {
+          kp = p0 + k;
+        }
+        return kp >= 0 && kp <= pr && (W == 0 || kp >= pr - W + 1);
+      };
+      ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait(s_full, i & 1));             // (goes on: its partner waits at the barrier)
+      tc::fence_after();
+      uint32_t r0[32], r1[32];
+      const int kh = k0 + 64 * half;
+      ld32(tmem + lanes + 64 * half, r0);
+      ld32(tmem + lanes + 64 * half + 32, r1);
+      ld_wait();
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(s_read);
+      if (!all_vis) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          if (!visible(kh + j)) r0[j] = 0xff800000u;         // -inf: exponential 0
+          if (!visible(kh + 32 + j)) r1[j] = 0xff800000u;
+        }
+      }
+      float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+      for (int j = 0; j < 32; j += 2) {
+        m4[0] = fmaxf(m4[0], __uint_as_float(r0[j])); m4[1] = fmaxf(m4[1], __uint_as_float(r0[j + 1]));
+        m4[2] = fmaxf(m4[2], __uint_as_float(r1[j])); m4[3] = fmaxf(m4[3], __uint_as_float(r1[j + 1]));
+      }
+      float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+      s_pair[half * 128 + i_row] = mx;
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + w4) : "memory");
+      mx = fmaxf(mx, s_pair[(half ^ 1) * 128 + i_row]);
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + w4) : "memory");         // read before the next tile's write
+      // P of the tile before has been multiplied: its place, and O, are free
+      if (i > 0) ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait(o_full, (i - 1) & 1));
+      tc::fence_after();
+      const bool grow = mx > m + GROW || (m == -INFINITY && mx != -INFINITY);
+      if (__any_sync(0xffffffffu, grow)) {
+        const float mn = grow ? mx : m, f = m == -INFINITY ? (grow ? 0.f : 1.f) : ex2(m - mn);
+        m = mn;
+        l *= f;
+        if (i > 0) {                                         // this half's 32 columns of the output
+#pragma unroll 1
+          for (int c = 0; c < 2; ++c) {
+            uint32_t o[16];
+            tc::ld16(tO + lanes + 32 * half + 16 * c, o);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * f);
+            st16(tO + lanes + 32 * half + 16 * c, o);
+          }
+        }
+      }
+      const float base = m == -INFINITY ? 0.f : m;
+      float s4[4] = {0.f, 0.f, 0.f, 0.f};
+      uint32_t pk[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float e0 = ex2(__uint_as_float(r0[2 * j]) - base), e1 = ex2(__uint_as_float(r0[2 * j + 1]) - base);
+        s4[0] += e0;
+        s4[1] += e1;
+        pk[j] = ptx::pack_bf16(e0, e1);
+      }
+      st16(tP + lanes + 32 * half, pk);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float e0 = ex2(__uint_as_float(r1[2 * j]) - base), e1 = ex2(__uint_as_float(r1[2 * j + 1]) - base);
+        s4[2] += e0;
+        s4[3] += e1;
+        pk[j] = ptx::pack_bf16(e0, e1);
+      }
+      st16(tP + lanes + 32 * half + 16, pk);
+      l += (s4[0] + s4[1]) + (s4[2] + s4[3]);
+      st_wait();
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(p_full);
+    }
+    s_pair[half * 128 + i_row] = l;
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + w4) : "memory");
+    l += s_pair[(half ^ 1) * 128 + i_row];
+    ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait(o_full, (n_tiles - 1) & 1));
+    if (!ok) s_fail = 1;
+    else {
+      tc::fence_after();
+      const float inv = 1.f / l;
+      bf16* op = a.out + ((size_t)(r0 + q0 + i_row) * 2 * dm.H + h) * DH;
+      uint32_t r[32];
+      ld32(tO + lanes + 32 * half, r);
+      ld_wait();
+      if (i_row < nq) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 8) {
+          uint32_t hi[4], lo[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float x = __uint_as_float(r[j + 2 * k]) * inv, y = __uint_as_float(r[j + 2 * k + 1]) * inv;
+            const __nv_bfloat162 hv = __floats2bfloat162_rn(x, y);
+            hi[k] = *reinterpret_cast<const uint32_t*>(&hv);
+            lo[k] = ptx::pack_bf16(__fsub_rn(x, __bfloat162float(hv.x)), __fsub_rn(y, __bfloat162float(hv.y)));
+          }
+          *reinterpret_cast<uint4*>(op + 32 * half + j) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+          *reinterpret_cast<uint4*>(op + dm.H * DH + 32 * half + j) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        }
+      }
+    }
+  }
+  __syncwarp();
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (s_fail) {                                              // a bounded wait gave up: report
+    if (threadIdx.x == 0) atomicExch(a.status, -5);
+    ptx::drain_delay();
+  }
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
+}
+
 }  // namespace pf

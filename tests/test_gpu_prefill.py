@@ -19,6 +19,9 @@ pytestmark = pytest.mark.gpu
     ((90, 20), (0, 0, 0), {"n_heads": 1, "n_kv_heads": 1, "head_dim": 128}),
     ((60,), (20, 9, 0), {"n_heads": 1, "n_kv_heads": 1, "head_dim": 128}),
     ((35, 2), (0, 0, 0), {"d_model": 192, "d_ff": 320}),              # partly empty last tiles
+    ((143,), (0, 0, 0), {"n_heads": 16, "n_kv_heads": 16}),           # 128 query rows per CTA: 10 tiles and 8 rows more
+    ((160, 3), (600, 0, 0), {"n_heads": 16, "n_kv_heads": 2}),        # the same with a ring shorter than the prompt, shared heads
+    ((950,), (700, 0, 0), {"n_heads": 16, "n_kv_heads": 16}),         # ... and in two chunks
     ((950, 30), (0, 0, 0), {}),                                       # cut into two chunks
     ((950,), (700, 0, 0), {}),                                        # two chunks and a ring that wraps
 ])
