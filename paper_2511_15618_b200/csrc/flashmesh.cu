@@ -149,6 +149,7 @@ struct fm_ctx {
   bool call_graphs_off;   // plain launches only (diagnostic modes, calls that swap scratch buffers)
   int batch;
   bool gen_fresh;       // no fm_generate call since the last fm_prefill
+  bool advanced;        // ... and no fm_accept
   std::vector<int> plen_host;
   int phase;            // 0 created, 1 prefilled / accepted, 2 verified
   int64_t launches;
@@ -1333,13 +1334,18 @@ int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off)
   return FM_OK;
 }
 
-// one decode pass of fm_generate
-void step_body(fm_ctx* c) {
+// what ends a pass of fm_generate (all of it when no sequence is running)
+void step_end(fm_ctx* c) {
   const Dims& dm = c->dm;
-  draft(c, nullptr, nullptr, nullptr, (const GenOut*)c->gen_dev);
-  forward(c, nullptr, 0, nullptr, nullptr, nullptr);
   launch_pdl(c, dim3(1, 1, 1), accept_kernel, 1, accept_threads(c->batch), 0, dm, c->st, c->batch, (const int*)nullptr, (const int*)nullptr,
              (int*)nullptr, (int*)nullptr, (int*)nullptr, (const GenOut*)c->gen_dev, 1);
+}
+
+// one decode pass of fm_generate
+void step_body(fm_ctx* c) {
+  draft(c, nullptr, nullptr, nullptr, (const GenOut*)c->gen_dev);
+  forward(c, nullptr, 0, nullptr, nullptr, nullptr);
+  step_end(c);
 }
 
 // Walk through `body` without launching anything: afterwards the descriptors of its launches exist (they
@@ -1773,6 +1779,7 @@ int fm_prefill(fm_ctx* c, int32_t batch, const float* cond, const int32_t* promp
   if (c->launch_error != FM_OK) return c->launch_error;
   c->phase = 1;
   c->gen_fresh = true;
+  c->advanced = false;
   return FM_OK;
 }
 
@@ -1913,6 +1920,7 @@ int fm_accept(fm_ctx* c, const int32_t* force_len, const int32_t* force_tok, int
              (const GenOut*)nullptr, 0);
   CUDA_OK(cudaGetLastError());
   if (c->launch_error != FM_OK) return c->launch_error;
+  c->advanced = true;
   c->phase = 1;
   return FM_OK;
 }
@@ -1944,6 +1952,7 @@ int fm_generate(fm_ctx* c, int32_t max_faces, int32_t* out_tok, int32_t out_stri
   CUDA_OK(cudaMemcpyAsync(c->gen_dev, &g, sizeof(g), cudaMemcpyHostToDevice, c->stream));
   CUDA_OK(cudaMemsetAsync(c->stats_dev, 0, (FM_MAX_DRAFT + 4) * sizeof(long long), c->stream));
   if (out_len != nullptr && c->gen_fresh) CUDA_OK(cudaMemsetAsync(out_len, 0, c->batch * sizeof(int), c->stream));
+  const bool first = c->gen_fresh && !c->advanced;
   c->gen_fresh = false;
   CUDA_OK(cudaStreamSynchronize(c->stream));       // `g` lives on this stack frame
   if (!c->prof_on) ensure_graph(c);
@@ -1955,22 +1964,40 @@ int fm_generate(fm_ctx* c, int32_t max_faces, int32_t* out_tok, int32_t out_stri
   *c->host_done = c->batch;
   // upper bound on passes: every pass emits at least one token per unfinished sequence
   const long long bound = max_steps > 0 ? max_steps : 9ll * max_faces + 8;
-  long long steps = 0;
-  bool finished = false;
-  while (!finished && steps < bound) {
-    const long long poll = max_steps > 0 ? bound : 8;
-    for (long long i = 0; i < poll; ++i) {
-      if (use_graph) {
-        CUDA_OK(cudaGraphLaunch(c->graph_exec, c->stream));
-        c->launches += c->graph_launches;
-      } else {
-        step_body(c);
-      }
-      ++steps;
+  // Passes come in groups of eight; the host waits at the end of a group.  No sequence can have finished before every
+  // pass accepted all it can (EOS masked, lengths known), so up to `least` passes nothing is waited for.  From there on
+  // at most three passes are in flight, and once no sequence is running the rest of the group is its bookkeeping only.
+  long long steps = 0, least = 0;
+  if (first && !keep_limits && !dm.allow_eos) least = plain ? 9ll * max_faces : (9ll * max_faces + dm.R1 - 1) / dm.R1;
+  bool finished = false, idle = false;
+  cudaEvent_t ev[4] = {};
+  cudaError_t err = cudaSuccess;
+  for (int i = 0; i < 4 && max_steps <= 0 && err == cudaSuccess; ++i) err = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+  while (!finished && steps < bound && err == cudaSuccess) {
+    if (idle) {
+      step_end(c);
+    } else if (use_graph) {
+      err = cudaGraphLaunch(c->graph_exec, c->stream);
+      c->launches += c->graph_launches;
+    } else {
+      step_body(c);
     }
-    CUDA_OK(cudaStreamSynchronize(c->stream));
-    finished = *c->host_done == 0 || max_steps > 0;
+    ++steps;
+    if (max_steps > 0) {
+      if (steps == bound) finished = true;
+    } else if (steps >= least && err == cudaSuccess) {
+      err = cudaEventRecord(ev[steps & 3], c->stream);
+      const long long seen = steps % 8 == 0 ? steps : steps - 2;
+      if (!idle && seen >= least && seen > 0 && err == cudaSuccess) {
+        err = cudaEventSynchronize(ev[seen & 3]);
+        idle = *reinterpret_cast<volatile int*>(c->host_done) == 0;
+      }
+      finished = idle && steps % 8 == 0;
+    }
   }
+  for (int i = 0; i < 4; ++i) if (ev[i] != nullptr) cudaEventDestroy(ev[i]);
+  if (err == cudaSuccess) err = cudaStreamSynchronize(c->stream);
+  if (err != cudaSuccess) { cudaEventDestroy(e0); cudaEventDestroy(e1); return FM_ERR_CUDA; }
   CUDA_OK(cudaEventRecord(e1, c->stream));
   CUDA_OK(cudaEventSynchronize(e1));
   float ms = 0.f;
