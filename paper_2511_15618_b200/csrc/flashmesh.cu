@@ -1298,7 +1298,7 @@ int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off)
   const int prefix_total = B * dm.P, kvw = 2 * dm.Hkv * dm.dh;
   for (int r0 = 0; r0 < prefix_total; r0 += pr.prefix_rows) {
     const int rows = prefix_total - r0 < pr.prefix_rows ? prefix_total - r0 : pr.prefix_rows;
-    LAUNCH(c, pf::prefix_norm_kernel, dim3(rows, rows < 2048 ? 4 : 1), row_threads(dm.d / 4), 0, cond + (size_t)r0 * dm.d, pr.layers, pr.n_layers,
+    LAUNCH(c, pf::prefix_norm_kernel, dim3(rows, rows < 2048 ? 8 : 2), row_threads(dm.d / 4), 0, cond + (size_t)r0 * dm.d, pr.layers, pr.n_layers,
            pr.prefix_rows, pr.wide, dm.d, dm.eps);
     pf::Epi e{};
     e.dm = dm; e.layers = pr.layers; e.row_first = r0; e.rows_layer = pr.prefix_rows;

@@ -535,6 +535,7 @@ __global__ void prefix_norm_kernel(const float* __restrict__ c, const LayerPtr* 
   const float inv = rsqrtf(ss / (float)d + eps);
   for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
     const float4 v = make_float4(xr[4 * i], xr[4 * i + 1], xr[4 * i + 2], xr[4 * i + 3]);
+#pragma unroll 4
     for (int z = blockIdx.y; z < n_layers; z += gridDim.y) {
       const float4 g = reinterpret_cast<const float4*>(layers[z].g1)[i];
       uint2 o;
@@ -611,10 +612,8 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1)
   __syncthreads();
   if (warp == NW) {
     if (lane == 0) {
-      ptx::grid_dep_wait();
-      for (int i = 0; i < n_tiles; ++i) {
+      auto issue = [&](int i) {
         const int st = i % CF::STAGES;
-        if (i >= CF::STAGES && !ptx::mbar_wait(empty + st, ((i / CF::STAGES) - 1) & 1)) { s_fail = 1; break; }
         unsigned char* Ks = sm + st * CF::STAGE;
         unsigned char* Vs = Ks + CF::TILE;
         ptx::mbar_expect_tx(full + st, CF::STAGE);
@@ -629,6 +628,15 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1)
           ptx::tma_load_2d(Ks + hf * C * 128, mk, x, row, full + st);
           ptx::tma_load_2d(Vs + hf * C * 128, mv, x, row, full + st);
         }
+      };
+      // Entries of the prefix and of earlier chunks were complete before this chunk's first launch: they are requested
+      // before the dependency wait.  (Slots behind them in a shared tile may be written meanwhile; they are masked.)
+      const int pre = min(n_old, CF::STAGES);
+      for (int i = 0; i < pre; ++i) issue(i);
+      ptx::grid_dep_wait();
+      for (int i = pre; i < n_tiles; ++i) {
+        if (i >= CF::STAGES && !ptx::mbar_wait(empty + i % CF::STAGES, ((i / CF::STAGES) - 1) & 1)) { s_fail = 1; break; }
+        issue(i);
       }
     }
     __syncwarp();
@@ -892,12 +900,8 @@ __global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, c
   const uint32_t tmem = *tmem_slot, tO = tmem + 128, tP = tmem + 192;        // S in columns 0..127, then O, then P
   ptx::grid_dep_launch();
   if (warp == 0 && lane == 0) {
-    ptx::grid_dep_wait();
-    ptx::mbar_expect_tx(q_full, TILE);
-    ptx::tma_load_2d(sm, tmQ, h * DH, r0 + q0, q_full);
-    for (int i = 0; i < n_tiles; ++i) {
+    auto issue = [&](int i) {
       const int st = i % STAGES;
-      if (i >= STAGES && !ptx::mbar_wait(empty + st, ((i / STAGES) - 1) & 1)) { s_fail = 1; break; }
       const bool old = i < n_old, cached = old || a.tmKn == nullptr;
       const int row = !cached ? r0 + (tn0 + i - n_old) * C
                               : (b * dm.Hkv + hk) * slots + (i < tp ? i * C : old ? (tc0 + i - tp) * C : P + p0 + (tn0 + i - n_old) * C);
@@ -905,6 +909,15 @@ __global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, c
       ptx::mbar_expect_tx(full + st, STAGE);
       ptx::tma_load_2d(ring + st * STAGE, cached ? a.tmK : a.tmKn, x, row, full + st);
       ptx::tma_load_2d(ring + st * STAGE + TILE, cached ? a.tmV : a.tmVn, x, row, full + st);
+    };
+    const int pre = min(n_old, STAGES);                      // as in attn_kernel: old entries before the dependency wait
+    for (int i = 0; i < pre; ++i) issue(i);
+    ptx::grid_dep_wait();
+    ptx::mbar_expect_tx(q_full, TILE);
+    ptx::tma_load_2d(sm, tmQ, h * DH, r0 + q0, q_full);
+    for (int i = pre; i < n_tiles; ++i) {
+      if (i >= STAGES && !ptx::mbar_wait(empty + i % STAGES, ((i / STAGES) - 1) & 1)) { s_fail = 1; break; }
+      issue(i);
     }
   } else if (warp == 1 && lane == 0) {
     const uint32_t id_s = tc::instr_desc_bf16(128), id_o = tc::instr_desc_bf16(DH) | (1u << 16);       // B of P V is MN-major
