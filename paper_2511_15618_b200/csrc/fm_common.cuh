@@ -6,6 +6,11 @@
 
 typedef __nv_bfloat16 bf16;
 
+// Kernels with the programmatic-dependent-launch attribute start while their predecessors still run.  What an earlier
+// kernel of the chain writes (activations, rings, logits, candidates) is therefore written during such a kernel's lifetime:
+// it is read behind the dependency wait with __ldcg, and its pointers are never `const ... __restrict__`, which would let
+// the compiler read through the read-only path.  That qualifier is for weights, tables and the maps and prompts of a call.
+
 // Ring sizes (entries per sequence) of the hourglass carry state, indexed by level-local
 // position modulo the size.  A verify pass touches coordinate positions L-2 .. L+D, vertices
 // ceil(L/3)-2 .. floor((L+D)/3) and faces ceil(L/9)-1 .. floor((L+D)/9); with D <= 27 these

@@ -494,8 +494,13 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   if (IS_RESID && want_side && !use_side && tid < items) {
     const int ma = tile_m * BM + 2 * (z * PW + (tid & (PW - 1))), mb = ma + 1;
     const float* xr = k_x + (size_t)(k_row0 + (tid >> lgPW)) * k_ldx;
-    if (ma < k_M) pre_xa = xr[ma];
-    if (mb < k_M) pre_xb = xr[mb];
+    if (mb < k_M) {
+      const float2 x0 = __ldcg(reinterpret_cast<const float2*>(xr + ma));
+      pre_xa = x0.x;
+      pre_xb = x0.y;
+    } else if (ma < k_M) {
+      pre_xa = __ldcg(xr + ma);
+    }
   }
 
   __syncthreads();                                         // s_inv / row maps are written (long before the MMAs end)
@@ -506,7 +511,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     if (col < e.stash_d)
       for (int n = 0; n < ns; ++n)
         if (s_rb[n] >= 0)
-          e.stash_ring[((size_t)s_rb[n] * e.stash_rs + s_rp[n] % e.stash_rs) * e.stash_d + col] = e.stash_x[(size_t)(row0 + n) * e.stash_d + col];
+          e.stash_ring[((size_t)s_rb[n] * e.stash_rs + s_rp[n] % e.stash_rs) * e.stash_d + col] = __ldcg(e.stash_x + (size_t)(row0 + n) * e.stash_d + col);
   }
   // ---- every warp waits for the accumulator and sends its 32 columns of the partial tile to
   // their owners.  A timeout is recorded; zeros are sent so that no owner waits in vain.
@@ -589,7 +594,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
         float2 x0 = make_float2(0.f, 0.f);
         if (use_side) x0 = *reinterpret_cast<const float2*>(side + n * 128 + ca);
         else if (first) x0 = make_float2(pre_xa, pre_xb);
-        else if (want_side) x0 = *reinterpret_cast<const float2*>(xr + ma);
+        else if (want_side) x0 = __ldcg(reinterpret_cast<const float2*>(xr + ma));
         xa = x0.x + ya;
         xb = x0.y + yb;
         if (MODE == EPI_RESID_CAT && s_rb[n] >= 0) {
@@ -611,7 +616,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
         *reinterpret_cast<float2*>(xr + ma) = make_float2(xa, xb);
         if (k_aout != nullptr) store_hi_lo2(k_aout + row * k_lda + ma, __fmul_rn(xa, pre_ga), __fmul_rn(xb, pre_gb), k_lo);
       } else if (a_ok) {
-        xa = (use_side ? side[n * 128 + ca] : (first ? pre_xa : (want_side ? xr[ma] : 0.f))) + ya;
+        xa = (use_side ? side[n * 128 + ca] : (first ? pre_xa : (want_side ? __ldcg(xr + ma) : 0.f))) + ya;
         xr[ma] = xa;
         if (k_aout != nullptr) store_hi_lo(k_aout + row * k_lda + ma, __fmul_rn(xa, pre_ga), k_lo);
       }

@@ -63,9 +63,9 @@ __device__ inline int fm_first_pos(const SeqState& st, int b, int level) {
 // ------------------------------------------------------------------------------------------
 // a1. candidate embedding: x[row] = E[cand[b][j]]  (zeros for rows that are not fed)
 // ------------------------------------------------------------------------------------------
-__global__ void embed_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ cand_in, int merge, const bf16* __restrict__ E, float* __restrict__ x,
+__global__ void embed_kernel(Dims dm, SeqState st, int batch, const int* cand_in, int merge, const bf16* __restrict__ E, float* __restrict__ x,
                              const float* __restrict__ g, bf16* __restrict__ a_out, float* __restrict__ ssq, int ld_ssq,
-                             int rows, const float* __restrict__ hc_ring, const float* __restrict__ hv_ring,
+                             int rows, const float* hc_ring, const float* hv_ring,
                              bf16* __restrict__ cat_v, bf16* __restrict__ cat_f, int rows_v, int rows_f) {
   // Launched with the programmatic attribute: whatever precedes the pass has completed behind the wait, and only then
   // may the prologues of the pass's kernels start, which read the per-pass state.
@@ -89,7 +89,7 @@ __global__ void embed_kernel(Dims dm, SeqState st, int batch, const int* __restr
     const bool ok = valid && pos >= 0;
     const float* src = (lb == 0 ? hc_ring : hv_ring) + ((size_t)b * rs + ((pos + rs) % rs)) * d;
     bf16* out = (level_out == 1 ? cat_v : cat_f) + (size_t)row * 6 * d + part * d;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) store_hi_lo(out + i, ok ? src[i] : 0.f, 3 * d);
+    for (int i = threadIdx.x; i < d; i += blockDim.x) store_hi_lo(out + i, ok ? __ldcg(src + i) : 0.f, 3 * d);
     return;
   }
   const int row = blockIdx.x;
@@ -100,9 +100,9 @@ __global__ void embed_kernel(Dims dm, SeqState st, int batch, const int* __restr
     // the candidates of the pass: those of the draft step, the caller's (slot 0 has to be the pending main token), or
     // (merge) the caller's where they are >= 0, never in slot 0
     const int bb = row / dm.R1, j = row - bb * dm.R1;
-    const int own = cand_in != nullptr ? cand_in[row] : -1;
+    const int own = cand_in != nullptr ? __ldcg(cand_in + row) : -1;
     const bool take = cand_in != nullptr && (!merge || (own >= 0 && j != 0));
-    tok = take ? own : st.cand[row];
+    tok = take ? own : __ldcg(st.cand + row);
     if (take && threadIdx.x == 0) {
       if (j == 0 && st.nrow[bb] > 0 && own != st.main_tok[bb]) atomicExch(st.status, -1);
       st.cand[row] = own;
@@ -120,19 +120,19 @@ __global__ void embed_kernel(Dims dm, SeqState st, int batch, const int* __restr
   stack_entry_row(x + (size_t)row * dm.d, row, dm.d, g, a_out, ssq, ld_ssq);
 }
 
-// RMSNorm of read-only fp32 rows (conditioning vectors, draft features) -> bf16 operand rows
-__global__ void rmsnorm_kernel(const float* __restrict__ x, const float* __restrict__ g, bf16* __restrict__ out,
+// RMSNorm of fp32 rows (draft features) -> bf16 operand rows
+__global__ void rmsnorm_kernel(const float* x, const float* __restrict__ g, bf16* __restrict__ out,
                                int d, float eps) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   __shared__ float sh[32];
   const float* xr = x + (size_t)blockIdx.x * d;
   float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) { const float v = xr[i]; ss += v * v; }
+  for (int i = threadIdx.x; i < d; i += blockDim.x) { const float v = __ldcg(xr + i); ss += v * v; }
   ss = block_sum(ss, sh);
   const float inv = rsqrtf(ss / (float)d + eps);
   for (int i = threadIdx.x; i < d; i += blockDim.x)
-    out[(size_t)blockIdx.x * d + i] = __float2bfloat16(xr[i] * inv * g[i]);
+    out[(size_t)blockIdx.x * d + i] = __float2bfloat16(__ldcg(xr + i) * inv * g[i]);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -157,8 +157,8 @@ __global__ void rope_table_kernel(float2* __restrict__ tab, const double* __rest
 // rows that are not fed) as [hi | lo] terms, row length 6d; a hidden of this pass is read from
 // x_below, an older one from the carry ring.  Blocks [rows_out, rows_out + rows_below): this pass's
 // hiddens of the level below go into its ring for later passes.
-__global__ void shorten_gather_kernel(Dims dm, SeqState st, int batch, int level_out, const float* __restrict__ x_below,
-                                      float* __restrict__ ring, bf16* __restrict__ out, int rows_out) {
+__global__ void shorten_gather_kernel(Dims dm, SeqState st, int batch, int level_out, const float* x_below,
+                                      float* ring, bf16* __restrict__ out, int rows_out) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int lb = level_out - 1, rs = fm_ring(lb), d = dm.d;
@@ -169,7 +169,7 @@ __global__ void shorten_gather_kernel(Dims dm, SeqState st, int batch, int level
     if (!fm_row_map(dm, st, batch, lb, row, b, p)) return;
     float* dst = ring + ((size_t)b * rs + (p % rs)) * d;
     const float* src = x_below + (size_t)row * d;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) dst[i] = src[i];
+    for (int i = threadIdx.x; i < d; i += blockDim.x) dst[i] = __ldcg(src + i);
     return;
   }
   const int row = blockIdx.x;
@@ -183,7 +183,7 @@ __global__ void shorten_gather_kernel(Dims dm, SeqState st, int batch, int level
     const float* src = (ok && pos >= p0) ? x_below + ((size_t)b * m_below + (pos - p0)) * d
                                          : ring + ((size_t)b * rs + ((pos + rs) % rs)) * d;
     for (int i = threadIdx.x; i < d; i += blockDim.x)
-      store_hi_lo(out + (size_t)row * 6 * d + part * d + i, ok ? src[i] : 0.f, 3 * d);
+      store_hi_lo(out + (size_t)row * 6 * d + part * d + i, ok ? __ldcg(src + i) : 0.f, 3 * d);
   }
 }
 
@@ -193,8 +193,8 @@ __global__ void shorten_gather_kernel(Dims dm, SeqState st, int batch, int level
 // `tri_new` if its parent row belongs to this pass, else from the ring; the row is then handed to
 // the first layer of the stack above (operand row and sum of squares).  Blocks [rows, rows +
 // rows_up): this pass's triples go into the ring.
-__global__ void upsample_add_kernel(Dims dm, SeqState st, int batch, int level, const float* __restrict__ h_ring,
-                                    const float* __restrict__ tri_new, float* __restrict__ tri_ring, float* __restrict__ x,
+__global__ void upsample_add_kernel(Dims dm, SeqState st, int batch, int level, const float* h_ring,
+                                    const float* tri_new, float* tri_ring, float* __restrict__ x,
                                     const float* __restrict__ g, bf16* __restrict__ a_out, float* __restrict__ ssq, int ld_ssq, int rows) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
@@ -205,7 +205,7 @@ __global__ void upsample_add_kernel(Dims dm, SeqState st, int batch, int level, 
     if (!fm_row_map(dm, st, batch, level + 1, row, b, p)) return;
     float* dst = tri_ring + ((size_t)b * rsu + (p % rsu)) * 3 * d;
     const float* src = tri_new + (size_t)row * 3 * d;
-    for (int i = threadIdx.x; i < 3 * d; i += blockDim.x) dst[i] = src[i];
+    for (int i = threadIdx.x; i < 3 * d; i += blockDim.x) dst[i] = __ldcg(src + i);
     return;
   }
   const int row = blockIdx.x;
@@ -215,7 +215,7 @@ __global__ void upsample_add_kernel(Dims dm, SeqState st, int batch, int level, 
   const int up = p / 3, p0u = valid ? fm_first_pos(st, b, level + 1) : 0;
   const float* t = (valid && up >= p0u) ? tri_new + ((size_t)b * fm_rows_per_seq(dm, level + 1) + (up - p0u)) * 3 * d + (p % 3) * d
                                         : tri_ring + ((size_t)b * rsu + (up % rsu)) * 3 * d + (p % 3) * d;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) x[(size_t)row * d + i] = valid ? h[i] + t[i] : 0.f;
+  for (int i = threadIdx.x; i < d; i += blockDim.x) x[(size_t)row * d + i] = valid ? __ldcg(h + i) + __ldcg(t + i) : 0.f;
   __syncthreads();
   stack_entry_row(x + (size_t)row * d, row, d, g, a_out, ssq, ld_ssq);
 }
@@ -235,13 +235,13 @@ __device__ inline void top2_merge(Top2& a, const Top2& b) {
   if (b.v1 > a.v1 || (b.v1 == a.v1 && b.i1 < a.i1)) { const float lose = a.v1; a.v1 = b.v1; a.i1 = b.i1; a.v2 = fmaxf(fmaxf(a.v2, b.v2), lose); }
   else a.v2 = fmaxf(fmaxf(a.v2, b.v2), b.v1);
 }
-__device__ inline Top2 block_top2(const float* __restrict__ z, const Dims& dm, int target_index) {
+__device__ inline Top2 block_top2(const float* z, const Dims& dm, int target_index) {
   Top2 t{-INFINITY, -1, -INFINITY};
   const bool eos_ok = dm.allow_eos && (target_index % 9 == 0);
   const int n = dm.n_bins + (eos_ok ? 2 : 0);
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     if (i == dm.n_bins) continue;                    // BOS
-    top2_push(t, z[i], i);
+    top2_push(t, __ldcg(z + i), i);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -261,7 +261,7 @@ __device__ inline Top2 block_top2(const float* __restrict__ z, const Dims& dm, i
   return r;
 }
 
-__global__ void verify_top2_kernel(Dims dm, SeqState st, int batch, const float* __restrict__ logits,
+__global__ void verify_top2_kernel(Dims dm, SeqState st, int batch, const float* logits,
                                    float* __restrict__ logits_out, int* __restrict__ o_out, float* __restrict__ margin_out) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
@@ -271,7 +271,7 @@ __global__ void verify_top2_kernel(Dims dm, SeqState st, int batch, const float*
   if (row / dm.R1 >= batch) return;
   if (logits_out != nullptr)
     for (int i = threadIdx.x; i < dm.V; i += blockDim.x)
-      logits_out[(size_t)row * dm.V + i] = valid ? logits[(size_t)row * dm.Vpad + i] : 0.f;
+      logits_out[(size_t)row * dm.V + i] = valid ? __ldcg(logits + (size_t)row * dm.Vpad + i) : 0.f;
   if (!valid) {
     if (threadIdx.x == 0) {
       st.o[row] = -1;
@@ -299,16 +299,16 @@ struct GenOut {            // where fm_generate collects tokens (device-resident
   volatile int* host_done; // mapped pinned flag: number of unfinished sequences
 };
 
-__device__ inline void accept_one(const Dims& dm, const SeqState& st, int b, int lane, const int* __restrict__ force_len,
-                                  const int* __restrict__ force_tok, int* __restrict__ n_acc, int* __restrict__ emitted,
+__device__ inline void accept_one(const Dims& dm, const SeqState& st, int b, int lane, const int* force_len,
+                                  const int* force_tok, int* __restrict__ n_acc, int* __restrict__ emitted,
                                   int* __restrict__ kv_len, const GenOut* __restrict__ gen) {
   const int R1 = dm.R1, eos = dm.n_bins + 1;
   // everything the decision needs, in one round of loads
   const int rows = st.nrow[b], done = st.done[b], t_end = st.t_end[b];
   int L = st.L[b];
-  const int ov = lane < R1 ? (force_tok != nullptr ? force_tok : st.o)[b * R1 + lane] : -1;
-  const int cand = lane < R1 ? st.cand[b * R1 + lane] : -1;
-  const int forced = force_len != nullptr ? force_len[b] : 0;
+  const int ov = lane < R1 ? __ldcg((force_tok != nullptr ? force_tok : st.o) + b * R1 + lane) : -1;
+  const int cand = lane < R1 ? __ldcg(st.cand + b * R1 + lane) : -1;
+  const int forced = force_len != nullptr ? __ldcg(force_len + b) : 0;
   const bool plain = gen != nullptr && gen->plain;
   int* out_tok = gen != nullptr ? gen->out_tok : nullptr;
   int* out_len = gen != nullptr ? gen->out_len : nullptr;
@@ -382,8 +382,8 @@ __device__ inline void count_rows(const Dims& dm, const SeqState& st, int batch)
 // One block; its warps walk over the sequences.  Afterwards thread 0 counts the rows of the next
 // pass and, inside fm_generate (step_end != 0), bumps the pass counter and tells the host when no
 // sequence is running any more.
-__global__ void accept_kernel(Dims dm, SeqState st, int batch, const int* __restrict__ force_len,
-                              const int* __restrict__ force_tok, int* __restrict__ n_acc, int* __restrict__ emitted,
+__global__ void accept_kernel(Dims dm, SeqState st, int batch, const int* force_len,
+                              const int* force_tok, int* __restrict__ n_acc, int* __restrict__ emitted,
                               int* __restrict__ kv_len, const GenOut* __restrict__ gen, int step_end) {
   ptx::grid_dep_wait();
   const int lane = threadIdx.x & 31;
@@ -424,8 +424,8 @@ __device__ inline const float* head_split_node(const Dims& dm, int h, int b, int
 
 // Head inputs.  Row (h, b): a[h][b] = bf16(rms(z) * g_h) with z the stashed split-node hidden of
 // the pending position.
-__global__ void draft_prep_kernel(Dims dm, SeqState st, int batch, const float* __restrict__ zc, const float* __restrict__ zv,
-                                  const float* __restrict__ zf, const float* __restrict__ gains /*[NH,d]*/,
+__global__ void draft_prep_kernel(Dims dm, SeqState st, int batch, const float* zc, const float* zv,
+                                  const float* zf, const float* __restrict__ gains /*[NH,d]*/,
                                   bf16* __restrict__ a /*[NH, max_batch, d]*/) {
   ptx::grid_dep_wait();                              // first: the prologues behind this kernel read the per-pass state
   ptx::grid_dep_launch();
@@ -435,17 +435,17 @@ __global__ void draft_prep_kernel(Dims dm, SeqState st, int batch, const float* 
   const int n = max(0, st.L[b] - 1);
   const float* z = head_split_node(dm, h, b, n, zc, zv, zf);
   float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) ss += z[i] * z[i];
+  for (int i = threadIdx.x; i < d; i += blockDim.x) { const float v = __ldcg(z + i); ss += v * v; }
   ss = block_sum(ss, sh);
   const float inv = rsqrtf(ss / (float)d + dm.eps);
   bf16* dst = a + ((size_t)h * dm.max_batch + b) * d;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) dst[i] = __float2bfloat16(z[i] * inv * gains[(size_t)h * d + i]);
+  for (int i = threadIdx.x; i < d; i += blockDim.x) dst[i] = __float2bfloat16(__ldcg(z + i) * inv * gains[(size_t)h * d + i]);
 }
 
 // y = z + A a  (Eq. 1 reduced to Linear + residual).  Coordinate-head features go straight to the
 // feature matrix (rows h*B+b); vertex/face head features become bf16 inputs of the upsample GEMMs.
-__global__ void draft_residual_kernel(Dims dm, SeqState st, int batch, const float* __restrict__ zc, const float* __restrict__ zv,
-                                      const float* __restrict__ zf, const float* __restrict__ y /*[NH,max_batch,d]*/,
+__global__ void draft_residual_kernel(Dims dm, SeqState st, int batch, const float* zc, const float* zv,
+                                      const float* zf, const float* y /*[NH,max_batch,d]*/,
                                       float* __restrict__ feat /*[NF*B, d]*/, bf16* __restrict__ up_in_v /*[2B + 3*Ef*B, d]*/,
                                       bf16* __restrict__ up_in_f /*[Ef*B, d]*/) {
   ptx::grid_dep_launch();
@@ -456,7 +456,7 @@ __global__ void draft_residual_kernel(Dims dm, SeqState st, int batch, const flo
   const float* z = head_split_node(dm, h, b, n, zc, zv, zf);
   const float* yr = y + ((size_t)h * dm.max_batch + b) * d;
   for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float v = z[i] + yr[i];
+    const float v = __ldcg(z + i) + __ldcg(yr + i);
     if (h < dm.nc) feat[((size_t)h * batch + b) * d + i] = v;
     else if (h < dm.nc + dm.nv) up_in_v[((size_t)(h - dm.nc) * batch + b) * d + i] = __float2bfloat16(v);
     else up_in_f[((size_t)(h - dm.nc - dm.nv) * batch + b) * d + i] = __float2bfloat16(v);
@@ -498,17 +498,17 @@ __global__ void hf_prep_kernel(Dims dm, SeqState st, int batch, int stage, float
   if (b >= batch) return;
   const float* x = hf_feature(dm, stage, t, b, batch, xv_pre, feat);
   float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) ss += x[i] * x[i];
+  for (int i = threadIdx.x; i < d; i += blockDim.x) { const float v = __ldcg(x + i); ss += v * v; }
   ss = block_sum(ss, sh);
   const float inv = rsqrtf(ss / (float)d + dm.eps);
   bf16* dst = a + ((size_t)t * dm.max_batch + b) * d;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) dst[i] = __float2bfloat16(x[i] * inv * gains[(size_t)t * d + i]);
+  for (int i = threadIdx.x; i < d; i += blockDim.x) dst[i] = __float2bfloat16(__ldcg(x + i) * inv * gains[(size_t)t * d + i]);
 }
 
 // queries of the draft modules: rotate to the query's level position, scale, round; rows
 // [t0, t0 + T) of the projection's output become rows (b * T + (t - t0)) of the attention's q
 __global__ void draft_q_kernel(Dims dm, SeqState st, int batch, int stage, int level, int t0, int T,
-                               const float* __restrict__ qf /*[sets*max_batch, H*dh]*/, const float2* __restrict__ rope_tab,
+                               const float* qf /*[sets*max_batch, H*dh]*/, const float2* __restrict__ rope_tab,
                                float qscale, bf16* __restrict__ q /*[B*T, H*dh]*/) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
@@ -522,7 +522,7 @@ __global__ void draft_q_kernel(Dims dm, SeqState st, int batch, int stage, int l
     const int head = i / half, k = i - head * half;
     float2 cs = make_float2(1.f, 0.f);
     if (dm.theta != 0.f) cs = rope_tab[(size_t)pos * half + k];
-    const float x1 = src[head * dm.dh + k], x2 = src[head * dm.dh + half + k];
+    const float x1 = __ldcg(src + head * dm.dh + k), x2 = __ldcg(src + head * dm.dh + half + k);
     // the caches hold rotary pairs side by side
     *reinterpret_cast<__nv_bfloat162*>(dst + head * dm.dh + 2 * k) =
         __floats2bfloat162_rn((x1 * cs.x - x2 * cs.y) * qscale, (x2 * cs.x + x1 * cs.y) * qscale);
@@ -530,8 +530,8 @@ __global__ void draft_q_kernel(Dims dm, SeqState st, int batch, int stage, int l
 }
 
 // SP-Block, between its attention and its linear layer: y = z + Wo o, a[h][b] = bf16(rms(y) * g_h)
-__global__ void sp_mid_kernel(Dims dm, SeqState st, int batch, const float* __restrict__ zc, const float* __restrict__ zv,
-                              const float* __restrict__ zf, const float* __restrict__ u /*[NH*max_batch, d]*/,
+__global__ void sp_mid_kernel(Dims dm, SeqState st, int batch, const float* zc, const float* zv,
+                              const float* zf, const float* u /*[NH*max_batch, d]*/,
                               const float* __restrict__ gains, bf16* __restrict__ a) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
@@ -542,17 +542,17 @@ __global__ void sp_mid_kernel(Dims dm, SeqState st, int batch, const float* __re
   const float* z = head_split_node(dm, h, b, n, zc, zv, zf);
   const float* ur = u + ((size_t)h * dm.max_batch + b) * d;
   float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) { const float y = z[i] + ur[i]; ss += y * y; }
+  for (int i = threadIdx.x; i < d; i += blockDim.x) { const float y = __ldcg(z + i) + __ldcg(ur + i); ss += y * y; }
   ss = block_sum(ss, sh);
   const float inv = rsqrtf(ss / (float)d + dm.eps);
   bf16* dst = a + ((size_t)h * dm.max_batch + b) * d;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) dst[i] = __float2bfloat16((z[i] + ur[i]) * inv * gains[(size_t)h * d + i]);
+  for (int i = threadIdx.x; i < d; i += blockDim.x) dst[i] = __float2bfloat16((__ldcg(z + i) + __ldcg(ur + i)) * inv * gains[(size_t)h * d + i]);
 }
 
 // HF-Block, last step: x += FFN output; the vertex-level blocks also hand the refined vertex
 // feature to the next upsample GEMM (bf16 operand row)
 __global__ void hf_finish_kernel(Dims dm, SeqState st, int batch, int stage, float* xv_pre, float* feat,
-                                 const float* __restrict__ y /*[T*max_batch, d]*/, bf16* __restrict__ up_in_v) {
+                                 const float* y /*[T*max_batch, d]*/, bf16* __restrict__ up_in_v) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int b = blockIdx.x, t = blockIdx.y, d = dm.d;
@@ -561,7 +561,7 @@ __global__ void hf_finish_kernel(Dims dm, SeqState st, int batch, int stage, flo
   const float* yr = y + ((size_t)t * dm.max_batch + b) * d;
   bf16* up = stage == DS_HF_V ? up_in_v + ((size_t)dm.nv * batch + 3 * ((size_t)(t / 3) * batch + b) + t % 3) * d : nullptr;
   for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float v = x[i] + yr[i];
+    const float v = __ldcg(x + i) + __ldcg(yr + i);
     x[i] = v;
     if (up != nullptr) up[i] = __float2bfloat16(v);
   }
@@ -597,9 +597,9 @@ __device__ inline int draft_point_row(const Dims& dm, int level, int head, int s
 // With a teacher (fm_generate's benchmark stand-in for trained heads, sitting where the Correct stage
 // edits drafts) the drafts 1..keep are then replaced by the known continuation and draft keep+1 by a
 // different coordinate id.
-__global__ void draft_pick_kernel(Dims dm, SeqState st, int batch, const float* __restrict__ logits /*[NF*B, Vpad]*/,
+__global__ void draft_pick_kernel(Dims dm, SeqState st, int batch, const float* logits /*[NF*B, Vpad]*/,
                                   float* __restrict__ logits_out, float* __restrict__ margin_out,
-                                  const GenOut* __restrict__ gen, const bf16* __restrict__ point_feat /*[(nv+3Ef)*B, d]*/,
+                                  const GenOut* __restrict__ gen, const bf16* point_feat /*[(nv+3Ef)*B, d]*/,
                                   const float* __restrict__ label_g, const float* __restrict__ label_W,
                                   int* __restrict__ labels /*[B, R1]*/, float* __restrict__ label_margin,
                                   float* __restrict__ avg_rows /*[B*R1, Vpad] scratch of the averaged merge*/,
@@ -622,7 +622,7 @@ __global__ void draft_pick_kernel(Dims dm, SeqState st, int batch, const float* 
       const bf16* f = point_feat + (size_t)draft_point_row(dm, level, head, slot, b, batch) * dm.d;
       float ss = 0.f, z0 = 0.f, z1 = 0.f, z2 = 0.f;
       for (int i = threadIdx.x; i < dm.d; i += blockDim.x) {
-        const float v = __bfloat162float(f[i]), vg = v * label_g[i];
+        const float v = __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(f) + i))), vg = v * label_g[i];
         ss += v * v;
         z0 += label_W[i] * vg; z1 += label_W[dm.d + i] * vg; z2 += label_W[2 * dm.d + i] * vg;
       }
@@ -675,24 +675,24 @@ __global__ void draft_pick_kernel(Dims dm, SeqState st, int batch, const float* 
     float mx[3], inv_sum[3];
     for (int k = 0; k < ns; ++k) {
       float m = -INFINITY;
-      for (int i = threadIdx.x; i < dm.V; i += blockDim.x) m = fmaxf(m, zs[k][i]);
+      for (int i = threadIdx.x; i < dm.V; i += blockDim.x) m = fmaxf(m, __ldcg(zs[k] + i));
       m = block_max(m, sha);
       float e = 0.f;
-      for (int i = threadIdx.x; i < dm.V; i += blockDim.x) e += expf(zs[k][i] - m);
+      for (int i = threadIdx.x; i < dm.V; i += blockDim.x) e += expf(__ldcg(zs[k] + i) - m);
       e = block_sum(e, sha);
       mx[k] = m; inv_sum[k] = 1.f / e;
     }
     float* row = avg_rows + (size_t)(b * dm.R1 + j) * dm.Vpad;
     for (int i = threadIdx.x; i < dm.V; i += blockDim.x) {
       float pr = 0.f;
-      for (int k = 0; k < ns; ++k) pr += expf(zs[k][i] - mx[k]) * inv_sum[k];
+      for (int k = 0; k < ns; ++k) pr += expf(__ldcg(zs[k] + i) - mx[k]) * inv_sum[k];
       row[i] = logf(pr / (float)ns);
     }
     __syncthreads();
     z = row;
   }
   if (logits_out)
-    for (int i = threadIdx.x; i < dm.V; i += blockDim.x) logits_out[((size_t)b * dm.D + j - 1) * dm.V + i] = z[i];
+    for (int i = threadIdx.x; i < dm.V; i += blockDim.x) logits_out[((size_t)b * dm.D + j - 1) * dm.V + i] = __ldcg(z + i);
   const Top2 t = block_top2(z, dm, n + j);
   if (threadIdx.x == 0) {
     int tok = t.i1;

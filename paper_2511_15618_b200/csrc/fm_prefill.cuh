@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
           if (e.add) {
             float x0[32];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) x0[j] = (j < nv && m_ok) ? xr[(size_t)j * e.ldx] : 0.f;
+            for (int j = 0; j < 32; ++j) x0[j] = (j < nv && m_ok) ? __ldcg(xr + (size_t)j * e.ldx) : 0.f;
 #pragma unroll
             for (int j = 0; j < 32; ++j) y[j] += x0[j];
           }
@@ -422,7 +422,7 @@ __global__ void embed_kernel(Dims dm, SeqState st, const Row* __restrict__ rows,
 // operand rows of a shorten GEMM: row u of level `lu` <- hiddens 3u-2, 3u-1, 3u of the level below,
 // from its residual rows or, before the segment, from the carry ring; grid (rows of the level, 3)
 __global__ void gather_kernel(Dims dm, const Seg* __restrict__ segs, const Row* __restrict__ rows, int lu,
-                              const float* __restrict__ x_low, const float* __restrict__ ring, bf16* __restrict__ out) {
+                              const float* x_low, const float* ring, bf16* __restrict__ out) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int row = blockIdx.x, part = blockIdx.y, d = dm.d, lb = lu - 1, rs = fm_ring(lb);
@@ -433,7 +433,7 @@ __global__ void gather_kernel(Dims dm, const Seg* __restrict__ segs, const Row* 
                                                                       : ring + ((size_t)r.b * rs + ((pos + rs) % rs)) * d);
   bf16* o = out + (size_t)row * 6 * d + part * d;
   for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
-    const float4 v = pos >= 0 ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 v = pos >= 0 ? __ldcg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     tc::store_hi_lo2(o + 4 * i, v.x, v.y, 3 * d);
     tc::store_hi_lo2(o + 4 * i + 2, v.z, v.w, 3 * d);
   }
@@ -443,8 +443,8 @@ __global__ void gather_kernel(Dims dm, const Seg* __restrict__ segs, const Row* 
 // segment go into the carry rings for what comes after it; operand row and sum of squares for the stack
 // above.  The parent of every row is a row of the same segment.
 __global__ void upsample_kernel(Dims dm, const Seg* __restrict__ segs, const Row* __restrict__ rows, int level,
-                                const float* __restrict__ tri, float* __restrict__ h_ring, float* __restrict__ tri_ring,
-                                float* __restrict__ x, const float* __restrict__ g, bf16* __restrict__ a, float* __restrict__ ssq, int ld_ssq) {
+                                const float* tri, float* __restrict__ h_ring, float* __restrict__ tri_ring,
+                                float* x, const float* __restrict__ g, bf16* __restrict__ a, float* __restrict__ ssq, int ld_ssq) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int row = blockIdx.x, d = dm.d, rs = fm_ring(level), rsu = fm_ring(level + 1);
@@ -457,16 +457,16 @@ __global__ void upsample_kernel(Dims dm, const Seg* __restrict__ segs, const Row
   // a triple is stored whole, by the block of its first child (its other children may lie behind the segment)
   float4* tr = slot == 0 && up >= s.p0[level + 1] + s.n[level + 1] - rsu ? reinterpret_cast<float4*>(tri_ring + ((size_t)r.b * rsu + up % rsu) * 3 * d) : nullptr;
   for (int i = threadIdx.x; i < d / 4; i += blockDim.x) {
-    const float4 h = xr[i], u = t[i];
+    const float4 h = __ldcg(xr + i), u = __ldcg(t + i);
     if (hr != nullptr) hr[i] = h;
-    if (tr != nullptr) { tr[i] = u; tr[d / 4 + i] = t[d / 4 + i]; tr[d / 2 + i] = t[d / 2 + i]; }
+    if (tr != nullptr) { tr[i] = u; tr[d / 4 + i] = __ldcg(t + d / 4 + i); tr[d / 2 + i] = __ldcg(t + d / 2 + i); }
     xr[i] = make_float4(h.x + u.x, h.y + u.y, h.z + u.z, h.w + u.w);
   }
   entry_row(xr, row, d, g, a, ssq, ld_ssq);
 }
 
 // the residual row of a prompt's last position, as it enters the last layer of a stack (split node)
-__global__ void stash_kernel(Dims dm, const Seg* __restrict__ segs, int level, const float* __restrict__ x, float* __restrict__ ring) {
+__global__ void stash_kernel(Dims dm, const Seg* __restrict__ segs, int level, const float* x, float* __restrict__ ring) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const Seg& s = segs[blockIdx.x];
@@ -474,12 +474,12 @@ __global__ void stash_kernel(Dims dm, const Seg* __restrict__ segs, int level, c
   const int k = s.n[level] - 1, p = s.p0[level] + k, rs = fm_ring(level);
   const float4* src = reinterpret_cast<const float4*>(x + (size_t)(s.r0[level] + k) * dm.d);
   float4* dst = reinterpret_cast<float4*>(ring + ((size_t)s.b * rs + p % rs) * dm.d);
-  for (int i = threadIdx.x; i < dm.d / 4; i += blockDim.x) dst[i] = src[i];
+  for (int i = threadIdx.x; i < dm.d / 4; i += blockDim.x) dst[i] = __ldcg(src + i);
 }
 
 // keys and values of the chunk -> cache, where its attention still needed entries that they replace
-__global__ void cache_kernel(Dims dm, const Seg* __restrict__ segs, const Row* __restrict__ rows, int level, const bf16* __restrict__ kbuf,
-                             const bf16* __restrict__ vbuf, bf16* __restrict__ Kc, bf16* __restrict__ Vc) {
+__global__ void cache_kernel(Dims dm, const Seg* __restrict__ segs, const Row* __restrict__ rows, int level, const bf16* kbuf,
+                             const bf16* vbuf, bf16* __restrict__ Kc, bf16* __restrict__ Vc) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
   const int row = blockIdx.x, cap = dm.cap[level], kvw = dm.Hkv * dm.dh;
@@ -490,13 +490,13 @@ __global__ void cache_kernel(Dims dm, const Seg* __restrict__ segs, const Row* _
   for (int i = threadIdx.x; i < kvw / 8; i += blockDim.x) {
     const int hk = 8 * i / dm.dh, c = 8 * i - hk * dm.dh;
     const size_t to = (((size_t)r.b * dm.Hkv + hk) * slots + dm.P + r.slot) * dm.dh + c;
-    *reinterpret_cast<uint4*>(Kc + to) = reinterpret_cast<const uint4*>(kbuf + (size_t)row * kvw)[i];
-    *reinterpret_cast<uint4*>(Vc + to) = reinterpret_cast<const uint4*>(vbuf + (size_t)row * kvw)[i];
+    *reinterpret_cast<uint4*>(Kc + to) = __ldcg(reinterpret_cast<const uint4*>(kbuf + (size_t)row * kvw) + i);
+    *reinterpret_cast<uint4*>(Vc + to) = __ldcg(reinterpret_cast<const uint4*>(vbuf + (size_t)row * kvw) + i);
   }
 }
 
 // attention output and residual row of a prompt's last position -> row b of the decode buffers
-__global__ void last_rows_kernel(Dims dm, const Seg* __restrict__ segs, const bf16* __restrict__ attn, const float* __restrict__ x,
+__global__ void last_rows_kernel(Dims dm, const Seg* __restrict__ segs, const bf16* attn, const float* x,
                                  bf16* __restrict__ attn_out, float* __restrict__ x_out) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
@@ -505,13 +505,13 @@ __global__ void last_rows_kernel(Dims dm, const Seg* __restrict__ segs, const bf
   const size_t row = s.r0[0] + s.n[0] - 1;
   const int hd = dm.H * dm.dh;
   for (int i = threadIdx.x; i < hd / 4; i += blockDim.x)
-    reinterpret_cast<uint4*>(attn_out + (size_t)s.b * 2 * hd)[i] = reinterpret_cast<const uint4*>(attn + row * 2 * hd)[i];
+    reinterpret_cast<uint4*>(attn_out + (size_t)s.b * 2 * hd)[i] = __ldcg(reinterpret_cast<const uint4*>(attn + row * 2 * hd) + i);
   for (int i = threadIdx.x; i < dm.d / 4; i += blockDim.x)
-    reinterpret_cast<float4*>(x_out + (size_t)s.b * dm.d)[i] = reinterpret_cast<const float4*>(x + row * dm.d)[i];
+    reinterpret_cast<float4*>(x_out + (size_t)s.b * dm.d)[i] = __ldcg(reinterpret_cast<const float4*>(x + row * dm.d) + i);
 }
 
 // state behind the prompt: the first main token is the argmax of the last position
-__global__ void finish_kernel(Dims dm, SeqState st, const float* __restrict__ logits, const int* __restrict__ prompt,
+__global__ void finish_kernel(Dims dm, SeqState st, const float* logits, const int* __restrict__ prompt,
                               const int* __restrict__ prompt_off) {
   ptx::grid_dep_launch();
   ptx::grid_dep_wait();
@@ -577,6 +577,15 @@ struct AttnCfg {
   static constexpr int BYTES = STAGES * STAGE + 64 + 1024;
   static constexpr int THREADS = (NW + 1) * 32;
 };
+
+// word t of the quad's lane c -> word c of its lane t
+__device__ inline void quad_transpose(uint4& v, int t4) {
+  const bool odd = t4 & 1, high = t4 & 2;
+  uint32_t a = __shfl_xor_sync(0xffffffffu, odd ? v.x : v.y, 1), b = __shfl_xor_sync(0xffffffffu, odd ? v.z : v.w, 1);
+  if (odd) { v.x = a; v.z = b; } else { v.y = a; v.w = b; }
+  a = __shfl_xor_sync(0xffffffffu, high ? v.x : v.z, 2), b = __shfl_xor_sync(0xffffffffu, high ? v.y : v.w, 2);
+  if (high) { v.x = a; v.y = b; } else { v.z = a; v.w = b; }
+}
 
 template <int DH, int C, int QW>
 __global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1) attn_kernel(const Attn a) {
@@ -651,10 +660,18 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1)
       const int i = g + hr * 8;
       const bool ok = qw * 16 + i < nq;
       const bf16* qp = a.q + ((size_t)(r0 + w0 + (ok ? i : 0)) * dm.H + h) * DH;
+      // A lane takes 16-byte chunks of its row, the quad transposes them into fragments.  (A 4-byte load per fragment
+      // register asks L2 for every sector twice: 0.8 us a launch at 73 rows.)
+      uint4 v[KS / 2];
 #pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        qa[ks][hr] = ok ? *reinterpret_cast<const uint32_t*>(qp + ks * 16 + 2 * t4) : 0u;
-        qa[ks][2 + hr] = ok ? *reinterpret_cast<const uint32_t*>(qp + ks * 16 + 8 + 2 * t4) : 0u;
+      for (int k = 0; k < KS / 2; ++k) v[k] = __ldcg(reinterpret_cast<const uint4*>(qp) + 4 * k + t4);
+#pragma unroll
+      for (int k = 0; k < KS / 2; ++k) {
+        quad_transpose(v[k], t4);
+        qa[2 * k][hr] = ok ? v[k].x : 0u;
+        qa[2 * k][2 + hr] = ok ? v[k].y : 0u;
+        qa[2 * k + 1][hr] = ok ? v[k].z : 0u;
+        qa[2 * k + 1][2 + hr] = ok ? v[k].w : 0u;
       }
     }
     float o[DH / 8][4];
