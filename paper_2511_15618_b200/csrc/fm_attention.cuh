@@ -58,6 +58,10 @@ struct AttnCfg {
   static constexpr int BYTES = RING + 128;                  // + barriers
   static constexpr int MAX_GROUPS = 24;                     // a lane per group in the merge
   static constexpr int THREADS = (NW + 1) * 32;
+  // CTAs per SM that the ring depth was chosen for.  The launch bound holds the registers to it (at most 200 per thread
+  // for two; 143 and 168 are in use), this the shared memory: 228 KB per SM, of which a CTA takes 1 KB for itself.
+  static constexpr int CTAS = STAGES <= 3 ? 2 : 1;
+  static_assert(CTAS * (BYTES + 1024) <= 228 * 1024, "the CTAs of an SM share its shared memory");
 };
 
 namespace attn {
@@ -105,7 +109,7 @@ __device__ inline size_t attn_out_at(const AttnArgs& a, const AttnWork& w, int b
 
 // grid (max_groups, Hkv * MT, batch); block (NW + 1) warps: NW compute warps and one producer warp.
 template <int DH, int C, int NW, int ST>
-__global__ void __launch_bounds__((NW + 1) * 32, 1) attn_stream_kernel(const AttnArgs a) {
+__global__ void __launch_bounds__(AttnCfg<DH, C, NW, ST>::THREADS, AttnCfg<DH, C, NW, ST>::CTAS) attn_stream_kernel(const AttnArgs a) {
   using CF = AttnCfg<DH, C, NW, ST>;
   constexpr int KS = DH / 16, KB = CF::KPW / 16, NT = CF::KPW / 8;     // k-steps of Q K^T; 16-slot blocks and 8-slot tiles per warp
   const Dims& dm = a.dm;
