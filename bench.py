@@ -215,7 +215,7 @@ def run_ours(args):
                               "gemm": {"launches": g_n, "us_per_launch": 1e3 * g_ms / max(1, g_n), "weight_bytes": g_b},
                               "attention": {"launches": a_n, "us_per_launch": 1e3 * a_ms / max(1, a_n)},
                               "batch": B, "ms_per_step": ms / max(1, steps), "steps": steps, "gpu_launches": launches,
-                              "mean_accept_len": emitted / max(1, steps * B),
+                              "mean_accept_len": st.mean_accept_len,
                               "verify_step_frac_of_hbm_peak": sb / (ms / max(1, steps) * 1e-3) / 1e9 / peak,
                               "note": "timed passes only"}), flush=True)
         return
@@ -243,8 +243,8 @@ def run_ours(args):
     e2e = run_e2e(dev, cfg, truth, keep, prompts, max(8, min(K, 64)))
 
     peak, peak_kind = _peaks()
-    (ms, e2e_s), (emitted, launches, e2e_tok) = reduce_over_ranks(
-        [ms, e2e["seconds"]], [float(emitted), float(launches), e2e["tokens"]], "cuda")
+    (ms, e2e_s), (emitted, launches, e2e_tok, seq_passes) = reduce_over_ranks(
+        [ms, e2e["seconds"]], [float(emitted), float(launches), e2e["tokens"], float(sum(st.accept_hist))], "cuda")
     emitted, launches = int(emitted), int(launches)
     e2e["tokens"], e2e["seconds"] = e2e_tok, e2e_s
     value = emitted / (ms * 1e-3)
@@ -261,8 +261,8 @@ def run_ours(args):
                    "acceptance": f"teacher drafts, seeded schedule, mean {MEAN_DRAFTS} drafts kept per pass",
                    "l2": "weights streamed per pass exceed the 126 MB L2; no flush between passes",
                    "parallelism": f"replicas x{world}"},
-        "mean_accept_len": emitted / max(1, steps * B * world),
-        "natural_accept_len": st_nat.emitted / max(1, st_nat.steps * B),
+        "mean_accept_len": emitted / max(1.0, seq_passes),
+        "natural_accept_len": st_nat.mean_accept_len,
         "natural_tokens_per_s": st_nat.emitted / (st_nat.ms * 1e-3),
         # the same D-draft pass with acceptance forced to one token (NOT T_ori of Sec. 4.1, which is
         # the D = 0 run reported under "plain_decoding")
@@ -383,11 +383,11 @@ def run_full_length(args, cfg, rank, local):
     peak, peak_kind = _peaks()
     est_steps = max(1, int(sum(stops) * 9 / B / (1 + MEAN_DRAFTS)))
     seg = max(20, est_steps // 40)
-    out, windows, total_ms, total_tok, total_steps = None, [], 0.0, 0, 0
+    out, windows, total_ms, total_tok, total_steps, seq_passes = None, [], 0.0, 0, 0, 0
     for _ in range(100000):
         tok, ln, st = dev.generate(-1, truth=truth_d, keep=keep_d, max_steps=seg, out=out, stride=stride)
         out = (tok, ln)
-        total_ms += float(st.ms); total_tok += int(st.emitted); total_steps += int(st.steps)
+        total_ms += float(st.ms); total_tok += int(st.emitted); total_steps += int(st.steps); seq_passes += sum(st.accept_hist)
         cand, _, _ = dev.draft()
         o, _, _ = dev.verify(cand)
         act = (o[:, 0] >= 0).cpu().numpy()
@@ -406,7 +406,7 @@ def run_full_length(args, cfg, rank, local):
     line = {"metric": METRIC, "mode": "full_run", "value": total_tok / (total_ms * 1e-3), "unit": "tokens/s", "workload": cfg.name,
             "batch": B, "draft_len": D, "draft_heads": cfg.draft_heads, "n_kv_heads": cfg.n_kv_heads,
             "faces_per_sequence": stops, "steps": total_steps, "emitted": total_tok, "ms_total": total_ms,
-            "tokens_per_pass": total_tok / max(1, total_steps),
+            "tokens_per_pass": total_tok / max(1, total_steps), "mean_accept_len": total_tok / max(1, seq_passes),
             "plain_run": {"tokens_per_s": float(pl.sum()) / (st_plain.ms * 1e-3), "ms_per_pass": st_plain.ms / max(1, st_plain.steps)},
             "windows": [{"after_steps": a, "ms_per_step": m, "emitted": e, "active_sequences": act, "verify_step_frac_of_hbm_peak": fr}
                         for a, m, e, act, fr in (windows[0], windows[len(windows) // 2], windows[-2] if len(windows) > 1 else windows[-1])],

@@ -172,9 +172,13 @@ typedef struct fm_teacher {
 } fm_teacher;
 
 typedef struct fm_stats {
-  int64_t steps;                          /* draft+verify+accept passes executed             */
+  int64_t steps;                          /* passes of the loop: exactly max_steps, or, without it,
+                                             counted in groups of eight, the last one whole (its
+                                             passes behind the end are not run)              */
   int64_t emitted;                        /* mesh tokens emitted, all sequences              */
-  int64_t accept_hist[FM_MAX_DRAFT + 2];  /* accept_hist[a] = passes that accepted a tokens  */
+  int64_t accept_hist[FM_MAX_DRAFT + 2];  /* accept_hist[a] = passes in which a running sequence
+                                             accepted a tokens, all sequences: the mean accept
+                                             length is emitted / sum(accept_hist)            */
   float   ms;                             /* device time of the decode loop (CUDA events)    */
 } fm_stats;
 

@@ -64,6 +64,11 @@ class FmStats(C.Structure):
     _fields_ = [("steps", C.c_int64), ("emitted", C.c_int64), ("accept_hist", C.c_int64 * (FM_MAX_DRAFT + 2)),
                 ("ms", C.c_float)]
 
+    @property
+    def mean_accept_len(self) -> float:
+        """Tokens accepted per pass and running sequence (`steps` counts the loop's last group of passes whole)."""
+        return self.emitted / max(1, sum(self.accept_hist))
+
 
 class FmProfile(C.Structure):
     _fields_ = [("gemm_ms", C.c_double), ("gemm_bytes", C.c_double), ("gemm_launches", C.c_int64),

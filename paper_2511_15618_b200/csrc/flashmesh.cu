@@ -1334,7 +1334,7 @@ int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off)
   return FM_OK;
 }
 
-// what ends a pass of fm_generate (all of it when no sequence is running)
+// what ends a pass of fm_generate
 void step_end(fm_ctx* c) {
   const Dims& dm = c->dm;
   launch_pdl(c, dim3(1, 1, 1), accept_kernel, 1, accept_threads(c->batch), 0, dm, c->st, c->batch, (const int*)nullptr, (const int*)nullptr,
@@ -1966,17 +1966,16 @@ int fm_generate(fm_ctx* c, int32_t max_faces, int32_t* out_tok, int32_t out_stri
   const long long bound = max_steps > 0 ? max_steps : 9ll * max_faces + 8;
   // Passes come in groups of eight; the host waits at the end of a group.  No sequence can have finished before every
   // pass accepted all it can (EOS masked, lengths known), so up to `least` passes nothing is waited for.  From there on
-  // at most three passes are in flight, and once no sequence is running the rest of the group is its bookkeeping only.
-  long long steps = 0, least = 0;
+  // at most three passes are in flight.  Once no sequence is running nothing more is launched; the rest of the group is
+  // only counted (fm_stats.steps).
+  long long steps = 0, least = 0, rest = 0;
   if (first && !keep_limits && !dm.allow_eos) least = plain ? 9ll * max_faces : (9ll * max_faces + dm.R1 - 1) / dm.R1;
-  bool finished = false, idle = false;
+  bool finished = false;
   cudaEvent_t ev[4] = {};
   cudaError_t err = cudaSuccess;
   for (int i = 0; i < 4 && max_steps <= 0 && err == cudaSuccess; ++i) err = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
   while (!finished && steps < bound && err == cudaSuccess) {
-    if (idle) {
-      step_end(c);
-    } else if (use_graph) {
+    if (use_graph) {
       err = cudaGraphLaunch(c->graph_exec, c->stream);
       c->launches += c->graph_launches;
     } else {
@@ -1988,11 +1987,11 @@ int fm_generate(fm_ctx* c, int32_t max_faces, int32_t* out_tok, int32_t out_stri
     } else if (steps >= least && err == cudaSuccess) {
       err = cudaEventRecord(ev[steps & 3], c->stream);
       const long long seen = steps % 8 == 0 ? steps : steps - 2;
-      if (!idle && seen >= least && seen > 0 && err == cudaSuccess) {
+      if (seen >= least && seen > 0 && err == cudaSuccess) {
         err = cudaEventSynchronize(ev[seen & 3]);
-        idle = *reinterpret_cast<volatile int*>(c->host_done) == 0;
+        finished = *reinterpret_cast<volatile int*>(c->host_done) == 0;
+        rest = (8 - steps % 8) % 8;
       }
-      finished = idle && steps % 8 == 0;
     }
   }
   for (int i = 0; i < 4; ++i) if (ev[i] != nullptr) cudaEventDestroy(ev[i]);
@@ -2008,7 +2007,7 @@ int fm_generate(fm_ctx* c, int32_t max_faces, int32_t* out_tok, int32_t out_stri
     long long h[FM_MAX_DRAFT + 4];
     CUDA_OK(cudaMemcpy(h, c->stats_dev, sizeof(h), cudaMemcpyDeviceToHost));
     memset(stats, 0, sizeof(*stats));
-    stats->steps = h[0];
+    stats->steps = h[0] + (finished ? rest : 0);
     stats->emitted = h[1];
     for (int a = 0; a < FM_MAX_DRAFT + 2; ++a) stats->accept_hist[a] = h[2 + a];
     stats->ms = ms;
