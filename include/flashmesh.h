@@ -47,6 +47,12 @@
  *     is rounded explicitly), so the tokens a speculative run emits are those of one-token-per-
  *     pass decoding with the same context, whatever the drafts were.  Two contexts (another
  *     batch size, draft count or capacity) may group reductions differently.
+ *   - This is a statement about passes behind one prefill.  A prefill packs all prompts of the call
+ *     into launches whose forms and tiles follow the prompt lengths of all sequences: the same call
+ *     leaves the same bits, but a sequence prefilled in other company, or a prompt and the same
+ *     tokens decoded in passes, agree to rounding only (tokens may then differ where two are all but
+ *     tied).  To continue a run to the bit, repeat its prefill and feed the tokens it had emitted as
+ *     drafts (fm_generate with a teacher, or cand of fm_verify) instead of a longer prompt.
  *   - Token ids: [0, n_bins) coordinate bins, BOS = n_bins, EOS = n_bins+1, PAD = n_bins+2.
  *     Emitted ids are always coordinate bins, or EOS at a face boundary when allow_eos != 0;
  *     ties in an argmax go to the lowest id.
@@ -198,7 +204,8 @@ int fm_destroy(fm_ctx* ctx);
 /* Start `batch` sequences.  cond: DEV float32 [batch, P, d] conditioning vectors, projected by
  * every layer's own K/V matrices into prefix cache slots.  prompt: DEV int32, the sequences'
  * mesh tokens concatenated; prompt_off: HOST int32 [batch+1] offsets into it (lengths must be
- * multiples of 9).  Runs BOS + prompt through the multi-row forward in chunks of D+1 rows.
+ * multiples of 9).  Runs BOS + prompt of all sequences as one packed multi-row forward, in chunks
+ * of up to 8192 rows.
  * Afterwards L[b] = 1 + prompt_len[b] and the first main token is pending.
  * Errors: INVALID_ARG, CAPACITY. */
 int fm_prefill(fm_ctx* ctx, int32_t batch, const float* cond /*DEV*/, const int32_t* prompt /*DEV*/,
