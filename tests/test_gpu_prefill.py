@@ -40,3 +40,17 @@ def test_prefill_lockstep(faces, window, kw):
     rep = run_lockstep(cfg, w, conds, prompts, dev, 2, 60, prefill_chunk=512)
     assert rep["done"] and rep["emitted"] == 18 * B and dev.device_status() == 0
     print(faces, {k: rep[k] for k in ("steps", "max_logit_err", "max_draft_err", "overrides")})
+
+
+@pytest.mark.parametrize("faces,window,kw", [
+    ((143,), (0, 0, 0), {}),                                          # 10 tiles and 8 rows more
+    ((160, 3), (600, 0, 0), {"n_kv_heads": 2}),                       # a ring shorter than the prompt, shared heads, a tile of few rows
+    ((950,), (700, 0, 0), {}),                                        # two chunks, a ring that wraps
+])
+def test_prefill_lockstep_128_query_rows_per_cta_heads_of_128(faces, window, kw):
+    """Heads of 128 take 128 query rows per CTA only where that gives every SM one."""
+    import torch
+    heads = 16
+    rows = [9 * f + 1 for f in faces]
+    assert sum(-(-min(r, 8190) // 128) for r in rows) * heads >= torch.cuda.get_device_properties(0).multi_processor_count
+    test_prefill_lockstep(faces, window, {"n_heads": heads, "n_kv_heads": heads, "head_dim": 128, **kw})
