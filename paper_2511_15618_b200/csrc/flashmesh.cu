@@ -678,25 +678,31 @@ cudaError_t allow_rows_smem() {
   return r;
 }
 
-// The tensor-memory form (fm_gemm_tc.cuh).  The K split (= cluster size) depends on the shapes only.
-void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_rows_alloc, int a_row0, int M, int K, int R,
-                const int* n_active, int mode, tc::Epi e, int a_parts, int stacked, int z_rows, int z_w_rows) {
-  const int tiles = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
+// How a launch of the tensor-memory form (fm_gemm_tc.cuh) is cut.  The K split (= cluster size) depends on the shapes only.
+struct SplitCut { int tiles, slabs, N, n_tiles, split; };
+SplitCut split_cut(const fm_ctx* c, int M, int K, int R, int stacked) {
+  SplitCut s{(M + tc::BM - 1) / tc::BM, K / tc::BK};
   // Few rows: one N tile, K split over a cluster so that enough SMs stream weights.  Many rows:
   // N tiles of 32 rows as well (each weight slab then comes from HBM once and from L2 for the other
   // N tiles), which keeps the K split, and with it the cluster reduction, small.
   const int Rpad = round_up(R, 16);
-  const int N = Rpad <= 32 ? Rpad : 32;
-  const int n_tiles = stacked > 1 ? stacked : (Rpad + N - 1) / N;   // stacked problems share a launch through grid.z
+  s.N = Rpad <= 32 ? Rpad : 32;
+  s.n_tiles = stacked > 1 ? stacked : (Rpad + s.N - 1) / s.N;       // stacked problems share a launch through grid.z
   // K split: up to about one CTA per SM; while a CTA would still stream more than 8 slabs (or the
   // launch has several N tiles) up to two CTAs per SM, whose rings are then kept small enough to share it.
-  const bool tiled = n_tiles > 1 && stacked == 1;
-  int split = 1;
-  while (split * 2 <= tc::MAX_SPLIT && split * 2 <= slabs) {
-    const bool deep = tiled || slabs / split > 8;
-    if (tiles * n_tiles * split * 2 > (deep ? c->split_target_deep : c->split_target)) break;
-    split *= 2;
+  const bool tiled = s.n_tiles > 1 && stacked == 1;
+  s.split = 1;
+  while (s.split * 2 <= tc::MAX_SPLIT && s.split * 2 <= s.slabs) {
+    const bool deep = tiled || s.slabs / s.split > 8;
+    if (s.tiles * s.n_tiles * s.split * 2 > (deep ? c->split_target_deep : c->split_target)) break;
+    s.split *= 2;
   }
+  return s;
+}
+
+void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_rows_alloc, int a_row0, int M, int K, int R,
+                const int* n_active, int mode, tc::Epi e, int a_parts, int stacked, int z_rows, int z_w_rows) {
+  const auto [tiles, slabs, N, n_tiles, split] = split_cut(c, M, K, R, stacked);
   const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, N, (uint32_t)a_parts);
   if (tA < 0) { c->launch_error = FM_ERR_CUDA; return; }
   // only the residual and the QKV epilogue have side rows, and only when a thread gets more than two items
@@ -732,20 +738,26 @@ void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_ro
   if (mode == tc::EPI_UP && e.ssq_out != nullptr) c->ssq_n = (c->dm.d / tc::BM) * split * (split == 1 ? 2 : 1);   // tiles within d
 }
 
-// The tiled form (fm_prefill.cuh).  Rows per tile: the choice that minimises waves x (slabs x the longer of a
-// slab's copy at 64 B per clock and its MMAs, + about 2000 clocks of start-up and epilogue).
-void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, pf::Epi e, int layers = 1, int w_tile0 = 0,
-             const int* n_active = nullptr) {
-  if (R <= 0) return;
-  const int parts = mode == pf::PF_PREFIX ? 1 : 2, tiles_m = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
-  int NT = 32;
+// How a launch of the tiled form (fm_prefill.cuh) is cut.  Rows per tile: the choice that minimises waves x (slabs x the
+// longer of a slab's copy at 64 B per clock and its MMAs, + about 2000 clocks of start-up and epilogue).
+struct TiledCut { int NT; double waves; };
+TiledCut tiled_cut(const fm_ctx* c, int M, int K, int R, int parts, int layers) {
+  const int tiles_m = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
+  TiledCut t{32, 0.0};
   double best = 0.0;
   for (int nt = 32; nt <= 256 / parts; nt *= 2) {
     const double tiles = (double)tiles_m * ((R + nt - 1) / nt) * layers, waves = ceil(tiles / c->n_sm);
     const double copy = (tc::BM * 128 + parts * nt * 128) / 64.0, mma = 2.0 * (parts * nt > 64 ? parts * nt : 64);
     const double cost = waves * (slabs * (copy > mma ? copy : mma) + 12.0 * parts * nt) + 2000.0;
-    if (nt == 32 || cost < best) { best = cost; NT = nt; }
+    if (nt == 32 || cost < best) { best = cost; t = TiledCut{nt, waves}; }
   }
+  return t;
+}
+
+void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, pf::Epi e, int layers = 1, int w_tile0 = 0,
+             const int* n_active = nullptr) {
+  if (R <= 0) return;
+  const int parts = mode == pf::PF_PREFIX ? 1 : 2, tiles_m = (M + tc::BM - 1) / tc::BM, NT = tiled_cut(c, M, K, R, parts, layers).NT;
   const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, NT, TMAP_STAGE + (uint32_t)parts);
   if (tA < 0) { c->launch_error = FM_ERR_CUDA; return; }
   int stages = (200 * 1024) / pf::stage_bytes(NT, parts);
@@ -764,13 +776,33 @@ void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_al
   }
 }
 
-// Whether a projection of more than 16 rows goes to the tiled form, whose CTAs hold all of K and need no exchange, or
-// to the split-K form.  Measured at d = 1024 (us, tiled / split): 73 rows QKV 6.9 / 10.2, first FFN matrix 9.0 / 10.1,
-// output projection 9.0 / 6.2; 253 rows 7.5 / 12.9, 9.6 / 15.2, 9.1 / 9.0, second FFN matrix 23 / 14; 20 rows 6.8 / 5.8.
+// Whether a projection of 64 rows or more goes to the tiled form, whose CTAs hold all of K and need no exchange, or to the
+// split-K form (below 64 rows the pass of the Large model and requests on Small were slower with the tiled form).  A
+// tiled launch is bound by one SM's copies: its time grows with the slabs of K and the waves of tiles.  A split launch
+// has its slabs divided by the split, but more CTAs to start and, with a small split, more of the epilogue per thread.
+// The estimates (us) are fitted to chains of launches with 64 to 480 rows at d = 256, 384, 512, 768, 1024 and 2048, the
+// six shapes of the path each (540 pairs; the chosen form is 0.5 % slower than the better one on average; row counts
+// alone, 64 without and 257 or 401 with a residual, were 3.3 % and up to 79 % slower).  Some of them, split / tiled:
+//               d = 256, 73 rows   d = 1024, 73 rows   d = 1024, 256 rows   d = 2048, 64 rows   d = 2048, 320 rows
+//   QKV            6.5 / 6.2          12.3 /  9.8         17.7 / 10.6          15.6 / 14.4         47.2 / 23.3
+//   output proj.   6.2 / 5.4           6.7 /  9.3          9.4 /  9.3           9.0 / 13.7         24.7 / 14.6
+//   first FFN      5.7 / 5.7          10.0 /  9.3         15.5 /  9.9          14.9 / 14.1         60.7 / 34.3
+//   second FFN     5.4 / 8.8           9.2 / 22.7         14.1 / 22.8          14.1 / 40.8         61.5 / 41.9
+//   logits         5.4 / 3.6           6.1 /  7.0         12.6 /  7.2           6.5 / 11.6         12.5 / 11.8
+bool tiled_is_faster(const fm_ctx* c, int M, int K, int R, bool plain_store) {
+  if (R < 64 || R > 480) return R > 480;                   // (beyond what was measured: every 32 rows read the weights again)
+  const SplitCut s = split_cut(c, M, K, R, 1);
+  const TiledCut t = tiled_cut(c, M, K, R, 2, 1);
+  const double per = (double)s.slabs / s.split, ctas = (double)s.tiles * s.n_tiles * s.split / c->n_sm;
+  const double split = 3.3 + 0.42 * per + 6.4 / s.split + 1.8 * ctas + 0.5 * per * (ceil(ctas / 2) - 1);
+  const double tiled = (plain_store ? 2.6 : 4.6) + s.slabs * t.waves * (0.22 + 0.05 * t.NT / 32);
+  return tiled < split;
+}
+
 bool tiled_gemm(fm_ctx* c, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, const int* n_active, int mode, const tc::Epi& e) {
   const bool resid = mode == tc::EPI_RESID;
   if (!resid && mode != tc::EPI_F32 && mode != tc::EPI_GELU && !(mode == tc::EPI_QKV && e.rows != nullptr && e.stash_ring == nullptr)) return false;
-  if (R < (resid ? (K <= 1536 ? 257 : 401) : 64)) return false;
+  if (!tiled_is_faster(c, M, K, R, mode == tc::EPI_F32)) return false;
   pf::Epi t{};
   t.ssq_in = e.ssq_in; t.ssq_n = e.ssq_n; t.ld_ssq = resid ? e.ld_ssq_out : e.ld_ssq; t.inv_d = e.inv_d_in; t.eps = e.eps;
   t.out = e.out; t.ldo = e.ldo; t.lo_off = e.lo_off;

@@ -1,5 +1,4 @@
-"""The packed prefill against the oracle at the sizes where it changes form: one query tile and a row more, the
-last size of the split-K GEMMs and the first of the tiled ones, ragged batches, windows whose ring is shorter
+"""The packed prefill against the oracle at the sizes where it changes form: one query tile and a row more, ragged batches, windows whose ring is shorter
 than a chunk (keys of the chunk outside the cache), more positions than one chunk holds."""
 import numpy as np
 import pytest
@@ -54,3 +53,14 @@ def test_prefill_lockstep_128_query_rows_per_cta_heads_of_128(faces, window, kw)
     rows = [9 * f + 1 for f in faces]
     assert sum(-(-min(r, 8190) // 128) for r in rows) * heads >= torch.cuda.get_device_properties(0).multi_processor_count
     test_prefill_lockstep(faces, window, {"n_heads": heads, "n_kv_heads": heads, "head_dim": 128, **kw})
+
+
+# The rows on both sides of each change between the split-K and the tiled form, at d = 128: 64 coordinate rows (most
+# projections), 225 (second FFN matrix of 256 columns), 481 (what is split up to there, here the second FFN matrix of 2048).
+@pytest.mark.parametrize("faces,d_ff", [
+    ((6, 0, 0, 0, 0, 0, 0, 0, 0), 256), ((7,), 256),                  # 63 and 64 rows
+    ((24, 0, 0, 0, 0, 0, 0, 0), 256), ((24, 0, 0, 0, 0, 0, 0, 0, 0), 256),        # 224 and 225
+    ((52, 1, 0), 2048), ((52, 1, 0, 0), 2048),                        # 480 and 481
+])
+def test_prefill_lockstep_where_projections_change_form(faces, d_ff):
+    test_prefill_lockstep(faces, (0, 0, 0), {"d_ff": d_ff, "weight_std": 0.1 if d_ff <= 256 else 0.05})
