@@ -27,6 +27,7 @@ namespace {
 
 constexpr int STACK_LEVEL[5] = {0, 1, 2, 1, 0};
 constexpr int PREFILL_ROWS = 8192;      // coordinate rows of a prefill chunk, at most
+constexpr int LAYOUT_SMS = 148;         // SMs of a B200: the workspace, which has no device yet, and the groups cut in it are laid out for them
 constexpr int FM_ROPE_SLACK = 64;       // the HF-Blocks of the face level query positions up to 4 faces ahead
 
 struct LayerDev {
@@ -321,17 +322,18 @@ void carve(fm_ctx* c, Carver& cv) {
     c->attn_two[l] = false;
     for (int ng = 1; ng <= g_cap && ng <= max_chunks; ++ng) {
       const int Gc = (max_chunks + ng - 1) / ng, groups = (max_chunks + Gc - 1) / Gc;
-      const long n = (long)tiles_l * groups, r = n % 296;
+      const long n = (long)tiles_l * groups, pairs = 2 * LAYOUT_SMS, r = n % pairs;
       const double fix = groups == 1 ? 3.0 : 6.0;
-      const bool two = n > 148;
-      const double cost = !two ? Gc + fix : (n / 296) * 2.0 * Gc + (r > 148 ? Gc * (r / 148.0) : r > 0 ? Gc : 0.0) + fix * ((n + 295) / 296);
+      const bool two = n > LAYOUT_SMS;
+      const double cost = !two ? Gc + fix
+                               : (n / pairs) * 2.0 * Gc + (r > LAYOUT_SMS ? Gc * (r / (double)LAYOUT_SMS) : r > 0 ? Gc : 0.0) + fix * ((n + pairs - 1) / pairs);
       if (ng == 1 || cost < best * (two && !c->attn_two[l] ? 0.8 : 1.0)) { best = cost; G = Gc; c->attn_two[l] = two; }
     }
     const char* gm = getenv("FM_ATTN_G");                 // tuning knob: chunks per group, all levels
     if (gm != nullptr && atoi(gm) > 0) {
       const int G_min = (max_chunks + g_cap - 1) / g_cap;
       G = atoi(gm) < G_min ? G_min : atoi(gm);
-      c->attn_two[l] = (long)tiles_l * ((max_chunks + G - 1) / G) > 148;
+      c->attn_two[l] = (long)tiles_l * ((max_chunks + G - 1) / G) > LAYOUT_SMS;
     }
     c->attn_G[l] = G;
     c->attn_max_groups[l] = (max_chunks + G - 1) / G;
@@ -1684,9 +1686,9 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
     c->rows_max = rm != nullptr && atoi(rm) < rg::MAX_ROWS ? atoi(rm) : rg::MAX_ROWS;
     const char* t = getenv("FM_SPLIT_TARGET");
     c->split_target = t != nullptr && atoi(t) > 0 ? atoi(t) : 160;
-    int dev = 0, sms = 148;
+    int dev = 0, sms = LAYOUT_SMS;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    c->n_sm = sms > 0 ? sms : 148;
+    c->n_sm = sms > 0 ? sms : LAYOUT_SMS;
     c->device = dev;
     const char* tt = getenv("FM_SPLIT_TARGET_DEEP");
     c->split_target_deep = tt != nullptr && atoi(tt) > 0 ? atoi(tt) : 296;
