@@ -68,6 +68,21 @@ def rank_sequences(rank, batch_per_rank):
 NCU_TRAFFIC = {}
 
 
+FEW_ROWS = 16              # rows up to which a projection takes the few-row form (rg::MAX_ROWS)
+
+
+def gemm_kernels(cfg):
+    """The kernels that the projections of a verify pass run through: every level has at most batch * (D + 1) rows."""
+    return "rg::gemm_rows_kernel" if cfg.batch * (cfg.draft_len + 1) <= FEW_ROWS else "rg::gemm_rows_kernel, tc::gemm_tc_kernel, pf::gemm_kernel"
+
+
+def attention_entry(cfg, ms, launches):
+    """The attention launches of a verify pass: one streaming launch per layer and, where a level's cache is cut into several
+    groups, its merge.  Time is per layer, both together."""
+    layers = sum(cfg.layers)
+    return {"launches": int(launches), "merges": int(launches) - layers, "us_per_layer": 1e3 * ms / layers}
+
+
 class ClockSampler:
     Q = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,clocks_event_reasons.hw_slowdown,"
          "clocks_event_reasons.hw_thermal_slowdown,clocks_event_reasons.sw_thermal_slowdown,"
@@ -213,7 +228,7 @@ def run_ours(args):
         if rank == 0:
             print(json.dumps({"metric": METRIC, "value": emitted / (ms * 1e-3), "unit": "tokens/s", "workload": args.workload,
                               "gemm": {"launches": g_n, "us_per_launch": 1e3 * g_ms / max(1, g_n), "weight_bytes": g_b},
-                              "attention": {"launches": a_n, "us_per_launch": 1e3 * a_ms / max(1, a_n)},
+                              "attention": attention_entry(cfg, a_ms, a_n),
                               "batch": B, "ms_per_step": ms / max(1, steps), "steps": steps, "gpu_launches": launches,
                               "mean_accept_len": st.mean_accept_len,
                               "verify_step_frac_of_hbm_peak": sb / (ms / max(1, steps) * 1e-3) / 1e9 / peak,
@@ -273,17 +288,17 @@ def run_ours(args):
                 "what": "fm_step_host once per pass with the host in the loop: candidates from pinned host memory "
                         "in, draft + verify + accept, accepted tokens copied back, per pass"},
         "gpu_launches": launches,
-        "roofline": {"bound": "hbm", "kernel": "tc::gemm_tc_kernel (all GEMM launches of one verify pass, timed alone as a graph)",
+        "roofline": {"bound": "hbm", "kernel": gemm_kernels(cfg) + " (all GEMM launches of one verify pass, timed alone as a graph)",
                      "achieved": gemm_gbs, "peak": peak, "unit": "GB/s", "frac": gemm_gbs / peak,
                      "peak_kind": peak_kind + " copy bandwidth (burst figure: the kernel is timed alone)",
                      "traffic": NCU_TRAFFIC.get(args.workload, {}).get("bytes_per_launch"),
                      "traffic_source": NCU_TRAFFIC.get(args.workload, {}).get("summary"),
                      "algorithmic_bytes_per_launch": gemm_bytes / max(1, gemm_n),
                      "launches_per_pass": int(gemm_n), "us_per_launch": gemm_ms * 1e3 / max(1, gemm_n),
-                     "second_kernel": {"kernel": "attn_stream_kernel (all attention launches of one verify pass)",
+                     "second_kernel": {"kernel": "attn_stream_kernel and its attn_merge_kernel (all attention launches of one verify pass)",
                                        "achieved": kv_bytes / (attn_ms * 1e-3) / 1e9 if attn_ms > 0 else 0.0,
                                        "frac": kv_bytes / (attn_ms * 1e-3) / 1e9 / peak if attn_ms > 0 else 0.0,
-                                       "launches_per_pass": int(attn_n), "us_per_launch": attn_ms * 1e3 / max(1, attn_n)}},
+                                       **attention_entry(cfg, attn_ms, attn_n)}},
         "verify_step": {"algorithmic_bytes": step_bytes, "ms": step_ms, "GB/s": step_bytes / (step_ms * 1e-3) / 1e9,
                         "frac_of_hbm_peak": step_bytes / (step_ms * 1e-3) / 1e9 / peak, "kv_len": kv_len[0],
                         "note": "whole pass (draft heads + verify + accept) against the verify bytes"},
