@@ -1408,7 +1408,7 @@ void drop_call_graph(fm_ctx::CallGraph& g) {
 // Runs `body` (which only enqueues work on the context's stream).  The first time a set of caller
 // pointers is seen the kernels are launched one by one (this also creates every descriptor the
 // path needs); when the same pointers come again the launches are captured into a graph, and
-// from then on the graph is replayed: a pass is 180 launches, and a host that drives the loop
+// from then on the graph is replayed: a pass is 208 launches (Medium), and a host that drives the loop
 // call by call would otherwise pay for each of them.  All state the kernels read lives in device
 // memory, so the same graph serves every pass.
 template <typename F>

@@ -36,6 +36,10 @@ struct LayerPtr { const bf16* Wqkv; const float* g1; bf16* K; bf16* V; int level
 // One thread needs about 420 clocks to request a weight slab and an operand slab of 64 k, and 128 threads
 // need 35 000 clocks for the GELU of a tile (its MMAs take 8 200): hence a producer warp for each of the two
 // streams, (for narrow tiles) stages of two slabs and eight epilogue warps.
+// 6994 rows, d = 1024: QKV 99 us, first FFN matrix 125, second 110, output projection 41, with the tensor pipe active
+// 43, 46, 53 and 33 % of the time.  A slab of a 128 x 128 tile is 48 KB and 512 MMA clocks; it takes 970 clocks where the
+// epilogue does not matter (second FFN matrix: 51 B per clock and SM; the L2 slices are at 27 to 35 % of their rate, DRAM
+// under 21 %), so the MMAs wait for the copies.
 enum Mode { PF_F32 = 0, PF_GELU = 1, PF_RESID = 2, PF_QKV = 3, PF_PREFIX = 4 };
 
 constexpr int THREADS = 384;     // weight producer, operand producer, MMA warp, one idle warp, eight epilogue warps
@@ -264,7 +268,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(acc_empty + buf);
         }
-      const int nv = min(32, nrows - c0);
+        const int nv = min(32, nrows - c0);
         const size_t row = (size_t)(n0 + c0);
         if (MODE != PF_PREFIX) {
 #pragma unroll
@@ -844,9 +848,10 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1)
 // row.  S = Q K^T goes to tensor memory; a thread reads its half of a row once, the two exchange maxima, and P
 // (bfloat16) goes back to tensor memory as the A operand of O += P V.  V is multiplied as it lies (keys x features: the
 // B operand's MN-major form).  S of the next tile is multiplied as soon as S is in registers, i.e. under the
-// exponentials.  The output is rescaled only when a row's maximum has grown by more than 2^8.  Bound: the special-
-// function units (1024 clocks for a tile's exponentials); two CTAs per SM keep them busy.  6994 rows, 16 heads:
-// 206 us a launch (MMAs of warps, attn_kernel: 505 us; a thread per row without the overlap: 462 us).
+// exponentials.  The output is rescaled only when a row's maximum has grown by more than 2^8 (the conditional rescaling of
+// FlashAttention-4, T. Dao et al., Hot Chips 2025).  Nearest bound: the special-function units (1024 clocks for a tile's
+// exponentials; 58 % of their rate in use, tensor pipe 27 %), which two CTAs per SM share.  6994 rows, 16 heads: 207 us a
+// launch (MMAs of warps, attn_kernel: 505 us; a thread per row without the overlap: 462 us).
 namespace fa {
 constexpr int THREADS = 320;     // producer warp, MMA warp, eight softmax warps
 constexpr int STAGES = 2, TILE = 128 * 128, STAGE = 2 * TILE;            // bytes of 128 keys (or values) of 64

@@ -4,7 +4,7 @@ A host that commits all its device memory once at start-up (a serving process wi
 plan, a plug-in that must not call cudaMalloc under its real-time loop) can run the verify pass with
 the attention kernel's split-KV scratch in a fixed array inside the library instead.  The call must
 give what fm_verify gives.  It is called twice in a row because every call reuses the same array,
-which still holds the previous call's partial results and counters.
+which still holds the previous call's partial results.
 
 This file is named so that pytest collects it last."""
 import numpy as np
@@ -21,7 +21,7 @@ def test_static_scratch_verify_matches_fm_verify_twice_in_a_row(monkeypatch):
 
     # One chunk per group (the library's tuning knob, read when the context is created), so that the
     # 72-face prompt spreads a head's cache over several CTAs at all three levels: only then do the
-    # partial results and the ticket counters, i.e. the static array, come into play.
+    # partial results, i.e. the static array, come into play.
     monkeypatch.setenv("FM_ATTN_G", "1")
     cfg = S.get_config("tiny").with_(prompt_faces=(72, 72), max_tokens=1 + 9 * (72 + 32) + 3 + 2)
     w = S.make_weights(cfg)
