@@ -104,12 +104,12 @@ def test_toy_lockstep_windows_and_mqa_and_eos():
     print({k: rep[k] for k in ("steps", "emitted", "max_logit_err", "max_draft_err", "overrides")})
 
 
-@pytest.mark.parametrize("prompt_faces", [100, 150])
-def test_toy_head_dim_128_long_cache_many_groups(prompt_faces):
-    """Head dimension 128 with a cache of 15 to 22 chunks: 100 faces give the largest number of
-    groups the last CTA can merge from shared memory (15, one chunk each), 150 faces give groups
-    of two chunks."""
+@pytest.mark.parametrize("prompt_faces,groups", [(100, 15), (150, 22), (165, 24), (250, 18)])
+def test_toy_head_dim_128_long_cache_many_groups(prompt_faces, groups):
+    """Head dimension 128 with a cache of 15 to 36 chunks: up to 24 groups of one chunk each (as many as
+    a warp of the merge takes), then groups of two chunks."""
     from oracle.lockstep import run_lockstep
+    from paper_2511_15618_b200 import fm_attention_layout
     faces = 3
     cfg = S.toy_config(d_model=128, n_heads=1, n_kv_heads=1, head_dim=128, d_ff=256, weight_std=0.1, out_std=0.02, draft_len=3,
                        layers=(1, 1, 1, 1, 1), prompt_faces=(prompt_faces, prompt_faces), prompt_subdiv=2, gen_faces=faces,
@@ -117,9 +117,10 @@ def test_toy_head_dim_128_long_cache_many_groups(prompt_faces):
     w, conds, prompts = _setup(cfg, batch=1)
     assert len(prompts[0]) == 9 * prompt_faces
     dev = _dev(cfg, w)
+    assert fm_attention_layout(dev.ctx, 0) == (0, (64, 2 if prompt_faces == 250 else 1, groups))
     rep = run_lockstep(cfg, w, conds, prompts, dev, faces, 60, tol=TOY_TOL, margin=TOY_MARGIN)
     assert rep["done"] and rep["emitted"] == 9 * faces
-    assert dev.device_status() == 0                  # in particular: the group-count guard did not fire
+    assert dev.device_status() == 0
     print({k: rep[k] for k in ("steps", "max_logit_err", "max_draft_err", "overrides")})
 
 
