@@ -659,23 +659,26 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1)
     const int qw = warp % QW, kw = warp / QW;
     const int w0 = q0 + qw * 16;                             // this warp's first query row of the segment
     const bool live = qw * 16 < nq;
+    // A lane takes 16-byte chunks of its two rows, the quad transposes them into fragments.  (A 4-byte load per fragment
+    // register asks L2 for every sector twice: 0.8 us a launch at 73 rows.)  All requests first: one L2 latency, not two.
+    uint4 v[2][KS / 2];
 #pragma unroll
     for (int hr = 0; hr < 2; ++hr) {
-      const int i = g + hr * 8;
-      const bool ok = qw * 16 + i < nq;
-      const bf16* qp = a.q + ((size_t)(r0 + w0 + (ok ? i : 0)) * dm.H + h) * DH;
-      // A lane takes 16-byte chunks of its row, the quad transposes them into fragments.  (A 4-byte load per fragment
-      // register asks L2 for every sector twice: 0.8 us a launch at 73 rows.)
-      uint4 v[KS / 2];
+      const int i = w0 + g + hr * 8;
+      const bf16* qp = a.q + ((size_t)(r0 + (i < q0 + nq ? i : q0)) * dm.H + h) * DH;      // (rows behind the tile: any row of it)
 #pragma unroll
-      for (int k = 0; k < KS / 2; ++k) v[k] = __ldcg(reinterpret_cast<const uint4*>(qp) + 4 * k + t4);
+      for (int k = 0; k < KS / 2; ++k) v[hr][k] = __ldcg(reinterpret_cast<const uint4*>(qp) + 4 * k + t4);
+    }
+#pragma unroll
+    for (int hr = 0; hr < 2; ++hr) {
+      const bool ok = w0 + g + hr * 8 < q0 + nq;
 #pragma unroll
       for (int k = 0; k < KS / 2; ++k) {
-        quad_transpose(v[k], t4);
-        qa[2 * k][hr] = ok ? v[k].x : 0u;
-        qa[2 * k][2 + hr] = ok ? v[k].y : 0u;
-        qa[2 * k + 1][hr] = ok ? v[k].z : 0u;
-        qa[2 * k + 1][2 + hr] = ok ? v[k].w : 0u;
+        quad_transpose(v[hr][k], t4);
+        qa[2 * k][hr] = ok ? v[hr][k].x : 0u;
+        qa[2 * k][2 + hr] = ok ? v[hr][k].y : 0u;
+        qa[2 * k + 1][hr] = ok ? v[hr][k].z : 0u;
+        qa[2 * k + 1][2 + hr] = ok ? v[hr][k].w : 0u;
       }
     }
     float o[DH / 8][4];

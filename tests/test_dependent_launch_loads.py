@@ -50,3 +50,19 @@ def test_residual_rows_of_earlier_launches_are_read_at_l2():
         assert not re.search(r"=\s*e\.stash_x\[", text), f
         assert not re.search(r"(?:=|\?)\s*xr\[\(size_t\)j \* e\.ldx\]", text), f
         assert not re.search(r"(?:=|\?)\s*\*reinterpret_cast<const float2\*>\(xr", text), f
+
+
+def test_prefill_attention_requests_query_rows_of_its_tile_only():
+    """The row expression of attn_kernel's query loads, evaluated for every lane of every tile height."""
+    text = open(os.path.join(CSRC, "fm_prefill.cuh")).read()
+    first = re.search(r"const int i = (w0 \+ g \+ hr \* 8);\s*const bf16\* qp = a\.q \+ \(\(size_t\)\(r0 \+ \((i < q0 \+ nq) \? (i) : (q0)\)\)", text)
+    assert first, "the query loads are not bounded by the tile"
+    q0 = 256
+    for nq in range(1, 129):
+        for w0 in range(q0, q0 + 128, 16):
+            for g in range(8):
+                for hr in range(2):
+                    env = {"w0": w0, "g": g, "hr": hr, "q0": q0, "nq": nq}
+                    env["i"] = eval(first.group(1), {}, env)
+                    row = eval(first.group(3) if eval(first.group(2), {}, env) else first.group(4), {}, env)
+                    assert q0 <= row < q0 + nq
