@@ -89,17 +89,23 @@ class ClockSampler:
          "clocks_event_reasons.sw_power_cap")
 
     def __init__(self, index):
-        self.index, self.proc, self.path = index, None, None
+        self.index, self.proc, self.path, self.skip = index, None, None, 0
 
     def start(self):
         try:
             fd, self.path = tempfile.mkstemp(suffix=".csv")
             os.close(fd)
             self.proc = subprocess.Popen(["nvidia-smi", f"--query-gpu={self.Q}", "--format=csv,noheader,nounits",
-                                          "-lms", "100", "-i", str(self.index)], stdout=open(self.path, "w"),
+                                          "-lms", "50", "-i", str(self.index)], stdout=open(self.path, "w"),
                                          stderr=subprocess.DEVNULL)
         except Exception:
             self.proc = None
+            return
+        # the timed region can be shorter than the tool's start-up: wait for its first sample, which does not count
+        limit = time.time() + 5.0
+        while self.skip == 0 and self.proc.poll() is None and time.time() < limit:
+            time.sleep(0.02)
+            self.skip = os.path.getsize(self.path)
 
     def stop(self):
         out = {"sm_mhz": None, "sm_max_mhz": None, "reasons": []}
@@ -111,7 +117,9 @@ class ClockSampler:
         except Exception:
             self.proc.kill()
         sm, reasons = [], set()
-        for ln in open(self.path):
+        lines = open(self.path)
+        lines.seek(self.skip)
+        for ln in lines:
             f = [x.strip() for x in ln.split(",")]
             if len(f) < 9:
                 continue
