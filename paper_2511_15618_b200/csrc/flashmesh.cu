@@ -783,7 +783,7 @@ void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_al
 // tiled launch is bound by one SM's copies: its time grows with the slabs of K and the waves of tiles.  A split launch
 // has its slabs divided by the split, but more CTAs to start and, with a small split, more of the epilogue per thread.
 // The estimates (us) are fitted to chains of launches with 64 to 480 rows at d = 256, 384, 512, 768, 1024 and 2048, the
-// six shapes of the path each (540 pairs; the chosen form is 0.5 % slower than the better one on average; row counts
+// six shapes of the path each (540 pairs; by them the chosen form is 0.5 % slower than the better one on average; row counts
 // alone, 64 without and 257 or 401 with a residual, were 3.3 % and up to 79 % slower).  Some of them, split / tiled:
 //               d = 256, 73 rows   d = 1024, 73 rows   d = 1024, 256 rows   d = 2048, 64 rows   d = 2048, 320 rows
 //   QKV            6.5 / 6.2          12.3 /  9.8         17.7 / 10.6          15.6 / 14.4         47.2 / 23.3
@@ -791,20 +791,24 @@ void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_al
 //   first FFN      5.7 / 5.7          10.0 /  9.3         15.5 /  9.9          14.9 / 14.1         60.7 / 34.3
 //   second FFN     5.4 / 8.8           9.2 / 22.7         14.1 / 22.8          14.1 / 40.8         61.5 / 41.9
 //   logits         5.4 / 3.6           6.1 /  7.0         12.6 /  7.2           6.5 / 11.6         12.5 / 11.8
-bool tiled_is_faster(const fm_ctx* c, int M, int K, int R, bool plain_store) {
+// In a forward the tiled form of a projection with a residual has to win by 3 us: its CTAs (200 KB) take the room in which the
+// weights of the launch behind it would arrive.  Prefills and passes at 18 sizes, us with that margin / without / by row counts
+// alone: d = 640, 1522 rows 1458 / 1486 / 1459; d = 768, 8 x 271 rows 4325 / 4426 / 4327; d = 1024, 901 rows 3228 / 3288 / 3269,
+// 8 sequences of 181 to 541 rows 5812 / 5897 / 5868; d = 2048, 2701 rows 13 914 / 13 813 / 14 320.
+bool tiled_is_faster(const fm_ctx* c, int M, int K, int R, bool plain_store, bool resid) {
   if (R < 64 || R > 480) return R > 480;                   // (beyond what was measured: every 32 rows read the weights again)
   const SplitCut s = split_cut(c, M, K, R, 1);
   const TiledCut t = tiled_cut(c, M, K, R, 2, 1);
   const double per = (double)s.slabs / s.split, ctas = (double)s.tiles * s.n_tiles * s.split / c->n_sm;
   const double split = 3.3 + 0.42 * per + 6.4 / s.split + 1.8 * ctas + 0.5 * per * (ceil(ctas / 2) - 1);
   const double tiled = (plain_store ? 2.6 : 4.6) + s.slabs * t.waves * (0.22 + 0.05 * t.NT / 32);
-  return tiled < split;
+  return tiled + (resid ? 3.0 : 0.0) < split;
 }
 
 bool tiled_gemm(fm_ctx* c, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, const int* n_active, int mode, const tc::Epi& e) {
   const bool resid = mode == tc::EPI_RESID;
   if (!resid && mode != tc::EPI_F32 && mode != tc::EPI_GELU && !(mode == tc::EPI_QKV && e.rows != nullptr && e.stash_ring == nullptr)) return false;
-  if (!tiled_is_faster(c, M, K, R, mode == tc::EPI_F32)) return false;
+  if (!tiled_is_faster(c, M, K, R, mode == tc::EPI_F32, resid)) return false;
   pf::Epi t{};
   t.ssq_in = e.ssq_in; t.ssq_n = e.ssq_n; t.ld_ssq = resid ? e.ld_ssq_out : e.ld_ssq; t.inv_d = e.inv_d_in; t.eps = e.eps;
   t.out = e.out; t.ldo = e.ldo; t.lo_off = e.lo_off;

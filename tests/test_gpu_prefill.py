@@ -55,12 +55,14 @@ def test_prefill_lockstep_128_query_rows_per_cta_heads_of_128(faces, window, kw)
     test_prefill_lockstep(faces, window, {"n_heads": heads, "n_kv_heads": heads, "head_dim": 128, **kw})
 
 
-# The rows on both sides of each change between the split-K and the tiled form, at d = 128: 64 coordinate rows (most
-# projections), 225 (second FFN matrix of 256 columns), 481 (what is split up to there, here the second FFN matrix of 2048).
-@pytest.mark.parametrize("faces,d_ff", [
-    ((6, 0, 0, 0, 0, 0, 0, 0, 0), 256), ((7,), 256),                  # 63 and 64 rows
-    ((24, 0, 0, 0, 0, 0, 0, 0), 256), ((24, 0, 0, 0, 0, 0, 0, 0, 0), 256),        # 224 and 225
-    ((52, 1, 0), 2048), ((52, 1, 0, 0), 2048),                        # 480 and 481
+# The rows on both sides of each change between the split-K and the tiled form: 64 coordinate rows (projections without a
+# residual), 481 (those with one, at d = 128), 321 (the output projection of d = 1024).
+@pytest.mark.parametrize("faces,kw", [
+    ((6, 0, 0, 0, 0, 0, 0, 0, 0), {}), ((7,), {}),                    # 63 and 64 rows
+    ((52, 1, 0), {}), ((52, 1, 0, 0), {}),                            # 480 and 481
+    ((52, 1, 0, 0), {"d_ff": 2048, "weight_std": 0.05}),
+    ((33, 2, 0, 0, 0), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),              # 320 and 321
+    ((33, 2, 0, 0, 0, 0), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),
 ])
-def test_prefill_lockstep_where_projections_change_form(faces, d_ff):
-    test_prefill_lockstep(faces, (0, 0, 0), {"d_ff": d_ff, "weight_std": 0.1 if d_ff <= 256 else 0.05})
+def test_prefill_lockstep_where_projections_change_form(faces, kw):
+    test_prefill_lockstep(faces, (0, 0, 0), kw)
