@@ -502,9 +502,9 @@ EncodeTiledFn encode_tiled_fn() {
   return fn;
 }
 
-// 2-D bf16 tensor [rows, cols] row-major, box [box_rows, 64 columns] (128 bytes), 128-byte swizzle.
+// 2-D bf16 tensor [rows, cols] row-major, box [box_rows, 64 columns] (128 bytes), 128-byte swizzle (`plain`: none).
 // Returns the index of the new map in ctx->tmaps_host, or -1.
-int add_tmap_bf16(fm_ctx* c, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+int add_tmap_bf16(fm_ctx* c, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, bool plain = false) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (fn == nullptr) return -1;
   CUtensorMap m;
@@ -513,7 +513,7 @@ int add_tmap_bf16(fm_ctx* c, const void* base, uint64_t rows, uint64_t cols, uin
   const cuuint32_t box[2] = {64, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   if (fn(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), gdim, gstride, box, estr,
-         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, plain ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return -1;
   c->tmaps_host.push_back(m);
@@ -540,14 +540,15 @@ int add_tmap_operand(fm_ctx* c, const void* base, uint64_t rows, uint64_t K, uin
 }
 
 // The same rows for stages of one or two K slabs: a 4-D tensor (64 columns, rows, parts, K / 64) whose box brings, slab
-// after slab, the hi and the lo tile; what lies behind the last slab reads as zero.
-int add_tmap_stage(fm_ctx* c, const void* base, uint64_t rows, uint64_t K, uint32_t parts, uint32_t box_rows) {
+// after slab, the hi and the lo tile (`pair`: one CTA's share of them, see pf::gemm_kernel); what lies behind the last
+// slab reads as zero.
+int add_tmap_stage(fm_ctx* c, const void* base, uint64_t rows, uint64_t K, uint32_t parts, uint32_t box_rows, bool pair) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (fn == nullptr) return -1;
   CUtensorMap m;
   const cuuint64_t gdim[4] = {64, rows, parts, K / 64};
   const cuuint64_t gstride[3] = {parts * K * 2, K * 2, 128};
-  const cuuint32_t box[4] = {64, box_rows, parts, (cuuint32_t)pf::stage_slabs((int)box_rows, (int)parts)};
+  const cuuint32_t box[4] = {64, box_rows, pair ? 1 : parts, (cuuint32_t)pf::stage_slabs((int)(pair ? 2 * box_rows / parts : box_rows), (int)parts)};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   if (fn(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), gdim, gstride, box, estr,
          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -559,15 +560,16 @@ int add_tmap_stage(fm_ctx* c, const void* base, uint64_t rows, uint64_t K, uint3
 
 // index of the tensor map for a bf16 matrix / box, created on first use (all call sites are
 // visited by the first pass, before any timing or capture)
-constexpr uint32_t TMAP_STAGE = 16;      // added to `parts`: the 4-D form; parts = 0: a plain 2-D map
+constexpr uint32_t TMAP_STAGE = 16, TMAP_PAIR = 32;      // added to `parts`: the 4-D form, of a pair of CTAs
+constexpr uint32_t TMAP_PLAIN = 64;                      // as `parts`: a 2-D map without the swizzle; 0: with it
 int tmap_for(fm_ctx* c, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t parts) {
   for (size_t i = 0; i < c->tmap_keys.size(); ++i) {
     const auto& k = c->tmap_keys[i];
     if (k.base == base && k.rows == rows && k.cols == cols && k.box_rows == box_rows && k.parts == parts) return (int)i;
   }
   if (c->tmaps_host.size() >= c->tmaps_cap || c->capturing) return -1;   // descriptors are made before capture
-  const int idx = parts == 0 ? add_tmap_bf16(c, base, rows, cols, box_rows)
-                  : parts >= TMAP_STAGE ? add_tmap_stage(c, base, rows, cols, parts - TMAP_STAGE, box_rows)
+  const int idx = parts == 0 || parts == TMAP_PLAIN ? add_tmap_bf16(c, base, rows, cols, box_rows, parts == TMAP_PLAIN)
+                  : parts >= TMAP_STAGE ? add_tmap_stage(c, base, rows, cols, parts & (TMAP_STAGE - 1), box_rows, (parts & TMAP_PAIR) != 0)
                                         : add_tmap_operand(c, base, rows, cols, parts, box_rows);
   if (idx < 0) return -1;
   c->tmap_keys.push_back({base, rows, cols, box_rows, parts});
@@ -740,41 +742,56 @@ void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_ro
   if (mode == tc::EPI_UP && e.ssq_out != nullptr) c->ssq_n = (c->dm.d / tc::BM) * split * (split == 1 ? 2 : 1);   // tiles within d
 }
 
-// How a launch of the tiled form (fm_prefill.cuh) is cut.  Rows per tile: the choice that minimises waves x (slabs x the
-// longer of a slab's copy at 64 B per clock and its MMAs, + about 2000 clocks of start-up and epilogue).
-struct TiledCut { int NT; double waves; };
+// How a launch of the tiled form (fm_prefill.cuh) is cut.  Rows per tile and CTAs per tile (one, or a pair that shares the
+// operand rows): the choice that minimises waves x (slabs x the longer of a slab's copy at 64 B per clock and its MMAs, + about
+// 2000 clocks of start-up and epilogue).  Single CTAs / pairs in whole requests up to the first pass, us: 6994 rows 8105 / 7852,
+// 16 prompts of 73 to 577 rows 7946 / 7654, 73 rows 2104 / 2116 (d = 1024).
+struct TiledCut { int NT, cg; double waves; };
 TiledCut tiled_cut(const fm_ctx* c, int M, int K, int R, int parts, int layers) {
   const int tiles_m = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
-  TiledCut t{32, 0.0};
+  TiledCut t{32, 1, 0.0};
   double best = 0.0;
-  for (int nt = 32; nt <= 256 / parts; nt *= 2) {
-    const double tiles = (double)tiles_m * ((R + nt - 1) / nt) * layers, waves = ceil(tiles / c->n_sm);
-    const double copy = (tc::BM * 128 + parts * nt * 128) / 64.0, mma = 2.0 * (parts * nt > 64 ? parts * nt : 64);
-    const double cost = waves * (slabs * (copy > mma ? copy : mma) + 12.0 * parts * nt) + 2000.0;
-    if (nt == 32 || cost < best) { best = cost; t = TiledCut{nt, waves}; }
+  for (int cg = 1; cg <= 2; ++cg) {
+    if (cg == 2 && tiles_m == 1) continue;
+    for (int nt = 32; nt <= 256 / parts; nt *= 2) {
+      const double tiles = (double)((tiles_m + cg - 1) / cg) * ((R + nt - 1) / nt) * layers, waves = ceil(tiles / (c->n_sm / cg));
+      const double copy = (tc::BM * 128 + parts * nt / cg * 128) / 64.0, mma = 2.0 * (parts * nt > 64 ? parts * nt : 64);
+      const double cost = waves * (slabs * (copy > mma ? copy : mma) + 12.0 * parts * nt) + 2000.0;
+      if (best == 0.0 || cost < best) { best = cost; t = TiledCut{nt, cg, waves}; }
+    }
   }
   return t;
+}
+
+template <int MODE, int PARTS>
+void launch_tiled(fm_ctx* c, int cg, dim3 grid, int smem, const pf::Gemm& g, const pf::Epi& e) {
+  if (cg == 1) launch_pdl(c, dim3(1, 1, 1), pf::gemm_kernel<MODE, PARTS, 1>, grid, pf::THREADS, smem, g, e);
+  else launch_pdl(c, dim3(2, 1, 1), pf::gemm_kernel<MODE, PARTS, 2>, grid, pf::THREADS, smem, g, e);
 }
 
 void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, pf::Epi e, int layers = 1, int w_tile0 = 0,
              const int* n_active = nullptr) {
   if (R <= 0) return;
-  const int parts = mode == pf::PF_PREFIX ? 1 : 2, tiles_m = (M + tc::BM - 1) / tc::BM, NT = tiled_cut(c, M, K, R, parts, layers).NT;
-  const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, NT, TMAP_STAGE + (uint32_t)parts);
-  if (tA < 0) { c->launch_error = FM_ERR_CUDA; return; }
-  int stages = (200 * 1024) / pf::stage_bytes(NT, parts);
-  stages = stages > pf::MAX_STAGES ? pf::MAX_STAGES : stages;
+  const int parts = mode == pf::PF_PREFIX ? 1 : 2, tiles_w = (M + tc::BM - 1) / tc::BM;
+  const TiledCut cut = tiled_cut(c, M, K, R, parts, layers);
+  const int NT = cut.NT, cg = cut.cg, slabs = pf::stage_slabs(NT, parts), tiles_m = (tiles_w + cg - 1) / cg;
+  const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, parts * NT / cg / (cg == 1 ? parts : 1), TMAP_STAGE + (cg == 2 ? TMAP_PAIR : 0) + (uint32_t)parts);
+  const int tW = cg == 2 ? tmap_for(c, c->ws, c->ws_bytes / 128, tc::BK, slabs * tc::BM, TMAP_PLAIN) : 0;
+  if (tA < 0 || tW < 0) { c->launch_error = FM_ERR_CUDA; return; }
+  const int stages = pf::ring_stages(NT, parts, cg);
   const int tiles_n = (R + NT - 1) / NT, tiles = tiles_m * tiles_n * layers;
-  if (mode == pf::PF_RESID && e.ssq_out != nullptr) c->ssq_n = tiles_m * 4;        // slots the next consumer adds
-  pf::Gemm g{W, c->tmaps + tA, M, K, R, NT, stages, pf::stage_slabs(NT, parts), tiles_m, tiles_n, tiles, w_tile0, n_active, c->st.status};
-  const dim3 grid(tiles < c->n_sm ? tiles : c->n_sm), one(1, 1, 1);
-  const int smem = pf::smem_bytes(NT, parts, stages);
+  if (mode == pf::PF_RESID && e.ssq_out != nullptr) c->ssq_n = tiles_w * 4;        // slots the next consumer adds
+  pf::Gemm g{W, c->tmaps + tA, M, K, R, NT, stages, slabs, tiles_m, tiles_n, tiles, reinterpret_cast<const bf16*>(c->ws), c->tmaps + tW, w_tile0, tiles_w,
+             n_active, c->st.status};
+  const int workers = c->n_sm / cg;
+  const dim3 grid(cg * (tiles < workers ? tiles : workers));
+  const int smem = pf::smem_bytes(NT, parts, cg, stages);
   switch (mode) {
-    case pf::PF_F32: launch_pdl(c, one, pf::gemm_kernel<pf::PF_F32, 2>, grid, pf::THREADS, smem, g, e); break;
-    case pf::PF_GELU: launch_pdl(c, one, pf::gemm_kernel<pf::PF_GELU, 2>, grid, pf::THREADS, smem, g, e); break;
-    case pf::PF_RESID: launch_pdl(c, one, pf::gemm_kernel<pf::PF_RESID, 2>, grid, pf::THREADS, smem, g, e); break;
-    case pf::PF_QKV: launch_pdl(c, one, pf::gemm_kernel<pf::PF_QKV, 2>, grid, pf::THREADS, smem, g, e); break;
-    default: launch_pdl(c, one, pf::gemm_kernel<pf::PF_PREFIX, 1>, grid, pf::THREADS, smem, g, e); break;
+    case pf::PF_F32: launch_tiled<pf::PF_F32, 2>(c, cg, grid, smem, g, e); break;
+    case pf::PF_GELU: launch_tiled<pf::PF_GELU, 2>(c, cg, grid, smem, g, e); break;
+    case pf::PF_RESID: launch_tiled<pf::PF_RESID, 2>(c, cg, grid, smem, g, e); break;
+    case pf::PF_QKV: launch_tiled<pf::PF_QKV, 2>(c, cg, grid, smem, g, e); break;
+    default: launch_tiled<pf::PF_PREFIX, 1>(c, cg, grid, smem, g, e); break;
   }
 }
 
@@ -808,6 +825,7 @@ bool tiled_is_faster(const fm_ctx* c, int M, int K, int R, bool plain_store, boo
 bool tiled_gemm(fm_ctx* c, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, const int* n_active, int mode, const tc::Epi& e) {
   const bool resid = mode == tc::EPI_RESID;
   if (!resid && mode != tc::EPI_F32 && mode != tc::EPI_GELU && !(mode == tc::EPI_QKV && e.rows != nullptr && e.stash_ring == nullptr)) return false;
+  if (mode == tc::EPI_F32 && (e.ldo & 3) != 0) return false; // rows stored in 16-byte pieces
   if (!tiled_is_faster(c, M, K, R, mode == tc::EPI_F32, resid)) return false;
   pf::Epi t{};
   t.ssq_in = e.ssq_in; t.ssq_n = e.ssq_n; t.ld_ssq = resid ? e.ld_ssq_out : e.ld_ssq; t.inv_d = e.inv_d_in; t.eps = e.eps;
@@ -1637,12 +1655,17 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
   TRYCUDA(allow_rows_smem<tc::EPI_UP>());
   TRYCUDA(allow_rows_smem<tc::EPI_QKV>());
   {
-    const int most = 216 * 1024;                             // a ring of at most 200 KB and what lies behind it
-    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_F32, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_GELU, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_RESID, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_QKV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_PREFIX, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    const int most = pf::SMEM_MOST;
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_F32, 2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_F32, 2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_GELU, 2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_GELU, 2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_RESID, 2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_RESID, 2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_QKV, 2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_QKV, 2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_PREFIX, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRYCUDA(cudaFuncSetAttribute(pf::gemm_kernel<pf::PF_PREFIX, 1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRYCUDA(cudaFuncSetAttribute(pf::attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::fa::BYTES));
     TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<64, 128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<64, 128, 2>::BYTES));
     TRYCUDA(cudaFuncSetAttribute(pf::attn_kernel<64, 128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::AttnCfg<64, 128, 1>::BYTES));

@@ -250,7 +250,11 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
         if (b_ok) o[1] = yb;
       }
     } else if (MODE == EPI_BF16 || MODE == EPI_GELU) {
-      if (MODE == EPI_GELU) { ya = gelu_erf_f(ya); yb = gelu_erf_f(yb); }
+      if (MODE == EPI_GELU) {
+        const float2 y = gelu2(ya, yb);
+        ya = y.x;
+        yb = y.y;
+      }
       bf16* o = reinterpret_cast<bf16*>(e.out) + row * e.ldo + ma;
       if (active && b_ok) store_hi_lo2(o, ya, yb, e.lo_off);
       else if (active && a_ok) store_hi_lo(o, ya, e.lo_off);

@@ -112,9 +112,9 @@ __device__ inline uint64_t smem_desc_sw128(uint32_t addr) {
   return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
          ((uint64_t)2 << 61);
 }
-__device__ inline uint32_t instr_desc_bf16(int n) {
-  // fp32 accumulate, bf16 x bf16, both K-major, M = 128, N = n
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+__device__ inline uint32_t instr_desc_bf16(int n, int m = BM) {
+  // fp32 accumulate, bf16 x bf16, both K-major, M = m (128, of a pair of CTAs 256), N = n
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 __device__ inline void mma_ss(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -223,7 +223,27 @@ __device__ inline void store_hi_lo2(bf16* p, float a, float b, int lo_off) {
     *reinterpret_cast<__nv_bfloat162*>(p + lo_off) = __floats2bfloat162_rn(__fsub_rn(a, __bfloat162float(hi.x)), __fsub_rn(b, __bfloat162float(hi.y)));
 }
 
-__device__ inline float gelu_erf_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
+// GELU of two values, x Phi(x) = max(x, 0) - |x| Phi(-|x|), with Phi(-c) = 2^q(c).  q(c) = log2 Phi(-c) on [0, 7] (behind
+// that the second term is under 1e-11) as a polynomial of degree 10 with q(0) = -1, fitted to SciPy's log_ndtr by
+// iteratively reweighted least squares (Lawson) with the weight c Phi(-c), i.e. for the smallest absolute error.  Packed
+// multiply-adds, one exponential, no branch: the first FFN matrix of 6994 rows takes 85 us, with erff 92.  Against 64 bits,
+// largest absolute error on [-9, 9] 2.4e-7 where 0.5 x (1 + erff(x / sqrt 2)) has 4.9e-7 (root mean square over a standard
+// normal 2.0e-8 and 2.5e-8; the negative tail, where that form cancels, is better by orders of magnitude).
+__device__ inline float2 gelu2(float a, float b) {
+  auto pack = [](float lo, float hi) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; };
+  const float ca = fminf(fabsf(a), 7.f), cb = fminf(fabsf(b), 7.f);
+  const uint64_t c = pack(ca, cb);
+  uint64_t q = pack(-3.9760344350270316e-08f, -3.9760344350270316e-08f);
+  constexpr float K[10] = {1.0968196875182912e-06f, -1.3029140973230824e-05f, 8.565230382373556e-05f, -0.00030231187702156603f, 3.0413037165999413e-05f,
+                           0.006926937960088253f, -0.052437372505664825f, -0.4592195749282837f, -1.1511045694351196f, -1.f};
+#pragma unroll
+  for (int k = 0; k < 10; ++k) asm("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(q) : "l"(c), "l"(pack(K[k], K[k])));
+  float qa, qb, ea, eb;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(qa), "=f"(qb) : "l"(q));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ea) : "f"(qa));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(eb) : "f"(qb));
+  return make_float2(__fmaf_rn(0.5f, a + fabsf(a), -__fmul_rn(ca, ea)), __fmaf_rn(0.5f, b + fabsf(b), -__fmul_rn(cb, eb)));       // (a NaN stays one)
+}
 
 // Pair slot q (0..63) of a 128-column tile holds columns (2q, 2q + 1): a thread's two values leave in one
 // store, and in the QKV projection, whose weight rows are stored with the rotary pairs (i, i + dh/2) of
@@ -585,8 +605,9 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
       else if (a_ok) store_hi_lo(o + ma, ya, k_lo);
     } else if (MODE == EPI_GELU) {
       bf16* o = reinterpret_cast<bf16*>(k_out) + row * k_ldo;
-      if (b_ok) store_hi_lo2(o + ma, gelu_erf_f(ya), gelu_erf_f(yb), k_lo);
-      else if (a_ok) store_hi_lo(o + ma, gelu_erf_f(ya), k_lo);
+      const float2 y = gelu2(ya, yb);
+      if (b_ok) store_hi_lo2(o + ma, y.x, y.y, k_lo);
+      else if (a_ok) store_hi_lo(o + ma, y.x, k_lo);
     } else if (IS_RESID) {
       float* xr = k_x + row * k_ldx;
       float xa = 0.f, xb = 0.f;

@@ -26,31 +26,35 @@ struct LayerPtr { const bf16* Wqkv; const float* g1; bf16* K; bf16* V; int level
 // ------------------------------------------------------------------------------------------
 // GEMM
 // ------------------------------------------------------------------------------------------
-// y[n][m] = sum_k W[m, k] A[n, k].  Tile: 128 output features (the MMA's M axis) x NT rows (N axis).
+// y[n][m] = sum_k W[m, k] A[n, k].  Tile: 128 output features per CTA (the MMA's M axis) x NT rows (N axis).
 // Operand rows with two bfloat16 terms lie as [hi | lo] tiles behind one another and form one operand of
-// 2 NT rows, so a weight slab is loaded once for both.  One persistent CTA per SM walks over the tiles
+// 2 NT rows, so a weight slab is loaded once for both.  Persistent CTAs walk over the tiles
 // (feature tiles innermost: neighbouring CTAs share their operand rows in L2); a ring of shared-memory
-// stages decouples the copies from the MMA thread, and two accumulators in tensor memory let the
-// epilogue of a tile run under the MMAs of the next.  A thread of the epilogue owns one feature (its
-// tensor-memory lane), so a warp stores 32 neighbouring features of a row at a time.
-// One thread needs about 420 clocks to request a weight slab and an operand slab of 64 k, and 128 threads
-// need 35 000 clocks for the GELU of a tile (its MMAs take 8 200): hence a producer warp for each of the two
-// streams, (for narrow tiles) stages of two slabs and eight epilogue warps.
-// 6994 rows, d = 1024: QKV 99 us, first FFN matrix 125, second 110, output projection 41, with the tensor pipe active
-// 43, 46, 53 and 33 % of the time.  A slab of a 128 x 128 tile is 48 KB and 512 MMA clocks; it takes 970 clocks where the
-// epilogue does not matter (second FFN matrix: 51 B per clock and SM; the L2 slices are at 27 to 35 % of their rate, DRAM
-// under 21 %), so the MMAs wait for the copies.
+// stages decouples the copies from the warp that issues the MMAs, and two accumulators in tensor memory let the
+// epilogue of a tile run under the MMAs of the next.
+// CG = 2: two CTAs of a cluster multiply together (tcgen05 cta_group::2, M = 256).  Each keeps its own 128 features of
+// weights; of the operand rows the first holds the hi and the second the lo tile, so an SM copies 32 instead of
+// 48 KB per slab and its MMAs read a third less shared memory.  The first CTA issues; both CTAs' copies count on its barriers.
+// What a slab (512 MMA clocks) waited for, 6994 rows, d = 1024, K = 4096: one thread per role behind `lane == 0`, whose
+// every descriptor went from general to uniform registers: 970 clocks; whole warps in step with one elected lane: 740.
+// The epilogue runs beside that, and must not take longer than a tile's MMAs (8 200 clocks at K = 1024).  A warp turns
+// CW rows x 32 features in shared memory so that a lane works on four neighbouring features of a row (no shuffles, 8- and
+// 16-byte stores, a row's address once for all of them), sixteen warps hide each other's latencies, the rows' scales
+// come from a warp of their own, and what an epilogue reads is requested a step ahead.
+// QKV / output projection / first / second FFN matrix, 6994 rows, d = 1024, us: 99 / 41 / 125 / 110 before these, 63 / 32 / 85 / 83
+// now (without any epilogue 57 / 22 / 73 / 69; tensor pipe 75 % active in the last).
 enum Mode { PF_F32 = 0, PF_GELU = 1, PF_RESID = 2, PF_QKV = 3, PF_PREFIX = 4 };
 
-constexpr int THREADS = 384;     // weight producer, operand producer, MMA warp, one idle warp, eight epilogue warps
-constexpr int EPI_WARPS = 8;
-constexpr int MAX_STAGES = 4;     // (deeper rings were no faster)
+constexpr int EPI_WARPS = 16, CW = 16;           // epilogue warps; rows a warp takes at a time
+constexpr int THREADS = 128 + 32 * EPI_WARPS;    // weight producer, operand producer, MMA warp, one idle warp, the epilogue
+constexpr int MAX_STAGES = 6;
 
 struct Gemm {
   const bf16* W; const CUtensorMap* tmA;
   int M, K, R, NT, stages, slabs;  // slabs of 64 k per stage: 1 or 2
-  int tiles_m, tiles_n, tiles;   // tiles = tiles_m * tiles_n * layers (PF_PREFIX), else tiles_m * tiles_n
-  int w_tile0;
+  int tiles_m, tiles_n, tiles;   // tiles = tiles_m * tiles_n * layers (PF_PREFIX), else tiles_m * tiles_n; a pair's tile has 256 features
+  const bf16* w_base; const CUtensorMap* tmW;      // pairs: weights through one map over the workspace [bytes / 128][64]
+  int w_tile0, w_tiles;          // first and number of 128-feature tiles of the matrix
   const int* n_active;           // skip when *n_active == 0 (may be null)
   int* status;
 };
@@ -64,8 +68,51 @@ struct Epi {
 };
 
 inline int stage_slabs(int NT, int parts) { return parts * NT > 128 ? 1 : 2; }      // slabs of 64 k per stage
-inline int stage_bytes(int NT, int parts) { return stage_slabs(NT, parts) * (tc::BM * 128 + parts * NT * 128); }
-inline int smem_bytes(int NT, int parts, int stages) { return stages * stage_bytes(NT, parts) + 2 * 256 * 4 + 256 + 1024; }
+inline int stage_bytes(int NT, int parts, int cg) { return stage_slabs(NT, parts) * (tc::BM * 128 + parts * NT / cg * 128); }
+// behind the ring: the epilogue's scratch, the rows' scales of two tiles, barriers, room to align
+constexpr int SMEM_MOST = 227 * 1024, SMEM_REST = EPI_WARPS * CW * 32 * 4 + 2 * 128 * 4 + 256 + 1024;
+inline int ring_stages(int NT, int parts, int cg) {
+  const int n = (SMEM_MOST - SMEM_REST) / stage_bytes(NT, parts, cg);
+  return n < MAX_STAGES ? n : MAX_STAGES;
+}
+inline int smem_bytes(int NT, int parts, int cg, int stages) { return stages * stage_bytes(NT, parts, cg) + SMEM_REST; }
+
+// tcgen05 instructions of a CTA (CG = 1) or of a pair of CTAs (CG = 2)
+template <int CG>
+__device__ inline void tmem_alloc(uint32_t* slot, uint32_t ncols) {
+  if (CG == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(slot)), "r"(ncols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  } else {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(slot)), "r"(ncols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+}
+template <int CG>
+__device__ inline void tmem_free(uint32_t tmem, uint32_t ncols) {
+  if (CG == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+  else asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+}
+template <int CG>
+__device__ inline void mma(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+  if (CG == 1) tc::mma_ss(tmem_d, da, db, idesc, accumulate);
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// arrives on the barrier (of both CTAs of a pair) once the MMAs issued so far are done
+template <int CG>
+__device__ inline void commit(uint64_t* bar) {
+  if (CG == 1) tc::commit(bar);
+  else
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(ptx::smem_u32(bar)),
+                 "h"((uint16_t)3)
+                 : "memory");
+}
 
 __device__ inline void ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -77,39 +124,23 @@ __device__ inline void ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
+__device__ inline void ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
 __device__ inline void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ inline bool epi_sync_or(bool v) {                 // barrier of the epilogue warps; true if it was true for any thread
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-               : "=r"(r) : "r"((uint32_t)v) : "memory");
-  return r != 0;
+// [hi | lo] operand values of four neighbouring features
+__device__ inline void store_hi_lo4(bf16* p, float a, float b, float c, float d, int lo_off) {
+  const __nv_bfloat162 h0 = __floats2bfloat162_rn(a, b), h1 = __floats2bfloat162_rn(c, d);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+  *reinterpret_cast<uint2*>(p + lo_off) = make_uint2(ptx::pack_bf16(__fsub_rn(a, __bfloat162float(h0.x)), __fsub_rn(b, __bfloat162float(h0.y))),
+                                                     ptx::pack_bf16(__fsub_rn(c, __bfloat162float(h1.x)), __fsub_rn(d, __bfloat162float(h1.y))));
 }
 
-// One step of a transposing butterfly: afterwards a lane holds half as many rows, summed over pairs of lanes.
-template <int H>
-__device__ inline void fold(float* v, int lane) {
-#pragma unroll
-  for (int i = 0; i < H; ++i) {
-    const float send = (lane & H) ? v[i] : v[i + H], keep = (lane & H) ? v[i + H] : v[i];
-    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, H);
-  }
-}
-
-// [hi | lo] operand values of 32 rows: neighbouring lanes hold neighbouring features; of two rows the even
-// lane stores the first and the odd lane the second, both features in one 4-byte store per term.  `p`: the
-// lane pair's first feature of the first row.
-__device__ inline void store_rows_hi_lo(bf16* p, int ld, int lo_off, const float (&y)[32], int nv, bool ok, int lane) {
-  const bool odd = lane & 1;
-#pragma unroll
-  for (int j = 0; j < 32; j += 2) {
-    const float other = __shfl_xor_sync(0xffffffffu, odd ? y[j] : y[j + 1], 1);
-    const float a = odd ? other : y[j], b = odd ? y[j + 1] : other;
-    const int n = j + (odd ? 1 : 0);
-    if (n < nv && ok) tc::store_hi_lo2(p + (size_t)n * ld, a, b, lo_off);
-  }
-}
-
-template <int MODE, int PARTS>
+template <int MODE, int PARTS, int CG>
 __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Epi e) {
   if (g.n_active != nullptr && *g.n_active == 0) {           // the whole grid leaves; keep the launch chain ordered
     ptx::grid_dep_launch();
@@ -119,16 +150,20 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int NT = g.NT, ST = g.stages, SLABS = g.slabs;
-  const int w_slab = tc::BM * 128, a_slab = PARTS * NT * 128, stage = SLABS * (w_slab + a_slab);
-  float* s_inv = reinterpret_cast<float*>(sm + ST * stage);                  // [2][256]
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_inv + 512);
+  const int HN = PARTS * NT / CG;                            // operand rows of a slab in this CTA
+  const int w_slab = tc::BM * 128, a_slab = HN * 128, stage = SLABS * (w_slab + a_slab);
+  float* s_turn = reinterpret_cast<float*>(sm + ST * stage);                 // [epilogue warp][CW rows][32 features]
+  float* s_inv = s_turn + EPI_WARPS * CW * 32;               // [2][128]
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_inv + 2 * 128);
   uint64_t* empty = full + MAX_STAGES;
   uint64_t* acc_full = empty + MAX_STAGES;
   uint64_t* acc_empty = acc_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
-  __shared__ int s_fail;
-  __shared__ Row s_row[2][MODE == PF_QKV ? 128 : 1];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint64_t *inv_full = acc_empty + 2, *inv_empty = inv_full + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(inv_empty + 2);
+  int& s_fail = *reinterpret_cast<int*>(tmem_slot + 1);
+  const int tid = threadIdx.x, warp = (int)ptx::uniform(tid >> 5), lane = tid & 31;
+  const int rank = CG == 2 ? (int)ptx::uniform(tc::cluster_rank()) : 0;    // place in the pair
+  const int worker = (int)blockIdx.x / CG, workers = (int)gridDim.x / CG;
   const int slabs = g.K / tc::BK, steps = (slabs + SLABS - 1) / SLABS;
   uint32_t ncols = 32;
   while ((int)ncols < 2 * PARTS * NT) ncols <<= 1;
@@ -136,19 +171,20 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
   if (tid == 0) {
     s_fail = 0;
     for (int i = 0; i < ST; ++i) { ptx::mbar_init(full + i, 2); ptx::mbar_init(empty + i, 1); }
-    for (int i = 0; i < 2; ++i) { ptx::mbar_init(acc_full + i, 1); ptx::mbar_init(acc_empty + i, EPI_WARPS); }
+    for (int i = 0; i < 2; ++i) { ptx::mbar_init(acc_full + i, 1); ptx::mbar_init(acc_empty + i, CG * EPI_WARPS); ptx::mbar_init(inv_full + i, 1); ptx::mbar_init(inv_empty + i, EPI_WARPS); }
     ptx::fence_mbar_init();
     ptx::prefetch_tmap(g.tmA);
+    if (CG == 2) ptx::prefetch_tmap(g.tmW);
   }
-  if (warp == 2) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(tmem_slot)), "r"(ncols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
+  if (warp == 2) tmem_alloc<CG>(tmem_slot, ncols);
   tc::fence_before();
   __syncthreads();
+  if (CG == 2) tc::cluster_sync();                           // the peer's barriers are initialised
   tc::fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = ptx::uniform(*tmem_slot);
   ptx::grid_dep_launch();
+  const bool scaled = MODE != PF_PREFIX && MODE != PF_RESID && e.ssq_in != nullptr;
+  bool failed = false;                                       // a bounded wait of this warp gave up
   const int per_z = g.tiles_m * g.tiles_n;
   auto tile_of = [&](int t, int& z, int& tm, int& tn) {
     z = MODE == PF_PREFIX ? t / per_z : 0;
@@ -156,210 +192,286 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
     tn = u / g.tiles_m;
     tm = u - tn * g.tiles_m;
   };
-  if (warp == 0 && lane == 0) {
+  auto wait = [](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity)) != 0; };
+  if (warp == 0) {
     // ---- weights: they do not depend on the previous kernel and start before the dependency wait
-    int it = 0;
-    for (int t = blockIdx.x; t < g.tiles && !s_fail; t += gridDim.x) {
+    int st = 0, round = 0;                                   // stage, times the ring has been walked through
+    for (int t = worker; t < g.tiles && !failed; t += workers) {
       int z, tm, tn;
       tile_of(t, z, tm, tn);
-      const bf16* W = (MODE == PF_PREFIX ? e.layers[z].Wqkv : g.W) + (size_t)(g.w_tile0 + tm) * slabs * (tc::BM * tc::BK);
-      for (int s = 0; s < steps; ++s, ++it) {
-        const int st = it % ST, bytes = min(SLABS, slabs - s * SLABS) * w_slab;
-        if (it >= ST && !ptx::mbar_wait(empty + st, ((it / ST) - 1) & 1)) { s_fail = 1; break; }
-        ptx::mbar_expect_tx(full + st, bytes);
-        ptx::bulk_load(sm + st * stage, W + (size_t)s * SLABS * (tc::BM * tc::BK), bytes, full + st);
+      // (an odd number of 128-feature tiles: the last pair's second CTA repeats the first one's weights and stores nothing)
+      const int tw = CG == 2 ? min(CG * tm + rank, g.w_tiles - 1) : tm;
+      const bf16* W = (MODE == PF_PREFIX ? e.layers[z].Wqkv : g.W) + (size_t)(g.w_tile0 + tw) * slabs * (tc::BM * tc::BK);
+      const int w_row = CG == 2 ? (int)((W - g.w_base) / tc::BK) : 0;
+      for (int s = 0; s < steps; ++s) {
+        if (round > 0 && !wait(empty + st, (round - 1) & 1)) { failed = true; break; }
+        if (ptx::elect_one()) {
+          if (CG == 1) {
+            const int bytes = min(SLABS, slabs - s * SLABS) * w_slab;
+            ptx::mbar_expect_tx(full + st, bytes);
+            ptx::bulk_load(sm + st * stage, W + (size_t)s * SLABS * (tc::BM * tc::BK), bytes, full + st);
+          } else {                                           // (behind the last slab: whatever follows, never multiplied)
+            if (rank == 0) ptx::mbar_expect_tx(full + st, CG * SLABS * w_slab);
+            ptx::tma_load_2d_pair(sm + st * stage, g.tmW, 0, w_row + s * SLABS * tc::BM, tc::map_peer(ptx::smem_u32(full + st), 0));
+          }
+        }
+        if (++st == ST) { st = 0; ++round; }
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---- operand rows: one copy brings the hi and lo tiles of a stage (zeros behind the last slab)
+    // the MMA thread's last arrivals (of the other CTA of a pair) land before this CTA leaves
+    for (int i = 0; CG == 2 && i < ST && !failed; ++i) {
+      const int uses = round + (i < st ? 1 : 0);
+      if (uses > 0 && !wait(empty + i, (uses - 1) & 1)) failed = true;
+    }
+    if (failed) s_fail = 1;
+  } else if (warp == 1) {
+    // ---- operand rows: one copy brings the hi and lo tiles of a stage (zeros behind the last slab); of a pair, the first
+    // CTA holds the hi and the second the lo tile (one term: half of the rows each)
     ptx::grid_dep_wait();
-    int it = 0;
-    for (int t = blockIdx.x; t < g.tiles && !s_fail; t += gridDim.x) {
+    int st = 0, round = 0;                                   // stage, times the ring has been walked through
+    for (int t = worker; t < g.tiles && !failed; t += workers) {
       int z, tm, tn;
       tile_of(t, z, tm, tn);
-      const int row = tn * NT + (MODE == PF_PREFIX ? z * e.rows_layer : 0);
-      for (int s = 0; s < steps; ++s, ++it) {
-        const int st = it % ST;
-        if (it >= ST && !ptx::mbar_wait(empty + st, ((it / ST) - 1) & 1)) { s_fail = 1; break; }
-        ptx::mbar_expect_tx(full + st, SLABS * a_slab);
-        ptx::tma_load_4d(sm + st * stage + SLABS * w_slab, g.tmA, 0, row, 0, s * SLABS, full + st);
+      const int row = tn * NT + (MODE == PF_PREFIX ? z * e.rows_layer : 0) + (CG == 2 && PARTS == 1 ? rank * HN : 0);
+      for (int s = 0; s < steps; ++s) {
+        if (round > 0 && !wait(empty + st, (round - 1) & 1)) { failed = true; break; }
+        if (ptx::elect_one()) {
+          if (rank == 0) ptx::mbar_expect_tx(full + st, CG * SLABS * a_slab);
+          unsigned char* dst = sm + st * stage + SLABS * w_slab;
+          if (CG == 1) ptx::tma_load_4d(dst, g.tmA, 0, row, 0, s * SLABS, full + st);
+          else ptx::tma_load_4d_pair(dst, g.tmA, 0, row, PARTS == 2 ? rank : 0, s * SLABS, tc::map_peer(ptx::smem_u32(full + st), 0));
+        }
+        if (++st == ST) { st = 0; ++round; }
       }
     }
-  } else if (warp == 2 && lane == 0) {
+    if (failed) s_fail = 1;
+  } else if (warp == 2 && rank == 0) {
     // ---- MMA issuer
-    const uint32_t idesc = tc::instr_desc_bf16(PARTS * NT);
-    int it = 0, k = 0;
-    for (int t = blockIdx.x; t < g.tiles; t += gridDim.x, ++k) {
+    const uint32_t idesc = tc::instr_desc_bf16(PARTS * NT, CG * tc::BM);
+    int st = 0, round = 0, k = 0;
+    for (int t = worker; t < g.tiles; t += workers, ++k) {
       const int buf = k & 1;
-      if (k >= 2 && !ptx::mbar_wait(acc_empty + buf, ((k >> 1) - 1) & 1)) { s_fail = 1; break; }
+      if (k >= 2 && !(CG == 2 ? __all_sync(0xffffffffu, tc::mbar_wait_cluster(acc_empty + buf, ((k >> 1) - 1) & 1)) != 0 : wait(acc_empty + buf, ((k >> 1) - 1) & 1))) { failed = true; break; }
       tc::fence_after();
-      bool bad = false;
-      for (int s = 0; s < steps; ++s, ++it) {
-        const int st = it % ST, n = min(SLABS, slabs - s * SLABS);
-        if (!ptx::mbar_wait(full + st, (it / ST) & 1)) { s_fail = 1; bad = true; break; }
+      for (int s = 0; s < steps; ++s) {
+        const int n = min(SLABS, slabs - s * SLABS);
+        if (!wait(full + st, round & 1)) { failed = true; break; }
         tc::fence_after();
         const uint32_t base = ptx::smem_u32(sm + st * stage);
-        for (int j = 0; j < n; ++j) {
-          const uint64_t da = tc::smem_desc_sw128(base + j * w_slab), db = tc::smem_desc_sw128(base + SLABS * w_slab + j * a_slab);
+        if (ptx::elect_one()) {
+          for (int j = 0; j < n; ++j) {
+            const uint64_t da = tc::smem_desc_sw128(base + j * w_slab), db = tc::smem_desc_sw128(base + SLABS * w_slab + j * a_slab);
 #pragma unroll
-          for (int kk = 0; kk < tc::BK / 16; ++kk)
-            tc::mma_ss(tmem + buf * acc_cols, da + 2 * kk, db + 2 * kk, idesc, (s > 0 || j > 0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < tc::BK / 16; ++kk)
+              mma<CG>(tmem + buf * acc_cols, da + 2 * kk, db + 2 * kk, idesc, (s > 0 || j > 0 || kk > 0) ? 1u : 0u);
+          }
+          commit<CG>(empty + st);
+          if (s == steps - 1) commit<CG>(acc_full + buf);
         }
-        tc::commit(empty + st);
+        __syncwarp();
+        if (++st == ST) { st = 0; ++round; }
       }
-      if (bad) break;
-      tc::commit(acc_full + buf);
+      if (failed) break;
     }
-  } else if (warp >= 4) {
-    // ---- epilogue: warp w reads tensor-memory lanes 32 (w mod 4) .. + 31; warps w and w + 4 share the rows
-    const int w4 = warp & 3, et = tid - 128;
+    if (failed) s_fail = 1;
+  } else if (warp == 3 && scaled) {
+    // ---- scales of the operand rows, a tile ahead of the epilogue (its own loads cost it 2 us a tile: nothing hides their latency there)
     ptx::grid_dep_wait();
     int k = 0;
-    for (int t = blockIdx.x; t < g.tiles; t += gridDim.x, ++k) {
+    for (int t = worker; t < g.tiles; t += workers, ++k) {
       int z, tm, tn;
       tile_of(t, z, tm, tn);
       const int buf = k & 1, n0 = tn * NT, nrows = min(NT, g.R - n0);
-      const int m = tm * tc::BM + w4 * 32 + lane;
-      const bool m_ok = m < g.M;
-      float* inv = s_inv + buf * 256;
-      if (MODE != PF_PREFIX) {
-        for (int n = et; n < nrows; n += EPI_WARPS * 32) {
-          float v = 1.f;
-          if (e.ssq_in != nullptr) {
-            const float* sq = e.ssq_in + (size_t)(n0 + n) * e.ld_ssq;
-            float ss = 0.f;
-            if ((e.ssq_n & 3) == 0) {                        // (one round of wide loads: a scalar loop cost the epilogue 2 000 clocks)
-#pragma unroll 8
-              for (int s = 0; s < e.ssq_n; s += 4) { const float4 q = __ldcg(reinterpret_cast<const float4*>(sq + s)); ss += (q.x + q.y) + (q.z + q.w); }
-            } else {
-              for (int s = 0; s < e.ssq_n; ++s) ss += __ldcg(sq + s);
-            }
-            v = rsqrtf(ss * e.inv_d + e.eps);
+      if (k >= 2 && !wait(inv_empty + buf, ((k >> 1) - 1) & 1)) { failed = true; break; }
+      for (int r0 = 0; r0 < nrows; r0 += 32) {               // eight lanes add the partial sums of a row
+        float ss[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        const float* sq = e.ssq_in + (size_t)(n0 + r0 + (lane >> 3)) * e.ld_ssq;
+        const int rows = nrows - r0 - (lane >> 3);           // (the eight requests of a round travel together)
+        if ((e.ssq_n & 3) == 0) {
+          for (int s0 = 0; s0 < e.ssq_n; s0 += 32) {
+            const int s = s0 + 4 * (lane & 7);
+            float4 q[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              q[i] = 4 * i < rows && s < e.ssq_n ? __ldcg(reinterpret_cast<const float4*>(sq + (size_t)4 * i * e.ld_ssq + s)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ss[i] += (q[i].x + q[i].y) + (q[i].z + q[i].w);
           }
-          inv[n] = v;
-          if (MODE == PF_QKV) s_row[buf][n] = e.rows[n0 + n];
+        } else {
+          for (int s = lane & 7; s < e.ssq_n; s += 8)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ss[i] += 4 * i < rows ? __ldcg(sq + (size_t)4 * i * e.ld_ssq + s) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], 1);
+          ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], 2);
+          ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], 4);
+          if ((lane & 7) == 0) s_inv[buf * 128 + r0 + 4 * i + (lane >> 3)] = rsqrtf(ss[i] * e.inv_d + e.eps);
         }
       }
-      float gain = 1.f;
-      if (MODE == PF_RESID && e.gain != nullptr && m_ok) gain = e.gain[m];
-      // (the barrier also publishes inv; all epilogue threads leave together when a wait ran out)
-      const bool late = !ptx::mbar_wait(acc_full + buf, (k >> 1) & 1);
-      if (epi_sync_or(late)) { if (late) s_fail = 1; break; }
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(inv_full + buf);
+    }
+    if (failed) s_fail = 1;
+  } else if (warp >= 4) {
+    // ---- epilogue: warp w reads tensor-memory lanes 32 (w mod 4) .. + 31 (a feature each); four warps share the rows, CW
+    // at a time.  A warp turns its CW rows x 32 features in a scratch of its own: behind that a lane holds four
+    // neighbouring features of rows tl, tl + 4, .., and everything it reads and writes is 8 or 16 bytes wide.
+    const int w4 = warp & 3, tl = lane >> 3, f4 = 4 * (lane & 7);
+    float* turn = s_turn + (warp - 4) * (CW * 32);
+    ptx::grid_dep_wait();
+    auto release = [&](int buf) {                            // this warp has read its share of the accumulator
+      if (rank == 0) ptx::mbar_arrive(acc_empty + buf);
+      else ptx::mbar_arrive_peer(tc::map_peer(ptx::smem_u32(acc_empty + buf), 0));
+    };
+    int k = 0;
+    for (int t = worker; t < g.tiles; t += workers, ++k) {
+      int z, tm, tn;
+      tile_of(t, z, tm, tn);
+      tm = CG * tm + rank;                                   // this CTA's tile of 128 features
+      const int buf = k & 1, n0 = tn * NT, nrows = min(NT, g.R - n0);
+      const int m = tm * tc::BM + w4 * 32 + f4;              // this lane's features m .. m + 3 (M is a multiple of 4 but for plain stores)
+      const bool m_ok = m < g.M;
+      const int c_first = CW * ((warp - 4) >> 2);
+      // ---- under the tile's MMAs: residual values of the warp's first rows
+      float4 gain = make_float4(1.f, 1.f, 1.f, 1.f);
+      float4 x0[4];                                          // PF_RESID: residual values, PF_QKV: rotary angles of the lane's two pairs
+      Row rw[4];
+      const int dh = e.dm.dh, H = e.dm.H, Hkv = e.dm.Hkv;
+      const int head = MODE == PF_QKV || MODE == PF_PREFIX ? m / dh : 0, f = m - head * dh;       // (the same head for the whole warp: dh is 64 or 128)
+      const bool rotate = MODE == PF_QKV && head < H + Hkv && e.dm.theta != 0.f;
+      auto load_x = [&](float4 (&x)[4], int c0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int n = c0 + tl + 4 * i;
+          x[i] = e.add && n < nrows && m_ok ? __ldcg(reinterpret_cast<const float4*>(e.x + (size_t)(n0 + n) * e.ldx + m)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      };
+      auto load_rows = [&](int c0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) rw[i] = e.rows[min(n0 + c0 + tl + 4 * i, g.R - 1)];
+      };
+      if (MODE == PF_RESID) {
+        if (e.gain != nullptr && m_ok) gain = *reinterpret_cast<const float4*>(e.gain + m);
+        load_x(x0, c_first);
+      }
+      if (MODE == PF_QKV) load_rows(c_first);
+      if (!__all_sync(0xffffffffu, ptx::mbar_wait(acc_full + buf, (k >> 1) & 1))) { s_fail = 1; break; }
       tc::fence_after();
-      const int c_first = (warp >= 8 ? 32 : 0);
-      if (c_first >= nrows && lane == 0) ptx::mbar_arrive(acc_empty + buf);          // nothing to read for this warp
-      for (int c0 = c_first; c0 < nrows; c0 += 64) {
-        uint32_t r[32];
-        float y[32];
-        ld32(tmem + buf * acc_cols + ((uint32_t)(w4 * 32) << 16) + c0, r);
-        if (PARTS == 2) {
-          uint32_t r2[32];
-          ld32(tmem + buf * acc_cols + ((uint32_t)(w4 * 32) << 16) + NT + c0, r2);
-          ld_wait();
+      float inv[2][4];
+      if (scaled) {
+        if (!__all_sync(0xffffffffu, ptx::mbar_wait(inv_full + buf, (k >> 1) & 1))) { s_fail = 1; break; }
 #pragma unroll
-          for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(r[j]) + __uint_as_float(r2[j]);
-        } else {
-          ld_wait();
+        for (int c = 0; c < 2; ++c)
 #pragma unroll
-          for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(r[j]);
+          for (int i = 0; i < 4; ++i) inv[c][i] = s_inv[buf * 128 + ((c_first + c * 4 * CW + tl + 4 * i) & 127)];
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(inv_empty + buf);
+      }
+      if (c_first >= nrows && lane == 0) release(buf);       // nothing to read for this warp
+#pragma unroll 1
+      for (int c0 = c_first; c0 < nrows; c0 += 4 * CW) {
+        if (MODE == PF_QKV) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) x0[i] = rotate ? *reinterpret_cast<const float4*>(e.rope + (size_t)rw[i].p * (dh >> 1) + (f >> 1)) : make_float4(1.f, 0.f, 1.f, 0.f);
         }
-        if (c0 + 64 >= nrows) {                              // this warp's share is in registers
-          tc::fence_before();
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(acc_empty + buf);
-        }
-        const int nv = min(32, nrows - c0);
-        const size_t row = (size_t)(n0 + c0);
-        if (MODE != PF_PREFIX) {
+        {
+          uint32_t r[CW];
+          ld16(tmem + buf * acc_cols + ((uint32_t)(w4 * 32) << 16) + c0, r);
+          if (PARTS == 2) {
+            uint32_t r2[CW];
+            ld16(tmem + buf * acc_cols + ((uint32_t)(w4 * 32) << 16) + NT + c0, r2);
+            ld_wait();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) y[j] *= inv[c0 + j];  // (rows behind nrows: stale scale, never stored)
-        }
-        if (MODE == PF_F32) {
-          float* o = reinterpret_cast<float*>(e.out) + row * e.ldo + m;
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (j < nv && m_ok) o[(size_t)j * e.ldo] = y[j];
-        } else if (MODE == PF_GELU) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) y[j] = tc::gelu_erf_f(y[j]);
-          store_rows_hi_lo(reinterpret_cast<bf16*>(e.out) + row * e.ldo + (m & ~1), e.ldo, e.lo_off, y, nv, m_ok, lane);
-        } else if (MODE == PF_RESID) {
-          float* xr = e.x + row * e.ldx + m;
-          if (e.add) {
-            float x0[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) x0[j] = (j < nv && m_ok) ? __ldcg(xr + (size_t)j * e.ldx) : 0.f;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) y[j] += x0[j];
-          }
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (j < nv && m_ok) xr[(size_t)j * e.ldx] = y[j];
-          if (e.a_out != nullptr) {
-            float v[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = __fmul_rn(y[j], gain);
-            store_rows_hi_lo(e.a_out + row * e.lda + (m & ~1), e.lda, e.lo_off, v, nv, m_ok, lane);
-          }
-          if (e.ssq_out != nullptr) {
-            // sums of squares of 32 rows over the warp's 32 features: lane i ends up with row c0 + i
-#pragma unroll
-            for (int j = 0; j < 32; ++j) y[j] = m_ok ? y[j] * y[j] : 0.f;
-            fold<16>(y, lane); fold<8>(y, lane); fold<4>(y, lane); fold<2>(y, lane); fold<1>(y, lane);
-            if (lane < nv) e.ssq_out[(row + lane) * e.ld_ssq + tm * 4 + w4] = y[0];
-          }
-        } else if (MODE == PF_QKV) {
-          // Q and K heads are stored with their rotary pairs side by side: the partner is the neighbouring lane
-          const int dh = e.dm.dh, H = e.dm.H, Hkv = e.dm.Hkv;
-          const int head = m / dh, i = m - head * dh;        // (the same head for the whole warp: dh is 64 or 128)
-          if (head < H + Hkv && e.dm.theta != 0.f) {
-            const float2* tab = e.rope + (i >> 1);
-            float2 cs[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) cs[j] = j < nv ? tab[(size_t)s_row[buf][c0 + j].p * (dh >> 1)] : make_float2(1.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const float o = __shfl_xor_sync(0xffffffffu, y[j], 1);
-              y[j] = (lane & 1) ? y[j] * cs[j].x + o * cs[j].y : y[j] * cs[j].x - o * cs[j].y;
-            }
-          }
-          if (head < H) {
-            bf16* o = e.q + row * (size_t)(H * dh) + m;
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (j < nv && m_ok) o[(size_t)j * (H * dh)] = __float2bfloat16(y[j] * e.qscale);
+            for (int j = 0; j < CW; ++j) turn[j * 32 + lane] = __uint_as_float(r[j]) + __uint_as_float(r2[j]);
           } else {
-            const bool is_k = head < H + Hkv;
-            const int hk = head - H - (is_k ? 0 : Hkv);
-            if (e.Kc != nullptr) {
-              const size_t slots = e.dm.P + e.dm.cap[e.level];
-              bf16* o = (is_k ? e.Kc : e.Vc) + (hk * slots + e.dm.P) * dh + i;
+            ld_wait();
 #pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                const Row rw = s_row[buf][c0 + j];
-                if (j < nv && m_ok && rw.b >= 0) o[(rw.b * (Hkv * slots) + rw.slot) * dh] = __float2bfloat16(y[j]);
-              }
-            } else {
-              bf16* o = (is_k ? e.kbuf : e.vbuf) + row * (size_t)(Hkv * dh) + hk * dh + i;
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (j < nv && m_ok) o[(size_t)j * (Hkv * dh)] = __float2bfloat16(y[j]);
-            }
-          }
-        } else {  // PF_PREFIX
-          const int dh = e.dm.dh, Hkv = e.dm.Hkv, P = e.dm.P;
-          const LayerPtr L = e.layers[z];
-          const int head = m / dh, i = m - head * dh;
-          const int hk = head < Hkv ? head : head - Hkv;
-          const int slots = P + e.dm.cap[L.level];
-          bf16* dst = (head < Hkv ? L.K : L.V) + i;
-          int b = (e.row_first + (int)row) / P, s = e.row_first + (int)row - b * P;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (j < nv && m_ok) dst[(((size_t)b * Hkv + hk) * slots + s) * dh] = __float2bfloat16(y[j]);
-            if (++s == P) { s = 0; ++b; }
+            for (int j = 0; j < CW; ++j) turn[j * 32 + lane] = __uint_as_float(r[j]);
           }
         }
+        tc::fence_before();
+        __syncwarp();
+        if (c0 + 4 * CW >= nrows && lane == 0) release(buf); // this warp's share has been read
+        const bool more = c0 + 4 * CW < nrows;
+        float4 xn[4];                                        // of the next rows, under the work on these
+        if (MODE == PF_RESID && more) load_x(xn, c0 + 4 * CW);
+        float4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const float4*>(turn + (tl + 4 * i) * 32 + f4);
+        __syncwarp();                                        // the scratch may be written again
+        if (scaled) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float s = c0 == c_first ? inv[0][i] : inv[1][i];
+            v[i].x *= s; v[i].y *= s; v[i].z *= s; v[i].w *= s;
+          }
+        }
+        if (MODE == PF_RESID) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) { v[i].x += x0[i].x; v[i].y += x0[i].y; v[i].z += x0[i].z; v[i].w += x0[i].w; x0[i] = xn[i]; }
+        }
+        int pb = 0, ps = 0;                                  // PF_PREFIX: sequence and prefix slot of the lane's first row
+        if (MODE == PF_PREFIX) { const int r = e.row_first + n0 + c0 + tl; pb = r / e.dm.P; ps = r - pb * e.dm.P; }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int n = c0 + tl + 4 * i;
+          const size_t row = (size_t)(n0 + n);
+          const bool ok = n < nrows && m_ok;
+          if (MODE == PF_F32) {
+            float* o = reinterpret_cast<float*>(e.out) + row * e.ldo + m;
+            if (ok && m + 3 < g.M) *reinterpret_cast<float4*>(o) = v[i];
+            else if (ok) {                                   // the last columns of a width that is not a multiple of 4
+              o[0] = v[i].x;
+              if (m + 1 < g.M) o[1] = v[i].y;
+              if (m + 2 < g.M) o[2] = v[i].z;
+            }
+          } else if (MODE == PF_GELU) {
+            const float2 a = tc::gelu2(v[i].x, v[i].y), b = tc::gelu2(v[i].z, v[i].w);
+            if (ok) store_hi_lo4(reinterpret_cast<bf16*>(e.out) + row * e.ldo + m, a.x, a.y, b.x, b.y, e.lo_off);
+          } else if (MODE == PF_RESID) {
+            if (ok) {
+              *reinterpret_cast<float4*>(e.x + row * e.ldx + m) = v[i];
+              if (e.a_out != nullptr)
+                store_hi_lo4(e.a_out + row * e.lda + m, __fmul_rn(v[i].x, gain.x), __fmul_rn(v[i].y, gain.y), __fmul_rn(v[i].z, gain.z),
+                             __fmul_rn(v[i].w, gain.w), e.lo_off);
+            }
+            if (e.ssq_out != nullptr) {                      // sum of squares over the warp's 32 features
+              float ss = m_ok ? (v[i].x * v[i].x + v[i].y * v[i].y) + (v[i].z * v[i].z + v[i].w * v[i].w) : 0.f;
+              ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+              ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+              ss += __shfl_xor_sync(0xffffffffu, ss, 4);
+              if (f4 == 0 && n < nrows && tm < g.w_tiles) e.ssq_out[row * e.ld_ssq + tm * 4 + w4] = ss;
+            }
+          } else if (MODE == PF_QKV) {
+            // Q and K heads are stored with their rotary pairs side by side
+            const float4 cs = x0[i];
+            float4 y = v[i];
+            if (rotate) y = make_float4(v[i].x * cs.x - v[i].y * cs.y, v[i].y * cs.x + v[i].x * cs.y, v[i].z * cs.z - v[i].w * cs.w, v[i].w * cs.z + v[i].z * cs.w);
+            bf16* o;
+            bool there = ok;
+            if (head < H) {
+              o = e.q + row * (size_t)(H * dh) + m;
+              y.x *= e.qscale; y.y *= e.qscale; y.z *= e.qscale; y.w *= e.qscale;
+            } else {
+              const bool is_k = head < H + Hkv;
+              const int hk = head - H - (is_k ? 0 : Hkv);
+              if (e.Kc == nullptr) o = (is_k ? e.kbuf : e.vbuf) + row * (size_t)(Hkv * dh) + hk * dh + f;
+              else {
+                there = ok && rw[i].b >= 0;
+                o = (is_k ? e.Kc : e.Vc) + (size_t)((rw[i].b * Hkv + hk) * (e.dm.P + e.dm.cap[e.level]) + e.dm.P + rw[i].slot) * dh + f;
+              }
+            }
+            if (there) *reinterpret_cast<uint2*>(o) = make_uint2(ptx::pack_bf16(y.x, y.y), ptx::pack_bf16(y.z, y.w));
+          } else {  // PF_PREFIX
+            const LayerPtr& L = e.layers[z];
+            bf16* o = (head < Hkv ? L.K : L.V) + (size_t)((pb * Hkv + (head < Hkv ? head : head - Hkv)) * (e.dm.P + e.dm.cap[L.level]) + ps) * dh + f;
+            if (ok) *reinterpret_cast<uint2*>(o) = make_uint2(ptx::pack_bf16(v[i].x, v[i].y), ptx::pack_bf16(v[i].z, v[i].w));
+            for (ps += 4; ps >= e.dm.P; ps -= e.dm.P) ++pb;
+          }
+        }
+        if (MODE == PF_QKV && more) load_rows(c0 + 4 * CW);
       }
     }
   }
@@ -371,7 +483,11 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
     if (tid == 0) atomicExch(g.status, -5);
     ptx::drain_delay();                                      // stages already requested may still be landing
   }
-  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+  if (CG == 2) {                                             // the pair's MMAs read this CTA's shared memory
+    tc::cluster_sync();
+    tc::fence_after();
+  }
+  if (warp == 1) tmem_free<CG>(tmem, ncols);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -895,7 +1011,7 @@ __global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, c
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_full + 1);
   __shared__ int s_fail;
   const Dims& dm = a.dm;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)ptx::uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int h = blockIdx.x, hk = h / (dm.H / dm.Hkv), level = a.level;
   const int2 tile = a.tiles[blockIdx.y];
   const Seg& sg = a.segs[tile.x];
@@ -922,10 +1038,12 @@ __global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, c
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  const uint32_t tmem = *tmem_slot, tO = tmem + 128, tP = tmem + 192;        // S in columns 0..127, then O, then P
+  const uint32_t tmem = ptx::uniform(*tmem_slot), tO = tmem + 128, tP = tmem + 192;        // S in columns 0..127, then O, then P
   ptx::grid_dep_launch();
-  if (warp == 0 && lane == 0) {
+  auto wait = [](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity)) != 0; };
+  if (warp == 0) {
     auto issue = [&](int i) {
+      if (!ptx::elect_one()) return;
       const int st = i % STAGES;
       const bool old = i < n_old, cached = old || a.tmKn == nullptr;
       const int row = !cached ? r0 + (tn0 + i - n_old) * C
@@ -938,42 +1056,48 @@ __global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, c
     const int pre = min(n_old, STAGES);                      // as in attn_kernel: old entries before the dependency wait
     for (int i = 0; i < pre; ++i) issue(i);
     ptx::grid_dep_wait();
-    ptx::mbar_expect_tx(q_full, TILE);
-    ptx::tma_load_2d(sm, tmQ, h * DH, r0 + q0, q_full);
+    if (ptx::elect_one()) {
+      ptx::mbar_expect_tx(q_full, TILE);
+      ptx::tma_load_2d(sm, tmQ, h * DH, r0 + q0, q_full);
+    }
     for (int i = pre; i < n_tiles; ++i) {
-      if (i >= STAGES && !ptx::mbar_wait(empty + i % STAGES, ((i / STAGES) - 1) & 1)) { s_fail = 1; break; }
+      if (i >= STAGES && !wait(empty + i % STAGES, ((i / STAGES) - 1) & 1)) { s_fail = 1; break; }
       issue(i);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     const uint32_t id_s = tc::instr_desc_bf16(128), id_o = tc::instr_desc_bf16(DH) | (1u << 16);       // B of P V is MN-major
     const uint64_t dq = tc::smem_desc_sw128(ptx::smem_u32(sm));
-    bool ok = ptx::mbar_wait(q_full, 0);
+    bool ok = wait(q_full, 0);
     auto scores = [&](int i) {
       const int st = i % STAGES;
-      if (!ptx::mbar_wait(full + st, (i / STAGES) & 1)) return false;
+      if (!wait(full + st, (i / STAGES) & 1)) return false;
       tc::fence_after();
       const uint64_t dk = tc::smem_desc_sw128(ptx::smem_u32(ring + st * STAGE));
+      if (ptx::elect_one()) {
 #pragma unroll
-      for (int k = 0; k < DH / 16; ++k) tc::mma_ss(tmem, dq + 2 * k, dk + 2 * k, id_s, k > 0 ? 1u : 0u);
-      tc::commit(s_full);
+        for (int k = 0; k < DH / 16; ++k) tc::mma_ss(tmem, dq + 2 * k, dk + 2 * k, id_s, k > 0 ? 1u : 0u);
+        tc::commit(s_full);
+      }
       return true;
     };
     ok = ok && scores(0);
     for (int i = 0; i < n_tiles && ok; ++i) {
-      if (!(ok = ptx::mbar_wait(s_read, i & 1))) break;
+      if (!(ok = wait(s_read, i & 1))) break;
       if (i + 1 < n_tiles && !(ok = scores(i + 1))) break;
-      if (!(ok = ptx::mbar_wait(p_full, i & 1))) break;
+      if (!(ok = wait(p_full, i & 1))) break;
       tc::fence_after();
       const uint64_t dv = tc::smem_desc_sw128(ptx::smem_u32(ring + (i % STAGES) * STAGE + TILE));
+      if (ptx::elect_one()) {
 #pragma unroll
-      for (int k = 0; k < C / 16; ++k) mma_ts(tO, tP + 8 * k, dv + 128 * k, id_o, (i > 0 || k > 0) ? 1u : 0u);
-      tc::commit(empty + i % STAGES);
-      tc::commit(o_full);
+        for (int k = 0; k < C / 16; ++k) mma_ts(tO, tP + 8 * k, dv + 128 * k, id_o, (i > 0 || k > 0) ? 1u : 0u);
+        tc::commit(empty + i % STAGES);
+        tc::commit(o_full);
+      }
     }
     if (!ok) {
       s_fail = 1;
-      tc::commit(q_full);                                    // what was issued ends before the CTA does
-      ptx::mbar_wait(q_full, 1);
+      if (ptx::elect_one()) tc::commit(q_full);              // what was issued ends before the CTA does
+      wait(q_full, 1);
     }
   } else if (warp >= 2) {
     // ---- softmax: warps w and w + 4 share 32 query rows, 64 of a tile's keys each

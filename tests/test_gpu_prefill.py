@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
     ((90, 20), (0, 0, 0), {"n_heads": 1, "n_kv_heads": 1, "head_dim": 128}),
     ((60,), (20, 9, 0), {"n_heads": 1, "n_kv_heads": 1, "head_dim": 128}),
     ((35, 2), (0, 0, 0), {"d_model": 192, "d_ff": 320}),              # partly empty last tiles
+    ((61, 2), (0, 0, 0), {"d_model": 384, "n_heads": 6, "n_kv_heads": 1, "d_ff": 320}),      # pairs of feature tiles: an odd number, a last one half empty
+    ((143, 1), (0, 0, 0), {"d_model": 640, "n_heads": 10, "n_kv_heads": 10, "d_ff": 704, "weight_std": 0.04}),
     ((143,), (0, 0, 0), {"n_heads": 16, "n_kv_heads": 16}),           # 128 query rows per CTA: 10 tiles and 8 rows more
     ((160, 3), (600, 0, 0), {"n_heads": 16, "n_kv_heads": 2}),        # the same with a ring shorter than the prompt, shared heads
     ((950,), (700, 0, 0), {"n_heads": 16, "n_kv_heads": 16}),         # ... and in two chunks
