@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, NW, ST>::THREADS, AttnCfg<DH, C
   const int hk = a.MT == 1 ? (int)blockIdx.y : (int)blockIdx.y / a.MT;
   const int mt = (int)blockIdx.y - hk * a.MT;
   const int b = blockIdx.z;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
+  const int warp = (int)ptx::uniform(threadIdx.x >> 5), lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
   ptx::grid_dep_launch();
   // ---- what this CTA has to do (per-pass state is final before the pass's first kernel starts)
   const AttnWork w = attn_work(a, b, C);
@@ -134,7 +134,6 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, NW, ST>::THREADS, AttnCfg<DH, C
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + CF::RING);
   uint64_t* empty = full + CF::STAGES;
   int& s_fail = *reinterpret_cast<int*>(empty + CF::STAGES);   // (no static shared memory: the ring must start at a 1024-byte boundary)
-  int& s_pre = *(&s_fail + 1);
 
   // slots written by this pass: P + (p mod cap), p = p0..p_max: one run of nq slots from new_lo,
   // which may wrap around the end of the ring once
@@ -148,6 +147,7 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, NW, ST>::THREADS, AttnCfg<DH, C
   };
   const int row_base = (b * dm.Hkv + hk) * slots;
   auto issue = [&](int i) {
+    if (!ptx::elect_one()) return;                           // one lane of the producer warp, which stays in step
     const int st = i % CF::STAGES;
     unsigned char* Ks = sm + st * CF::STAGE;
     unsigned char* Vs = Ks + CF::TILE;
@@ -159,15 +159,17 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, NW, ST>::THREADS, AttnCfg<DH, C
       ptx::tma_load_2d(Vs + h * C * 128, a.tmV, h * 64, row0, full + st);
     }
   };
-  if (threadIdx.x == 0) {
-    s_fail = 0;
-    for (int i = 0; i < CF::STAGES; ++i) { ptx::mbar_init(full + i, 1); ptx::mbar_init(empty + i, NW); }
-    ptx::fence_mbar_init();
+  int n_pre = 0;                                             // producer: chunks requested
+  if (warp == NW) {
+    if (lane == 0) {
+      s_fail = 0;
+      for (int i = 0; i < CF::STAGES; ++i) { ptx::mbar_init(full + i, 1); ptx::mbar_init(empty + i, NW); }
+      ptx::fence_mbar_init();
+    }
+    __syncwarp();
     // chunks that hold old entries only are requested at once, before the dependency wait
-    int i = 0;
     const int pre = n_my < CF::STAGES ? n_my : CF::STAGES;
-    while (i < pre && !has_new(u + i * NG)) { issue(i); ++i; }
-    s_pre = i;
+    while (n_pre < pre && !has_new(u + n_pre * NG)) { issue(n_pre); __syncwarp(); ++n_pre; }
   }
   __syncthreads();
 
@@ -179,14 +181,12 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, NW, ST>::THREADS, AttnCfg<DH, C
 
   if (warp == NW) {
     // ---- producer
-    if (lane == 0) {
-      ptx::grid_dep_wait();
-      for (int i = s_pre; i < n_my; ++i) {
-        if (i >= CF::STAGES && !ptx::mbar_wait(empty + i % CF::STAGES, ((i / CF::STAGES) - 1) & 1)) { s_fail = 1; break; }
-        issue(i);
-      }
+    ptx::grid_dep_wait();
+    for (int i = n_pre; i < n_my; ++i) {
+      if (i >= CF::STAGES && !__all_sync(0xffffffffu, ptx::mbar_wait(empty + i % CF::STAGES, ((i / CF::STAGES) - 1) & 1))) { s_fail = 1; break; }
+      issue(i);
+      __syncwarp();
     }
-    __syncwarp();
   } else {
     // ---- compute warps
     ptx::grid_dep_wait();                          // queries come from the previous kernel

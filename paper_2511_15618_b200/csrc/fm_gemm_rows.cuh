@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
   __shared__ float s_inv[MAX_ROWS];
   __shared__ int s_rb[MAX_ROWS], s_rp[MAX_ROWS], s_ra[MAX_ROWS], s_rl[MAX_ROWS];
   __shared__ int s_carry[CARRY_MAX], s_ncarry;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
+  const int tid = threadIdx.x, warp = (int)ptx::uniform(tid >> 5), lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
   const int f0 = blockIdx.x * FT, slabs = g.K / BK, R = g.R;
   const int row0 = e.row0 + (int)blockIdx.y * g.z_rows;      // first output row
   if (tid == 0) {
@@ -82,7 +82,9 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
   if (warp == 0) {
     __syncwarp();
     const bf16* src = g.W + ((size_t)(g.w_tile0 + (int)blockIdx.y * g.z_w_tiles + f0 / BM) * slabs * BM + f0 % BM) * BK;
-    for (int s = lane; s < slabs; s += 32) ptx::bulk_load(sm + s * FT * 128, src + (size_t)s * (BM * BK), FT * 128, &full);
+    if (ptx::elect_one())                                    // (one lane of a warp in step: the copies' operands stay in uniform registers)
+      for (int s = 0; s < slabs; ++s) ptx::bulk_load(sm + s * FT * 128, src + (size_t)s * (BM * BK), FT * 128, &full);
+    __syncwarp();
   }
   ptx::grid_dep_launch();
   // ---- what does not depend on the previous kernel: row maps (positions are per-pass state), the first item's gain and angle

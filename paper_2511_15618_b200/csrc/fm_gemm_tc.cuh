@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   __shared__ int s_ra[ROWS_AUX], s_rl[ROWS_AUX];             // EPI_RESID_CAT / EPI_UP: see the row maps below
   __shared__ int s_carry[CARRY_MAX], s_ncarry;               // EPI_UP: child rows whose parent is not in this pass
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = (int)ptx::uniform(tid >> 5), lane = tid & 31;
   const int tile_m = blockIdx.x;
   // token rows of this CTA: N tile blockIdx.z of the launch's rows
   const int row_lo = (int)blockIdx.z * (g.z_rows > 0 ? g.z_rows : g.N);
@@ -290,33 +290,40 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   const int row0 = e.row0 + row_lo;                        // first output row
   const int a_row = g.a_row0 + row_lo;                     // first operand row
   const int S = g.split;
-  const int z = (int)cluster_rank();                 // == blockIdx.y: the cluster spans the grid's y extent
+  const int z = (int)ptx::uniform(cluster_rank());   // == blockIdx.y: the cluster spans the grid's y extent
   const int slabs = g.K / BK;
   const int s0 = (int)((long long)slabs * z / S), s1 = (int)((long long)slabs * (z + 1) / S);
   const int n_slabs = s1 - s0;
   uint32_t ncols = 32;
   while ((int)ncols < g.a_parts * g.N) ncols <<= 1;
 
-  if (tid == 0) {
-    s_fail = 0;
-    for (int i = 0; i < STAGES; ++i) { ptx::mbar_init(full + i, 1); ptx::mbar_init(empty + i, 1); }
-    ptx::mbar_init(accum, 1);
-    ptx::mbar_init(rbar, 1);
-    ptx::mbar_init(sbar, 1);
-    ptx::fence_mbar_init();
-    // rows are sent in groups of 16: groups x 16 rows x 128/S columns x S ranks x 4 bytes
-    ptx::mbar_expect_tx(rbar, (uint32_t)((ns + 15) / 16) * 16u * 512u);
-    ptx::prefetch_tmap(g.tmA);
+  // (Copies and MMAs are issued by one elected lane of a warp that stays in step: behind `lane == 0` their operands go from
+  // general to uniform registers one instruction at a time, a slab's four MMAs then take 900 clocks to issue.)
+  if (warp == 0) {
+    if (lane == 0) {
+      s_fail = 0;
+      for (int i = 0; i < STAGES; ++i) { ptx::mbar_init(full + i, 1); ptx::mbar_init(empty + i, 1); }
+      ptx::mbar_init(accum, 1);
+      ptx::mbar_init(rbar, 1);
+      ptx::mbar_init(sbar, 1);
+      ptx::fence_mbar_init();
+      // rows are sent in groups of 16: groups x 16 rows x 128/S columns x S ranks x 4 bytes
+      ptx::mbar_expect_tx(rbar, (uint32_t)((ns + 15) / 16) * 16u * 512u);
+    }
+    __syncwarp();
     // The weight slabs of the first stages do not depend on the previous kernel: request them at
     // once, so that they travel while the rest of the prologue runs.
     const bf16* wsrc = g.W + ((size_t)(w_tile + tile_m) * slabs + s0) * (BM * BK);
     const int pre = n_slabs < STAGES ? n_slabs : STAGES;
-    for (int i = 0; i < pre; ++i) {
-      ptx::mbar_expect_tx(full + i, BM * 128 + g.a_parts * g.N * 128);
-      ptx::bulk_load(sm + i * stage_bytes, wsrc + (size_t)i * (BM * BK), BM * 128, full + i);
+    if (ptx::elect_one()) {
+      for (int i = 0; i < pre; ++i) {
+        ptx::mbar_expect_tx(full + i, BM * 128 + g.a_parts * g.N * 128);
+        ptx::bulk_load(sm + i * stage_bytes, wsrc + (size_t)i * (BM * BK), BM * 128, full + i);
+      }
+      ptx::prefetch_tmap(g.tmA);
     }
-  }
-  if (warp == 0) {
+    __syncwarp();
+  } else if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(tmem_slot)), "r"(ncols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -324,7 +331,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = ptx::uniform(*tmem_slot);
   // This CTA now holds its tensor memory and shared memory: the next kernel may start its own
   // prologue beside us.
   ptx::grid_dep_launch();
@@ -346,35 +353,41 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     // copy per slab brings the hi and the lo tile; lanes issue them side by side
     const int pre = n_slabs < STAGES ? n_slabs : STAGES;
     ptx::grid_dep_wait();
-    if (lane < pre) ptx::tma_load_3d(sm + lane * stage_bytes + BM * 128, g.tmA, (s0 + lane) * BK, a_row, 0, full + lane);
-  }
-  if (warp == 0 && lane == 0) {
+    if (ptx::elect_one())
+      for (int i = 0; i < pre; ++i) ptx::tma_load_3d(sm + i * stage_bytes + BM * 128, g.tmA, (s0 + i) * BK, a_row, 0, full + i);
+    __syncwarp();
     // ---- producer: stream the rest of this CTA's K range through the stage ring
     const bf16* wsrc = g.W + ((size_t)(w_tile + tile_m) * slabs + s0) * (BM * BK);
-    const int pre = n_slabs < STAGES ? n_slabs : STAGES;
-    for (int i = pre; i < n_slabs; ++i) {
-      const int st = i % STAGES;
-      if (!ptx::mbar_wait(empty + st, ((i / STAGES) - 1) & 1)) { s_fail = 1; break; }
-      unsigned char* a_dst = sm + st * stage_bytes;
-      ptx::mbar_expect_tx(full + st, BM * 128 + g.a_parts * g.N * 128);
-      ptx::bulk_load(a_dst, wsrc + (size_t)i * (BM * BK), BM * 128, full + st);
-      ptx::tma_load_3d(a_dst + BM * 128, g.tmA, (s0 + i) * BK, a_row, 0, full + st);
+    for (int i = pre, st = 0, round = 0; i < n_slabs; ++i) {           // (pre == STAGES here)
+      if (!__all_sync(0xffffffffu, ptx::mbar_wait(empty + st, round & 1))) { s_fail = 1; break; }
+      if (ptx::elect_one()) {
+        unsigned char* a_dst = sm + st * stage_bytes;
+        ptx::mbar_expect_tx(full + st, BM * 128 + g.a_parts * g.N * 128);
+        ptx::bulk_load(a_dst, wsrc + (size_t)i * (BM * BK), BM * 128, full + st);
+        ptx::tma_load_3d(a_dst + BM * 128, g.tmA, (s0 + i) * BK, a_row, 0, full + st);
+      }
+      __syncwarp();
+      if (++st == STAGES) { st = 0; ++round; }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---- MMA issuer
     const uint32_t idesc = instr_desc_bf16(g.a_parts * g.N);   // hi and lo tiles: one operand of 2N rows
-    for (int i = 0; i < n_slabs; ++i) {
-      const int st = i % STAGES;
-      if (!ptx::mbar_wait(full + st, (i / STAGES) & 1)) { s_fail = 1; break; }
+    for (int i = 0, st = 0, round = 0; i < n_slabs; ++i) {
+      if (!__all_sync(0xffffffffu, ptx::mbar_wait(full + st, round & 1))) { s_fail = 1; break; }
       fence_after();
       const uint32_t a_addr = ptx::smem_u32(sm + st * stage_bytes);
-      const uint64_t da = smem_desc_sw128(a_addr), db = smem_desc_sw128(a_addr + BM * 128);
+      if (ptx::elect_one()) {
+        const uint64_t da = smem_desc_sw128(a_addr), db = smem_desc_sw128(a_addr + BM * 128);
 #pragma unroll
-      for (int k = 0; k < BK / 16; ++k)                    // +32 bytes along K per step (encoded >> 4)
-        mma_ss(tmem, da + 2 * k, db + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
-      commit(empty + st);                                  // stage reusable once these MMAs retire
+        for (int k = 0; k < BK / 16; ++k)                  // +32 bytes along K per step (encoded >> 4)
+          mma_ss(tmem, da + 2 * k, db + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
+        commit(empty + st);                                // stage reusable once these MMAs retire
+      }
+      __syncwarp();
+      if (++st == STAGES) { st = 0; ++round; }
     }
-    commit(accum);                                         // accumulator complete
+    if (ptx::elect_one()) commit(accum);                   // accumulator complete
+    __syncwarp();
   }
   else if (warp >= 2) {
     // ---- warps 2 and 3, while the operands arrive: operand-row scales (the partial sums of
@@ -424,8 +437,9 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
       const int cols = min(BM, g.M - tile_m * BM);
       if (lane == 0) ptx::mbar_expect_tx(sbar, (uint32_t)(ns * cols) * 4u);
       __syncwarp();
-      for (int n = lane; n < ns; n += 32)
-        ptx::bulk_load(side + n * 128, e.x + (size_t)(row0 + n) * e.ldx + tile_m * BM, (uint32_t)cols * 4u, sbar);
+      if (ptx::elect_one())
+        for (int n = 0; n < ns; ++n) ptx::bulk_load(side + n * 128, e.x + (size_t)(row0 + n) * e.ldx + tile_m * BM, (uint32_t)cols * 4u, sbar);
+      __syncwarp();
     }
     const int t = tid - 64;
     if (e.ssq_in != nullptr) {
