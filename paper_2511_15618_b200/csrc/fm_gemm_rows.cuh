@@ -178,6 +178,9 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
 #pragma unroll
     for (int j = 0; j < FJ; ++j) acc[mt][j][0] = acc[mt][j][1] = acc[mt][j][2] = acc[mt][j][3] = 0.f;
   const bool ok = ptx::mbar_wait(&full, 0);
+  // MMA column q takes feature q / 2 + 4 (q mod 2) of its eight: the two features that eight lanes read together then lie in
+  // different halves of the swizzled 128 bytes (in order, every such read took two passes over the banks).
+  const int fq = (gq >> 1) | ((gq & 1) << 2);
   auto block = [&](int buf, int kb) {
 #pragma unroll
     for (int c = 0; c < CB; ++c) {
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
       const int k = kb + c;
       uint4 w[FJ];
 #pragma unroll
-      for (int j = 0; j < FJ; ++j) w[j] = *reinterpret_cast<const uint4*>(sm + ((k >> 1) * FT + j * 8 + gq) * 128 + (((4 * (k & 1) + t4) ^ gq) << 4));
+      for (int j = 0; j < FJ; ++j) w[j] = *reinterpret_cast<const uint4*>(sm + ((k >> 1) * FT + j * 8 + fq) * 128 + (((4 * (k & 1) + t4) ^ fq) << 4));
 #pragma unroll
       for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -209,9 +212,9 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
   for (int mt = 0; mt < MTN; ++mt)
 #pragma unroll
     for (int j = 0; j < FJ; ++j) {
-      float* p = red + ((warp * MTN + mt) * 16 + gq) * S + j * 8 + 2 * t4;
-      *reinterpret_cast<float2*>(p) = make_float2(acc[mt][j][0], acc[mt][j][1]);
-      *reinterpret_cast<float2*>(p + 8 * S) = make_float2(acc[mt][j][2], acc[mt][j][3]);
+      float* p = red + ((warp * MTN + mt) * 16 + gq) * S + j * 8 + t4;        // MMA columns 2 t4 and 2 t4 + 1
+      p[0] = acc[mt][j][0]; p[4] = acc[mt][j][1];
+      p[8 * S] = acc[mt][j][2]; p[8 * S + 4] = acc[mt][j][3];
     }
   __syncthreads();
   if (!ok && tid == 0) atomicExch(g.status, -5);
