@@ -148,11 +148,9 @@ __device__ inline uint32_t cluster_rank() {
 __device__ inline void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// 16-byte store into a peer CTA's shared memory that reports its bytes to an mbarrier of that CTA
-__device__ inline void st_async_peer4(uint32_t remote_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t remote_bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(remote_addr),
-               "r"(a), "r"(b), "r"(c), "r"(d), "r"(remote_bar)
-               : "memory");
+// 4-byte store into a peer CTA's shared memory that reports its bytes to an mbarrier of that CTA
+__device__ inline void st_async_peer(uint32_t remote_addr, uint32_t a, uint32_t remote_bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(remote_addr), "r"(a), "r"(remote_bar) : "memory");
 }
 __device__ inline bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
@@ -179,9 +177,8 @@ __device__ inline uint32_t map_peer(uint32_t local_addr, uint32_t rank) {
 }
 
 // Shared memory: ring of `stages` x ([128 x 64] weight slab + [N x 64] operand slab), then the
-// receive buffer of the cluster reduction [split][64/split][2][N + 4] fp32 = (N + 4) * 512 bytes
-// (peers write into it while this CTA may still be multiplying, so it never aliases the ring;
-// the 4 floats of padding spread the readers over the banks), then the side rows [N][512 bytes]
+// receive buffer of the cluster reduction [split][N][128/split] fp32 = N * 512 bytes
+// (peers write into it while this CTA may still be multiplying, so it never aliases the ring), then the side rows [N][512 bytes]
 // (what the epilogue reads per row besides the product: the residual rows of the tile's 128
 // columns, or the rows' rotary angles; brought in by bulk copies while the MMAs run), then barriers.
 inline int stage_bytes(int N, int parts) { return BM * 128 + parts * (((N * 128 + 1023) / 1024) * 1024); }
@@ -192,13 +189,13 @@ __host__ __device__ inline int side_bytes(int N, int split) { return N * (64 / s
 // as many stages as the CTA has slabs (its whole K range is then requested at once), at most 8
 // and what fits beside the receive buffer
 inline int pick_stages(int N, int n_slabs, int parts, int side_b) {
-  int st = (200 * 1024 - (N + 4) * 512 - side_b) / stage_bytes(N, parts);
+  int st = (200 * 1024 - N * 512 - side_b) / stage_bytes(N, parts);
   st = st > MAX_STAGES ? MAX_STAGES : st;
   st = st > n_slabs ? n_slabs : st;
   return st < 2 ? 2 : st;
 }
 inline int smem_bytes(int N, int stages, int parts, int side_b) {
-  return stages * stage_bytes(N, parts) + (N + 4) * 512 + side_b + 1024 + 256;
+  return stages * stage_bytes(N, parts) + N * 512 + side_b + 1024 + 256;
 }
 
 inline int max_smem_bytes() {
@@ -266,10 +263,9 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   const int STAGES = g.stages;
   const int b_bytes = ((g.N * 128 + 1023) / 1024) * 1024;
   const int stage_bytes = BM * 128 + g.a_parts * b_bytes;
-  const int NP = g.N + 4;
-  float* recv = reinterpret_cast<float*>(sm + STAGES * stage_bytes);          // [S][PW][2][NP]
-  float* side = recv + NP * 128;                                              // [N][128] fp32 (or [N][64] float2)
-  uint64_t* full = reinterpret_cast<uint64_t*>(sm + STAGES * stage_bytes + NP * 512 + (SIDE ? g.N * 512 : 0));
+  float* recv = reinterpret_cast<float*>(sm + STAGES * stage_bytes);          // [S][N][128 / S]
+  float* side = recv + g.N * 128;                                             // [N][128] fp32 (or [N][64] float2)
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + STAGES * stage_bytes + g.N * 512 + (SIDE ? g.N * 512 : 0));
   uint64_t* empty = full + MAX_STAGES;
   uint64_t* accum = empty + MAX_STAGES;
   uint64_t* rbar = accum + 1;                                                 // partials of all ranks have arrived
@@ -307,8 +303,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
       ptx::mbar_init(rbar, 1);
       ptx::mbar_init(sbar, 1);
       ptx::fence_mbar_init();
-      // rows are sent in groups of 16: groups x 16 rows x 128/S columns x S ranks x 4 bytes
-      ptx::mbar_expect_tx(rbar, (uint32_t)((ns + 15) / 16) * 16u * 512u);
+      ptx::mbar_expect_tx(rbar, (uint32_t)ns * 512u);        // rows x 128/S columns x S ranks x 4 bytes
     }
     __syncwarp();
     // The weight slabs of the first stages do not depend on the previous kernel: request them at
@@ -469,22 +464,20 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   __syncwarp();
 
   // ---- where this thread's accumulator column goes, and its first item of the epilogue.  Column
-  // m of the tile is half h of pair slot q; slots [r*PW, (r+1)*PW) belong to rank r, which receives
-  // [source rank][slot][half][row].  Everything that does not depend on the previous kernel
+  // m of the tile is half of pair slot m / 2; slots [r*PW, (r+1)*PW) belong to rank r, which receives
+  // [source rank][row][column]: a row's columns of a warp travel together (128 bytes at a split of up to 4; 16 bytes of a
+  // column's rows at a time took 1.3 us for 32 rows).  Everything that does not depend on the previous kernel
   // (indices, gains, rotary angles) is prepared here, before the wait.
   const int lgS = 31 - __clz(S);                           // S is 1, 2, 4 or 8
   const int lgPW = 6 - lgS, PW = 1 << lgPW;
   const int items = ns * PW;
   uint32_t dst0 = 0, dbar = 0;
-  float* recv_own;                                         // S == 1: this thread's row run in the local buffer
-  {
-    const int q = tid >> 1, h = tid & 1;
-    const int owner = q >> lgPW, cc = q & (PW - 1);
-    recv_own = recv + (((size_t)z * PW + cc) * 2 + h) * NP;
-    if (S > 1) {
-      dst0 = map_peer(ptx::smem_u32(recv_own), (uint32_t)owner);
-      dbar = map_peer(ptx::smem_u32(rbar), (uint32_t)owner);
-    }
+  const int CW = 2 << lgPW;                                // columns a rank owns
+  float* recv_own = recv + z * g.N * CW + (tid & (CW - 1));  // this thread's column of row 0
+  if (S > 1) {
+    const uint32_t owner = (uint32_t)(tid >> (lgPW + 1));
+    dst0 = map_peer(ptx::smem_u32(recv_own), owner);
+    dbar = map_peer(ptx::smem_u32(rbar), owner);
   }
   // A thread keeps its pair slot in every item (items advance by 128, a multiple of PW): its two
   // columns, and with them the gains, are fixed.
@@ -568,11 +561,11 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     }
     if (S > 1) {
 #pragma unroll
-      for (int j = 0; j < 16; j += 4) st_async_peer4(dst0 + (uint32_t)(n0 + j) * 4u, r[j], r[j + 1], r[j + 2], r[j + 3], dbar);
+      for (int j = 0; j < 16; ++j)
+        if (n0 + j < k_ns) st_async_peer(dst0 + (uint32_t)((n0 + j) * CW) * 4u, r[j], dbar);
     } else {                                               // no split: the tile stays in this CTA
 #pragma unroll
-      for (int j = 0; j < 16; j += 4)
-        *reinterpret_cast<uint4*>(recv_own + n0 + j) = make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
+      for (int j = 0; j < 16; ++j) recv_own[(n0 + j) * CW] = __uint_as_float(r[j]);
     }
   }
   bool arrived = true;
@@ -589,17 +582,14 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     const bool active = it < items, first = it0 == 0;
     const int n = active ? it >> lgPW : 0, cc = active ? it & (PW - 1) : 0;
     const int ca = 2 * (z * PW + cc);
-    float va[MAX_SPLIT], vb[MAX_SPLIT];
+    float2 v[MAX_SPLIT];
 #pragma unroll
-    for (int r = 0; r < MAX_SPLIT; ++r) {                  // all loads first, then the sums in rank order
-      const float* src = recv + ((r << lgPW) + cc) * 2 * NP + n;
-      va[r] = (r < S && active) ? src[0] : 0.f;
-      vb[r] = (r < S && active) ? src[NP] : 0.f;
-    }
+    for (int r = 0; r < MAX_SPLIT; ++r)                    // all loads first, then the sums in rank order
+      v[r] = (r < S && active) ? *reinterpret_cast<const float2*>(recv + (r * g.N + n) * CW + 2 * cc) : make_float2(0.f, 0.f);
     float ya = 0.f, yb = 0.f;
 #pragma unroll
     for (int r = 0; r < MAX_SPLIT; ++r)
-      if (r < S) { ya += va[r]; yb += vb[r]; }
+      if (r < S) { ya += v[r].x; yb += v[r].y; }
     const float inv = s_inv[n];
     ya *= inv;
     yb *= inv;
