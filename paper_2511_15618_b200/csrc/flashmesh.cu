@@ -709,7 +709,7 @@ void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_ro
   const auto [tiles, slabs, N, n_tiles, split] = split_cut(c, M, K, R, stacked);
   const int tA = tmap_for(c, A, a_rows_alloc, (uint64_t)K, N, (uint32_t)a_parts);
   if (tA < 0) { c->launch_error = FM_ERR_CUDA; return; }
-  // only the residual and the QKV epilogue have side rows, and only when a thread gets more than two items
+  // only the residual and the QKV epilogue have side rows, and only when a thread gets more than one item
   const bool side = (mode == tc::EPI_RESID || mode == tc::EPI_QKV) && tc::side_bytes(N, split) > 0;
   const int side_b = side ? tc::side_bytes(N, split) : 0;
   int stages = tc::pick_stages(N, (slabs + split - 1) / split, a_parts, side_b);
@@ -738,8 +738,8 @@ void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_ro
       else launch_pdl(c, cl, tc::gemm_tc_kernel<tc::EPI_QKV, false>, grid, 128, smem, g, e);
       break;
   }
-  if ((mode == tc::EPI_RESID || mode == tc::EPI_RESID_CAT) && e.ssq_out != nullptr) c->ssq_n = tiles * split * (split == 1 ? 2 : 1);     // slots the next consumer adds
-  if (mode == tc::EPI_UP && e.ssq_out != nullptr) c->ssq_n = (c->dm.d / tc::BM) * split * (split == 1 ? 2 : 1);   // tiles within d
+  if ((mode == tc::EPI_RESID || mode == tc::EPI_RESID_CAT) && e.ssq_out != nullptr) c->ssq_n = tiles * split;     // slots the next consumer adds
+  if (mode == tc::EPI_UP && e.ssq_out != nullptr) c->ssq_n = (c->dm.d / tc::BM) * split;   // tiles within d
 }
 
 // How a launch of the tiled form (fm_prefill.cuh) is cut.  Rows per tile and CTAs per tile (one, or a pair that shares the

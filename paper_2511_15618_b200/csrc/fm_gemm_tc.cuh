@@ -182,8 +182,8 @@ __device__ inline uint32_t map_peer(uint32_t local_addr, uint32_t rank) {
 // (what the epilogue reads per row besides the product: the residual rows of the tile's 128
 // columns, or the rows' rotary angles; brought in by bulk copies while the MMAs run), then barriers.
 inline int stage_bytes(int N, int parts) { return BM * 128 + parts * (((N * 128 + 1023) / 1024) * 1024); }
-// The side rows exist only when a thread may get more than two items of the epilogue (N rows x
-// 64/split pair slots over 128 threads); otherwise the shared memory is better left to a
+// The side rows exist only when a thread may get more than one item of the epilogue (N rows x
+// 32/split quads over 128 threads); otherwise the shared memory is better left to a
 // neighbouring kernel's CTA.
 __host__ __device__ inline int side_bytes(int N, int split) { return N * (64 / split) > 256 ? N * 512 : 0; }
 // as many stages as the CTA has slabs (its whole K range is then requested at once), at most 8
@@ -220,6 +220,16 @@ __device__ inline void store_hi_lo2(bf16* p, float a, float b, int lo_off) {
     *reinterpret_cast<__nv_bfloat162*>(p + lo_off) = __floats2bfloat162_rn(__fsub_rn(a, __bfloat162float(hi.x)), __fsub_rn(b, __bfloat162float(hi.y)));
 }
 
+// four neighbouring values as [hi] and [lo] runs of 8 bytes
+__device__ inline void store_hi_lo4(bf16* p, float a, float b, float c, float d, int lo_off) {
+  const __nv_bfloat162 h0 = __floats2bfloat162_rn(a, b), h1 = __floats2bfloat162_rn(c, d);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+  if (lo_off > 0)
+    *reinterpret_cast<uint2*>(p + lo_off) = make_uint2(ptx::pack_bf16(__fsub_rn(a, __bfloat162float(h0.x)), __fsub_rn(b, __bfloat162float(h0.y))),
+                                                       ptx::pack_bf16(__fsub_rn(c, __bfloat162float(h1.x)), __fsub_rn(d, __bfloat162float(h1.y))));
+}
+__device__ inline float sum_sq4(const float4& x) { return __fmaf_rn(x.w, x.w, __fmaf_rn(x.z, x.z, __fmaf_rn(x.y, x.y, __fmul_rn(x.x, x.x)))); }
+
 // GELU of two values, x Phi(x) = max(x, 0) - |x| Phi(-|x|), with Phi(-c) = 2^q(c).  q(c) = log2 Phi(-c) on [0, 7] (behind
 // that the second term is under 1e-11) as a polynomial of degree 10 with q(0) = -1, fitted to SciPy's log_ndtr by
 // iteratively reweighted least squares (Lawson) with the weight c Phi(-c), i.e. for the smallest absolute error.  Packed
@@ -242,9 +252,9 @@ __device__ inline float2 gelu2(float a, float b) {
   return make_float2(__fmaf_rn(0.5f, a + fabsf(a), -__fmul_rn(ca, ea)), __fmaf_rn(0.5f, b + fabsf(b), -__fmul_rn(cb, eb)));       // (a NaN stays one)
 }
 
-// Pair slot q (0..63) of a 128-column tile holds columns (2q, 2q + 1): a thread's two values leave in one
-// store, and in the QKV projection, whose weight rows are stored with the rotary pairs (i, i + dh/2) of
-// a head side by side, they are one rotary pair.
+// Quad q (0..31) of a 128-column tile holds columns 4q .. 4q + 3: a thread's four values of a row leave together, and in the
+// QKV projection, whose weight rows are stored with the rotary pairs (i, i + dh/2) of a head side by side, they are two
+// rotary pairs.
 // grid (M/128 tiles, split, N tiles of the token rows), cluster (1, split, 1); block 128.  Warp 0 lane 0 feeds TMA, warp 1
 // lane 0 issues MMAs, all four warps read the accumulator back (warp w owns TMEM lanes 32w..32w+31).
 // SIDE: the launch has side rows (side_bytes(N, split) > 0); a separate instantiation, because the
@@ -336,7 +346,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
 
   // side rows: residual rows of this tile's columns (EPI_RESID that adds), or the rows' rotary
   // angles (EPI_QKV tiles that hold query or key heads)
-  // Only when a thread has more than two items: with fewer, loads straight into registers right
+  // Only when a thread has more than one item: with fewer, loads straight into registers right
   // after the dependency wait are quicker than the round through the copy engine (measured).
   constexpr bool IS_RESID = MODE == EPI_RESID || MODE == EPI_RESID_CAT;
   constexpr bool ROW_MAPS = MODE == EPI_QKV || MODE == EPI_RESID_CAT || MODE == EPI_UP;
@@ -464,40 +474,33 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   __syncwarp();
 
   // ---- where this thread's accumulator column goes, and its first item of the epilogue.  Column
-  // m of the tile is half of pair slot m / 2; slots [r*PW, (r+1)*PW) belong to rank r, which receives
+  // m of the tile is one of quad m / 4; quads [r*QW, (r+1)*QW) belong to rank r, which receives
   // [source rank][row][column]: a row's columns of a warp travel together (128 bytes at a split of up to 4; 16 bytes of a
   // column's rows at a time took 1.3 us for 32 rows).  Everything that does not depend on the previous kernel
   // (indices, gains, rotary angles) is prepared here, before the wait.
   const int lgS = 31 - __clz(S);                           // S is 1, 2, 4 or 8
-  const int lgPW = 6 - lgS, PW = 1 << lgPW;
-  const int items = ns * PW;
+  const int lgQ = 5 - lgS, QW = 1 << lgQ;                  // quads a rank owns
+  const int items = ns * QW;
   uint32_t dst0 = 0, dbar = 0;
-  const int CW = 2 << lgPW;                                // columns a rank owns
+  const int CW = 4 << lgQ;                                 // columns a rank owns
   float* recv_own = recv + z * g.N * CW + (tid & (CW - 1));  // this thread's column of row 0
   if (S > 1) {
-    const uint32_t owner = (uint32_t)(tid >> (lgPW + 1));
+    const uint32_t owner = (uint32_t)(tid >> (lgQ + 2));
     dst0 = map_peer(ptx::smem_u32(recv_own), owner);
     dbar = map_peer(ptx::smem_u32(rbar), owner);
   }
-  // A thread keeps its pair slot in every item (items advance by 128, a multiple of PW): its two
-  // columns, and with them the gains, are fixed.
-  float pre_ga = 1.f, pre_gb = 1.f;
-  float2 pre_cs = make_float2(1.f, 0.f);                   // first item's rotary angle when the side rows are not used
-  if (tid < items) {
-    const int ma = tile_m * BM + 2 * (z * PW + (tid & (PW - 1))), mb = ma + 1;
-    if (IS_RESID && e.gain != nullptr) {
-      if (ma < g.M) pre_ga = e.gain[ma];
-      if (mb < g.M) pre_gb = e.gain[mb];
-    }
-    if (MODE == EPI_UP && e.gain != nullptr) {             // gains of the child rows' next norm: column m mod d
-      if (ma < g.M) pre_ga = e.gain[ma % e.d_model];
-      if (mb < g.M) pre_gb = e.gain[mb % e.d_model];
-    }
-    if (MODE == EPI_QKV && want_side && !use_side) {
+  // A thread keeps its quad in every item (items advance by 128, a multiple of QW): its columns, and with them the gains,
+  // are fixed.
+  const int qc = 4 * (tid & (QW - 1)), ma = tile_m * BM + z * CW + qc;       // first column: of the rank's share, of the matrix
+  const bool m_ok = ma < g.M;                              // (M is a multiple of 4 but for plain stores)
+  float4 gain = make_float4(1.f, 1.f, 1.f, 1.f);
+  float4 pre = make_float4(1.f, 0.f, 1.f, 0.f);            // first item: rotary angles, or (below) residual values, when the side rows are not used
+  const bool rot = MODE == EPI_QKV && want_side && m_ok && ma / e.dm.dh < e.dm.H + e.dm.Hkv;
+  if (tid < items && m_ok) {
+    if ((IS_RESID || MODE == EPI_UP) && e.gain != nullptr) gain = *reinterpret_cast<const float4*>(e.gain + (MODE == EPI_UP ? ma % e.d_model : ma));
+    if (rot && !use_side) {
       int b, p;
-      const bool valid = row_of(e, row0 + (tid >> lgPW), b, p);
-      const int head = ma / e.dm.dh, i = (ma - head * e.dm.dh) >> 1;
-      if (valid && ma < g.M && head < e.dm.H + e.dm.Hkv) pre_cs = e.rope_tab[(size_t)p * (e.dm.dh >> 1) + i];
+      if (row_of(e, row0 + (tid >> lgQ), b, p)) pre = *reinterpret_cast<const float4*>(e.rope_tab + (size_t)p * (e.dm.dh >> 1) + ((ma % e.dm.dh) >> 1));
     }
   }
   // Kernel parameters the tail needs, read into registers now: a first touch of the parameter
@@ -517,17 +520,9 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   asm volatile("" : "+l"(k_out), "+l"(k_x), "+l"(k_aout), "+l"(k_ssqo), "+l"(k_q), "+l"(k_K), "+l"(k_V), "+l"(k_status));
   asm volatile("" : "+f"(k_qs), "+r"(k_H), "+r"(k_Hkv), "+r"(k_dh), "+r"(k_P), "+r"(k_cap));
   ptx::grid_dep_wait();                                    // everything below touches activations
-  float pre_xa = 0.f, pre_xb = 0.f;                        // first item's residual values, same case
-  if (IS_RESID && want_side && !use_side && tid < items) {
-    const int ma = tile_m * BM + 2 * (z * PW + (tid & (PW - 1))), mb = ma + 1;
-    const float* xr = k_x + (size_t)(k_row0 + (tid >> lgPW)) * k_ldx;
-    if (mb < k_M) {
-      const float2 x0 = __ldcg(reinterpret_cast<const float2*>(xr + ma));
-      pre_xa = x0.x;
-      pre_xb = x0.y;
-    } else if (ma < k_M) {
-      pre_xa = __ldcg(xr + ma);
-    }
+  if (IS_RESID) {
+    pre = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (want_side && !use_side && tid < items && m_ok) pre = __ldcg(reinterpret_cast<const float4*>(k_x + (size_t)(k_row0 + (tid >> lgQ)) * k_ldx + ma));
   }
 
   __syncthreads();                                         // s_inv / row maps are written (long before the MMAs end)
@@ -575,132 +570,119 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   if (!ok || !arrived || s_fail) {
     if (tid == 0) atomicExch(k_status, -5);
   }
-  // ---- this rank's share of the tile: pair slots [z*PW, (z+1)*PW), all rows
-  const int lgL = lgPW < 5 ? lgPW : 5, L = 1 << lgL;        // lanes that share a row
+  // ---- this rank's share of the tile: quads [z*QW, (z+1)*QW), all rows
   for (int it0 = 0; it0 < items; it0 += 128) {
     const int it = it0 + tid;
-    const bool active = it < items, first = it0 == 0;
-    const int n = active ? it >> lgPW : 0, cc = active ? it & (PW - 1) : 0;
-    const int ca = 2 * (z * PW + cc);
-    float2 v[MAX_SPLIT];
+    const bool active = it < items, first = it0 == 0, ok = active && m_ok;
+    const int n = active ? it >> lgQ : 0;
+    float4 v[MAX_SPLIT];
 #pragma unroll
     for (int r = 0; r < MAX_SPLIT; ++r)                    // all loads first, then the sums in rank order
-      v[r] = (r < S && active) ? *reinterpret_cast<const float2*>(recv + (r * g.N + n) * CW + 2 * cc) : make_float2(0.f, 0.f);
-    float ya = 0.f, yb = 0.f;
+      v[r] = (r < S && active) ? *reinterpret_cast<const float4*>(recv + (r * g.N + n) * CW + qc) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int r = 0; r < MAX_SPLIT; ++r)
-      if (r < S) { ya += v[r].x; yb += v[r].y; }
+      if (r < S) { y.x += v[r].x; y.y += v[r].y; y.z += v[r].z; y.w += v[r].w; }
     const float inv = s_inv[n];
-    ya *= inv;
-    yb *= inv;
-    const int ma = tile_m * BM + ca, mb = ma + 1;
-    const bool a_ok = active && ma < k_M, b_ok = active && mb < k_M;
+    y.x *= inv; y.y *= inv; y.z *= inv; y.w *= inv;
     const size_t row = (size_t)(k_row0 + n);
     if (MODE == EPI_F32) {
-      float* o = reinterpret_cast<float*>(k_out) + row * k_ldo;
-      if (b_ok && (k_ldo & 1) == 0) *reinterpret_cast<float2*>(o + ma) = make_float2(ya, yb);
-      else {
-        if (a_ok) o[ma] = ya;
-        if (b_ok) o[mb] = yb;
+      float* o = reinterpret_cast<float*>(k_out) + row * k_ldo + ma;
+      if (ok && ma + 3 < k_M && (k_ldo & 3) == 0) *reinterpret_cast<float4*>(o) = y;
+      else if (ok) {
+        o[0] = y.x;
+        if (ma + 1 < k_M) o[1] = y.y;
+        if (ma + 2 < k_M) o[2] = y.z;
+        if (ma + 3 < k_M) o[3] = y.w;
       }
-    } else if (MODE == EPI_BF16) {
-      bf16* o = reinterpret_cast<bf16*>(k_out) + row * k_ldo;
-      if (b_ok) store_hi_lo2(o + ma, ya, yb, k_lo);
-      else if (a_ok) store_hi_lo(o + ma, ya, k_lo);
-    } else if (MODE == EPI_GELU) {
-      bf16* o = reinterpret_cast<bf16*>(k_out) + row * k_ldo;
-      const float2 y = gelu2(ya, yb);
-      if (b_ok) store_hi_lo2(o + ma, y.x, y.y, k_lo);
-      else if (a_ok) store_hi_lo(o + ma, y.x, k_lo);
+    } else if (MODE == EPI_BF16 || MODE == EPI_GELU) {     // (rows and widths are multiples of 4 values)
+      if (MODE == EPI_GELU) {
+        const float2 a = gelu2(y.x, y.y), b = gelu2(y.z, y.w);
+        y = make_float4(a.x, a.y, b.x, b.y);
+      }
+      if (ok) store_hi_lo4(reinterpret_cast<bf16*>(k_out) + row * k_ldo + ma, y.x, y.y, y.z, y.w, k_lo);
     } else if (IS_RESID) {
-      float* xr = k_x + row * k_ldx;
-      float xa = 0.f, xb = 0.f;
-      if (b_ok) {                                          // both columns (M is even wherever the residual is used)
-        float2 x0 = make_float2(0.f, 0.f);
-        if (use_side) x0 = *reinterpret_cast<const float2*>(side + n * 128 + ca);
-        else if (first) x0 = make_float2(pre_xa, pre_xb);
-        else if (want_side) x0 = __ldcg(reinterpret_cast<const float2*>(xr + ma));
-        xa = x0.x + ya;
-        xb = x0.y + yb;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (ok) {
+        float* xr = k_x + row * k_ldx + ma;
+        if (use_side) x = *reinterpret_cast<const float4*>(side + n * 128 + z * CW + qc);
+        else if (first) x = pre;
+        else if (want_side) x = __ldcg(reinterpret_cast<const float4*>(xr));
+        x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
         if (MODE == EPI_RESID_CAT && s_rb[n] >= 0) {
-          // (xa, xb) is the level's final hidden of position p: into the carry ring, into the operand
+          // x is the level's final hidden of position p: into the carry ring, into the operand
           // row of the parent that pools it (if that parent is a row of this pass), and, where the
           // position's own parent p / 3 was computed in an earlier pass, that parent's stored slot
           // is added at once (the up-stack then finds h + upsampled slot in the residual row)
           const int b = s_rb[n], p = s_rp[n], dd = e.d_model, rs = fm_ring(e.level), rsu = fm_ring(e.level + 1);
-          *reinterpret_cast<float2*>(e.cat_ring + ((size_t)b * rs + p % rs) * dd + ma) = make_float2(xa, xb);
+          *reinterpret_cast<float4*>(e.cat_ring + ((size_t)b * rs + p % rs) * dd + ma) = x;
           const int u = (p + 2) / 3, part = p - 3 * u + 2;
           if (3 * u <= s_rl[n])
-            store_hi_lo2(e.cat_out + ((size_t)(b * fm_rows_per_seq(e.dm, e.level + 1) + u - s_ra[n]) * 6 + part) * dd + ma, xa, xb, 3 * dd);
+            store_hi_lo4(e.cat_out + ((size_t)(b * fm_rows_per_seq(e.dm, e.level + 1) + u - s_ra[n]) * 6 + part) * dd + ma, x.x, x.y, x.z, x.w, 3 * dd);
           if (p < 3 * s_ra[n]) {
-            const float2 t = __ldcg(reinterpret_cast<const float2*>(e.cat_tri + (((size_t)b * rsu + (p / 3) % rsu) * 3 + p % 3) * dd + ma));
-            xa += t.x;
-            xb += t.y;
+            const float4 t = __ldcg(reinterpret_cast<const float4*>(e.cat_tri + (((size_t)b * rsu + (p / 3) % rsu) * 3 + p % 3) * dd + ma));
+            x.x += t.x; x.y += t.y; x.z += t.z; x.w += t.w;
           }
         }
-        *reinterpret_cast<float2*>(xr + ma) = make_float2(xa, xb);
-        if (k_aout != nullptr) store_hi_lo2(k_aout + row * k_lda + ma, __fmul_rn(xa, pre_ga), __fmul_rn(xb, pre_gb), k_lo);
-      } else if (a_ok) {
-        xa = (use_side ? side[n * 128 + ca] : (first ? pre_xa : (want_side ? __ldcg(xr + ma) : 0.f))) + ya;
-        xr[ma] = xa;
-        if (k_aout != nullptr) store_hi_lo(k_aout + row * k_lda + ma, __fmul_rn(xa, pre_ga), k_lo);
+        *reinterpret_cast<float4*>(xr) = x;
+        if (k_aout != nullptr)
+          store_hi_lo4(k_aout + row * k_lda + ma, __fmul_rn(x.x, gain.x), __fmul_rn(x.y, gain.y), __fmul_rn(x.z, gain.z), __fmul_rn(x.w, gain.w), k_lo);
       }
       if (k_ssqo != nullptr) {
-        // per-row sums of squares of this rank's columns: a fixed shuffle tree over the L lanes that
-        // share the row; the next GEMM adds the (tile, rank, lane group) partials in slot order
-        float sqv = __fmaf_rn(xa, xa, __fmul_rn(xb, xb));
-        for (int o = L >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
-        if (active && (cc & (L - 1)) == 0)
-          k_ssqo[row * k_ldssq + ((((tile_m << lgS) + z) << (lgPW - lgL)) + (cc >> lgL))] = sqv;
+        // per-row sums of squares of this rank's columns: a fixed shuffle tree over the QW lanes that
+        // share the row; the next GEMM adds the (tile, rank) partials in slot order
+        float sqv = sum_sq4(x);
+        for (int o = QW >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
+        if (active && qc == 0) k_ssqo[row * k_ldssq + (tile_m << lgS) + z] = sqv;
       }
     } else if (MODE == EPI_UP) {
-      // (ya, yb): columns (ma, ma + 1) of the triple of parent row n = slot ma / d, column ma % d
+      // y: columns ma .. ma + 3 of the triple of parent row n = slot ma / d, columns ma % d ..
       const int dd = e.d_model;
-      float xa = 0.f, xb = 0.f;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
       bool child = false;
       size_t crow = 0;
-      if (b_ok && s_rb[n] >= 0) {
+      if (ok && s_rb[n] >= 0) {
         const int b = s_rb[n], pu = s_rp[n], rsu = fm_ring(e.level);
-        *reinterpret_cast<float2*>(e.tri_ring + ((size_t)b * rsu + pu % rsu) * 3 * dd + ma) = make_float2(ya, yb);
+        *reinterpret_cast<float4*>(e.tri_ring + ((size_t)b * rsu + pu % rsu) * 3 * dd + ma) = y;
         const int slot = ma / dd, col = ma - slot * dd, p = 3 * pu + slot;
         if (p <= s_rl[n]) {                                // the child is a row of this pass
           child = true;
           crow = (size_t)b * fm_rows_per_seq(e.dm, e.level - 1) + (p - s_ra[n]);
           float* xr = k_x + crow * k_ldx + col;
-          const float2 x0 = __ldcg(reinterpret_cast<const float2*>(xr));
-          xa = x0.x + ya;
-          xb = x0.y + yb;
-          *reinterpret_cast<float2*>(xr) = make_float2(xa, xb);
-          if (k_aout != nullptr) store_hi_lo2(k_aout + crow * k_lda + col, __fmul_rn(xa, pre_ga), __fmul_rn(xb, pre_gb), k_lo);
+          x = __ldcg(reinterpret_cast<const float4*>(xr));
+          x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+          *reinterpret_cast<float4*>(xr) = x;
+          if (k_aout != nullptr)
+            store_hi_lo4(k_aout + crow * k_lda + col, __fmul_rn(x.x, gain.x), __fmul_rn(x.y, gain.y), __fmul_rn(x.z, gain.z), __fmul_rn(x.w, gain.w), k_lo);
         }
       }
       if (k_ssqo != nullptr) {                             // as EPI_RESID, for the child row; tiles count within d
-        float sqv = __fmaf_rn(xa, xa, __fmul_rn(xb, xb));
-        for (int o = L >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
-        if (active && child && (cc & (L - 1)) == 0)
-          k_ssqo[crow * k_ldssq + (((((tile_m % (dd / BM)) << lgS) + z) << (lgPW - lgL)) + (cc >> lgL))] = sqv;
+        float sqv = sum_sq4(x);
+        for (int o = QW >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
+        if (active && child && qc == 0) k_ssqo[crow * k_ldssq + ((tile_m % (dd / BM)) << lgS) + z] = sqv;
       }
-    } else {  // EPI_QKV: (ya, yb) is the rotary pair (i, i + dh/2) of one head, stored at (c, c + 1), c = 2i
+    } else {  // EPI_QKV: y holds the rotary pairs (i, i + dh/2) and (i + 1, i + 1 + dh/2) of one head, stored at c .. c + 3, c = 2i
       const int dh = k_dh, H = k_H, Hkv = k_Hkv;
       const int head = ma / dh, c = ma - head * dh;
-      if (a_ok && head < H + 2 * Hkv) {
+      if (ok && head < H + 2 * Hkv) {
         const int b = s_rb[n], p = s_rp[n];
         const bool valid = b >= 0;
         const int slots = k_P + k_cap;
-        if (head < H + Hkv) {
-          float2 cs = make_float2(1.f, 0.f);
-          if (use_side) { if (valid) cs = reinterpret_cast<const float2*>(side)[n * 64 + (c >> 1)]; }
-          else if (first) cs = pre_cs;
-          else if (want_side && valid) cs = e.rope_tab[(size_t)p * (dh >> 1) + (c >> 1)];
-          const float y1 = ya * cs.x - yb * cs.y, y2 = yb * cs.x + ya * cs.y;
-          if (head < H)
-            *reinterpret_cast<__nv_bfloat162*>(k_q + (row * H + head) * dh + c) =
-                valid ? __floats2bfloat162_rn(y1 * k_qs, y2 * k_qs) : __floats2bfloat162_rn(0.f, 0.f);
-          else if (valid)
-            *reinterpret_cast<__nv_bfloat162*>(k_K + (((size_t)b * Hkv + (head - H)) * slots + k_P + (p % k_cap)) * dh + c) = __floats2bfloat162_rn(y1, y2);
-        } else if (valid) {
-          *reinterpret_cast<__nv_bfloat162*>(k_V + (((size_t)b * Hkv + (head - H - Hkv)) * slots + k_P + (p % k_cap)) * dh + c) = __floats2bfloat162_rn(ya, yb);
+        if (rot) {
+          float4 cs = pre;
+          if (use_side) cs = valid ? *reinterpret_cast<const float4*>(side + n * 128 + c) : make_float4(1.f, 0.f, 1.f, 0.f);
+          else if (!first) cs = valid ? *reinterpret_cast<const float4*>(e.rope_tab + (size_t)p * (dh >> 1) + (c >> 1)) : make_float4(1.f, 0.f, 1.f, 0.f);
+          y = make_float4(y.x * cs.x - y.y * cs.y, y.y * cs.x + y.x * cs.y, y.z * cs.z - y.w * cs.w, y.w * cs.z + y.z * cs.w);
         }
+        bf16* dst;
+        if (head < H) {
+          dst = k_q + (row * H + head) * dh + c;
+          y = valid ? make_float4(y.x * k_qs, y.y * k_qs, y.z * k_qs, y.w * k_qs) : make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+          const bool is_k = head < H + Hkv;
+          dst = (is_k ? k_K : k_V) + (((size_t)b * Hkv + (head - H - (is_k ? 0 : Hkv))) * slots + k_P + (p % k_cap)) * dh + c;
+        }
+        if (valid || head < H) *reinterpret_cast<uint2*>(dst) = make_uint2(ptx::pack_bf16(y.x, y.y), ptx::pack_bf16(y.z, y.w));
       }
     }
   }
@@ -708,24 +690,20 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     // child rows of this tile's slot whose parent was computed in an earlier pass: their residual
     // rows are final already (the last layer below added the stored slot); what is missing is the
     // next operand and the sums of squares, for this rank's columns
-    const int dd = e.d_model, nci = s_ncarry << lgPW;
+    const int dd = e.d_model, nci = s_ncarry << lgQ, col = ma % dd;
+    const float4 cg = e.gain != nullptr && m_ok ? *reinterpret_cast<const float4*>(e.gain + col) : make_float4(1.f, 1.f, 1.f, 1.f);
     for (int it0 = 0; it0 < nci; it0 += 128) {
       const int it = it0 + tid;
       const bool active = it < nci;
-      const int cc = it & (PW - 1);
-      const size_t crow = active ? (size_t)s_carry[it >> lgPW] : 0;
-      const int col = (tile_m * BM + 2 * (z * PW + cc)) % dd;
-      float2 x0 = make_float2(0.f, 0.f);
-      if (active) x0 = __ldcg(reinterpret_cast<const float2*>(k_x + crow * k_ldx + col));
-      if (active && k_aout != nullptr) {
-        const float ga = e.gain != nullptr ? e.gain[col] : 1.f, gb = e.gain != nullptr ? e.gain[col + 1] : 1.f;
-        store_hi_lo2(k_aout + crow * k_lda + col, __fmul_rn(x0.x, ga), __fmul_rn(x0.y, gb), k_lo);
-      }
+      const size_t crow = active ? (size_t)s_carry[it >> lgQ] : 0;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (active) x = __ldcg(reinterpret_cast<const float4*>(k_x + crow * k_ldx + col));
+      if (active && k_aout != nullptr)
+        store_hi_lo4(k_aout + crow * k_lda + col, __fmul_rn(x.x, cg.x), __fmul_rn(x.y, cg.y), __fmul_rn(x.z, cg.z), __fmul_rn(x.w, cg.w), k_lo);
       if (k_ssqo != nullptr) {
-        float sqv = __fmaf_rn(x0.x, x0.x, __fmul_rn(x0.y, x0.y));
-        for (int o = L >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
-        if (active && (cc & (L - 1)) == 0)
-          k_ssqo[crow * k_ldssq + (((((tile_m % (dd / BM)) << lgS) + z) << (lgPW - lgL)) + (cc >> lgL))] = sqv;
+        float sqv = sum_sq4(x);
+        for (int o = QW >> 1; o > 0; o >>= 1) sqv += __shfl_xor_sync(0xffffffffu, sqv, o);
+        if (active && qc == 0) k_ssqo[crow * k_ldssq + ((tile_m % (dd / BM)) << lgS) + z] = sqv;
       }
     }
   }

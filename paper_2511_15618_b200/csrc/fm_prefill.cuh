@@ -132,14 +132,6 @@ __device__ inline void ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr));
 }
 __device__ inline void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// [hi | lo] operand values of four neighbouring features
-__device__ inline void store_hi_lo4(bf16* p, float a, float b, float c, float d, int lo_off) {
-  const __nv_bfloat162 h0 = __floats2bfloat162_rn(a, b), h1 = __floats2bfloat162_rn(c, d);
-  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
-  *reinterpret_cast<uint2*>(p + lo_off) = make_uint2(ptx::pack_bf16(__fsub_rn(a, __bfloat162float(h0.x)), __fsub_rn(b, __bfloat162float(h0.y))),
-                                                     ptx::pack_bf16(__fsub_rn(c, __bfloat162float(h1.x)), __fsub_rn(d, __bfloat162float(h1.y))));
-}
-
 template <int MODE, int PARTS, int CG>
 __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Epi e) {
   if (g.n_active != nullptr && *g.n_active == 0) {           // the whole grid leaves; keep the launch chain ordered
@@ -429,12 +421,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
             }
           } else if (MODE == PF_GELU) {
             const float2 a = tc::gelu2(v[i].x, v[i].y), b = tc::gelu2(v[i].z, v[i].w);
-            if (ok) store_hi_lo4(reinterpret_cast<bf16*>(e.out) + row * e.ldo + m, a.x, a.y, b.x, b.y, e.lo_off);
+            if (ok) tc::store_hi_lo4(reinterpret_cast<bf16*>(e.out) + row * e.ldo + m, a.x, a.y, b.x, b.y, e.lo_off);
           } else if (MODE == PF_RESID) {
             if (ok) {
               *reinterpret_cast<float4*>(e.x + row * e.ldx + m) = v[i];
               if (e.a_out != nullptr)
-                store_hi_lo4(e.a_out + row * e.lda + m, __fmul_rn(v[i].x, gain.x), __fmul_rn(v[i].y, gain.y), __fmul_rn(v[i].z, gain.z),
+                tc::store_hi_lo4(e.a_out + row * e.lda + m, __fmul_rn(v[i].x, gain.x), __fmul_rn(v[i].y, gain.y), __fmul_rn(v[i].z, gain.z),
                              __fmul_rn(v[i].w, gain.w), e.lo_off);
             }
             if (e.ssq_out != nullptr) {                      // sum of squares over the warp's 32 features
