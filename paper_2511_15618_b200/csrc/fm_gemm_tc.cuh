@@ -396,8 +396,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   }
   else if (warp >= 2) {
     // ---- warps 2 and 3, while the operands arrive: operand-row scales (the partial sums of
-    // squares of a row are gathered by 8 lanes, each adding its slots in slot order, then combined by
-    // a fixed shuffle tree) and row maps
+    // squares of a row are gathered by 8 lanes, then combined by a fixed shuffle tree) and row maps
     if (ROW_MAPS && warp == 3) {
       // row maps, and the rows' rotary angles into the side buffer: positions are per-pass state
       // and the table is constant, so nothing here waits for the previous kernel
@@ -448,24 +447,34 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
     }
     const int t = tid - 64;
     if (e.ssq_in != nullptr) {
+      // (the requests of 32 rows travel together: eight rows at a time waited for L2 four times, 1.5 us in front of the epilogue)
       const int sub = t & 7;
-      for (int n0 = 0; n0 < ns; n0 += 8) {
-        const int n = n0 + (t >> 3);
-        float v[8];
+      for (int n0 = 0; n0 < ns; n0 += 32) {
+        float ss[4] = {0.f, 0.f, 0.f, 0.f};
+        const float* sq = e.ssq_in + (size_t)(row0 + n0 + (t >> 3)) * e.ld_ssq + 4 * sub;        // (rows of ssq are a multiple of 16 floats)
+        const int rows = ns - n0 - (t >> 3);
+        for (int s0 = 0; s0 < e.ssq_n; s0 += 64) {
+          float4 q[4][2];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int slot = sub + 8 * k;
-          v[k] = (n < ns && slot < e.ssq_n) ? __ldcg(e.ssq_in + (size_t)(row0 + n) * e.ld_ssq + slot) : 0.f;
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+              q[i][k] = 8 * i < rows && s0 + 32 * k + 4 * sub < e.ssq_n ? __ldcg(reinterpret_cast<const float4*>(sq + (size_t)8 * i * e.ld_ssq + s0 + 32 * k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              const int left = e.ssq_n - (s0 + 32 * k + 4 * sub);
+              ss[i] += (q[i][k].x + (left > 1 ? q[i][k].y : 0.f)) + ((left > 2 ? q[i][k].z : 0.f) + (left > 3 ? q[i][k].w : 0.f));
+            }
         }
-        float ss = 0.f;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) ss += v[k];
-        for (int slot = sub + 64; slot < e.ssq_n; slot += 8)             // more than 64 slots: not expected
-          ss += (n < ns) ? __ldcg(e.ssq_in + (size_t)(row0 + n) * e.ld_ssq + slot) : 0.f;
-        ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-        ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-        ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-        if (sub == 0 && n < ns) s_inv[n] = rsqrtf(ss * e.inv_d_in + e.eps);
+        for (int i = 0; i < 4; ++i) {
+          ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], 1);
+          ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], 2);
+          ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], 4);
+          if (sub == 0 && 8 * i < rows) s_inv[n0 + 8 * i + (t >> 3)] = rsqrtf(ss[i] * e.inv_d_in + e.eps);
+        }
       }
     } else {
       for (int n = t; n < ns; n += 64) s_inv[n] = 1.f;
