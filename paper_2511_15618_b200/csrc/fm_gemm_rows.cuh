@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
   constexpr int FT = FJ * 8, PAIRS = FT / 2, S = FT == 8 ? 8 : FT + 8;
   constexpr bool IS_RESID = MODE == EPI_RESID || MODE == EPI_RESID_CAT;
   constexpr bool ROW_MAPS = MODE == EPI_QKV || MODE == EPI_RESID_CAT || MODE == EPI_UP;
+  constexpr bool SCALED = MODE != EPI_UP && !IS_RESID;
   constexpr int CARRY_MAX = MODE == EPI_UP ? 128 : 1;
   if (g.n_active != nullptr && *g.n_active == 0) {           // the whole grid leaves; keep the launch chain ordered
     ptx::grid_dep_launch();
@@ -144,6 +145,14 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
   const int nkb = g.K / 32, kb0 = nkb * warp / NW, kb1 = nkb * (warp + 1) / NW;
   __syncthreads();                                           // barrier and row maps are initialised
   ptx::grid_dep_wait();                                      // everything below touches activations
+  // The partial sums of squares of rows warp and warp + NW are requested first, 16 bytes a lane (rows of ssq are a multiple
+  // of 16 floats; 4 bytes at a time a row of 128 slots took four round trips).
+  float4 sq[2];
+  if (SCALED && e.ssq_in != nullptr) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      sq[j] = warp + NW * j < R && 4 * lane < e.ssq_n ? __ldcg(reinterpret_cast<const float4*>(e.ssq_in + (size_t)(row0 + warp + NW * j) * e.ld_ssq) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   constexpr int CB = 2;                                      // blocks of 32 k per request, two requests in flight
   uint4 va[2][CB][MTN][2];
   auto load = [&](int buf, int kb) {
@@ -160,17 +169,24 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const Args g, con
   // residual values of the first item, and the rows' scales, while the operands travel
   float2 x0 = make_float2(0.f, 0.f);
   if (IS_RESID && e.add && tid < items && b_ok) x0 = __ldcg(reinterpret_cast<const float2*>(e.x + (size_t)(row0 + tid / PAIRS) * e.ldx + ma));
-  if (MODE != EPI_UP && !IS_RESID) {
-    for (int n = warp; n < R; n += NW) {
-      float v = 1.f;
-      if (e.ssq_in != nullptr) {
-        const float* sq = e.ssq_in + (size_t)(row0 + n) * e.ld_ssq;
-        float ss = 0.f;
-        for (int s = lane; s < e.ssq_n; s += 32) ss += __ldcg(sq + s);
-        v = rsqrtf(warp_sum(ss) * e.inv_d_in + e.eps);
+  if (SCALED && warp < R) {
+    float ss[2] = {0.f, 0.f};
+    if (e.ssq_in != nullptr) {
+      const int left = e.ssq_n - 4 * lane;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        ss[j] = (sq[j].x + (left > 1 ? sq[j].y : 0.f)) + ((left > 2 ? sq[j].z : 0.f) + (left > 3 ? sq[j].w : 0.f));
+        if (warp + NW * j < R)
+          for (int s = 128 + lane; s < e.ssq_n; s += 32) ss[j] += __ldcg(e.ssq_in + (size_t)(row0 + warp + NW * j) * e.ld_ssq + s);     // more than 128 slots
       }
-      if (lane == 0) s_inv[n] = v;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float a = __shfl_xor_sync(0xffffffffu, ss[0], o), b = __shfl_xor_sync(0xffffffffu, ss[1], o);
+        ss[0] += a;
+        ss[1] += b;
+      }
     }
+    if (lane < 2 && warp + NW * lane < R) s_inv[warp + NW * lane] = e.ssq_in != nullptr ? rsqrtf((lane == 0 ? ss[0] : ss[1]) * e.inv_d_in + e.eps) : 1.f;
   }
   float acc[MTN][FJ][4];
 #pragma unroll
