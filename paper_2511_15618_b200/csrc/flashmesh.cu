@@ -643,12 +643,20 @@ void launch_rows(fm_ctx* c, int mtn, int fj, dim3 grid, int smem, const rg::Args
   }
 }
 // The few-row form (fm_gemm_rows.cuh), with as few features per CTA as give every SM at most one CTA.  For
-// up to 16 rows (above that the operand rows that every CTA reads cost more than the cluster exchange of the
-// other form: 24 rows 4.0 / 9.8 us for the output projection and the second FFN matrix) whose weights per
-// CTA fit beside a neighbour's; returns false where it does not apply.
+// up to 16 rows whose weights per CTA fit beside a neighbour's; returns false where it does not apply.
+// Above 16 MMA rows (8 rows of two terms) it has two row tiles, and its time grows with the features per CTA and with K, while
+// the split-K form takes as long as for one row: there it keeps the output projections and the narrow QKV only.  From one
+// launch's dependency wait to the next one's, us, few-row / split-K:
+//                      d = 256, 10 rows   512, 10 rows   640, 10 rows   1024, 10 rows   1024, 16 rows   1024, 4 rows
+//   QKV                  3.4 / 3.6          3.3 / 3.5      3.5 / 3.3      5.6 / 3.6       5.9 / 3.2       3.3 / 3.3
+//   output projection    2.0 / 3.0          2.4 / 3.7      2.7 / 3.7      2.9 / 3.7       3.4 / 4.0       2.7 / 3.8
+//   first FFN matrix     2.9 / 2.2          3.3 / 3.0      4.8 / 3.0      6.0 / 3.4       6.5 / 3.3       3.4 / 3.6
+//   second FFN matrix    2.4 / 3.6          4.7 / 4.3      5.7 / 4.8      5.8 / 5.7       6.3 / 6.2       4.2 / 5.6
+// (second FFN matrix: K = 1536 3.1 / 4.0, K = 2048 4.7 / 4.3, K = 3072 7.0 / 5.0, K = 3584 5.2 / 5.4)
 bool gemm_rows(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, int a_row0, int M, int K, int R, const int* n_active, int mode,
                const tc::Epi& e, int parts, int stacked, int z_rows, int z_w_rows) {
   if (R > c->rows_max || M < 8) return false;
+  if (parts * R > 16 && (mode == tc::EPI_GELU || (mode == tc::EPI_QKV && K >= 640) || K > 1536)) return false;
   int FT = K > 1536 ? 16 : 8;                              // long K: fewer CTAs, each of which reads all operand rows
   while (FT < 32 && (M + FT - 1) / FT * stacked > c->n_sm) FT *= 2;
   const int mtn = (parts * R + 15) / 16, smem = rg::smem_bytes(FT, K, mtn);
