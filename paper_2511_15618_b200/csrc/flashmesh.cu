@@ -1329,12 +1329,14 @@ int prefill_run(fm_ctx* c, const float* cond, const int* prompt, const int* off)
     for (int l = 0; l < 3; ++l) {
       const size_t t0 = tiles.size();
       tile_at.push_back(t0);
-      // query rows per CTA: the most that still give every SM one (see pf::AttnCfg)
+      // Query rows per CTA: the most that still give every SM one (see pf::AttnCfg); 128 on the tensor cores (heads of 64)
+      // already where 60 % of the SMs get one.  Prefills, d = 1024, with that line at 100 / 60 / 40 %, us: 60 faces 1556 / 1556 / 1592,
+      // 100 faces 1939 / 1894 / 1895, 300 faces 3157 / 3110 / 3111, four of 30 2033 / 2035 / 2166, four of 100 3582 / 3589 / 3642.
       ch.tile_rows[l] = dm.dh == 64 ? 16 : 32;
       for (int rows = 128; rows >= 32; rows /= 4) {
         int n = 0;
         for (int k = 0; k < ch.n_segs; ++k) n += (segs[seg_at.back() + k].n[l] + rows - 1) / rows;
-        if (n * dm.H >= c->n_sm) { ch.tile_rows[l] = rows; break; }
+        if (n * dm.H * 5 >= c->n_sm * (rows == 128 && dm.dh == 64 ? 3 : 5)) { ch.tile_rows[l] = rows; break; }
       }
       for (int k = 0; k < ch.n_segs; ++k)
         for (int q = 0; q < segs[seg_at.back() + k].n[l]; q += ch.tile_rows[l]) tiles.push_back(make_int2(k, q));

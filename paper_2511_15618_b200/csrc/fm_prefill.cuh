@@ -961,18 +961,39 @@ __global__ void __launch_bounds__(AttnCfg<DH, C, QW>::THREADS, DH == 64 ? 2 : 1)
 // B operand's MN-major form).  S of the next tile is multiplied as soon as S is in registers, i.e. under the
 // exponentials.  The output is rescaled only when a row's maximum has grown by more than 2^8 (the conditional rescaling of
 // FlashAttention-4, T. Dao et al., Hot Chips 2025).  Nearest bound: the special-function units (1024 clocks for a tile's
-// exponentials; 58 % of their rate in use, tensor pipe 27 %), which two CTAs per SM share.  6994 rows, 16 heads: 207 us a
-// launch (MMAs of warps, attn_kernel: 505 us; a thread per row without the overlap: 462 us).
+// exponentials, which two CTAs per SM share; 65 % of their rate in use), beside them the issue slots of the softmax warps: hence
+// sums and differences in pairs, maxima of three, one barrier a tile.  6994 rows, 16 heads: 180 us a launch (187 without these,
+// 201 with copies and MMAs issued behind `lane == 0`; MMAs of warps, attn_kernel: 505 us; a thread per row without the overlap: 462 us).
 namespace fa {
 constexpr int THREADS = 320;     // producer warp, MMA warp, eight softmax warps
 constexpr int STAGES = 2, TILE = 128 * 128, STAGE = 2 * TILE;            // bytes of 128 keys (or values) of 64
-constexpr int BYTES = TILE + STAGES * STAGE + 256 * 4 + 128 + 1024;
+constexpr int BYTES = TILE + STAGES * STAGE + 512 * 4 + 128 + 1024;
 constexpr float GROW = 8.f;
 
 __device__ inline float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+__device__ inline uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ inline float2 unpack2(uint64_t r) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
+  return v;
+}
+__device__ inline uint64_t add2(uint64_t a, uint64_t b) {              // two sums in one instruction
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ inline float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
 __device__ inline void st16(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" ::"r"(r[0]), "r"(r[1]),
@@ -997,8 +1018,8 @@ __global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, c
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* ring = sm + TILE;                           // behind the query tile
-  float* s_pair = reinterpret_cast<float*>(ring + STAGES * STAGE);         // [half][row]
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_pair + 256);
+  float* s_pair = reinterpret_cast<float*>(ring + STAGES * STAGE);         // [tile mod 2][half][row]
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_pair + 512);
   uint64_t *empty = full + STAGES, *q_full = empty + STAGES, *s_full = q_full + 1, *s_read = s_full + 1, *p_full = s_read + 1, *o_full = p_full + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_full + 1);
   __shared__ int s_fail;
@@ -1136,15 +1157,15 @@ __global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, c
       }
       float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) {
-        m4[0] = fmaxf(m4[0], __uint_as_float(r0[j])); m4[1] = fmaxf(m4[1], __uint_as_float(r0[j + 1]));
-        m4[2] = fmaxf(m4[2], __uint_as_float(r1[j])); m4[3] = fmaxf(m4[3], __uint_as_float(r1[j + 1]));
+      for (int j = 0; j < 32; j += 4) {
+        m4[0] = max3(m4[0], __uint_as_float(r0[j]), __uint_as_float(r0[j + 1])); m4[1] = max3(m4[1], __uint_as_float(r0[j + 2]), __uint_as_float(r0[j + 3]));
+        m4[2] = max3(m4[2], __uint_as_float(r1[j]), __uint_as_float(r1[j + 1])); m4[3] = max3(m4[3], __uint_as_float(r1[j + 2]), __uint_as_float(r1[j + 3]));
       }
       float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-      s_pair[half * 128 + i_row] = mx;
+      float* pair = s_pair + (i & 1) * 256;                  // (two of them: written again behind the next tile's barrier)
+      pair[half * 128 + i_row] = mx;
       asm volatile("bar.sync %0, 64;" ::"r"(1 + w4) : "memory");
-      mx = fmaxf(mx, s_pair[(half ^ 1) * 128 + i_row]);
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + w4) : "memory");         // read before the next tile's write
+      mx = fmaxf(mx, pair[(half ^ 1) * 128 + i_row]);
       // P of the tile before has been multiplied: its place, and O, are free
       if (i > 0) ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait(o_full, (i - 1) & 1));
       tc::fence_after();
@@ -1165,33 +1186,36 @@ __global__ void __launch_bounds__(fa::THREADS, 2) attn_tc_kernel(const Attn a, c
         }
       }
       const float base = m == -INFINITY ? 0.f : m;
-      float s4[4] = {0.f, 0.f, 0.f, 0.f};
+      const uint64_t nb = pack2(-base, -base);
+      uint64_t s2[2] = {0ull, 0ull};
       uint32_t pk[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const float e0 = ex2(__uint_as_float(r0[2 * j]) - base), e1 = ex2(__uint_as_float(r0[2 * j + 1]) - base);
-        s4[0] += e0;
-        s4[1] += e1;
+        const float2 d = unpack2(add2(pack2(__uint_as_float(r0[2 * j]), __uint_as_float(r0[2 * j + 1])), nb));
+        const float e0 = ex2(d.x), e1 = ex2(d.y);
+        s2[0] = add2(s2[0], pack2(e0, e1));
         pk[j] = ptx::pack_bf16(e0, e1);
       }
       st16(tP + lanes + 32 * half, pk);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const float e0 = ex2(__uint_as_float(r1[2 * j]) - base), e1 = ex2(__uint_as_float(r1[2 * j + 1]) - base);
-        s4[2] += e0;
-        s4[3] += e1;
+        const float2 d = unpack2(add2(pack2(__uint_as_float(r1[2 * j]), __uint_as_float(r1[2 * j + 1])), nb));
+        const float e0 = ex2(d.x), e1 = ex2(d.y);
+        s2[1] = add2(s2[1], pack2(e0, e1));
         pk[j] = ptx::pack_bf16(e0, e1);
       }
       st16(tP + lanes + 32 * half + 16, pk);
-      l += (s4[0] + s4[1]) + (s4[2] + s4[3]);
+      const float2 sa = unpack2(s2[0]), sb = unpack2(s2[1]);
+      l += (sa.x + sa.y) + (sb.x + sb.y);
       st_wait();
       tc::fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(p_full);
     }
-    s_pair[half * 128 + i_row] = l;
+    float* pair = s_pair + (n_tiles & 1) * 256;
+    pair[half * 128 + i_row] = l;
     asm volatile("bar.sync %0, 64;" ::"r"(1 + w4) : "memory");
-    l += s_pair[(half ^ 1) * 128 + i_row];
+    l += pair[(half ^ 1) * 128 + i_row];
     ok = ok && __all_sync(0xffffffffu, ptx::mbar_wait(o_full, (n_tiles - 1) & 1));
     if (!ok) s_fail = 1;
     else {

@@ -20,7 +20,9 @@ pytestmark = pytest.mark.gpu
     ((35, 2), (0, 0, 0), {"d_model": 192, "d_ff": 320}),              # partly empty last tiles
     ((61, 2), (0, 0, 0), {"d_model": 384, "n_heads": 6, "n_kv_heads": 1, "d_ff": 320}),      # pairs of feature tiles: an odd number, a last one half empty
     ((143, 1), (0, 0, 0), {"d_model": 640, "n_heads": 10, "n_kv_heads": 10, "d_ff": 704, "weight_std": 0.04}),
-    ((143,), (0, 0, 0), {"n_heads": 16, "n_kv_heads": 16}),           # 128 query rows per CTA: 10 tiles and 8 rows more
+    ((71,), (0, 0, 0), {"n_heads": 16, "n_kv_heads": 16}),            # 640 rows, 5 tiles of 128 on 16 heads: 32 query rows per CTA
+    ((71, 0), (30, 0, 0), {"n_heads": 16, "n_kv_heads": 4}),          # a row more, 6 tiles: 128
+    ((143,), (0, 0, 0), {"n_heads": 16, "n_kv_heads": 16}),           # 10 tiles and 8 rows more
     ((160, 3), (600, 0, 0), {"n_heads": 16, "n_kv_heads": 2}),        # the same with a ring shorter than the prompt, shared heads
     ((950,), (700, 0, 0), {"n_heads": 16, "n_kv_heads": 16}),         # ... and in two chunks
     ((950, 30), (0, 0, 0), {}),                                       # cut into two chunks
