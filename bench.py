@@ -65,7 +65,7 @@ def rank_sequences(rank, batch_per_rank):
 # DRAM traffic of the dominant kernel per launch from ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum), keyed by workload, each with the summary under profiles/ that holds the
 # capture; None where the kernel changed since the capture or none was taken.
-NCU_TRAFFIC = {"medium": {"bytes_per_launch": 6.35e6, "summary": "profiles/gemm_and_attention_dram_traffic_medium.md (mean of a layer's four projections)"}}
+NCU_TRAFFIC = {"medium": {"bytes_per_launch": 6.38e6, "summary": "profiles/gemm_and_attention_dram_traffic_medium.md (mean of a layer's four projections)"}}
 
 
 FEW_ROWS = 16              # rows up to which a projection takes the few-row form (rg::MAX_ROWS)
@@ -296,7 +296,7 @@ def run_ours(args):
                 "what": "fm_step_host once per pass with the host in the loop: candidates from pinned host memory "
                         "in, draft + verify + accept, accepted tokens copied back, per pass"},
         "gpu_launches": launches,
-        "roofline": {"bound": "hbm", "kernel": gemm_kernels(cfg) + " (all GEMM launches of one verify pass, timed alone as a graph)",
+        "roofline": {"bound": "hbm", "kernel": gemm_kernels(cfg) + (", tc::gemm_tc_kernel (the wide ones of more than 8 rows)" if 8 < cfg.batch * (cfg.draft_len + 1) <= FEW_ROWS else "") + " (all GEMM launches of one verify pass, timed alone as a graph)",
                      "achieved": gemm_gbs, "peak": peak, "unit": "GB/s", "frac": gemm_gbs / peak,
                      "peak_kind": peak_kind + " copy bandwidth (burst figure: the kernel is timed alone)",
                      "traffic": NCU_TRAFFIC.get(args.workload, {}).get("bytes_per_launch"),
