@@ -9,7 +9,7 @@
 // 128-byte swizzle.  Weights are stored in HBM slab by slab, each [128 x 64] slab as the 16 KB
 // image the MMA reads from shared memory, so a CTA's K range is one contiguous stream fetched by
 // 16 KB bulk copies; the token rows come through a TMA tensor map.  A ring of shared-memory stages
-// decouples the copies from the one thread that issues the MMAs; accumulators live in tensor
+// decouples the copies from the warp that issues the MMAs; accumulators live in tensor
 // memory and are read back with tcgen05.ld.
 // Operand rows may come as two bfloat16 terms per value, [hi | lo] side by side (hi = bf16(v),
 // lo = bf16(v - hi)): the hi tile and the lo tile of a slab then sit one after the other in shared
@@ -19,7 +19,7 @@
 // The work is bandwidth bound: the grid is (M/128 tiles) x (S splits of K) so that many SMs
 // stream weights.  The S CTAs of one M tile form a thread-block cluster: every CTA owns 1/S of the
 // tile's columns; each CTA sends the columns of its partial tile to their owners' shared memory
-// with asynchronous distributed-shared-memory stores that count their bytes on an mbarrier of the
+// with asynchronous distributed-shared-memory stores, a row's columns of a warp at a time, that count their bytes on an mbarrier of the
 // owner, so an owner continues as soon as its own S partials are in, adds them in rank order (a
 // fixed order, so a row's result does not depend on how many rows the launch holds) and applies
 // the epilogue of the projection: RMSNorm scale of the operand rows, then one of
@@ -255,8 +255,8 @@ __device__ inline float2 gelu2(float a, float b) {
 // Quad q (0..31) of a 128-column tile holds columns 4q .. 4q + 3: a thread's four values of a row leave together, and in the
 // QKV projection, whose weight rows are stored with the rotary pairs (i, i + dh/2) of a head side by side, they are two
 // rotary pairs.
-// grid (M/128 tiles, split, N tiles of the token rows), cluster (1, split, 1); block 128.  Warp 0 lane 0 feeds TMA, warp 1
-// lane 0 issues MMAs, all four warps read the accumulator back (warp w owns TMEM lanes 32w..32w+31).
+// grid (M/128 tiles, split, N tiles of the token rows), cluster (1, split, 1); block 128.  Warp 0 feeds TMA, warp 1
+// issues MMAs (one elected lane each), all four warps read the accumulator back (warp w owns TMEM lanes 32w..32w+31).
 // SIDE: the launch has side rows (side_bytes(N, split) > 0); a separate instantiation, because the
 // mere presence of that path costs the few-row launches 0.4 us each (measured).
 template <int MODE, bool SIDE>

@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const Gemm g, const Ep
         if (++st == ST) { st = 0; ++round; }
       }
     }
-    // the MMA thread's last arrivals (of the other CTA of a pair) land before this CTA leaves
+    // the last arrivals of the MMAs (the first CTA's, for both CTAs of a pair) land before this CTA leaves
     for (int i = 0; CG == 2 && i < ST && !failed; ++i) {
       const int uses = round + (i < st ? 1 : 0);
       if (uses > 0 && !wait(empty + i, (uses - 1) & 1)) failed = true;
