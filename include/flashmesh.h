@@ -357,6 +357,21 @@ int fm_profile_end(fm_ctx* ctx, fm_profile* out /*HOST*/);
 int fm_attention_layout(const fm_ctx* ctx, int32_t level, int32_t* chunk_slots, int32_t* chunks_per_group,
                         int32_t* max_groups);
 
+/* The form in which a projection of the model runs on `rows` rows of a level (no counterpart in the paper; for reports and
+ * tests): FM_FORM_* for an FM_PROJ_* of the backbone, decided as the library does on a device of 148 SMs without the
+ * environment switches.  (The QKV projection of a layer whose inputs the draft heads read, the last one of an up-stack or of the
+ * face stack, takes the split-K form where the others are tiled, in decode passes.)  HOST only, needs no device.  Negative: error. */
+#define FM_PROJ_QKV 0
+#define FM_PROJ_OUT 1
+#define FM_PROJ_FFN1 2
+#define FM_PROJ_FFN2 3
+#define FM_PROJ_LOGITS 4
+#define FM_FORM_FEW_ROWS 0
+#define FM_FORM_SPLIT_K 1
+#define FM_FORM_TILED 2
+#define FM_FORM_TILED_PAIRS 3
+int fm_projection_form(const fm_config* cfg, int32_t projection, int32_t rows);
+
 /* Number of kernels launched by this context since creation (for launch accounting). */
 int64_t fm_launch_count(const fm_ctx* ctx);
 

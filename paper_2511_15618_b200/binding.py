@@ -128,6 +128,8 @@ def load_library():
     lib.fm_profile_class.argtypes = [vp, i32, i32, C.POINTER(FmProfile)]
     lib.fm_attention_layout.restype = C.c_int
     lib.fm_attention_layout.argtypes = [vp, i32, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
+    lib.fm_projection_form.restype = C.c_int
+    lib.fm_projection_form.argtypes = [C.POINTER(FmConfig), i32, i32]
     lib.fm_launch_count.restype = C.c_int64
     lib.fm_launch_count.argtypes = [vp]
     lib.fm_selftest_wait_timeout.restype = C.c_int
@@ -239,6 +241,18 @@ def fm_attention_layout(ctx, level):
     a, b, c = C.c_int32(), C.c_int32(), C.c_int32()
     rc = load_library().fm_attention_layout(ctx, int(level), C.byref(a), C.byref(b), C.byref(c))
     return rc, (a.value, b.value, c.value)
+
+
+PROJECTIONS = ("qkv", "out", "ffn1", "ffn2", "logits")
+FORMS = ("few_rows", "split_k", "tiled", "tiled_pairs")
+
+
+def fm_projection_form(cfg, projection, rows):
+    """The form (of FORMS) in which a projection (of PROJECTIONS) of the model `cfg` runs on `rows` rows."""
+    rc = load_library().fm_projection_form(C.byref(cfg), PROJECTIONS.index(projection), int(rows))
+    if rc < 0:
+        raise FmError(rc, "fm_projection_form")
+    return FORMS[rc]
 
 
 def fm_launch_count(ctx):

@@ -28,6 +28,7 @@ namespace {
 constexpr int STACK_LEVEL[5] = {0, 1, 2, 1, 0};
 constexpr int PREFILL_ROWS = 8192;      // coordinate rows of a prefill chunk, at most
 constexpr int LAYOUT_SMS = 148;         // SMs of a B200: the workspace, which has no device yet, and the groups cut in it are laid out for them
+constexpr int SPLIT_TARGET = 160, SPLIT_TARGET_DEEP = 296;        // CTAs a split-K launch aims for (see split_cut)
 constexpr int FM_ROPE_SLACK = 64;       // the HF-Blocks of the face level query positions up to 4 faces ahead
 
 struct LayerDev {
@@ -653,17 +654,25 @@ void launch_rows(fm_ctx* c, int mtn, int fj, dim3 grid, int smem, const rg::Args
 //   first FFN matrix     2.9 / 2.2          3.3 / 3.0      4.8 / 3.0      6.0 / 3.4       6.5 / 3.3       3.4 / 3.6
 //   second FFN matrix    2.4 / 3.6          4.7 / 4.3      5.7 / 4.8      5.8 / 5.7       6.3 / 6.2       4.2 / 5.6
 // (second FFN matrix: K = 1536 3.1 / 4.0, K = 2048 4.7 / 4.3, K = 3072 7.0 / 5.0, K = 3584 5.2 / 5.4)
-bool gemm_rows(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, int a_row0, int M, int K, int R, const int* n_active, int mode,
-               const tc::Epi& e, int parts, int stacked, int z_rows, int z_w_rows) {
-  if (R > c->rows_max || M < 8) return false;
-  if (parts * R > 16 && (mode == tc::EPI_GELU || (mode == tc::EPI_QKV && K >= 640) || K > 1536)) return false;
+struct RowsCut { int FT, mtn, smem; };       // FT = 0: the form does not apply
+RowsCut rows_cut(const fm_ctx* c, int M, int K, int R, int mode, int parts, int stacked, bool sums) {
+  const RowsCut none{0, 0, 0};
+  if (R > c->rows_max || M < 8) return none;
+  if (parts * R > 16 && (mode == tc::EPI_GELU || (mode == tc::EPI_QKV && K >= 640) || K > 1536)) return none;
   int FT = K > 1536 ? 16 : 8;                              // long K: fewer CTAs, each of which reads all operand rows
   while (FT < 32 && (M + FT - 1) / FT * stacked > c->n_sm) FT *= 2;
   const int mtn = (parts * R + 15) / 16, smem = rg::smem_bytes(FT, K, mtn);
   // (weights of more than 64 KB only where an SM gets one CTA: a ring of slabs for larger ones was slower than the
   // other form, 11.4 against 10.7 us per launch on the Large model)
-  if (smem > 140 * 1024 || (smem > 100 * 1024 && (M + FT - 1) / FT * stacked > c->n_sm)) return false;
-  if (e.ssq_out != nullptr && c->dm.d % FT != 0) return false;
+  if (smem > 140 * 1024 || (smem > 100 * 1024 && (M + FT - 1) / FT * stacked > c->n_sm)) return none;
+  if (sums && c->dm.d % FT != 0) return none;
+  return RowsCut{FT, mtn, smem};
+}
+
+bool gemm_rows(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, int a_row0, int M, int K, int R, const int* n_active, int mode,
+               const tc::Epi& e, int parts, int stacked, int z_rows, int z_w_rows) {
+  const auto [FT, mtn, smem] = rows_cut(c, M, K, R, mode, parts, stacked, e.ssq_out != nullptr);
+  if (FT == 0) return false;
   const rg::Args g{W, A, parts * K, M, K, R, parts, w_row0 / tc::BM, a_row0, stacked > 1 ? z_rows : 0, stacked > 1 ? z_w_rows / tc::BM : 0,
                    n_active, c->st.status};
   const dim3 grid((M + FT - 1) / FT, stacked);
@@ -750,10 +759,19 @@ void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_ro
   if (mode == tc::EPI_UP && e.ssq_out != nullptr) c->ssq_n = (c->dm.d / tc::BM) * split;   // tiles within d
 }
 
-// How a launch of the tiled form (fm_prefill.cuh) is cut.  Rows per tile and CTAs per tile (one, or a pair that shares the
-// operand rows): the choice that minimises waves x (slabs x the longer of a slab's copy at 64 B per clock and its MMAs, + about
-// 2000 clocks of start-up and epilogue).  Single CTAs / pairs in whole requests up to the first pass, us: 6994 rows 8105 / 7852,
-// 16 prompts of 73 to 577 rows 7946 / 7654, 73 rows 2104 / 2116 (d = 1024).
+// How a launch of the tiled form (fm_prefill.cuh) is cut: rows per tile and CTAs per tile (one, or a pair that shares the
+// operand rows), by an estimate of its clocks.  A wave of tiles takes, per slab, the longer of its copy (72 bytes per clock) and
+// its MMAs, and then what of the epilogue the next tile's MMAs do not cover; a last wave that is nearly empty takes 0.58 of a full
+// one.  A pair copies less per slab, but takes 1000 clocks more a wave and 630 a launch, and its tiles are coarser.  Fitted to
+// chains of launches with 33 to 8100 rows at d = 256 .. 2048, the shapes of the path and the conditioning's (1921 launches, six or
+// eight cuts each): the cut chosen is 0.9 % slower than the best one on average (1.3 % at d = 1280 and 1536, which are not in the
+// fit), single CTAs throughout 3.5 %, pairs wherever their slabs are shorter 7.7 % and up to 1.7 times the time.  Some of them, us,
+// best single / best pair:
+//               d = 256, 480 rows   d = 512, 320 rows   d = 1024, 73 rows   d = 1024, 2334 rows   d = 1024, 6994 rows   d = 2048, 320 rows
+//   QKV             4.0 / 5.1           4.9 / 5.6           6.0 / 6.5           29.6 / 26.6           69.2 / 67.4           17.8 / 18.0
+//   output proj.    3.5 / 4.1           4.3 / 4.6           5.7 / 5.8           13.4 / 13.4           35.7 / 33.0           11.5 / 11.1
+//   first FFN       4.1 / 5.2           5.5 / 6.3           6.1 / 6.7           40.1 / 33.6           97.7 / 91.4           30.0 / 26.3
+//   second FFN      5.7 / 5.6           8.7 / 8.2          14.3 / 13.2          42.8 / 34.7           92.8 / 87.2           32.9 / 27.5
 struct TiledCut { int NT, cg; double waves; };
 TiledCut tiled_cut(const fm_ctx* c, int M, int K, int R, int parts, int layers) {
   const int tiles_m = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
@@ -762,10 +780,12 @@ TiledCut tiled_cut(const fm_ctx* c, int M, int K, int R, int parts, int layers) 
   for (int cg = 1; cg <= 2; ++cg) {
     if (cg == 2 && tiles_m == 1) continue;
     for (int nt = 32; nt <= 256 / parts; nt *= 2) {
-      const double tiles = (double)((tiles_m + cg - 1) / cg) * ((R + nt - 1) / nt) * layers, waves = ceil(tiles / (c->n_sm / cg));
-      const double copy = (tc::BM * 128 + parts * nt / cg * 128) / 64.0, mma = 2.0 * (parts * nt > 64 ? parts * nt : 64);
-      const double cost = waves * (slabs * (copy > mma ? copy : mma) + 12.0 * parts * nt) + 2000.0;
-      if (best == 0.0 || cost < best) { best = cost; t = TiledCut{nt, cg, waves}; }
+      const double tiles = (double)((tiles_m + cg - 1) / cg) * ((R + nt - 1) / nt) * layers;
+      const double full = floor(tiles / (c->n_sm / cg)), last = tiles / (c->n_sm / cg) - full;
+      const double waves = full == 0.0 ? 1.0 : full + (last > 0.0 ? 0.58 + 0.42 * last : 0.0);
+      const double copy = (tc::BM * 128 + parts * nt / cg * 128) / 72.0, mma = 2.28 * (parts * nt > 64 ? parts * nt : 64);
+      const double cost = waves * (slabs * (copy > mma ? copy : mma) + 18.4 * parts * nt + (cg == 2 ? 1000.0 : 0.0)) + (cg == 2 ? 630.0 : 0.0);
+      if (best == 0.0 || cost < best) { best = cost; t = TiledCut{nt, cg, ceil(waves)}; }
     }
   }
   return t;
@@ -1722,13 +1742,13 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
     const char* rm = getenv("FM_ROWS_MAX");
     c->rows_max = rm != nullptr && atoi(rm) < rg::MAX_ROWS ? atoi(rm) : rg::MAX_ROWS;
     const char* t = getenv("FM_SPLIT_TARGET");
-    c->split_target = t != nullptr && atoi(t) > 0 ? atoi(t) : 160;
+    c->split_target = t != nullptr && atoi(t) > 0 ? atoi(t) : SPLIT_TARGET;
     int dev = 0, sms = LAYOUT_SMS;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     c->n_sm = sms > 0 ? sms : LAYOUT_SMS;
     c->device = dev;
     const char* tt = getenv("FM_SPLIT_TARGET_DEEP");
-    c->split_target_deep = tt != nullptr && atoi(tt) > 0 ? atoi(tt) : 296;
+    c->split_target_deep = tt != nullptr && atoi(tt) > 0 ? atoi(tt) : SPLIT_TARGET_DEEP;
     const char* nf = getenv("FM_NO_FUSE");
     // (the upsampling epilogue lists at most 128 carried rows per slot: one per sequence)
     c->fuse_hourglass = c->dm.d % tc::BM == 0 && c->dm.max_batch <= 128 && !(nf != nullptr && nf[0] == '1');
@@ -2121,6 +2141,20 @@ int fm_attention_layout(const fm_ctx* c, int32_t level, int32_t* chunk_slots, in
   if (chunks_per_group != nullptr) *chunks_per_group = c->attn_G[level];
   if (max_groups != nullptr) *max_groups = c->attn_max_groups[level];
   return FM_OK;
+}
+
+int fm_projection_form(const fm_config* cfg, int32_t projection, int32_t rows) {
+  if (check_config(cfg) != FM_OK || projection < FM_PROJ_QKV || projection > FM_PROJ_LOGITS || rows < 1) return FM_ERR_INVALID_ARG;
+  fm_ctx c{};
+  c.dm = make_dims(*cfg);
+  c.n_sm = LAYOUT_SMS; c.rows_max = rg::MAX_ROWS; c.split_target = SPLIT_TARGET; c.split_target_deep = SPLIT_TARGET_DEEP;
+  const Dims& dm = c.dm;
+  const int hd = dm.H * dm.dh, shape[5][3] = {{hd + 2 * dm.Hkv * dm.dh, dm.d, tc::EPI_QKV}, {dm.d, hd, tc::EPI_RESID}, {dm.dff, dm.d, tc::EPI_GELU},
+                                              {dm.d, dm.dff, tc::EPI_RESID}, {dm.V, dm.d, tc::EPI_F32}};
+  const auto [M, K, mode] = shape[projection];
+  if (rows_cut(&c, M, K, rows, mode, 2, 1, mode == tc::EPI_RESID).FT > 0) return FM_FORM_FEW_ROWS;
+  if (!tiled_is_faster(&c, M, K, rows, mode == tc::EPI_F32, mode == tc::EPI_RESID)) return FM_FORM_SPLIT_K;
+  return tiled_cut(&c, M, K, rows, 2, 1).cg == 1 ? FM_FORM_TILED : FM_FORM_TILED_PAIRS;
 }
 
 int64_t fm_launch_count(const fm_ctx* c) { return c ? c->launches : 0; }
