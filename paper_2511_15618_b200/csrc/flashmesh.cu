@@ -772,7 +772,7 @@ void gemm_split(fm_ctx* c, const bf16* W, int w_row0, const bf16* A, size_t a_ro
 //   output proj.    3.5 / 4.1           4.3 / 4.6           5.7 / 5.8           13.4 / 13.4           35.7 / 33.0           11.5 / 11.1
 //   first FFN       4.1 / 5.2           5.5 / 6.3           6.1 / 6.7           40.1 / 33.6           97.7 / 91.4           30.0 / 26.3
 //   second FFN      5.7 / 5.6           8.7 / 8.2          14.3 / 13.2          42.8 / 34.7           92.8 / 87.2           32.9 / 27.5
-struct TiledCut { int NT, cg; double waves; };
+struct TiledCut { int NT, cg; double clocks; };
 TiledCut tiled_cut(const fm_ctx* c, int M, int K, int R, int parts, int layers) {
   const int tiles_m = (M + tc::BM - 1) / tc::BM, slabs = K / tc::BK;
   TiledCut t{32, 1, 0.0};
@@ -785,7 +785,7 @@ TiledCut tiled_cut(const fm_ctx* c, int M, int K, int R, int parts, int layers) 
       const double waves = full == 0.0 ? 1.0 : full + (last > 0.0 ? 0.58 + 0.42 * last : 0.0);
       const double copy = (tc::BM * 128 + parts * nt / cg * 128) / 72.0, mma = 2.28 * (parts * nt > 64 ? parts * nt : 64);
       const double cost = waves * (slabs * (copy > mma ? copy : mma) + 18.4 * parts * nt + (cg == 2 ? 1000.0 : 0.0)) + (cg == 2 ? 630.0 : 0.0);
-      if (best == 0.0 || cost < best) { best = cost; t = TiledCut{nt, cg, ceil(waves)}; }
+      if (best == 0.0 || cost < best) { best = cost; t = TiledCut{nt, cg, cost}; }
     }
   }
   return t;
@@ -824,37 +824,34 @@ void pf_gemm(fm_ctx* c, int mode, const bf16* W, const bf16* A, size_t a_rows_al
 }
 
 // Whether a projection of 64 rows or more goes to the tiled form, whose CTAs hold all of K and need no exchange, or to the
-// split-K form (below 64 rows the pass of the Large model and requests on Small were slower with the tiled form).  A
-// tiled launch is bound by one SM's copies: its time grows with the slabs of K and the waves of tiles.  A split launch
-// has its slabs divided by the split, but more CTAs to start and, with a small split, more of the epilogue per thread.
-// The estimates (us) are fitted to chains of launches with 64 to 480 rows at d = 256, 384, 512, 768, 1024 and 2048, the
-// six shapes of the path each (540 pairs; by them the chosen form is 0.5 % slower than the better one on average; row counts
-// alone, 64 without and 257 or 401 with a residual, were 3.3 % and up to 79 % slower).  Some of them, split / tiled:
-//               d = 256, 73 rows   d = 1024, 73 rows   d = 1024, 256 rows   d = 2048, 64 rows   d = 2048, 320 rows
-//   QKV            6.5 / 6.2          12.3 /  9.8         17.7 / 10.6          15.6 / 14.4         47.2 / 23.3
-//   output proj.   6.2 / 5.4           6.7 /  9.3          9.4 /  9.3           9.0 / 13.7         24.7 / 14.6
-//   first FFN      5.7 / 5.7          10.0 /  9.3         15.5 /  9.9          14.9 / 14.1         60.7 / 34.3
-//   second FFN     5.4 / 8.8           9.2 / 22.7         14.1 / 22.8          14.1 / 40.8         61.5 / 41.9
-//   logits         5.4 / 3.6           6.1 /  7.0         12.6 /  7.2           6.5 / 11.6         12.5 / 11.8
-// In a forward the tiled form of a projection with a residual has to win by 3 us: its CTAs (200 KB) take the room in which the
-// weights of the launch behind it would arrive.  Prefills and passes at 18 sizes, us with that margin / without / by row counts
-// alone: d = 640, 1522 rows 1458 / 1486 / 1459; d = 768, 8 x 271 rows 4325 / 4426 / 4327; d = 1024, 901 rows 3228 / 3288 / 3269,
-// 8 sequences of 181 to 541 rows 5812 / 5897 / 5868; d = 2048, 2701 rows 13 914 / 13 813 / 14 320.
-bool tiled_is_faster(const fm_ctx* c, int M, int K, int R, bool plain_store, bool resid) {
-  if (R < 64 || R > 480) return R > 480;                   // (beyond what was measured: every 32 rows read the weights again)
+// split-K form (33 to 63 rows: the split-K form is 1.0 % above the better one on average, and passes of 39 to 57 rows took up to 0.8 %
+// more with a line at 33).  A tiled launch takes its clocks (tiled_cut) and a start.  A split launch has its slabs divided by the
+// split, but more CTAs to start and, with a small split, more of the epilogue per thread; clusters do not fill the SMs, so more than
+// 1.92 CTAs per SM take a second wave.  The estimates (us) are fitted to chains of launches with 64 to 480 rows at d = 256 .. 2048, the
+// seven shapes of the path (915 launches; by them the chosen form is 0.3 % slower than the better one on average; with the constants
+// of the kernels before 1.9 % and up to 77 %; 225 launches at d = 1280 and 1536, not in the fit: 0.4 %).  Some of them, split / tiled:
+//               d = 256, 73 rows   d = 512, 320 rows   d = 1024, 73 rows   d = 1024, 256 rows   d = 2048, 64 rows   d = 2048, 320 rows
+//   QKV            4.2 / 3.7          7.8 / 4.9           8.7 /  6.0         12.1 /  7.6          11.9 / 10.0         35.8 / 17.8
+//   output proj.   3.7 / 3.3          4.8 / 4.3           3.9 /  5.7          6.2 /  5.9           6.9 /  9.0         16.7 / 11.1
+//   first FFN      3.6 / 3.6          7.5 / 5.5           7.1 /  6.1         10.6 /  7.9          11.6 / 10.3         50.5 / 26.3
+//   second FFN     3.2 / 5.4          6.7 / 8.2           6.7 / 13.2         10.2 / 13.0          11.3 / 24.0         44.9 / 27.5
+//   logits         3.3 / 3.2          5.7 / 4.3           4.2 /  5.4          8.7 /  5.5           6.9 /  8.7          9.2 /  8.6
+// Above 480 rows, where only the second FFN matrix of narrow models is faster split, always the tiled form: 0.3 % above the better one.
+// (A margin of 1, 2 or 3 us for projections with a residual, which the kernels before needed, gains nothing any more: prefills of
+// 64 to 3604 rows at d = 256 .. 2048 and passes of 40 to 448 rows are 0.0, 0.1 and 0.2 % slower with it.)
+bool tiled_is_faster(const fm_ctx* c, int M, int K, int R, bool plain_store) {
+  if (R < 64 || R > 480) return R > 480;
   const SplitCut s = split_cut(c, M, K, R, 1);
-  const TiledCut t = tiled_cut(c, M, K, R, 2, 1);
   const double per = (double)s.slabs / s.split, ctas = (double)s.tiles * s.n_tiles * s.split / c->n_sm;
-  const double split = 3.3 + 0.42 * per + 6.4 / s.split + 1.8 * ctas + 0.5 * per * (ceil(ctas / 2) - 1);
-  const double tiled = (plain_store ? 2.6 : 4.6) + s.slabs * t.waves * (0.22 + 0.05 * t.NT / 32);
-  return tiled + (resid ? 3.0 : 0.0) < split;
+  const double split = 2.8 + 0.3 * per + 3.6 / s.split + 0.8 * ctas + 0.7 * per * (ceil(ctas / 1.92) - 1);
+  return (plain_store ? 2.0 : 2.4) + 0.52e-3 * tiled_cut(c, M, K, R, 2, 1).clocks < split;
 }
 
 bool tiled_gemm(fm_ctx* c, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, const int* n_active, int mode, const tc::Epi& e) {
   const bool resid = mode == tc::EPI_RESID;
   if (!resid && mode != tc::EPI_F32 && mode != tc::EPI_GELU && !(mode == tc::EPI_QKV && e.rows != nullptr && e.stash_ring == nullptr)) return false;
   if (mode == tc::EPI_F32 && (e.ldo & 3) != 0) return false; // rows stored in 16-byte pieces
-  if (!tiled_is_faster(c, M, K, R, mode == tc::EPI_F32, resid)) return false;
+  if (!tiled_is_faster(c, M, K, R, mode == tc::EPI_F32)) return false;
   pf::Epi t{};
   t.ssq_in = e.ssq_in; t.ssq_n = e.ssq_n; t.ld_ssq = resid ? e.ld_ssq_out : e.ld_ssq; t.inv_d = e.inv_d_in; t.eps = e.eps;
   t.out = e.out; t.ldo = e.ldo; t.lo_off = e.lo_off;
@@ -2153,7 +2150,7 @@ int fm_projection_form(const fm_config* cfg, int32_t projection, int32_t rows) {
                                               {dm.d, dm.dff, tc::EPI_RESID}, {dm.V, dm.d, tc::EPI_F32}};
   const auto [M, K, mode] = shape[projection];
   if (rows_cut(&c, M, K, rows, mode, 2, 1, mode == tc::EPI_RESID).FT > 0) return FM_FORM_FEW_ROWS;
-  if (!tiled_is_faster(&c, M, K, rows, mode == tc::EPI_F32, mode == tc::EPI_RESID)) return FM_FORM_SPLIT_K;
+  if (!tiled_is_faster(&c, M, K, rows, mode == tc::EPI_F32)) return FM_FORM_SPLIT_K;
   return tiled_cut(&c, M, K, rows, 2, 1).cg == 1 ? FM_FORM_TILED : FM_FORM_TILED_PAIRS;
 }
 

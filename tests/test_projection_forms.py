@@ -57,6 +57,13 @@ def test_single_ctas_or_pairs(d, kv_heads, projection, rows, split, single, pair
         assert times[form] <= 1.1 * min(single, pairs)
 
 
+@pytest.mark.parametrize("d,kv_heads,projection,rows,split,single,pairs", [m for m in MEASURED if m[4] is not None])
+def test_split_k_or_tiled(d, kv_heads, projection, rows, split, single, pairs):
+    from paper_2511_15618_b200 import fm_projection_form
+    times = {"split_k": split, "tiled": single, "tiled_pairs": pairs}
+    assert times[fm_projection_form(_config(d, kv_heads), projection, rows)] <= 1.1 * min(times.values())
+
+
 def test_refuses_what_is_no_projection():
     from paper_2511_15618_b200 import FmError, fm_projection_form, load_library
     import ctypes as C
