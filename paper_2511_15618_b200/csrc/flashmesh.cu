@@ -644,23 +644,29 @@ void launch_rows(fm_ctx* c, int mtn, int fj, dim3 grid, int smem, const rg::Args
   }
 }
 // The few-row form (fm_gemm_rows.cuh), with as few features per CTA as give every SM at most one CTA.  For
-// up to 16 rows whose weights per CTA fit beside a neighbour's; returns false where it does not apply.
+// up to 16 rows whose weights per CTA fit beside a neighbour's.
 // Above 16 MMA rows (8 rows of two terms) it has two row tiles, and its time grows with the features per CTA and with K, while
-// the split-K form takes as long as for one row: there it keeps the output projections and the narrow QKV only.  From one
-// launch's dependency wait to the next one's, us, few-row / split-K:
-//                      d = 256, 10 rows   512, 10 rows   640, 10 rows   1024, 10 rows   1024, 16 rows   1024, 4 rows
-//   QKV                  3.4 / 3.6          3.3 / 3.5      3.5 / 3.3      5.6 / 3.6       5.9 / 3.2       3.3 / 3.3
-//   output projection    2.0 / 3.0          2.4 / 3.7      2.7 / 3.7      2.9 / 3.7       3.4 / 4.0       2.7 / 3.8
-//   first FFN matrix     2.9 / 2.2          3.3 / 3.0      4.8 / 3.0      6.0 / 3.4       6.5 / 3.3       3.4 / 3.6
-//   second FFN matrix    2.4 / 3.6          4.7 / 4.3      5.7 / 4.8      5.8 / 5.7       6.3 / 6.2       4.2 / 5.6
-// (second FFN matrix: K = 1536 3.1 / 4.0, K = 2048 4.7 / 4.3, K = 3072 7.0 / 5.0, K = 3584 5.2 / 5.4)
+// the split-K form takes as long as for one row.  There it keeps what has eight features per CTA (output projections up to d = 1184, second
+// FFN and shortening matrices up to K = 1536, QKV with few key/value heads, upsampling of narrow models), any width below K = 640, and
+// neither the first FFN matrix nor the logits (of two terms: the draft heads' have one).  Chains of launches, us, few-row / split-K:
+//                      d = 256, 10 rows   512, 10 rows   768, 10 rows   1024, 10 rows   1024, 16 rows   1024, 4 rows
+//   QKV                  2.6 / 3.1          3.2 / 3.2      3.7 / 3.6      5.3 / 4.5       5.7 / 4.6       3.3 / 4.1
+//   ..., one kv head     2.5 / 3.1          2.7 / 3.1      3.2 / 3.3      3.5 / 3.3       3.8 / 3.5       2.6 / 3.0
+//   output projection    1.6 / 2.4          1.9 / 2.5      2.0 / 2.8      2.9 / 3.1       3.3 / 3.2       2.1 / 3.0
+//   first FFN matrix     2.6 / 2.3          3.0 / 2.6      4.4 / 3.0      5.3 / 4.0       5.8 / 4.2       3.3 / 4.0
+//   second FFN matrix    2.2 / 2.6          3.5 / 3.4      5.1 / 4.5      6.7 / 6.0       7.1 / 6.2       4.7 / 6.0
+//   logits               2.6 / 2.5          2.7 / 2.6      2.9 / 2.7      3.3 / 2.8       3.7 / 3.0       2.7 / 2.7
+//   upsampling           2.1 / 2.5          2.6 / 2.6      3.1 / 3.0      3.7 / 3.2       3.9 / 3.3       2.7 / 3.1
+// Where a chain shows no difference a pass does: QKV with one kv head as split-K launches (10 rows, us) 625 instead of 608 at d = 640,
+// 670 / 661 at d = 896, 714 / 703 at d = 1024; QKV of d = 512 (16 features) 323 / 314; output projections of d = 1280 (16 features)
+// as few-row launches 474 / 470.
 struct RowsCut { int FT, mtn, smem; };       // FT = 0: the form does not apply
 RowsCut rows_cut(const fm_ctx* c, int M, int K, int R, int mode, int parts, int stacked, bool sums) {
   const RowsCut none{0, 0, 0};
   if (R > c->rows_max || M < 8) return none;
-  if (parts * R > 16 && (mode == tc::EPI_GELU || (mode == tc::EPI_QKV && K >= 640) || K > 1536)) return none;
   int FT = K > 1536 ? 16 : 8;                              // long K: fewer CTAs, each of which reads all operand rows
   while (FT < 32 && (M + FT - 1) / FT * stacked > c->n_sm) FT *= 2;
+  if (parts * R > 16 && (mode == tc::EPI_GELU || mode == tc::EPI_F32 || (FT > 8 && K >= 640))) return none;
   const int mtn = (parts * R + 15) / 16, smem = rg::smem_bytes(FT, K, mtn);
   // (weights of more than 64 KB only where an SM gets one CTA: a ring of slabs for larger ones was slower than the
   // other form, 11.4 against 10.7 us per launch on the Large model)

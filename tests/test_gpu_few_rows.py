@@ -1,5 +1,5 @@
 """The few-row projections against the oracle where they change form: one and two MMA row tiles (up to 8 and 16
-rows with two terms each), with more than 8 rows only the narrow ones, the first row count of the split-K form for all, 16 and 32 features per CTA (long K, many
+rows with two terms each), with more than 8 rows only those with 8 features per CTA or short K, the first row count of the split-K form for all, 16 and 32 features per CTA (long K, many
 features), weights too large for a CTA, a last CTA with few features."""
 import pytest
 
@@ -17,8 +17,10 @@ pytestmark = pytest.mark.gpu
     (3, 1, {"d_ff": 4096}),                                           # 16 features per CTA, 128 KB of weights; 32 features
     (9, 1, {"d_ff": 4096}),
     (9, 1, {"d_ff": 8192, "n_bins": 133}),                            # weights too large: split K; ragged outputs
-    (7, 1, {"d_model": 640, "n_heads": 10, "n_kv_heads": 10, "weight_std": 0.04}),          # 8 rows: all of them; 9: the output projection alone
+    (7, 1, {"d_model": 640, "n_heads": 10, "n_kv_heads": 10, "weight_std": 0.04}),          # 8 rows: all of them; 9: the output projection and the second FFN matrix
     (8, 1, {"d_model": 640, "n_heads": 10, "n_kv_heads": 10, "weight_std": 0.04}),
+    (8, 1, {"d_model": 640, "n_heads": 10, "n_kv_heads": 1, "weight_std": 0.04}),           # 9 rows: QKV with 8 features per CTA
+    (15, 1, {"d_model": 640, "n_heads": 10, "n_kv_heads": 1, "weight_std": 0.04}),          # 16
 ])
 def test_few_rows_lockstep(D, batch, kw):
     from oracle.lockstep import run_lockstep

@@ -40,6 +40,26 @@ MEASURED = [
     (2048, 0, "ffn2", 1100, 116.5, 58.7, 57.9),
 ]
 
+# 9 to 16 rows; few-row form, split-K (whole passes where a chain of one projection shows no difference)
+MEASURED_FEW = [
+    (640, 1, "qkv", 10, 608, 625),
+    (768, 2, "qkv", 16, 662, 675),
+    (896, 1, "qkv", 10, 661, 670),
+    (1024, 1, "qkv", 10, 703, 714),
+    (512, 0, "qkv", 10, 314, 323),
+    (1280, 0, "out", 10, 474, 470),
+    (1024, 0, "qkv", 10, 5.3, 4.5),
+    (1024, 0, "out", 10, 2.9, 3.1),
+    (1024, 0, "ffn1", 10, 5.3, 4.0),
+    (1024, 0, "ffn2", 10, 6.7, 6.0),
+    (1024, 0, "logits", 10, 3.3, 2.8),
+    (256, 0, "qkv", 12, 2.7, 3.2),
+    (256, 0, "ffn1", 12, 2.6, 2.3),
+    (256, 0, "ffn2", 12, 2.2, 2.7),
+    (384, 0, "ffn2", 16, 2.8, 3.0),
+    (512, 0, "ffn2", 16, 3.8, 3.4),
+]
+
 
 def _config(d, kv_heads=0):
     from paper_2511_15618_b200 import binding as B
@@ -62,6 +82,12 @@ def test_split_k_or_tiled(d, kv_heads, projection, rows, split, single, pairs):
     from paper_2511_15618_b200 import fm_projection_form
     times = {"split_k": split, "tiled": single, "tiled_pairs": pairs}
     assert times[fm_projection_form(_config(d, kv_heads), projection, rows)] <= 1.1 * min(times.values())
+
+
+@pytest.mark.parametrize("d,kv_heads,projection,rows,few,split", MEASURED_FEW)
+def test_few_rows_or_split_k(d, kv_heads, projection, rows, few, split):
+    from paper_2511_15618_b200 import fm_projection_form
+    assert fm_projection_form(_config(d, kv_heads), projection, rows) == ("few_rows" if few < split else "split_k")
 
 
 def test_refuses_what_is_no_projection():
