@@ -630,6 +630,9 @@ tc::Epi epi_plain(void* out, int ldo) {
   return e;
 }
 
+// Modes that rows_cut gives two MMA row tiles (more than 8 rows of two terms); the others have one.
+constexpr bool rows_two_tiles(int mode) { return mode == tc::EPI_RESID || mode == tc::EPI_RESID_CAT || mode == tc::EPI_UP || mode == tc::EPI_QKV; }
+
 template <int MODE>
 void launch_rows(fm_ctx* c, int mtn, int fj, dim3 grid, int smem, const rg::Args& g, const tc::Epi& e) {
   const dim3 one(1, 1, 1);
@@ -637,10 +640,12 @@ void launch_rows(fm_ctx* c, int mtn, int fj, dim3 grid, int smem, const rg::Args
     if (fj == 1) launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 1, 1>, grid, rg::THREADS, smem, g, e);
     else if (fj == 2) launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 1, 2>, grid, rg::THREADS, smem, g, e);
     else launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 1, 4>, grid, rg::THREADS, smem, g, e);
-  } else {
+  } else if constexpr (rows_two_tiles(MODE)) {
     if (fj == 1) launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 2, 1>, grid, rg::THREADS, smem, g, e);
     else if (fj == 2) launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 2, 2>, grid, rg::THREADS, smem, g, e);
     else launch_pdl(c, one, rg::gemm_rows_kernel<MODE, 2, 4>, grid, rg::THREADS, smem, g, e);
+  } else {
+    c->launch_error = FM_ERR_UNSUPPORTED;
   }
 }
 // The few-row form (fm_gemm_rows.cuh), with as few features per CTA as give every SM at most one CTA.  For
@@ -666,7 +671,7 @@ RowsCut rows_cut(const fm_ctx* c, int M, int K, int R, int mode, int parts, int 
   if (R > c->rows_max || M < 8) return none;
   int FT = K > 1536 ? 16 : 8;                              // long K: fewer CTAs, each of which reads all operand rows
   while (FT < 32 && (M + FT - 1) / FT * stacked > c->n_sm) FT *= 2;
-  if (parts * R > 16 && (mode == tc::EPI_GELU || mode == tc::EPI_F32 || (FT > 8 && K >= 640))) return none;
+  if (parts * R > 16 && (!rows_two_tiles(mode) || (FT > 8 && K >= 640))) return none;
   const int mtn = (parts * R + 15) / 16, smem = rg::smem_bytes(FT, K, mtn);
   // (weights of more than 64 KB only where an SM gets one CTA: a ring of slabs for larger ones was slower than the
   // other form, 11.4 against 10.7 us per launch on the Large model)
@@ -701,7 +706,9 @@ cudaError_t allow_rows_smem() {
   cudaError_t r = cudaSuccess;
   auto set = [&](const void* k) { if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most); };
   set((const void*)rg::gemm_rows_kernel<MODE, 1, 1>); set((const void*)rg::gemm_rows_kernel<MODE, 1, 2>); set((const void*)rg::gemm_rows_kernel<MODE, 1, 4>);
-  set((const void*)rg::gemm_rows_kernel<MODE, 2, 1>); set((const void*)rg::gemm_rows_kernel<MODE, 2, 2>); set((const void*)rg::gemm_rows_kernel<MODE, 2, 4>);
+  if constexpr (rows_two_tiles(MODE)) {
+    set((const void*)rg::gemm_rows_kernel<MODE, 2, 1>); set((const void*)rg::gemm_rows_kernel<MODE, 2, 2>); set((const void*)rg::gemm_rows_kernel<MODE, 2, 4>);
+  }
   return r;
 }
 
@@ -856,7 +863,6 @@ bool tiled_is_faster(const fm_ctx* c, int M, int K, int R, bool plain_store) {
 bool tiled_gemm(fm_ctx* c, const bf16* W, const bf16* A, size_t a_rows_alloc, int M, int K, int R, const int* n_active, int mode, const tc::Epi& e) {
   const bool resid = mode == tc::EPI_RESID;
   if (!resid && mode != tc::EPI_F32 && mode != tc::EPI_GELU && !(mode == tc::EPI_QKV && e.rows != nullptr && e.stash_ring == nullptr)) return false;
-  if (mode == tc::EPI_F32 && (e.ldo & 3) != 0) return false; // rows stored in 16-byte pieces
   if (!tiled_is_faster(c, M, K, R, mode == tc::EPI_F32)) return false;
   pf::Epi t{};
   t.ssq_in = e.ssq_in; t.ssq_n = e.ssq_n; t.ld_ssq = resid ? e.ld_ssq_out : e.ld_ssq; t.inv_d = e.inv_d_in; t.eps = e.eps;

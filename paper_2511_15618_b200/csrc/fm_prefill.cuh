@@ -60,7 +60,7 @@ struct Gemm {
 };
 struct Epi {
   const float* ssq_in; int ssq_n, ld_ssq; float inv_d, eps;     // RMSNorm scale of the operand rows (null: none)
-  void* out; int ldo, lo_off;                                   // PF_F32: fp32, PF_GELU: [hi | lo] bf16
+  void* out; int ldo, lo_off;                                   // PF_F32: fp32 (rows a multiple of 4 apart), PF_GELU: [hi | lo] bf16
   float* x; int ldx, add; const float* gain; bf16* a_out; int lda; float* ssq_out;      // PF_RESID
   Dims dm; const Row* rows; int level; const float2* rope; float qscale;                // PF_QKV
   bf16 *q, *kbuf, *vbuf, *Kc, *Vc;                              // keys and values: into the cache, or (Kc null) into kbuf / vbuf
