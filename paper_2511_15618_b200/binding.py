@@ -429,7 +429,7 @@ class FlashMesh:
         B, D = self.batch, self.D
         cand = self._out("cand", (B, D + 1), t.int32, reuse)
         dl = self._out("dl", (B, D, self.V), t.float32, reuse) if want_logits else None
-        dm = self._empty((B, max(D, 1)), t.float32)[:, :D].contiguous() if want_logits else None
+        dm = self._out("dm", (B, D), t.float32, reuse) if want_logits else None
         self._before()
         self._check(fm_draft(self.ctx, cand.data_ptr(), dl.data_ptr() if dl is not None else None,
                              dm.data_ptr() if dm is not None and D > 0 else None), "fm_draft")
