@@ -68,12 +68,16 @@ def rank_sequences(rank, batch_per_rank):
 NCU_TRAFFIC = {"medium": {"bytes_per_launch": 6.38e6, "summary": "profiles/gemm_and_attention_dram_traffic_medium.md (mean of a layer's four projections)"}}
 
 
-FEW_ROWS = 16              # rows up to which a projection takes the few-row form (rg::MAX_ROWS)
+FORM_KERNELS = {"few_rows": "rg::gemm_rows_kernel", "split_k": "tc::gemm_tc_kernel", "tiled": "pf::gemm_kernel", "tiled_pairs": "pf::gemm_kernel"}
 
 
 def gemm_kernels(cfg):
-    """The kernels that the projections of a verify pass run through: every level has at most batch * (D + 1) rows."""
-    return "rg::gemm_rows_kernel" if cfg.batch * (cfg.draft_len + 1) <= FEW_ROWS else "rg::gemm_rows_kernel, tc::gemm_tc_kernel, pf::gemm_kernel"
+    """The kernels that the projections of a verify pass run through: every level's rows, as the library decides (a verify pass has
+    batch * ceil((D + 1) / 3) rows at the vertex and batch * ceil((D + 1) / 9) at the face level)."""
+    from paper_2511_15618_b200.binding import PROJECTIONS, fm_projection_form, make_config
+    c, r1 = make_config(cfg), cfg.draft_len + 1
+    forms = {fm_projection_form(c, p, cfg.batch * -(-r1 // ratio)) for ratio in (1, 3, 9) for p in PROJECTIONS if p != "logits" or ratio == 1}
+    return ", ".join(dict.fromkeys(FORM_KERNELS[f] for f in FORM_KERNELS if f in forms))
 
 
 def attention_entry(cfg, ms, launches):
@@ -296,7 +300,7 @@ def run_ours(args):
                 "what": "fm_step_host once per pass with the host in the loop: candidates from pinned host memory "
                         "in, draft + verify + accept, accepted tokens copied back, per pass"},
         "gpu_launches": launches,
-        "roofline": {"bound": "hbm", "kernel": gemm_kernels(cfg) + (", tc::gemm_tc_kernel (the wide ones of more than 8 rows)" if 8 < cfg.batch * (cfg.draft_len + 1) <= FEW_ROWS else "") + " (all GEMM launches of one verify pass, timed alone as a graph)",
+        "roofline": {"bound": "hbm", "kernel": gemm_kernels(cfg) + " (all GEMM launches of one verify pass, timed alone as a graph)",
                      "achieved": gemm_gbs, "peak": peak, "unit": "GB/s", "frac": gemm_gbs / peak,
                      "peak_kind": peak_kind + " copy bandwidth (burst figure: the kernel is timed alone)",
                      "traffic": NCU_TRAFFIC.get(args.workload, {}).get("bytes_per_launch"),

@@ -1,20 +1,17 @@
 """What the benchmark line calls its kernels."""
-import os
-import re
-
 import bench
 import fm_synth as S
 
-CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_15618_b200", "csrc")
+FEW, SPLIT, TILED = "rg::gemm_rows_kernel", "tc::gemm_tc_kernel", "pf::gemm_kernel"
 
 
 def test_the_projections_are_named_by_the_form_they_take():
-    text = open(os.path.join(CSRC, "fm_gemm_rows.cuh")).read()
-    assert bench.FEW_ROWS == int(re.search(r"MAX_ROWS = (\d+)", text).group(1))
-    for name, kernel in (("tiny", "rg::gemm_rows_kernel"), ("medium", "rg::gemm_rows_kernel")):
-        assert bench.gemm_kernels(S.get_config(name)) == kernel
-    for name in ("batched", "large"):
-        assert "tc::gemm_tc_kernel" in bench.gemm_kernels(S.get_config(name))
+    for name, kernels in (("tiny", [FEW]),                   # 4, 2 and 1 rows
+                          ("small", [FEW, SPLIT]),           # 10, 4 and 2: above 8 rows the first FFN matrix is split
+                          ("medium", [FEW, SPLIT]),
+                          ("batched", [SPLIT, TILED]),       # 160, 64 and 32
+                          ("large", [FEW, SPLIT])):          # 52, 20 and 8
+        assert bench.gemm_kernels(S.get_config(name)) == ", ".join(kernels)
 
 
 def test_merges_do_not_count_as_streaming_launches():
