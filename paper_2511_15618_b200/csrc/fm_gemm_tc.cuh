@@ -537,9 +537,9 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   __syncthreads();                                         // s_inv / row maps are written (long before the MMAs end)
   if (MODE == EPI_QKV && e.stash_ring != nullptr && z == 0) {
     // the rows' residual values, as they enter this layer, go into the carry ring (the draft heads
-    // read them after the pass); this CTA copies column tile_m*128 + tid
-    const int col = tile_m * BM + tid;
-    if (col < e.stash_d)
+    // read them after the pass); this CTA copies column tile_m*128 + tid, and where the matrix has fewer tiles than the rows have
+    // blocks of 128 columns (heads of together less than d) every gridDim.x-th block behind it
+    for (int col = tile_m * BM + tid; col < e.stash_d; col += (int)gridDim.x * BM)
       for (int n = 0; n < ns; ++n)
         if (s_rb[n] >= 0)
           e.stash_ring[((size_t)s_rb[n] * e.stash_rs + s_rp[n] % e.stash_rs) * e.stash_d + col] = __ldcg(e.stash_x + (size_t)(row0 + n) * e.stash_d + col);

@@ -21,6 +21,9 @@ pytestmark = pytest.mark.gpu
     (8, 1, {"d_model": 640, "n_heads": 10, "n_kv_heads": 10, "weight_std": 0.04}),
     (8, 1, {"d_model": 640, "n_heads": 10, "n_kv_heads": 1, "weight_std": 0.04}),           # 9 rows: QKV with 8 features per CTA
     (15, 1, {"d_model": 640, "n_heads": 10, "n_kv_heads": 1, "weight_std": 0.04}),          # 16
+    (16, 1, {"d_model": 512, "n_kv_heads": 1, "weight_std": 0.05}),   # 17, QKV with fewer features than the hidden that it keeps for the draft heads
+    (9, 2, {"d_model": 640, "n_kv_heads": 1, "weight_std": 0.04}),    # 20
+    (15, 1, {"d_model": 640, "n_kv_heads": 1, "weight_std": 0.04}),   # 16, few-row form
 ])
 def test_few_rows_lockstep(D, batch, kw):
     from oracle.lockstep import run_lockstep
