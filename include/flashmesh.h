@@ -366,6 +366,7 @@ int fm_attention_layout(const fm_ctx* ctx, int32_t level, int32_t* chunk_slots, 
 #define FM_PROJ_FFN1 2
 #define FM_PROJ_FFN2 3
 #define FM_PROJ_LOGITS 4
+#define FM_PROJ_CONDITIONING 5     /* keys and values of the prefix, all layers in one launch; rows: conditioning vectors of all sequences */
 #define FM_FORM_FEW_ROWS 0
 #define FM_FORM_SPLIT_K 1
 #define FM_FORM_TILED 2

@@ -243,7 +243,7 @@ def fm_attention_layout(ctx, level):
     return rc, (a.value, b.value, c.value)
 
 
-PROJECTIONS = ("qkv", "out", "ffn1", "ffn2", "logits")
+PROJECTIONS = ("qkv", "out", "ffn1", "ffn2", "logits", "conditioning")
 FORMS = ("few_rows", "split_k", "tiled", "tiled_pairs")
 
 

@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <mutex>
 #include <new>
+#include <numeric>
 #include <utility>
 #include <vector>
 
@@ -2153,13 +2154,15 @@ int fm_attention_layout(const fm_ctx* c, int32_t level, int32_t* chunk_slots, in
 }
 
 int fm_projection_form(const fm_config* cfg, int32_t projection, int32_t rows) {
-  if (check_config(cfg) != FM_OK || projection < FM_PROJ_QKV || projection > FM_PROJ_LOGITS || rows < 1) return FM_ERR_INVALID_ARG;
+  if (check_config(cfg) != FM_OK || projection < FM_PROJ_QKV || projection > FM_PROJ_CONDITIONING || rows < 1) return FM_ERR_INVALID_ARG;
   fm_ctx c{};
   c.dm = make_dims(*cfg);
   c.n_sm = LAYOUT_SMS; c.rows_max = rg::MAX_ROWS; c.split_target = SPLIT_TARGET; c.split_target_deep = SPLIT_TARGET_DEEP;
   const Dims& dm = c.dm;
   const int hd = dm.H * dm.dh, shape[5][3] = {{hd + 2 * dm.Hkv * dm.dh, dm.d, tc::EPI_QKV}, {dm.d, hd, tc::EPI_RESID}, {dm.dff, dm.d, tc::EPI_GELU},
                                               {dm.d, dm.dff, tc::EPI_RESID}, {dm.V, dm.d, tc::EPI_F32}};
+  if (projection == FM_PROJ_CONDITIONING)
+    return tiled_cut(&c, 2 * dm.Hkv * dm.dh, dm.d, rows, 1, std::accumulate(cfg->layers, cfg->layers + 5, 0)).cg == 1 ? FM_FORM_TILED : FM_FORM_TILED_PAIRS;
   const auto [M, K, mode] = shape[projection];
   if (rows_cut(&c, M, K, rows, mode, 2, 1, mode == tc::EPI_RESID).FT > 0) return FM_FORM_FEW_ROWS;
   if (!tiled_is_faster(&c, M, K, rows, mode == tc::EPI_F32)) return FM_FORM_SPLIT_K;

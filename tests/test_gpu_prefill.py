@@ -59,14 +59,37 @@ def test_prefill_lockstep_128_query_rows_per_cta_heads_of_128(faces, window, kw)
     test_prefill_lockstep(faces, window, {"n_heads": heads, "n_kv_heads": heads, "head_dim": 128, **kw})
 
 
-# The rows on both sides of each change between the split-K and the tiled form: 64 coordinate rows (projections without a
-# residual), 481 (those with one, at d = 128), 321 (the output projection of d = 1024).
+# The rows on both sides of each change between the split-K and the tiled form: 64 coordinate rows (every projection of d = 128), 481
+# (the second FFN matrix with K = 2048), at d = 1024 161 (the output projection) and 193 (QKV in pairs of CTAs).
 @pytest.mark.parametrize("faces,kw", [
     ((6, 0, 0, 0, 0, 0, 0, 0, 0), {}), ((7,), {}),                    # 63 and 64 rows
     ((52, 1, 0), {}), ((52, 1, 0, 0), {}),                            # 480 and 481
     ((52, 1, 0, 0), {"d_ff": 2048, "weight_std": 0.05}),
     ((33, 2, 0, 0, 0), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),              # 320 and 321
     ((33, 2, 0, 0, 0, 0), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),
+    ((17, 0, 0, 0, 0, 0, 0), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),        # 160 and 161
+    ((17, 0, 0, 0, 0, 0, 0, 0), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),
+    ((21, 0, 0), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),                    # 192 and 193
+    ((21, 0, 0, 0), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),
 ])
 def test_prefill_lockstep_where_projections_change_form(faces, kw):
+    test_prefill_lockstep(faces, (0, 0, 0), kw)
+
+
+# Pairs of CTAs: an even number of 128-feature tiles, an odd one whose last tile is half empty, the conditioning's with an odd one (its second
+# CTA repeats the first one's weights and stores nothing).
+@pytest.mark.parametrize("faces,projections,kw", [
+    ((86,), ("qkv", "out"), {"d_model": 1024, "n_heads": 16, "n_kv_heads": 16, "weight_std": 0.03}),
+    ((29,), ("ffn1", "ffn2"), {"d_model": 1088, "n_heads": 4, "n_kv_heads": 1, "d_ff": 2112, "weight_std": 0.03}),
+    ((13,), ("ffn2",), {"d_model": 1088, "n_heads": 4, "n_kv_heads": 1, "d_ff": 2112, "weight_std": 0.03}),
+    # (so many faces that all 512 conditioning vectors go through one launch)
+    ((110,), ("conditioning",), {"d_model": 1024, "n_heads": 6, "n_kv_heads": 3, "n_prefix": 512, "d_ff": 2048, "weight_std": 0.03}),
+    ((60, 55), ("conditioning",), {"d_model": 1024, "n_heads": 6, "n_kv_heads": 3, "n_prefix": 256, "d_ff": 2048, "weight_std": 0.03}),
+])
+def test_prefill_lockstep_pairs_of_ctas(faces, projections, kw):
+    from paper_2511_15618_b200 import binding as B
+    cfg = B.make_config(S.toy_config(**{"n_heads": 2, "n_kv_heads": 2, "head_dim": 64, "d_ff": 256, "layers": (1, 2, 2, 1, 2), **kw}))
+    for p in projections:
+        rows = len(faces) * cfg.n_prefix if p == "conditioning" else sum(9 * f + 1 for f in faces)
+        assert B.fm_projection_form(cfg, p, rows) == "tiled_pairs"
     test_prefill_lockstep(faces, (0, 0, 0), kw)

@@ -95,5 +95,5 @@ def test_refuses_what_is_no_projection():
     import ctypes as C
     with pytest.raises(FmError):
         fm_projection_form(_config(256), "qkv", 0)
-    assert load_library().fm_projection_form(C.byref(_config(256)), 5, 8) < 0
+    assert load_library().fm_projection_form(C.byref(_config(256)), 6, 8) < 0
     assert load_library().fm_projection_form(None, 0, 8) < 0
