@@ -11,7 +11,7 @@
 // form with K split over a cluster, fm_gemm_tc.cuh, spends 0.8 us on the operand copy, 0.5 us on the
 // round trip through tensor memory and 1 us on the exchange between the CTAs, and hardly more for more rows.)  From one
 // launch's dependency wait to the next one's, d = 1024, 2 rows, here / there: QKV 3.2 / 3.3 us, output projection 2.5 / 3.7, first
-// FFN matrix 3.3 / 3.5, second 4.0 / 5.6; more rows at gemm_rows in flashmesh.cu.
+// FFN matrix 3.3 / 3.5, second 4.0 / 5.6; more rows at rows_cut in flashmesh.cu.
 //
 // The token rows are the MMA's M axis: the hi terms of the R rows, then their lo terms, so 10 rows with two
 // terms take 20 of 32 MMA rows.  Eight features are the N axis.  Within a block of 32 k, lane t of a quad

@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const Args g, const Epi e)
   const bool use_side = SIDE && want_side;
   if (warp == 0) {
     // ---- operand rows of the first stages (their weight slabs are already on their way): one
-    // copy per slab brings the hi and the lo tile; lanes issue them side by side
+    // copy per slab brings the hi and the lo tile
     const int pre = n_slabs < STAGES ? n_slabs : STAGES;
     ptx::grid_dep_wait();
     if (ptx::elect_one())

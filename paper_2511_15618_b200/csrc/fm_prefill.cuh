@@ -35,6 +35,7 @@ struct LayerPtr { const bf16* Wqkv; const float* g1; bf16* K; bf16* V; int level
 // CG = 2: two CTAs of a cluster multiply together (tcgen05 cta_group::2, M = 256).  Each keeps its own 128 features of
 // weights; of the operand rows the first holds the hi and the second the lo tile, so an SM copies 32 instead of
 // 48 KB per slab and its MMAs read a third less shared memory.  The first CTA issues; both CTAs' copies count on its barriers.
+// tiled_cut (flashmesh.cu) says where that is faster: long K or many rows.
 // What a slab (512 MMA clocks) waited for, 6994 rows, d = 1024, K = 4096: one thread per role behind `lane == 0`, whose
 // every descriptor went from general to uniform registers: 970 clocks; whole warps in step with one elected lane: 740.
 // The epilogue runs beside that, and must not take longer than a tile's MMAs (8 200 clocks at K = 1024).  A warp turns
@@ -46,7 +47,7 @@ struct LayerPtr { const bf16* Wqkv; const float* g1; bf16* K; bf16* V; int level
 enum Mode { PF_F32 = 0, PF_GELU = 1, PF_RESID = 2, PF_QKV = 3, PF_PREFIX = 4 };
 
 constexpr int EPI_WARPS = 16, CW = 16;           // epilogue warps; rows a warp takes at a time
-constexpr int THREADS = 128 + 32 * EPI_WARPS;    // weight producer, operand producer, MMA warp, one idle warp, the epilogue
+constexpr int THREADS = 128 + 32 * EPI_WARPS;    // weight producer, operand producer, MMA warp, the rows' scales, the epilogue
 constexpr int MAX_STAGES = 6;
 
 struct Gemm {
