@@ -675,7 +675,7 @@ RowsCut rows_cut(const fm_ctx* c, int M, int K, int R, int mode, int parts, int 
   if (parts * R > 16 && (!rows_two_tiles(mode) || (FT > 8 && K >= 640))) return none;
   const int mtn = (parts * R + 15) / 16, smem = rg::smem_bytes(FT, K, mtn);
   // (weights of more than 64 KB only where an SM gets one CTA: a ring of slabs for larger ones was slower than the
-  // other form, 11.4 against 10.7 us per launch on the Large model)
+  // split-K form of its day, 11.4 against 10.7 us per launch on the Large model)
   if (smem > 140 * 1024 || (smem > 100 * 1024 && (M + FT - 1) / FT * stacked > c->n_sm)) return none;
   if (sums && c->dm.d % FT != 0) return none;
   return RowsCut{FT, mtn, smem};
@@ -1763,7 +1763,7 @@ int fm_create(const fm_config* cfg, const fm_weights* w, void* dev_workspace, si
     // (the upsampling epilogue lists at most 128 carried rows per slot: one per sequence)
     c->fuse_hourglass = c->dm.d % tc::BM == 0 && c->dm.max_batch <= 128 && !(nf != nullptr && nf[0] == '1');
     const char* sc = getenv("FM_STAGE_CAP");
-    c->stage_cap = sc != nullptr ? atoi(sc) : 3;        // (2 / 3 / 4 stages: 9.4 / 8.8 / 9.2 us per launch at batch 16, 11.5 / 10.1 / 10.7 us on Large)
+    c->stage_cap = sc != nullptr ? atoi(sc) : 3;        // (2 / 3 / 4 stages: 6.7 / 6.2 / 6.5 us per launch at batch 16, 9.3 / 8.3 / 8.5 us on Large)
   }
   *out = c;
   return FM_OK;
