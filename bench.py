@@ -10,11 +10,12 @@ and the teacher schedule resident in HBM.  One JSON line is printed by rank 0.
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import os
 import subprocess
 import sys
-import tempfile
+import threading
 import time
 
 import numpy as np
@@ -88,57 +89,55 @@ def attention_entry(cfg, ms, launches):
 
 
 class ClockSampler:
-    Q = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,clocks_event_reasons.hw_slowdown,"
-         "clocks_event_reasons.hw_thermal_slowdown,clocks_event_reasons.sw_thermal_slowdown,"
-         "clocks_event_reasons.sw_power_cap")
+    """SM clock and slowdown reasons of a GPU, read through NVML every few milliseconds (nvidia-smi takes 50 ms a sample, longer than
+    20 timed passes) between begin() and stop().  Reads only."""
+    REASONS = {0x8: "hw_slowdown", 0x40: "hw_thermal_slowdown", 0x20: "sw_thermal_slowdown", 0x4: "sw_power_cap"}
+    SM = 1                                                  # NVML_CLOCK_SM
 
-    def __init__(self, index):
-        self.index, self.proc, self.path, self.skip = index, None, None, 0
+    def __init__(self, uuid, nvml=None, interval=0.003):
+        self.nvml, self.dev, self.interval = nvml, ctypes.c_void_p(), interval
+        self.samples, self.ended, self.thread = [], threading.Event(), None
+        try:
+            if self.nvml is None:
+                self.nvml = ctypes.CDLL("libnvidia-ml.so.1")
+            ok = self.nvml.nvmlInit_v2() == 0 and self.nvml.nvmlDeviceGetHandleByUUID(f"GPU-{uuid}".encode(), ctypes.byref(self.dev)) == 0
+        except (OSError, AttributeError):
+            ok = False
+        if ok:
+            self.thread = threading.Thread(target=self._run, daemon=True)
+
+    def _sample(self):
+        mhz, why = ctypes.c_uint(), ctypes.c_ulonglong()
+        if self.nvml.nvmlDeviceGetClockInfo(self.dev, self.SM, ctypes.byref(mhz)) == 0 and \
+                self.nvml.nvmlDeviceGetCurrentClocksThrottleReasons(self.dev, ctypes.byref(why)) == 0:
+            self.samples.append((mhz.value, why.value))
+
+    def _run(self):
+        while not self.ended.is_set():
+            self._sample()
+            self.ended.wait(self.interval)
 
     def start(self):
-        try:
-            fd, self.path = tempfile.mkstemp(suffix=".csv")
-            os.close(fd)
-            self.proc = subprocess.Popen(["nvidia-smi", f"--query-gpu={self.Q}", "--format=csv,noheader,nounits",
-                                          "-lms", "50", "-i", str(self.index)], stdout=open(self.path, "w"),
-                                         stderr=subprocess.DEVNULL)
-        except Exception:
-            self.proc = None
-            return
-        # the timed region can be shorter than the tool's start-up: wait for its first sample, which does not count
-        limit = time.time() + 5.0
-        while self.skip == 0 and self.proc.poll() is None and time.time() < limit:
-            time.sleep(0.02)
-            self.skip = os.path.getsize(self.path)
+        if self.thread is not None:
+            self.thread.start()
+
+    def begin(self):
+        """What was sampled so far does not count."""
+        self.samples.clear()
 
     def stop(self):
         out = {"sm_mhz": None, "sm_max_mhz": None, "reasons": []}
-        if self.proc is None:
+        if self.thread is None:
             return out
-        self.proc.terminate()
-        try:
-            self.proc.wait(timeout=5)
-        except Exception:
-            self.proc.kill()
-        sm, reasons = [], set()
-        lines = open(self.path)
-        lines.seek(self.skip)
-        for ln in lines:
-            f = [x.strip() for x in ln.split(",")]
-            if len(f) < 9:
-                continue
-            try:
-                sm.append(float(f[1]))
-                out["sm_max_mhz"] = float(f[2])
-            except ValueError:
-                continue
-            for name, v in zip(("hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap"), f[5:9]):
-                if v.lower().startswith("active"):
-                    reasons.add(name)
-        os.unlink(self.path)
-        if sm:
-            out["sm_mhz"] = float(np.median(sm))
-        out["reasons"] = sorted(reasons)
+        self.ended.set()
+        self.thread.join(timeout=5)
+        top = ctypes.c_uint()
+        if self.nvml.nvmlDeviceGetMaxClockInfo(self.dev, self.SM, ctypes.byref(top)) == 0:
+            out["sm_max_mhz"] = float(top.value)
+        seen = list(self.samples)
+        if seen:
+            out["sm_mhz"] = float(np.median([m for m, _ in seen]))
+        out["reasons"] = sorted(name for bit, name in self.REASONS.items() if any(why & bit for _, why in seen))
         return out
 
 
@@ -211,11 +210,12 @@ def run_ours(args):
     if W > 0:
         tok, ln, _ = dev.generate(need_faces, truth=truth_d, keep=keep_d, max_steps=W)
         out = (tok, ln)
-    sampler = ClockSampler(local)
+    sampler = ClockSampler(torch.cuda.get_device_properties(local).uuid)
     sampler.start()
     l0 = dev.launch_count()
     sync_all()
     torch.cuda.profiler.start()           # lets `ncu --profile-from-start off` see only the timed passes
+    sampler.begin()
     tok, ln, st = dev.generate(need_faces, truth=truth_d, keep=keep_d, max_steps=K, out=out)
     sync_all()
     torch.cuda.profiler.stop()
